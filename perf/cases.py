@@ -600,7 +600,7 @@ def exact(case, seed):
     if path == "batch":
         out = []
         for p in _batch_list(case, seed):
-            if seconds(p["nx"], Q[case["kind"]] * p["ny"], 1, 2) > 4:
+            if seconds(p["nx"], Q[case["kind"]] * p["ny"], 1, 2) > 3:
                 out.append({m: None for m in ("sigma", "sigma_halko", "U", "V")})
                 continue
             ex = _Exact(case, seed, p["nx"], p["ny"])
