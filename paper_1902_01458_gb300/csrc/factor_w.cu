@@ -12,17 +12,13 @@
 // M = Q^T S^{-1} Q^T with (Q x)_j = x_{p_j}, so S^{-1}[j, p_m] = M[p_j, m].
 //
 // Levels, for every slab of W = 128 columns [c0, c1):
-//   inner, per panel K of 16 columns:
-//     panel  : one CTA per problem holds the tall panel M[:, K] in registers
-//              (one row per thread), first applies the previous panel's
-//              transformation to it, then the 16 eliminations, recording the
-//              pivot rows P (gjw_panel_kernel);
-//     update : the transformations of K applied to the rest of the slab but
-//              the next panel, M[r, m] += M[r, K] * M_old[P, m] for rows r not
-//              in P and M[P, m] = M[P, K] * M_old[P, m] (the pivot rows take
-//              T^{-1} B itself: adding (T^{-1} - I) B to B would cancel when
-//              T^{-1} is small), in FP32 on the CUDA cores, beside the next
-//              panel on a third stream (gjw_slab_update_kernel);
+//   inner: one cluster of CTAs per problem holds the slab on chip and runs
+//     its panels K of 16 columns (gjw_slab_kernel): the 16 eliminations,
+//     recording the pivot rows P, then the transformations of K applied to
+//     the rest of the slab, M[r, m] += M[r, K] * M_old[P, m] for rows r not
+//     in P and M[P, m] = M[P, K] * M_old[P, m] (the pivot rows take T^{-1} B
+//     itself: adding (T^{-1} - I) B to B would cancel when T^{-1} is small),
+//     in FP32 on the CUDA cores;
 //   outer:
 //     gather : B = M[P_slab, outside the slab] (the pivot rows, saved before
 //              they change);
@@ -44,314 +40,559 @@ namespace {
 
 constexpr int GW_W = 128;   // slab width (rank of the outer update)
 constexpr int GW_NB = 16;   // panel width (rank of the slab update)
-constexpr int GW_PANEL_MAX = 768;  // rows a panel CTA holds (two per thread)
+constexpr int GW_MAX = 768;  // largest block of the wide path
 
-// ------------------------------------------------------------------- panel
-// Eliminates columns K = [k0, k0 + nbk) of every row of M (problem =
-// blockIdx.x), one row per thread, the row's 16 entries of K held in
-// registers.  When kp0 >= 0 the previous panel [kp0, kp0 + 16) of the same
-// slab was factored last and its transformation has reached every slab
-// column except its own and K (gjw_slab_update_kernel); the kernel applies
-// it to K first:
-//   x += M[r, Kp] B   (rows not pivoted in Kp),   x = M[r, Kp] B   (its pivot rows),
-// B = the rows of Kp's pivots at K before this step.  Then per column j:
-// each warp finds its best eligible row (largest |.|^2, lowest row on ties)
-// and the winning lane publishes that whole row in shared memory; after one
-// block barrier every warp reduces the per-warp candidates itself, reads the
-// pivot row from shared memory and eliminates (candidates double-buffered
-// by step parity).  Outputs: the columns K of M, rowpiv[r] = pivot column of
-// the rows pivoted here, pivslot[k0 + j] = pivot row of column k0 + j.
-constexpr int GW_PANEL_THREADS = GW_PANEL_MAX;  // one row per thread up to 768 rows
+// -------------------------------------------------------------------- slab
+// Factors one slab: eliminates the columns [c0, c1) (at most 128) of every row
+// of M, the slab resident on chip for all of its steps.  A cluster of CL CTAs
+// owns one problem; CTA rank r holds the rows r, r + CL, r + 2 CL, ... of the
+// slab in shared memory (cyclic, so the pivot rows of a panel, which cluster
+// around the diagonal, are spread over the CTAs that send them).  Per panel K
+// of 16 columns:
+//   steps  : the panel warps hold the panel in registers, LPR lanes per row.
+//            Step j: the CTA's best eligible row of column j
+//            (largest |.|^2 to 18 bits, lowest warp and lane among equals) by
+//            warp reductions and a barrier of the panel warps, which send it,
+//            128 bytes, to every CTA of the cluster (st.async into the
+//            sender's candidate slot, completing on the receiver's mbarrier,
+//            so data and signal travel together; a CTA without an eligible
+//            row sends a zero pivot); every warp then reduces the CL
+//            candidates itself (lowest CTA among equals) and eliminates:
+//            x += m (pivot row), x_j = m with m = -x_j / pivot, and x = 0,
+//            m = 1 / pivot in the pivot row;
+//   B      : the CTAs that hold the panel's 16 pivot rows send them (the
+//            slab's columns, before this panel's step) to every CTA, the other
+//            warps' work as soon as a pivot is known;
+//   update : M[r, m] += M[r, K] B[:, m] for the slab's other columns m,
+//            M[r, m] = M[r, K] B[:, m] for the pivot rows (T^{-1} B itself), in
+//            exact FP32 on the CUDA cores.  The panel warps take the next
+//            panel's 16 columns as they load them; the rest is the other
+//            warps' work while the panel warps run the next panel's steps.
+// A problem that fits one CTA (SOLO) needs no exchange.
+// Candidate slots are double-buffered by step parity: a CTA sends for step
+// j + 2 only after it has received every CTA's candidate of step j + 1, each
+// sent after a barrier that follows its panel warps' last reads of step j.  B
+// is double-buffered by panel parity: a CTA sends for panel p + 2 only after
+// every CTA took part in panel p + 2, which each begins after its update of
+// panel p is complete.
+//
+// Bound: the chain of 128 dependent steps (reduce, send, receive, reduce,
+// eliminate).  768 rows in clusters of eight CTAs: 108 us a slab of 128 columns,
+// of which 58 in the local part of the steps, 22 in the exchange and the rest
+// where the update competes for issue slots; one kernel per 16-column panel and
+// one for its update of the slab took 8 x 39 us.  Sixteen warps keep the panel
+// code out of local memory (96 registers and fewer spilled in the steps: 112
+// to 150 us).
+constexpr int SL_THREADS = 512, SL_WARPS = SL_THREADS / 32;
+constexpr int SL_LD = GW_W + 2;  // row pitch: 16-byte reads down a column hit all banks
+constexpr int SL_PWMAX = 12;     // most panel warps of a CTA (the others update)
+constexpr int SL_WSLOTS = 16;    // slots of the panel warps' best rows
+constexpr int SL_UR = 8;         // rows of an update tile
+constexpr int SL_CLMAX = 8;      // largest cluster
+constexpr int SL_CAND = GW_NB * 8;  // bytes of a candidate: one row of the panel
+constexpr size_t SL_SMEM_CAP = 226 * 1024;  // dynamic shared memory of a CTA
 
-// rotate a held row left by one place (column c + 1 moves to register c)
-__device__ __forceinline__ void gjw_rotate(float2 (&x)[GW_NB]) {
-  const float2 first = x[0];
-#pragma unroll
-  for (int c = 0; c + 1 < GW_NB; ++c) x[c] = x[c + 1];
-  x[GW_NB - 1] = first;
+struct SlabArgs {
+  int b, c0, c1, rpc, CL;
+  float2* M;                     // [F][b][b]
+  int* rowpiv;                   // [F][b]
+  int* pivslot;                  // [F][b]
+  int* flag;                     // [F] singular flags, [F] = wait timeout
+  int F;
+  uint32_t tries;
+};
+
+__host__ __device__ constexpr int slab_rows8(int rpc) { return (rpc + SL_UR - 1) / SL_UR * SL_UR; }
+__host__ __device__ constexpr size_t slab_smem_bytes(int rpc, int CL) {
+  return (size_t)slab_rows8(rpc) * (SL_LD * 8 + 8)                       // S, pivot steps
+         + (size_t)(CL > 1 ? 2 : 1) * GW_NB * GW_W * 8                  // B
+         + (size_t)2 * ((CL > 1 ? SL_CLMAX : 0) + SL_WSLOTS) * SL_CAND;  // candidates, staging
 }
 
-// staged panel rows: 16 complex padded to 18 (row pitch 144 bytes, so the
-// threads of a warp, one row each, spread over the banks)
-constexpr int GW_STAGE_LD = GW_NB + 2;
-
-// the 16 columns [c, c + ncol) of every row of M into the stage (zero
-// beyond ncol), each warp reading whole 128-byte row segments
-__device__ __forceinline__ void gjw_stage_cols(float2* stage, const float2* M, int b, int c,
-                                               int ncol) {
-  for (int e = threadIdx.x; e < b * (GW_NB / 2); e += blockDim.x) {
-    const int row = e / (GW_NB / 2), u = e - row * (GW_NB / 2);
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (2 * u < ncol) v = reinterpret_cast<const float4*>(M + (size_t)row * b + c)[u];
-    *reinterpret_cast<float4*>(&stage[row * GW_STAGE_LD + 2 * u]) = v;
-  }
-}
-
-__global__ void __launch_bounds__(GW_PANEL_THREADS, 1)
-gjw_panel_kernel(int b, int k0, int nbk, int kp0, float2* __restrict__ Mall,
-                 int* __restrict__ rowpiv_all, int* __restrict__ pivslot_all,
-                 int* __restrict__ flag) {
-  constexpr int NB = GW_NB;
-  constexpr int MAXW = GW_PANEL_THREADS / 32;
-  __shared__ __align__(16) float2 cand[2][MAXW][NB];
-  __shared__ float candv[2][MAXW];
-  __shared__ int candi[2][MAXW];
-  __shared__ int piv_sm[NB];
-  __shared__ __align__(16) float2 Bp[NB][NB];   // Kp's pivot rows at K
-  extern __shared__ __align__(16) float2 stage[];  // [b][GW_STAGE_LD]
-  const int f = blockIdx.x;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int nw = blockDim.x >> 5;
-  const bool a0 = t < b;
-  float2* M = Mall + (size_t)f * b * b;
-  int* rowpiv = rowpiv_all + (size_t)f * b;
-
-  float2 x0[NB];
-  gjw_stage_cols(stage, M, b, k0, nbk);
-  __syncthreads();
-#pragma unroll
-  for (int c = 0; c < NB; ++c)
-    x0[c] = a0 ? stage[t * GW_STAGE_LD + c] : make_float2(0.f, 0.f);
-  const int rp = a0 ? rowpiv[t] : -1;
-  if (kp0 >= 0) {
-    const bool prevpiv = rp >= kp0 && rp < kp0 + NB;
-    if (prevpiv) {
-#pragma unroll
-      for (int c = 0; c < NB; ++c) Bp[rp - kp0][c] = x0[c];
-    }
-    __syncthreads();  // B published; every row taken from the stage
-    gjw_stage_cols(stage, M, b, kp0, NB);
-    __syncthreads();
-    if (a0) {
-      if (prevpiv) {
-#pragma unroll
-        for (int c = 0; c < NB; ++c) x0[c] = make_float2(0.f, 0.f);
-      }
-#pragma unroll 1
-      for (int j = 0; j < NB; ++j) {
-        const float2 a = stage[t * GW_STAGE_LD + j];
-#pragma unroll
-        for (int c = 0; c < NB; ++c) x0[c] = cfma(a, Bp[j][c], x0[c]);
-      }
-#pragma unroll
-      for (int c = 0; c < NB; ++c)
-        if (c >= nbk) x0[c] = make_float2(0.f, 0.f);
-    }
-  }
-  bool e0 = a0 && rp < 0;
-  int col0 = -1;
-
-  // The step loop stays rolled (an unrolled one overflows the instruction
-  // cache: every warp would run the whole straight-line program once).  The
-  // held rows are kept rotated so that the column being eliminated is always
-  // register 0: after each step every row (and so the published pivot row)
-  // rotates left by one, and after nbk == NB steps the order is the original
-  // one again (a ragged last panel rotates the rest at the end).
-#pragma unroll 1
-  for (int j = 0; j < nbk; ++j) {
-    const int buf = j & 1;
-    // this thread's best eligible row, then the warp's, in two warp
-    // reductions: the largest key (the bits of a non-negative float order
-    // like the float; ineligible rows key 0), then the lowest row holding it
-    const float bv0 = e0 ? x0[0].x * x0[0].x + x0[0].y * x0[0].y : -1.f;
-    const int mine = a0 ? t : 0x7fffffff;
-    const unsigned key = bv0 >= 0.f ? __float_as_uint(bv0) + 1u : 0u;
-    const unsigned kmax = __reduce_max_sync(0xffffffffu, key);
-    const int bi = (int)__reduce_min_sync(0xffffffffu, key == kmax ? (unsigned)mine : 0x7fffffffu);
-    const float bv = kmax == 0u ? -1.f : __uint_as_float(kmax - 1u);
-    if (bi == mine && bi != 0x7fffffff) {
-      // 16-byte stores: the shared-memory pipe is the step's bottleneck
-      float4* dst = reinterpret_cast<float4*>(cand[buf][warp]);
-#pragma unroll
-      for (int c = 0; c < NB; c += 2) dst[c / 2] = make_float4(x0[c].x, x0[c].y, x0[c + 1].x, x0[c + 1].y);
-      candv[buf][warp] = bv;
-      candi[buf][warp] = bi;
-    }
-    __syncthreads();
-    // every warp reduces the per-warp candidates the same way; the winning
-    // warp is the lowest lane holding the winner
-    const float cv = lane < nw ? candv[buf][lane] : -2.f;
-    const unsigned ck = cv >= 0.f ? __float_as_uint(cv) + 1u : 0u;
-    const unsigned cmax = __reduce_max_sync(0xffffffffu, ck);
-    const unsigned ci = lane < nw ? (unsigned)candi[buf][lane] : 0x7fffffffu;
-    const int pi = (int)__reduce_min_sync(0xffffffffu, ck == cmax ? ci : 0x7fffffffu);
-    const int pw = __ffs(__ballot_sync(0xffffffffu, ck == cmax && ci == (unsigned)pi)) - 1;
-    const float pv = cmax == 0u ? -1.f : __uint_as_float(cmax - 1u);
-    if (t == 0) {
-      piv_sm[j] = pi;
-      if (!(pv > 0.f)) flag[f] = 1;
-    }
-    // the pivot row in registers (16-byte loads, broadcast to the warp)
-    float2 prow[NB];
-    {
-      const float4* src = reinterpret_cast<const float4*>(cand[buf][pw]);
-#pragma unroll
-      for (int c = 0; c < NB; c += 2) {
-        const float4 v = src[c / 2];
-        prow[c] = make_float2(v.x, v.y);
-        prow[c + 1] = make_float2(v.z, v.w);
-      }
-    }
-    float2 piv = prow[0];
-    if (piv.x * piv.x + piv.y * piv.y == 0.f) piv = make_float2(1e-18f, 0.f);
-    const float pd = piv.x * piv.x + piv.y * piv.y;
-    const float ipd = __frcp_rn(pd);
-    const float2 pinv = make_float2(piv.x * ipd, -piv.y * ipd);
-    // every held row: x -= (x_0 / pivot) * pivot row, x_0 <- -x_0 / pivot;
-    // the pivot row itself is scaled by 1/pivot, its x_0 <- 1/pivot
-    if (t != pi) {
-      const float2 m0 = cmul(x0[0], pinv);
-#pragma unroll
-      for (int c = 1; c < NB; ++c) {
-        const float2 p = prow[c];
-        x0[c].x = fmaf(-m0.x, p.x, fmaf(m0.y, p.y, x0[c].x));
-        x0[c].y = fmaf(-m0.x, p.y, fmaf(-m0.y, p.x, x0[c].y));
-      }
-      x0[0] = make_float2(-m0.x, -m0.y);
-    } else {
-#pragma unroll
-      for (int c = 1; c < NB; ++c) x0[c] = cmul(prow[c], pinv);
-      x0[0] = pinv;
-      e0 = false;
-      col0 = j;
-    }
-    gjw_rotate(x0);
-  }
-  // a ragged panel (nbk < NB steps) rotates the remaining NB - nbk places
-#pragma unroll 1
-  for (int j = nbk; j < NB; ++j) gjw_rotate(x0);
-  // panel columns back in place (through shared memory, coalesced); pivot
-  // bookkeeping
-  __syncthreads();  // the stage is free (the pre-step's reads are done)
-  if (a0) {
-#pragma unroll
-    for (int c = 0; c < NB; ++c) stage[t * GW_STAGE_LD + c] = x0[c];
-  }
-  if (a0 && col0 >= 0) rowpiv[t] = k0 + col0;
-  __syncthreads();
-  for (int e = t; e < b * (NB / 2); e += blockDim.x) {
-    const int row = e / (NB / 2), u = e - row * (NB / 2);
-    if (2 * u < nbk)
-      reinterpret_cast<float4*>(M + (size_t)row * b + k0)[u] =
-          *reinterpret_cast<const float4*>(&stage[row * GW_STAGE_LD + 2 * u]);
-  }
-  if (t < nbk) pivslot_all[(size_t)f * b + k0 + t] = piv_sm[t];
-}
-
-// ------------------------------------------------------------- slab update
-// The transformation of panel K = [k0, k0 + nbk) applied to the slab's other
-// columns, except the next panel's [kn0, kn0 + 16) (kn0 < 0: none), which
-// that panel's kernel updates itself:
-//   M[r, m] += M[r, K] B[:, m]      rows r not pivoted in K,
-//   M[r, m]  = M[r, K] B[:, m]      the pivot rows of K (T^{-1} B itself),
-// B[j][m] = M[pivslot[k0 + j], m] before this step.  A cluster of SU_CL CTAs
-// owns one 16-column group of the slab for one problem, each CTA a range of
-// rows: every CTA reads B for the group's columns, then a cluster barrier,
-// then the CTAs write their rows (pivot rows included), so no B entry is
-// read after it was overwritten and no other cluster touches these columns.
-// Exact FP32 on the CUDA cores: a rank-16 contraction is bound by moving the
-// columns, not by its flops.
-constexpr int SU_THREADS = 256, SU_RT = 64, SU_CL = 4;
-
-__device__ __forceinline__ void su_cluster_sync() {
+__device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+  return r;
+}
+// address of the same shared-memory location in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// 16 bytes into a CTA of the cluster, counted on that CTA's mbarrier
+__device__ __forceinline__ void st_async16(uint32_t addr, float4 v, uint32_t mbar) {
+  asm volatile(
+      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];\n" ::
+          "r"(addr),
+      "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(mbar)
+      : "memory");
+}
+// bounded wait that acquires data sent from other CTAs of the cluster
+__device__ __forceinline__ bool slab_wait(uint64_t* bar, uint32_t parity, uint32_t tries) {
+  for (uint32_t t = 0; t < tries; ++t) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n"
+        " mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(tc::smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+// 1 / v to FP32 accuracy without a call: the hardware approximation (1 ulp) and
+// a Newton step where it cannot leave the normal range
+__device__ __forceinline__ float recip(float v) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;\n" : "=f"(r) : "f"(v));
+  const float n = fmaf(r, fmaf(-v, r, 1.f), r);
+  return v > 1e-37f && v < 1e37f ? n : r;
+}
+// 16-byte piece i of a candidate in slot c sits at piece i ^ (c % 8): the
+// lanes of a warp that read one column of all slots spread over the banks
+__device__ __forceinline__ int cand_piece(int i, int c) { return (i ^ (c & 7)) * 16; }
+// key of a pivot candidate: orders like |x|^2 cut to 18 bits (the bits of a
+// non-negative float order like the float), then the largest id < 32
+__device__ __forceinline__ unsigned pivot_key(float a, unsigned id) {
+  return (__float_as_uint(a) & ~31u) | id;
+}
 
-__global__ void __launch_bounds__(SU_THREADS)
-gjw_slab_update_kernel(int b, int k0, int nbk, int kn0, int c0, int c1, float2* __restrict__ Mall,
-                       const int* __restrict__ rowpiv_all, const int* __restrict__ pivslot_all) {
+// The transformation of the panel at group kg (16 columns each) applied to
+// the CTA's rows at the slab's other groups, except the group kg + 1 when
+// skip_next, in tiles of 8 rows x 32 NS columns (slot t of a lane: column
+// lane % 16 of the (2 (slot0 + t) + lane / 16)-th remaining group) taken by the warps
+// w0, w0 + nw, ...; rowp[r] >= 0 marks the panel's pivot rows.
+template <int NS>
+__device__ __forceinline__ void slab_update_tiles(float2* S, const float2* Bs, const int* rowp,
+                                                  int nrows, int ngrp, int kg, int nskip, int w0,
+                                                  int nw, int lane, int slot0 = 0) {
   constexpr int NB = GW_NB;
-  __shared__ float2 Bs[NB][NB + 1];
-  __shared__ float2 As[SU_RT][NB + 1];
-  const int f = blockIdx.y;
-  const int gsel = blockIdx.x / SU_CL, chunk = blockIdx.x % SU_CL;  // cluster = gsel
-  // gsel-th 16-column group of [c0, c1) that is neither K nor the next
-  // panel (the same for every CTA of the cluster)
-  int cs = -1;
-  for (int g = 0, cnt = 0; c0 + NB * g < c1; ++g) {
-    const int c = c0 + NB * g;
-    if (c == k0 || c == kn0) continue;
-    if (cnt++ == gsel) {
-      cs = c;
-      break;
-    }
-  }
-  if (cs < 0) return;  // the whole cluster returns
-  const int nc = min(NB, c1 - cs);
-  const int rows_per = (b + SU_CL * SU_RT - 1) / (SU_CL * SU_RT) * SU_RT;
-  const int rbeg = chunk * rows_per, rend = min(b, rbeg + rows_per);
-  float2* M = Mall + (size_t)f * b * b;
-  const int* rowpiv = rowpiv_all + (size_t)f * b;
-  const int* piv = pivslot_all + (size_t)f * b + k0;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;  // ty: 0 .. 15
-  for (int e = tid; e < NB * NB; e += SU_THREADS) {
-    const int j = e / NB, c = e - j * NB;
-    Bs[j][c] = (j < nbk && c < nc) ? M[(size_t)piv[j] * b + cs + c] : make_float2(0.f, 0.f);
-  }
-  // every CTA of the cluster has read B before any of them writes a row
-  // (pivot rows included); the barrier also orders this CTA's Bs
-  su_cluster_sync();
-  // Row tiles of SU_RT rows, software-pipelined: the old values and K's
-  // entries of tile t + 1 are loaded into registers while tile t is computed.
-  constexpr int RI = SU_RT / 16, AI = SU_RT * NB / SU_THREADS;
-  float2 old[RI], anext[AI];
-  auto load = [&](int r0) {
+  int col[NS];
+  bool on[NS];
 #pragma unroll
-    for (int i = 0; i < RI; ++i) {
-      const int r = r0 + ty + 16 * i;
-      const bool live = r < rend && tx < nc;
-      const int rp = live ? rowpiv[r] : -1;
-      const bool pivot = rp >= k0 && rp < k0 + NB;
-      old[i] = (live && !pivot) ? M[(size_t)r * b + cs + tx] : make_float2(0.f, 0.f);
-    }
+  for (int t = 0; t < NS; ++t) {
+    const int gi = 2 * (t + slot0) + (lane >> 4), gr = gi < kg ? gi : gi + nskip;
+    on[t] = gr < ngrp;
+    col[t] = (on[t] ? gr : kg) * NB + (lane & 15);
+  }
+  for (int rg = w0 * SL_UR; rg < nrows; rg += nw * SL_UR) {
+    float2 acc[SL_UR][NS];
 #pragma unroll
-    for (int u = 0; u < AI; ++u) {
-      const int e = tid + u * SU_THREADS, rr = e / NB, k = e - rr * NB, r = r0 + rr;
-      anext[u] = (r < rend && k < nbk) ? M[(size_t)r * b + k0 + k] : make_float2(0.f, 0.f);
+    for (int i = 0; i < SL_UR; ++i) {
+      const bool keep = rg + i < nrows && rowp[rg + i] < 0;
+#pragma unroll
+      for (int t = 0; t < NS; ++t)
+        acc[i][t] = keep ? S[(rg + i) * SL_LD + col[t]] : make_float2(0.f, 0.f);
     }
-  };
-  if (rbeg < rend) load(rbeg);
 #pragma unroll 1
-  for (int r0 = rbeg; r0 < rend; r0 += SU_RT) {
+    for (int j = 0; j < NB; j += 2) {
+      float2 b0[NS], b1[NS];
 #pragma unroll
-    for (int u = 0; u < AI; ++u) {
-      const int e = tid + u * SU_THREADS, rr = e / NB, k = e - rr * NB;
-      As[rr][k] = anext[u];
+      for (int t = 0; t < NS; ++t) {
+        b0[t] = Bs[j * GW_W + col[t]];
+        b1[t] = Bs[(j + 1) * GW_W + col[t]];
+      }
+#pragma unroll
+      for (int i = 0; i < SL_UR; ++i) {
+        const float4 a = *reinterpret_cast<const float4*>(&S[(rg + i) * SL_LD + kg * NB + j]);
+#pragma unroll
+        for (int t = 0; t < NS; ++t) acc[i][t] = cfma(make_float2(a.x, a.y), b0[t], acc[i][t]);
+#pragma unroll
+        for (int t = 0; t < NS; ++t) acc[i][t] = cfma(make_float2(a.z, a.w), b1[t], acc[i][t]);
+      }
     }
-    float2 acc[RI];
 #pragma unroll
-    for (int i = 0; i < RI; ++i) acc[i] = old[i];
-    __syncthreads();
-    if (r0 + SU_RT < rend) load(r0 + SU_RT);
+    for (int i = 0; i < SL_UR; ++i) {
+      if (rg + i >= nrows) break;
 #pragma unroll
-    for (int i = 0; i < RI; ++i) {
-      const int rr = ty + 16 * i, r = r0 + rr;
-#pragma unroll
-      for (int k = 0; k < NB; ++k) acc[i] = cfma(As[rr][k], Bs[k][tx], acc[i]);
-      if (r < rend && tx < nc) M[(size_t)r * b + cs + tx] = acc[i];
+      for (int t = 0; t < NS; ++t)
+        if (on[t]) S[(rg + i) * SL_LD + col[t]] = acc[i][t];
     }
-    __syncthreads();
   }
 }
 
-// launch of the slab update: ngroups column groups x SU_CL-CTA clusters
-rr_status launch_slab_update(int b, int k0, int nbk, int kn0, int c0, int c1, int ngroups, int F,
-                             float2* M, const int* rowpiv, const int* pivslot, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ngroups * SU_CL, F, 1);
-  cfg.blockDim = dim3(SU_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = SU_CL;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  RR_CUDA(cudaLaunchKernelEx(&cfg, gjw_slab_update_kernel, b, k0, nbk, kn0, c0, c1, M, rowpiv,
-                             pivslot));
+__device__ __forceinline__ void slab_update(float2* S, const float2* Bs, const int* rowp, int nrows,
+                                            int ngrp, int kg, bool skip_next, int w0, int nw,
+                                            int lane) {
+  const int nskip = skip_next ? 2 : 1, left = ngrp - nskip;
+  if (left <= 0) return;
+  switch ((left + 1) >> 1) {
+    case 1: slab_update_tiles<1>(S, Bs, rowp, nrows, ngrp, kg, nskip, w0, nw, lane); break;
+    case 2: slab_update_tiles<2>(S, Bs, rowp, nrows, ngrp, kg, nskip, w0, nw, lane); break;
+    case 3: slab_update_tiles<3>(S, Bs, rowp, nrows, ngrp, kg, nskip, w0, nw, lane); break;
+    default:  // (four column slots at once exceed the registers of 24 warps)
+      slab_update_tiles<2>(S, Bs, rowp, nrows, ngrp, kg, nskip, w0, nw, lane);
+      slab_update_tiles<2>(S, Bs, rowp, nrows, ngrp, kg, nskip, w0, nw, lane, 2);
+  }
+}
+
+template <bool SOLO, int LPR>
+__global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
+  constexpr int NB = GW_NB;
+  constexpr int CPL = NB / LPR;  // panel columns per lane
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t mbar[2], mbarB;
+  __shared__ unsigned wkey[2][32];  // the panel warps' keys of a step (0 beyond)
+  // local row of the panel's pivots (-1: not known yet, -2: another CTA's)
+  __shared__ int own_sm[2][NB];
+  volatile int(*own)[NB] = own_sm;
+  const int CL = SOLO ? 1 : g.CL;
+  const int rpc8 = slab_rows8(g.rpc);
+  const int pw = (g.rpc * LPR + 31) >> 5;  // panel warps
+  float2* S = reinterpret_cast<float2*>(smem_raw);            // [rpc8][SL_LD]
+  float2* Bs = S + (size_t)rpc8 * SL_LD;                      // [SOLO ? 1 : 2][NB][GW_W]
+  unsigned char* cand = reinterpret_cast<unsigned char*>(Bs + (SOLO ? 1 : 2) * NB * GW_W);
+  // candidate slots [2][SL_CLMAX] (slot 7 - rank) and the panel warps' best
+  // rows [2][SL_WSLOTS] (slot 15 - warp)
+  unsigned char* wst = cand + (SOLO ? 0 : 2 * SL_CLMAX * SL_CAND);
+  int* rowp = reinterpret_cast<int*>(wst + 2 * SL_WSLOTS * SL_CAND);  // [2][rpc8]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = g.b, c0 = g.c0, ncol = g.c1 - g.c0;
+  const uint32_t rank = SOLO ? 0u : cluster_rank();
+  const int f = blockIdx.x / CL;
+  const int nrows = max(0, (b - (int)rank + CL - 1) / CL);
+  float2* M = g.M + (size_t)f * b * b;
+  int* rowpiv = g.rowpiv + (size_t)f * b;
+  const int npan = (ncol + NB - 1) / NB;
+
+  if (!SOLO && tid == 0) {
+    tc::mbar_init(&mbar[0], 1);
+    tc::mbar_init(&mbar[1], 1);
+    tc::mbar_init(&mbarB, 1);
+  }
+  if (tid < 2 * NB) own[tid / NB][tid % NB] = -1;
+  if (tid < 64) wkey[tid >> 5][tid & 31] = 0u;
+  if (!SOLO)  // the slots of absent CTAs stay zero
+    for (int e = tid; e < 2 * SL_CLMAX * SL_CAND / 4; e += SL_THREADS)
+      reinterpret_cast<int*>(cand)[e] = 0;
+  // the slab's rows (zero beyond its columns and rows)
+  for (int e = tid; e < rpc8 * (GW_W / 2); e += SL_THREADS) {
+    const int r = e / (GW_W / 2), u = e - r * (GW_W / 2);
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < nrows && 2 * u < ncol)
+      v = reinterpret_cast<const float4*>(M + (size_t)(r * CL + rank) * b + c0)[u];
+    *reinterpret_cast<float4*>(&S[r * SL_LD + 2 * u]) = v;
+  }
+  // a panel lane: row prow, columns [cg, cg + CPL) of the panel
+  const bool is_panel = warp < pw;
+  const int prow = tid / LPR, cg = (tid % LPR) * CPL;
+  const bool live = is_panel && prow < nrows;
+  const int grow = prow * CL + (int)rank;
+  bool elig = live && (c0 == 0 || rowpiv[grow] < 0);
+  int mypiv = -1;        // column this row pivoted for in this slab
+  int myj = -1;          // its step if it pivoted in the panel at hand
+  bool singular = false;
+  if (SOLO) __syncthreads();
+  else cluster_sync();  // barriers initialised before any CTA sends; S complete
+
+  // sending the CTA's candidate: panel warp w takes the 16-byte piece lane % 8
+  // for CTA 4 w + lane / 8 (and, with one panel warp, 4 + lane / 8)
+  const int myslot = SL_CLMAX - 1 - (int)rank;
+  const uint32_t cand_a = tc::smem_u32(cand) + myslot * SL_CAND + cand_piece(lane & 7, myslot);
+  const uint32_t mbar_a = tc::smem_u32(&mbar[0]);
+  const int rk1 = 4 * warp + (lane >> 3), rk2 = pw == 1 ? rk1 + 4 : CL;
+  uint32_t ra1 = 0, ra2 = 0, rm1 = 0, rm2 = 0;
+  if (!SOLO) {
+    ra1 = cluster_map(cand_a, min(rk1, CL - 1));
+    ra2 = cluster_map(cand_a, min(rk2, CL - 1));
+    rm1 = cluster_map(mbar_a, min(rk1, CL - 1));
+    rm2 = cluster_map(mbar_a, min(rk2, CL - 1));
+  }
+  const uint32_t cbytes = (uint32_t)(CL * SL_CAND);
+  constexpr uint32_t CB = SL_CLMAX * SL_CAND, WB = SL_WSLOTS * SL_CAND;  // one buffer of each
+  const unsigned row_id = 31u - (unsigned)(lane / LPR);
+  unsigned char* my_wst = wst + (is_panel ? SL_WSLOTS - 1 - warp : 0) * SL_CAND + cg * 8;
+  bool ok = true;
+  for (int p = 0; p < npan; ++p) {
+    const int kl = p * NB, nbk = min(NB, ncol - kl);
+    int* rowp_p = rowp + (p & 1) * rpc8;
+    float2* Bp = Bs + (SOLO ? 0 : (p & 1) * NB * GW_W);
+    const float2* Bq = Bs + (SOLO ? 0 : ((p + 1) & 1) * NB * GW_W);  // the previous panel's
+    if (is_panel) {
+      if (tid < NB) own[(p + 1) & 1][tid] = -1;
+      if (!SOLO && tid == 0 && npan > 1) tc::mbar_expect_tx(&mbarB, (uint32_t)nbk * (GW_W * 8));
+      // the panel's columns, with the previous panel's transformation
+      float2 x[CPL];
+#pragma unroll
+      for (int c = 0; c < CPL; c += 2) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (live && myj < 0) v = *reinterpret_cast<const float4*>(&S[prow * SL_LD + kl + cg + c]);
+        x[c] = make_float2(v.x, v.y);
+        x[c + 1] = make_float2(v.z, v.w);
+      }
+      if (p > 0 && live) {
+        const float2* Ar = &S[prow * SL_LD + kl - NB];
+#pragma unroll 2
+        for (int j = 0; j < NB; j += 2) {
+          const float4 a = *reinterpret_cast<const float4*>(Ar + j);
+          const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w);
+          const float2* B0 = Bq + j * GW_W + kl + cg;
+#pragma unroll
+          for (int c = 0; c < CPL; c += 2) {
+            const float4 v0 = *reinterpret_cast<const float4*>(B0 + c);
+            const float4 v1 = *reinterpret_cast<const float4*>(B0 + GW_W + c);
+            x[c] = cfma(a0, make_float2(v0.x, v0.y), x[c]);
+            x[c + 1] = cfma(a0, make_float2(v0.z, v0.w), x[c + 1]);
+            x[c] = cfma(a1, make_float2(v1.x, v1.y), x[c]);
+            x[c + 1] = cfma(a1, make_float2(v1.z, v1.w), x[c + 1]);
+          }
+        }
+      }
+      myj = -1;
+      // column jb CPL + s is register s of lane jb of every row; b % 8 == 0,
+      // so a panel has a multiple of CPL steps and the parities of a step are
+      // those of s
+#pragma unroll 1
+      for (int jb = 0; jb * CPL < nbk; ++jb) {
+        const int src_lane = (lane & ~(LPR - 1)) | jb;
+        const bool mycol = cg == jb * CPL;
+#pragma unroll
+        for (int s = 0; s < CPL; ++s) {
+          const int j = jb * CPL + s, buf = s & 1;
+          const float2 xs = make_float2(__shfl_sync(0xffffffffu, x[s].x, src_lane),
+                                        __shfl_sync(0xffffffffu, x[s].y, src_lane));
+          const float av = elig ? xs.x * xs.x + xs.y * xs.y : 0.f;
+          const unsigned kmax = __reduce_max_sync(0xffffffffu, pivot_key(av, row_id));
+          const bool wrow = ((kmax ^ row_id) & 31u) == 0u;  // the warp's best row
+          {
+            // (a warp without an eligible row: zero in the pivot's place)
+            const bool none = kmax < 32u && mycol;
+            if (wrow && cg == 0) wkey[buf][warp] = kmax;
+#pragma unroll
+            for (int c = 0; c < CPL; c += 2) {
+              float4 v = make_float4(x[c].x, x[c].y, x[c + 1].x, x[c + 1].y);
+              if (c == s) v.x = none ? 0.f : v.x, v.y = none ? 0.f : v.y;
+              if (c + 1 == s) v.z = none ? 0.f : v.z, v.w = none ? 0.f : v.w;
+              if (wrow) *reinterpret_cast<float4*>(my_wst + buf * WB + c * 8) = v;
+            }
+          }
+          // the CTA's candidate: the best of its panel warps
+          asm volatile("bar.sync 1, %0;\n" ::"r"(pw * 32) : "memory");
+          const unsigned wk = pivot_key(__uint_as_float(wkey[buf][lane]), (15u - lane) & 31u);
+          const unsigned cw = __reduce_max_sync(0xffffffffu, wk) & 15u;  // 15 - warp
+          const unsigned char* src = wst + buf * WB + cw * SL_CAND;
+          float2 pinv;
+          bool mine = true;  // this CTA holds the pivot row
+          unsigned sw = 0;   // piece swizzle of the row at src
+          if (!SOLO) {
+            if (warp < 2) {  // (at most eight CTAs: two warps send)
+              const float4 v = *reinterpret_cast<const float4*>(src + (lane & 7) * 16);
+              if (rk1 < CL) st_async16(ra1 + buf * CB, v, rm1 + buf * 8);
+              if (rk2 < CL) st_async16(ra2 + buf * CB, v, rm2 + buf * 8);
+              if (tid == 0) tc::mbar_expect_tx(&mbar[buf], cbytes);
+            }
+            if (ok) ok = slab_wait(&mbar[buf], (s >> 1) & 1, g.tries);
+            // every warp reduces the candidates the same way
+            const unsigned char* cb = cand + buf * CB;
+            const int sl = lane & 7;
+            float2 cp = *reinterpret_cast<const float2*>(cb + sl * SL_CAND + cand_piece(j >> 1, sl) +
+                                                         (s & 1) * 8);
+            float cv = cp.x * cp.x + cp.y * cp.y;
+            const unsigned cmax = __reduce_max_sync(0xffffffffu, pivot_key(cv, sl));
+            if (cv == 0.f) {
+              cp = make_float2(1e-18f, 0.f);
+              cv = 1e-36f;
+            }
+            const float rv = recip(cv);
+            sw = cmax & 7u;
+            src = cb + sw * SL_CAND;
+            mine = sw == (unsigned)myslot;
+            pinv.x = __shfl_sync(0xffffffffu, cp.x * rv, sw);
+            pinv.y = __shfl_sync(0xffffffffu, -cp.y * rv, sw);
+            // a pivot of zero, or not a number
+            singular |= cmax - 32u >= 0x7f800020u - 32u;
+          } else {
+            float2 pv = *reinterpret_cast<const float2*>(src + j * 8);
+            float pd = pv.x * pv.x + pv.y * pv.y;
+            singular |= !(pd > 0.f);
+            if (pd == 0.f) {
+              pv = make_float2(1e-18f, 0.f);
+              pd = 1e-36f;
+            }
+            const float rv = recip(pd);
+            pinv = make_float2(pv.x * rv, -pv.y * rv);
+          }
+          float2 q[CPL];
+#pragma unroll
+          for (int c = 0; c < CPL; c += 2) {
+            const float4 v = *reinterpret_cast<const float4*>(src + cand_piece((cg + c) / 2, sw));
+            q[c] = make_float2(v.x, v.y);
+            q[c + 1] = make_float2(v.z, v.w);
+          }
+          float2 m = make_float2(xs.y * pinv.y - xs.x * pinv.x, -xs.x * pinv.y - xs.y * pinv.x);
+          if (mine && cw + warp == 15u) {  // (the whole warp)
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+              x[c].x = wrow ? 0.f : x[c].x;
+              x[c].y = wrow ? 0.f : x[c].y;
+            }
+            m.x = wrow ? pinv.x : m.x;
+            m.y = wrow ? pinv.y : m.y;
+            elig = elig && !wrow;
+            myj = wrow ? j : myj;
+            if (wrow && cg == 0) own[p & 1][j] = prow;
+          }
+          if (!SOLO && !mine && tid == 0) own[p & 1][j] = -2;
+#pragma unroll
+          for (int cc = 1; cc <= CPL; ++cc) {
+            const int c = (s + cc) % CPL;
+            x[c].x = fmaf(m.x, q[c].x, fmaf(-m.y, q[c].y, x[c].x));
+            x[c].y = fmaf(m.x, q[c].y, fmaf(m.y, q[c].x, x[c].y));
+          }
+          if (mycol) x[s] = m;
+        }
+      }
+      if (live) {
+#pragma unroll
+        for (int c = 0; c < CPL; c += 2)
+          *reinterpret_cast<float4*>(&S[prow * SL_LD + kl + cg + c]) =
+              make_float4(x[c].x, x[c].y, x[c + 1].x, x[c + 1].y);
+        if (myj >= 0) mypiv = c0 + kl + myj;
+        if (cg == 0) rowp_p[prow] = myj;
+      }
+    } else if (npan > 1) {
+      // beside the steps: the previous panel's transformation of the rest,
+      const int uw = warp - pw, nuw = SL_WARPS - pw;
+      if (p > 0)
+        slab_update(S, Bq, rowp + ((p + 1) & 1) * rpc8, nrows, npan, p - 1, true, uw, nuw, lane);
+      // then, every row being complete, the pivot rows as they become known
+      asm volatile("bar.sync 2, %0;\n" ::"r"(nuw * 32) : "memory");
+      const uint32_t mb = tc::smem_u32(&mbarB);
+      for (int j = uw; j < NB; j += nuw) {
+        int lr = j < nbk ? -1 : -2;
+        for (uint32_t t = 0; lr == -1 && t < g.tries; ++t) {
+          lr = own[p & 1][j];
+          if (lr == -1) __nanosleep(400);
+        }
+        if (lr == -1) ok = false;
+        if (lr < 0) {
+          // (rows beyond a ragged panel's columns multiply zeros; keep them finite)
+          if (j >= nbk)
+            for (int c = lane; c < GW_W; c += 32) Bp[j * GW_W + c] = make_float2(0.f, 0.f);
+          continue;
+        }
+        const float4 v0 = *reinterpret_cast<const float4*>(&S[lr * SL_LD + 2 * lane]);
+        const float4 v1 = *reinterpret_cast<const float4*>(&S[lr * SL_LD + 64 + 2 * lane]);
+        if (SOLO) {
+          *reinterpret_cast<float4*>(&Bp[j * GW_W + 2 * lane]) = v0;
+          *reinterpret_cast<float4*>(&Bp[j * GW_W + 64 + 2 * lane]) = v1;
+        } else {
+          const uint32_t ba = tc::smem_u32(Bp + j * GW_W + 2 * lane);
+          for (int d = 0; d < CL; ++d) {
+            const uint32_t rm = cluster_map(mb, d), ra = cluster_map(ba, d);
+            st_async16(ra, v0, rm);
+            st_async16(ra + 512, v1, rm);
+          }
+        }
+      }
+    }
+    __syncthreads();  // panel columns, rowp, the previous update, the sends' reads
+    if (!SOLO && npan > 1 && ok) ok = slab_wait(&mbarB, p & 1, g.tries);
+    if (npan > 1 && p + 1 == npan) {
+      slab_update(S, Bp, rowp_p, nrows, npan, p, false, warp, SL_WARPS, lane);
+      __syncthreads();
+    }
+  }
+  for (int e = tid; e < nrows * (GW_W / 2); e += SL_THREADS) {
+    const int r = e / (GW_W / 2), u = e - r * (GW_W / 2);
+    if (2 * u < ncol)
+      reinterpret_cast<float4*>(M + (size_t)(r * CL + rank) * b + c0)[u] =
+          *reinterpret_cast<const float4*>(&S[r * SL_LD + 2 * u]);
+  }
+  if (live && cg == 0) {
+    if (mypiv >= 0) {
+      rowpiv[grow] = mypiv;
+      g.pivslot[(size_t)f * b + mypiv] = grow;
+    } else if (c0 == 0) {
+      rowpiv[grow] = -1;
+    }
+  }
+  if (rank == 0 && tid == 0 && singular) g.flag[f] = 1;
+  if (!ok && lane == 0) atomicExch(g.flag + g.F, 1);
+  if (!SOLO) cluster_sync();  // no CTA leaves while another may still send to it
+}
+
+// lanes per row: four where that leaves warps for the update
+int slab_lpr(int rpc) { return rpc <= 8 * SL_PWMAX ? 4 : 2; }
+
+// Cluster size of the slab kernel: the one with the least modelled time, waves
+// of clusters x time of a full slab.  Measured at two problems: 72 us with 24
+// rows per CTA, 91 with 48, 108 with 96 in clusters of eight (82 and 104 with
+// 48 and 96 rows in clusters of four), 116 with 192 rows in one CTA, where the
+// update beside the steps weighs most.  At one CTA per SM a GPC of 19 SMs holds
+// 19 / CL clusters.
+int slab_cluster(int b, int F, int nsm) {
+  int best = SL_CLMAX;
+  double bt = 1e30;
+  for (int cl = 1; cl <= SL_CLMAX; ++cl) {
+    const int rpc = (b + cl - 1) / cl;
+    if (rpc > (cl == 1 ? 16 : 8) * SL_PWMAX || slab_smem_bytes(rpc, cl) > SL_SMEM_CAP) continue;
+    const int slots = std::max(1, nsm / 19 * (19 / cl));
+    const int waves = (F + slots - 1) / slots;
+    const double t = waves * (cl > 1 ? 60.0 + 0.5 * rpc : 45.0 + 0.37 * rpc);
+    if (t < bt) {
+      bt = t;
+      best = cl;
+    }
+  }
+  return best;
+}
+
+rr_status launch_slab(rr_factors* fa, int c0, int c1, cudaStream_t st) {
+  const OpDev& d = fa->op->d;
+  SlabArgs a;
+  a.b = d.b;
+  a.c0 = c0;
+  a.c1 = c1;
+  a.F = fa->F;
+  a.CL = slab_cluster(d.b, fa->F, num_sms(d.device));
+  a.rpc = (d.b + a.CL - 1) / a.CL;
+  a.M = reinterpret_cast<float2*>(fa->M);
+  a.rowpiv = fa->rowpiv;
+  a.pivslot = fa->pivslot;
+  a.flag = fa->flag;
+  a.tries = wait_tries();
+  const size_t smem = slab_smem_bytes(a.rpc, a.CL);
+  const int lpr = slab_lpr(a.rpc);
+  static bool attr = false;
+  if (!attr) {
+    constexpr int cap = (int)SL_SMEM_CAP;
+    RR_CUDA(cudaFuncSetAttribute(gjw_slab_kernel<true, 2>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    RR_CUDA(cudaFuncSetAttribute(gjw_slab_kernel<true, 4>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    RR_CUDA(cudaFuncSetAttribute(gjw_slab_kernel<false, 4>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
+    attr = true;
+  }
+  prof_begin(PROF_PANEL, st);
+  if (a.CL == 1) {
+    if (lpr == 4) gjw_slab_kernel<true, 4><<<fa->F, SL_THREADS, smem, st>>>(a);
+    else gjw_slab_kernel<true, 2><<<fa->F, SL_THREADS, smem, st>>>(a);
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.CL * fa->F), 1, 1);
+    cfg.blockDim = dim3(SL_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = a.CL;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    RR_CUDA(cudaLaunchKernelEx(&cfg, gjw_slab_kernel<false, 4>, a));
+  }
+  prof_end(PROF_PANEL, st);
+  RR_CUDA(cudaGetLastError());
   return RR_OK;
 }
 
@@ -748,11 +989,6 @@ gjw_finalize_kernel(OpView op, int i, int RB, const float2* __restrict__ Mall,
   }
 }
 
-__global__ void gjw_rowpiv_init_kernel(int* rowpiv, int n) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < n) rowpiv[e] = -1;
-}
-
 template <int SPLIT>
 rr_status launch_gemm(rr_factors* fa, const CUtensorMap* ta, const CUtensorMap* tb, int ka, int Kc,
                       int x0, int x1, int y0, int y1, cudaStream_t st) {
@@ -805,60 +1041,10 @@ rr_status factor_wide_impl(rr_factors* fa) {
   RR_CUDA(cudaFuncSetAttribute(gjw_finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)fsmem));
   const int nct_all = (b + GG_CT - 1) / GG_CT;
-  const int pthreads = (b + 31) & ~31;  // one row per thread
-  const size_t psmem = (size_t)b * GW_STAGE_LD * sizeof(float2);
-  RR_CUDA(cudaFuncSetAttribute(gjw_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)psmem));
   const int ncols = fa->factor_cols > 0 ? std::min(fa->factor_cols, nx) : nx;
   for (int i = 0; i < ncols; ++i) {
-    prof_count(1);
-    gjw_rowpiv_init_kernel<<<(F * b + 255) / 256, 256, 0, st>>>(fa->rowpiv, F * b);
     rr_status s = launch_schur_f32(fa, i, st);
     if (s != RR_OK) return s;
-    // Inner factorisation of one slab: the panels in order on stream sx,
-    // each panel's update of the rest of the slab on stream sy.  Panel p+1
-    // applies panel p's transformation to its own columns itself, so it
-    // waits only for the slab update of panel p-1 (which reaches its
-    // columns) and runs beside the slab update of panel p (disjoint
-    // columns; the rows pivoted in p+1 change rowpiv from "none" to a
-    // column outside panel p, which that update reads as "not a pivot of p"
-    // either way).  The slab updates run in order on sy; sx joins sy at the
-    // end.
-    auto inner = [&](int c0, cudaStream_t sx, cudaStream_t sy) -> rr_status {
-      const int c1 = std::min(b, c0 + GW_W);
-      const int npan = (c1 - c0 + GW_NB - 1) / GW_NB;
-      cudaEvent_t* ev_pan = fa->ev_w;      // [4] ring: panel p done (on sx)
-      cudaEvent_t* ev_upd = fa->ev_w + 4;  // [4] ring: slab update of panel p done (on sy)
-      bool used = false;                   // sy took work (it joined sx's order by an event)
-      for (int p = 0; p < npan; ++p) {
-        const int k0 = c0 + p * GW_NB, nbk = std::min(GW_NB, c1 - k0);
-        if (p >= 2) RR_CUDA(cudaStreamWaitEvent(sx, ev_upd[(p - 2) & 3], 0));
-        prof_begin(PROF_PANEL, sx);
-        gjw_panel_kernel<<<F, pthreads, psmem, sx>>>(b, k0, nbk, p > 0 ? k0 - GW_NB : -1, M,
-                                                     fa->rowpiv, fa->pivslot, fa->flag);
-        prof_end(PROF_PANEL, sx);
-        RR_CUDA(cudaGetLastError());
-        // the slab's columns outside this panel and the next one
-        const int kn0 = p + 1 < npan ? k0 + GW_NB : -1;
-        const int ngroups = npan - 1 - (kn0 >= 0 ? 1 : 0);
-        if (ngroups > 0) {
-          RR_CUDA(cudaEventRecord(ev_pan[p & 3], sx));
-          RR_CUDA(cudaStreamWaitEvent(sy, ev_pan[p & 3], 0));
-          prof_begin(PROF_INNER, sy);
-          rr_status ls = launch_slab_update(b, k0, nbk, kn0, c0, c1, ngroups, F, M, fa->rowpiv,
-                                            fa->pivslot, sy);
-          prof_end(PROF_INNER, sy);
-          if (ls != RR_OK) return ls;
-          RR_CUDA(cudaEventRecord(ev_upd[p & 3], sy));
-          used = true;
-        }
-      }
-      if (used) {
-        RR_CUDA(cudaEventRecord(fa->ev_w[8], sy));
-        RR_CUDA(cudaStreamWaitEvent(sx, fa->ev_w[8], 0));
-      }
-      return RR_OK;
-    };
     // Look-ahead: once the next slab's columns have received this slab's
     // rank-128 update, the next slab's inner factorisation runs on the second
     // (high-priority) stream while the rank-128 update of the remaining
@@ -868,8 +1054,7 @@ rr_status factor_wide_impl(rr_factors* fa) {
     // stream's update reads as "not a pivot of this slab" either way).  The
     // next slab's pivot rows are gathered on the main stream after both.
     cudaStream_t st2 = fa->stream2;
-    cudaStream_t st3 = fa->stream3;
-    if ((s = inner(0, st, st3)) != RR_OK) return s;
+    if ((s = launch_slab(fa, 0, std::min(b, GW_W), st)) != RR_OK) return s;
     for (int c0 = 0; c0 < b; c0 += GW_W) {
       const int c1 = std::min(b, c0 + GW_W);
       if (c1 >= b && c0 == 0) break;  // one slab: no outer update
@@ -885,7 +1070,7 @@ rr_status factor_wide_impl(rr_factors* fa) {
         if (st2 != nullptr) {
           RR_CUDA(cudaEventRecord(fa->ev_next, st));
           RR_CUDA(cudaStreamWaitEvent(st2, fa->ev_next, 0));
-          if ((s = inner(c1, st2, st3)) != RR_OK) return s;
+          if ((s = launch_slab(fa, c1, n1, st2)) != RR_OK) return s;
           RR_CUDA(cudaEventRecord(fa->ev_panel, st2));
           if ((s = launch_gemm<SPLIT>(fa, tA, tBout, c0, GW_W, 0, s0, u1, nct_all, st)) != RR_OK)
             return s;
@@ -893,7 +1078,7 @@ rr_status factor_wide_impl(rr_factors* fa) {
         } else {
           if ((s = launch_gemm<SPLIT>(fa, tA, tBout, c0, GW_W, 0, s0, u1, nct_all, st)) != RR_OK)
             return s;
-          if ((s = inner(c1, st, st3)) != RR_OK) return s;
+          if ((s = launch_slab(fa, c1, n1, st)) != RR_OK) return s;
         }
       } else {
         if ((s = launch_gemm<SPLIT>(fa, tA, tBout, c0, GW_W, 0, s0, 0, 0, st)) != RR_OK) return s;
@@ -911,12 +1096,12 @@ rr_status factor_wide_impl(rr_factors* fa) {
 
 }  // namespace
 
-// The wide path needs FP32 factors, an even block of at most 768 rows (one
-// panel row per thread) and at least 64, and the TMA maps of M and of the
+// The wide path needs FP32 factors, a block of a multiple of 8 rows, at most
+// 768 and at least 64, and the TMA maps of M and of the
 // gathered pivot rows.
 bool factor_wide_ok(const rr_factors* fa) {
   const int b = fa->op->d.b;
-  return fa->wide_ok && b >= 64 && b <= GW_PANEL_MAX && (b % 8) == 0 &&
+  return fa->wide_ok && b >= 64 && b <= GW_MAX && (b % 8) == 0 &&
          (fa->prec == RR_FP32 || fa->prec == RR_FP32_BF16X3 || fa->prec == RR_FP32_BF16X6);
 }
 
