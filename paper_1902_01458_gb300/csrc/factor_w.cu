@@ -32,6 +32,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "rr_internal.cuh"
 #include "tc.cuh"
@@ -109,44 +110,6 @@ __host__ __device__ constexpr size_t slab_smem_bytes(int rpc, int CL) {
          + (size_t)2 * ((CL > 1 ? SL_CLMAX : 0) + SL_WSLOTS) * SL_CAND;  // candidates, staging
 }
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
-  return r;
-}
-// address of the same shared-memory location in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-// 16 bytes into a CTA of the cluster, counted on that CTA's mbarrier
-__device__ __forceinline__ void st_async16(uint32_t addr, float4 v, uint32_t mbar) {
-  asm volatile(
-      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];\n" ::
-          "r"(addr),
-      "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(mbar)
-      : "memory");
-}
-// bounded wait that acquires data sent from other CTAs of the cluster
-__device__ __forceinline__ bool slab_wait(uint64_t* bar, uint32_t parity, uint32_t tries) {
-  for (uint32_t t = 0; t < tries; ++t) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n"
-        " mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(tc::smem_u32(bar)), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
 // 1 / v to FP32 accuracy without a call: the hardware approximation (1 ulp) and
 // a Newton step where it cannot leave the normal range
 __device__ __forceinline__ float recip(float v) {
@@ -255,7 +218,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
   int* rowp = reinterpret_cast<int*>(wst + 2 * SL_WSLOTS * SL_CAND);  // [2][rpc8]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = g.b, c0 = g.c0, ncol = g.c1 - g.c0;
-  const uint32_t rank = SOLO ? 0u : cluster_rank();
+  const uint32_t rank = SOLO ? 0u : tc::cluster_rank();
   const int f = blockIdx.x / CL;
   const int nrows = max(0, (b - (int)rank + CL - 1) / CL);
   float2* M = g.M + (size_t)f * b * b;
@@ -290,7 +253,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
   int myj = -1;          // its step if it pivoted in the panel at hand
   bool singular = false;
   if (SOLO) __syncthreads();
-  else cluster_sync();  // barriers initialised before any CTA sends; S complete
+  else tc::cluster_sync();  // barriers initialised before any CTA sends; S complete
 
   // sending the CTA's candidate: panel warp w takes the 16-byte piece lane % 8
   // for CTA 4 w + lane / 8 (and, with one panel warp, 4 + lane / 8)
@@ -300,10 +263,10 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
   const int rk1 = 4 * warp + (lane >> 3), rk2 = pw == 1 ? rk1 + 4 : CL;
   uint32_t ra1 = 0, ra2 = 0, rm1 = 0, rm2 = 0;
   if (!SOLO) {
-    ra1 = cluster_map(cand_a, min(rk1, CL - 1));
-    ra2 = cluster_map(cand_a, min(rk2, CL - 1));
-    rm1 = cluster_map(mbar_a, min(rk1, CL - 1));
-    rm2 = cluster_map(mbar_a, min(rk2, CL - 1));
+    ra1 = tc::cluster_map(cand_a, min(rk1, CL - 1));
+    ra2 = tc::cluster_map(cand_a, min(rk2, CL - 1));
+    rm1 = tc::cluster_map(mbar_a, min(rk1, CL - 1));
+    rm2 = tc::cluster_map(mbar_a, min(rk2, CL - 1));
   }
   const uint32_t cbytes = (uint32_t)(CL * SL_CAND);
   constexpr uint32_t CB = SL_CLMAX * SL_CAND, WB = SL_WSLOTS * SL_CAND;  // one buffer of each
@@ -384,11 +347,11 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
           if (!SOLO) {
             if (warp < 2) {  // (at most eight CTAs: two warps send)
               const float4 v = *reinterpret_cast<const float4*>(src + (lane & 7) * 16);
-              if (rk1 < CL) st_async16(ra1 + buf * CB, v, rm1 + buf * 8);
-              if (rk2 < CL) st_async16(ra2 + buf * CB, v, rm2 + buf * 8);
+              if (rk1 < CL) tc::st_async16(ra1 + buf * CB, v, rm1 + buf * 8);
+              if (rk2 < CL) tc::st_async16(ra2 + buf * CB, v, rm2 + buf * 8);
               if (tid == 0) tc::mbar_expect_tx(&mbar[buf], cbytes);
             }
-            if (ok) ok = slab_wait(&mbar[buf], (s >> 1) & 1, g.tries);
+            if (ok) ok = tc::cluster_wait(&mbar[buf], (s >> 1) & 1, g.tries);
             // every warp reduces the candidates the same way
             const unsigned char* cb = cand + buf * CB;
             const int sl = lane & 7;
@@ -486,15 +449,15 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
         } else {
           const uint32_t ba = tc::smem_u32(Bp + j * GW_W + 2 * lane);
           for (int d = 0; d < CL; ++d) {
-            const uint32_t rm = cluster_map(mb, d), ra = cluster_map(ba, d);
-            st_async16(ra, v0, rm);
-            st_async16(ra + 512, v1, rm);
+            const uint32_t rm = tc::cluster_map(mb, d), ra = tc::cluster_map(ba, d);
+            tc::st_async16(ra, v0, rm);
+            tc::st_async16(ra + 512, v1, rm);
           }
         }
       }
     }
     __syncthreads();  // panel columns, rowp, the previous update, the sends' reads
-    if (!SOLO && npan > 1 && ok) ok = slab_wait(&mbarB, p & 1, g.tries);
+    if (!SOLO && npan > 1 && ok) ok = tc::cluster_wait(&mbarB, p & 1, g.tries);
     if (npan > 1 && p + 1 == npan) {
       slab_update(S, Bp, rowp_p, nrows, npan, p, false, warp, SL_WARPS, lane);
       __syncthreads();
@@ -516,7 +479,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
   }
   if (rank == 0 && tid == 0 && singular) g.flag[f] = 1;
   if (!ok && lane == 0) atomicExch(g.flag + g.F, 1);
-  if (!SOLO) cluster_sync();  // no CTA leaves while another may still send to it
+  if (!SOLO) tc::cluster_sync();  // no CTA leaves while another may still send to it
 }
 
 // lanes per row: four where that leaves warps for the update
@@ -526,15 +489,14 @@ int slab_lpr(int rpc) { return rpc <= 8 * SL_PWMAX ? 4 : 2; }
 // of clusters x time of a full slab.  Measured at two problems: 72 us with 24
 // rows per CTA, 91 with 48, 108 with 96 in clusters of eight (82 and 104 with
 // 48 and 96 rows in clusters of four), 116 with 192 rows in one CTA, where the
-// update beside the steps weighs most.  At one CTA per SM a GPC of 19 SMs holds
-// 19 / CL clusters.
-int slab_cluster(int b, int F, int nsm) {
+// update beside the steps weighs most.
+int slab_cluster(int b, int F, int device) {
   int best = SL_CLMAX;
   double bt = 1e30;
   for (int cl = 1; cl <= SL_CLMAX; ++cl) {
     const int rpc = (b + cl - 1) / cl;
     if (rpc > (cl == 1 ? 16 : 8) * SL_PWMAX || slab_smem_bytes(rpc, cl) > SL_SMEM_CAP) continue;
-    const int slots = std::max(1, nsm / 19 * (19 / cl));
+    const int slots = cluster_slots(device, cl);
     const int waves = (F + slots - 1) / slots;
     const double t = waves * (cl > 1 ? 60.0 + 0.5 * rpc : 45.0 + 0.37 * rpc);
     if (t < bt) {
@@ -552,7 +514,7 @@ rr_status launch_slab(rr_factors* fa, int c0, int c1, cudaStream_t st) {
   a.c0 = c0;
   a.c1 = c1;
   a.F = fa->F;
-  a.CL = slab_cluster(d.b, fa->F, num_sms(d.device));
+  a.CL = slab_cluster(d.b, fa->F, d.device);
   a.rpc = (d.b + a.CL - 1) / a.CL;
   a.M = reinterpret_cast<float2*>(fa->M);
   a.rowpiv = fa->rowpiv;
@@ -1095,6 +1057,39 @@ rr_status factor_wide_impl(rr_factors* fa) {
 }
 
 }  // namespace
+
+// Clusters of cl CTAs (at most eight, one CTA per SM) resident at once: what the
+// GPCs hold, 152, 76, 46, 36, 28, 23, 15 and 15 on the GB300 measured.
+int cluster_slots(int device, int cl) {
+  static int cached[64][SL_CLMAX + 1];
+  static std::mutex mu;
+  if (cl < 1 || cl > SL_CLMAX) return 1;
+  const int dev = device >= 0 && device < 64 ? device : 0;
+  std::lock_guard<std::mutex> lock(mu);
+  int& n = cached[dev][cl];
+  if (n == 0) {
+    constexpr int smem = 200 * 1024;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cl * 64), 1, 1);
+    cfg.blockDim = dim3(SL_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(gjw_slab_kernel<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)SL_SMEM_CAP) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, gjw_slab_kernel<false, 4>, &cfg) != cudaSuccess ||
+        n <= 0) {
+      cudaGetLastError();
+      n = std::max(1, num_sms(device) / 19 * (19 / cl));  // (a GPC of 19 SMs)
+    }
+  }
+  return n;
+}
 
 // The wide path needs FP32 factors, a block of a multiple of 8 rows, at most
 // 768 and at least 64, and the TMA maps of M and of the

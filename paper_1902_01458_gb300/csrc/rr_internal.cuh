@@ -249,6 +249,12 @@ rr_status launch_factor_wide(rr_factors* f);
 // sweep.cu: x = A^{-1} b or A^{-H} b with the factors in precision T.
 // b and x are [F][N][k] in the factor precision; tmp same size (adjoint only).
 rr_status launch_solve_lo(rr_factors* f, int k, int adjoint, const void* b, void* x, void* tmp);
+// sweep_cl32.cu, sweep_cl64.cu: the same in one launch per solve, and its
+// modelled time in microseconds
+rr_status launch_sweep_cl32(rr_factors* f, int k, int adjoint, const void* b, void* x, void* tmp);
+rr_status launch_sweep_cl64(rr_factors* f, int k, int adjoint, const void* b, void* x, void* tmp);
+double sweep_cl32_us(const rr_factors* f, int k, int adjoint);
+double sweep_cl64_us(const rr_factors* f, int k, int adjoint);
 // true when the solves of k columns take the split tensor-core sweep, the
 // one path that can run on a subset of the problems (rr_factors::amap)
 bool sweep_tc2_ok(const rr_factors* f, int k);
@@ -321,3 +327,5 @@ uint32_t wait_tries();
 int take_stall();
 
 int num_sms(int device);
+// clusters of cl <= 8 CTAs, one per SM, that are resident at once (factor_w.cu)
+int cluster_slots(int device, int cl);

@@ -9,10 +9,12 @@
 // Adjoint solve (s I - L)^H w = g:
 //   forward  h_0 = g_0,          h_{i+1} = g_{i+1} - C_i^H (G_i^H h_i)
 //   backward w_{n-1} = G^H h,    w_i = G_i^H (h_i + L_{i+1,i}^T w_{i+1})
-// Only G_i is stored; every step is one dense (b x b) x (b x k) product
-// streamed from HBM, plus a sparse coupling product formed by a small kernel
-// into a b x k staging block before (or after) it.  One launch per streamwise
-// column covers all F problems of the batch.
+// Only G_i is stored.  Two forms: one launch per solve with a cluster of CTAs
+// per problem (sweep_cl.cuh), or, for large blocks and batches, two launches
+// per streamwise column for all problems of the batch: the dense (b x b) x
+// (b x k) product on the tensor cores, its contraction split over CTAs
+// (sweep_tc2_kernel), and the sum of the partial blocks with the sparse
+// coupling that forms the next column's right-hand side (sweep_couple_kernel).
 #include <algorithm>
 #include <type_traits>
 
@@ -23,438 +25,154 @@
 
 namespace {
 
-constexpr int SW_THREADS = 256;  // each thread owns a 4 x 2 output tile: RT * kp = 2048
+// Step s of a solve works on column sweep_col(s): forward, then back.
+__host__ __device__ __forceinline__ int sweep_col(int s, int nx) { return s < nx ? s : 2 * nx - 2 - s; }
 
-enum { FWD = 0, BWD = 1, ADJ_FWD = 2, ADJ_BWD = 3 };
-enum { EPI_STORE = 0, EPI_SUB = 1, EPI_TMP = 2 };
-
-__device__ __forceinline__ int slotv(int dx, int dy) { return (dx + 1) * 3 + (dy + 1); }
-
-// Staged right-hand side t (b x k per problem):
-//   FWD     (i > 0)      t = in_i + L_{i,i-1} out_{i-1}
-//   BWD                  t = C_i out_{i+1} = -L_{i,i+1} out_{i+1}
-//   ADJ_BWD (i < nx-1)   t = in_i + L_{i+1,i}^T out_{i+1}
-// Grid (ceil(b k / blockDim), active problems): problem f =
-// active_problem(amap, blockIdx.y), 32-bit indices within the problem.
-template <typename T, int MODE>
-__global__ void sweep_rhs_kernel(OpView op, int i, int k, const C_t<T>* in, const C_t<T>* out,
-                                 C_t<T>* __restrict__ tbuf, size_t tstride,
-                                 const int* __restrict__ amap) {
-  using C = C_t<T>;
-  const int b = op.b, q = op.q;
-  const size_t NK = (size_t)op.n * k;
-  const int f = active_problem(amap, blockIdx.y);
-  {
-    const int rem = blockIdx.x * blockDim.x + threadIdx.x;
-    if (rem >= b * k) return;
-    const int m = rem / k, j = rem - m * k;
-    const C* outf = out + (size_t)f * NK;
-    size_t row = (size_t)i * b + m;
-    C v = czero<C>();
-    if (MODE == FWD) {
-      v = in[(size_t)f * NK + row * k + j];
-      int iy = m / q;
-      const size_t cf = row * op.S;
-      for (int dy = -1; dy <= 1; ++dy) {
-        int jy = nbr_y(iy, dy, op.ny, op.periodic);
-        if (jy < 0) continue;
-        for (int cp = 0; cp < q; ++cp) {
-          T a = coefv<T>(op, cf + slotv(-1, dy) * q + cp);
-          if (a != (T)0) v = crfma(a, outf[((size_t)(i - 1) * b + jy * q + cp) * k + j], v);
-        }
-      }
-    } else if (MODE == BWD) {
-      int iy = m / q;
-      const size_t cf = row * op.S;
-      for (int dy = -1; dy <= 1; ++dy) {
-        int jy = nbr_y(iy, dy, op.ny, op.periodic);
-        if (jy < 0) continue;
-        for (int cp = 0; cp < q; ++cp) {
-          T a = coefv<T>(op, cf + slotv(1, dy) * q + cp);
-          if (a != (T)0) v = crfma(-a, outf[((size_t)(i + 1) * b + jy * q + cp) * k + j], v);
-        }
-      }
-    } else {
-      v = in[(size_t)f * NK + row * k + j];
-      int iym = m / q, cm = m - iym * q;
-      for (int dy = -1; dy <= 1; ++dy) {
-        int iyr = nbr_y(iym, -dy, op.ny, op.periodic);
-        if (iyr < 0) continue;
-        for (int cr = 0; cr < q; ++cr) {
-          size_t rrow = (size_t)(i + 1) * b + iyr * q + cr;
-          T a = coefv<T>(op, rrow * op.S + slotv(-1, dy) * q + cm);
-          if (a != (T)0) v = crfma(a, outf[rrow * k + j], v);
-        }
-      }
-    }
-    tbuf[(size_t)f * tstride + (size_t)m * k + j] = v;
-  }
+// Result of step s and right-hand side of step s + 1.  Per problem and tile of
+// CPL_Y grid points: o = the sum of the KS partial products in a fixed order
+// (back sweep: z_i minus it), of the tile's rows and of one point on either
+// side (recomputed, not exchanged), kept in shared memory; then
+//   t = in + L_{i,i-1} o (forward), -L_{i,i+1} o (back),
+//   t = in + L_{i-1,i}^T o (adjoint forward, stored as h too),
+//   t = h + L_{i+1,i}^T o (adjoint back)
+// for the next column i.  z goes to zh in the forward sweep, so the back sweep's
+// results (x) never overwrite a value a neighbouring tile still needs.
+// Bound: L2 latency (the partials were just written), so the coefficients and
+// inputs of the coupling are requested before the partials are summed, and a
+// thread has one element (two columns) of each phase at k <= 32.
+constexpr int CPL_Y = 4, CPL_MAXTHR = 512;
+inline int couple_threads(int q, int k) {
+  return std::min(CPL_MAXTHR, ((CPL_Y + 2) * q * (k / 2) + 31) & ~31);
 }
 
-// h_{i+1} -= C_i^H t, i.e. h_{i+1}[c] += sum_m L[(i,m),(i+1,c)] t[m] (L real).
-// Grid (ceil(b k / blockDim), F) as sweep_rhs_kernel.
-template <typename T>
-__global__ void adj_couple_kernel(OpView op, int i, int k, const C_t<T>* __restrict__ tbuf,
-                                  size_t tstride, C_t<T>* h, const int* __restrict__ amap) {
-  using C = C_t<T>;
-  const int b = op.b, q = op.q;
-  const size_t NK = (size_t)op.n * k;
-  const int f = active_problem(amap, blockIdx.y);
-  {
-    const int rem = blockIdx.x * blockDim.x + threadIdx.x;
-    if (rem >= b * k) return;
-    const int c = rem / k, j = rem - c * k;
-    const int iyc = c / q, cc = c - iyc * q;
-    const C* tf = tbuf + (size_t)f * tstride;
-    size_t idx = (size_t)f * NK + ((size_t)(i + 1) * b + c) * k + j;
-    C v = h[idx];
-    for (int dy = -1; dy <= 1; ++dy) {
-      int iym = nbr_y(iyc, -dy, op.ny, op.periodic);
-      if (iym < 0) continue;
-      for (int cm = 0; cm < q; ++cm) {
-        int m = iym * q + cm;
-        T a = coefv<T>(op, ((size_t)i * b + m) * op.S + slotv(1, dy) * q + cc);
-        if (a != (T)0) v = crfma(a, tf[(size_t)m * k + j], v);
-      }
-    }
-    h[idx] = v;
-  }
-}
-
-// Asynchronous global->shared copy of one complex element (cp.async;
-// zero-filled when pred is false).
-template <typename C>
-__device__ __forceinline__ void cp_async_elem(C* smem, const C* gmem, bool pred) {
-  const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-  if constexpr (sizeof(C) == 16) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem),
-                 "r"(pred ? 16 : 0));
-  } else {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(s), "l"(gmem),
-                 "r"(pred ? 8 : 0));
-  }
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
-}
-
-// acc[r][j] = sum_m op(G)[r][m] rhs[m][j] with op = identity or conjugate
-// transpose.  rhs is b x k (row stride k) at rhs + f * rstride.  The
-// contraction is staged through ST shared-memory stages filled by cp.async
-// while the previous stage is consumed; each thread owns a 4 x 2 register
-// tile of the RT x kp output.  Epilogue: store to block ob of out, subtract
-// from it, or store to the staging block tmp.
-template <typename T, bool TRANS, int EPI, int KC, int ST>
-__global__ void __launch_bounds__(SW_THREADS)
-sweep_step_kernel(int b, int k, int kp, int RT, size_t NK, int ob,
-                  const C_t<T>* __restrict__ Mat, size_t mstride, const C_t<T>* rhs,
-                  size_t rstride, C_t<T>* out, C_t<T>* tmp, size_t tstride) {
-  using C = C_t<T>;
+template <bool TRANS>
+__global__ void __launch_bounds__(CPL_MAXTHR)
+sweep_couple_kernel(OpView op, int s, int F, int k, int KS, const float2* __restrict__ part,
+                    const float2* __restrict__ in, float2* x, float2* zh,
+                    float2* __restrict__ tbuf, const int* __restrict__ amap) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* base = reinterpret_cast<C*>(smem_raw);
-  const int ms_elems = TRANS ? KC * (RT + 1) : RT * (KC + 1);
-  const int stage_elems = ms_elems + KC * kp;
-  const int f = blockIdx.y;
-  const int r0 = blockIdx.x * RT;
-  const C* Mf = Mat + (size_t)f * mstride;
-  const C* rf = rhs + (size_t)f * rstride;
-  const int tid = threadIdx.x;
-  const int TX = kp >> 1, TY = SW_THREADS / TX;
-  const int tx = tid % TX, ty = tid / TX;
-
-  auto load_stage = [&](int stage, int m0) {
-    C* Ms = base + stage * stage_elems;
-    C* Ts = Ms + ms_elems;
-    if (!TRANS) {
-      for (int e = tid; e < RT * KC; e += SW_THREADS) {
-        int rr = e / KC, mm = e - rr * KC;
-        int r = r0 + rr, m = m0 + mm;
-        bool ok = r < b && m < b;
-        cp_async_elem(&Ms[rr * (KC + 1) + mm], ok ? Mf + (size_t)r * b + m : Mf, ok);
-      }
-    } else {
-      for (int e = tid; e < RT * KC; e += SW_THREADS) {
-        int mm = e / RT, rr = e - mm * RT;
-        int r = r0 + rr, m = m0 + mm;
-        bool ok = r < b && m < b;
-        cp_async_elem(&Ms[mm * (RT + 1) + rr], ok ? Mf + (size_t)m * b + r : Mf, ok);
-      }
-    }
-    for (int e = tid; e < KC * kp; e += SW_THREADS) {
-      int mm = e / kp, j = e - mm * kp;
-      int m = m0 + mm;
-      bool ok = m < b && j < k;
-      cp_async_elem(&Ts[mm * kp + j], ok ? rf + (size_t)m * k + j : rf, ok);
-    }
+  float4* o = reinterpret_cast<float4*>(smem_raw);  // [(CPL_Y + 2) q][k / 2]
+  const int b = op.b, q = op.q, ny = op.ny, nx = op.nx, P = k >> 1;
+  const int f = active_problem(amap, blockIdx.y);
+  const int y0 = blockIdx.x * CPL_Y, npt = min(CPL_Y, ny - y0);
+  const size_t NK = (size_t)op.n * k, total = (size_t)F * b * k;
+  const int i = sweep_col(s, nx);
+  const bool last = s == 2 * nx - 2, fwd = s + 1 < nx;
+  const int i1 = last ? i : sweep_col(s + 1, nx);
+  const float* cb = op.coef32 + (size_t)(!TRANS ? i1 : fwd ? i1 - 1 : i1 + 1) * b * op.S;
+  // (h_0 is the input itself: no forward step stores it)
+  const float4* src = reinterpret_cast<const float4*>((fwd || i1 == 0 ? in : zh) + (size_t)f * NK +
+                                                      (size_t)i1 * b * k);
+  struct Term {
+    float cf[3][4];
+    float4 t;
   };
-
-  C acc[4][2];
+  auto load_term = [&](Term& w, int e) {
+    const int lrow = e / P, jp = e - lrow * P;
+    const int lp = lrow / q, c = lrow - lp * q, iy = y0 + lp, m = iy * q + c;
+    w.t = TRANS || fwd ? src[m * P + jp] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = czero<C>();
-
-  const int nch = (b + KC - 1) / KC;
-#pragma unroll
-  for (int s = 0; s < ST - 1; ++s) {
-    if (s < nch) load_stage(s, s * KC);
-    cp_async_commit();
-  }
-  for (int c = 0; c < nch; ++c) {
-    cp_async_wait<ST - 2>();
-    __syncthreads();
-    if (c + ST - 1 < nch) load_stage((c + ST - 1) % ST, (c + ST - 1) * KC);
-    cp_async_commit();
-    const C* Ms = base + (c % ST) * stage_elems;
-    const C* Ts = Ms + ms_elems;
-#pragma unroll 4
-    for (int mm = 0; mm < KC; ++mm) {
-      C a[4], bv[2];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        a[i] = TRANS ? cconj(Ms[mm * (RT + 1) + ty + TY * i]) : Ms[(ty + TY * i) * (KC + 1) + mm];
-      bv[0] = Ts[mm * kp + tx];
-      bv[1] = Ts[mm * kp + tx + TX];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        acc[i][0] = cfma(a[i], bv[0], acc[i][0]);
-        acc[i][1] = cfma(a[i], bv[1], acc[i][1]);
-      }
-    }
-  }
-  cp_async_wait<0>();
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int r = r0 + ty + TY * i;
-    if (r >= b) continue;
-#pragma unroll
-    for (int jj = 0; jj < 2; ++jj) {
-      int j = tx + TX * jj;
-      if (j >= k) continue;
-      if (EPI == EPI_TMP) {
-        tmp[(size_t)f * tstride + (size_t)r * k + j] = acc[i][jj];
-      } else {
-        size_t idx = (size_t)f * NK + ((size_t)ob * b + r) * k + j;
-        if (EPI == EPI_STORE) out[idx] = acc[i][jj];
-        else out[idx] = csub(out[idx], acc[i][jj]);
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Tensor-core sweep step (complex FP32 factors, tcgen05 kind::tf32).
-//
-// The complex product acc = op(G) t (128 rows of G per CTA, all k columns)
-// is one real GEMM: the interleaved rows of op(G) are the K-major A operand
-// (K = 2 * 32 reals per chunk) and the right-hand side chunk is expanded to
-// the 2k x 64 real matrix Bt with rows (Re t, -Im t, ...) and (Im t, Re t, ...),
-// so D = A Bt^T holds (Re, Im) pairs of the complex result.  FP32 accuracy
-// comes from splitting every operand into a round-to-nearest TF32 part and
-// its remainder, A Bt ~ Ahi Bhi + Ahi Blo + Alo Bhi (3 MMAs per K step).
-// Raw tiles arrive by cp.async (double-buffered); one thread issues the MMAs
-// into a TMEM accumulator and commits them to an mbarrier; warps 0-3 read the
-// 128 x 2k accumulator back with tcgen05.ld.  Waits are bounded: on timeout
-// the kernel sets *err, drains its copies, frees TMEM and returns.
-constexpr int TC_RT = 128, TC_KC = 32, TC_THREADS = 256;
-constexpr uint32_t TC_LBO = 128, TC_SBO = 2048;   // 64 reals of K per 8-row group
-constexpr uint32_t TC_WAIT_TRIES = 1u << 22;
-
-__host__ __device__ constexpr size_t tc_smem_bytes(int kp, bool trans) {
-  return 2 * 32768 + 2 * (size_t)(2 * kp / 8) * TC_SBO +
-         2 * (size_t)((trans ? TC_KC * (TC_RT + 1) : TC_RT * (TC_KC + 1)) + TC_KC * kp) * 8;
-}
-
-template <bool TRANS, int EPI>
-__global__ void __launch_bounds__(TC_THREADS, 1)
-sweep_tc_kernel(int b, int k, int kp, size_t NK, int ob, const float2* __restrict__ Mat,
-                size_t mstride, const float2* rhs, size_t rstride, float2* out, float2* tmp,
-                size_t tstride, int* err) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint64_t mbar;
-  __shared__ uint32_t tmem_base;
-  __shared__ int s_ok;
-  const int N = 2 * kp;
-  const uint32_t bt_bytes = (uint32_t)(N / 8) * TC_SBO;
-  // operand tiles start on a 1 KB boundary (the launch adds 1 KB of slack)
-  unsigned char* A_hi = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  unsigned char* A_lo = A_hi + 32768;
-  unsigned char* B_hi = A_lo + 32768;
-  unsigned char* B_lo = B_hi + bt_bytes;
-  float2* raw = reinterpret_cast<float2*>(B_lo + bt_bytes);
-  const int raw_ms = TRANS ? TC_KC * (TC_RT + 1) : TC_RT * (TC_KC + 1);
-  const int raw_elems = raw_ms + TC_KC * kp;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int f = blockIdx.y;
-  const int r0 = blockIdx.x * TC_RT;
-  const float2* Mf = Mat + (size_t)f * mstride;
-  const float2* rf = rhs + (size_t)f * rstride;
-  const uint32_t ncols = N <= 32 ? 32u : (N <= 64 ? 64u : 128u);
-
-  if (warp == 0) tc::tmem_alloc(&tmem_base, ncols);
-  if (tid == 0) {
-    tc::mbar_init(&mbar, 1);
-    s_ok = 1;
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = tmem_base;
-
-  auto load_raw = [&](int stage, int m0) {
-    float2* Ms = raw + stage * raw_elems;
-    float2* Ts = Ms + raw_ms;
-    if (!TRANS) {
-      for (int e = tid; e < TC_RT * TC_KC; e += TC_THREADS) {
-        int rr = e / TC_KC, mm = e - rr * TC_KC;
-        int r = r0 + rr, m = m0 + mm;
-        bool ok = r < b && m < b;
-        cp_async_elem(&Ms[rr * (TC_KC + 1) + mm], ok ? Mf + (size_t)r * b + m : Mf, ok);
-      }
-    } else {
-      for (int e = tid; e < TC_RT * TC_KC; e += TC_THREADS) {
-        int mm = e / TC_RT, rr = e - mm * TC_RT;
-        int r = r0 + rr, m = m0 + mm;
-        bool ok = r < b && m < b;
-        cp_async_elem(&Ms[mm * (TC_RT + 1) + rr], ok ? Mf + (size_t)m * b + r : Mf, ok);
-      }
-    }
-    for (int e = tid; e < TC_KC * kp; e += TC_THREADS) {
-      int mm = e / kp, j = e - mm * kp;
-      int m = m0 + mm;
-      bool ok = m < b && j < k;
-      cp_async_elem(&Ts[mm * kp + j], ok ? rf + (size_t)m * k + j : rf, ok);
-    }
-  };
-
-  const int nch = (b + TC_KC - 1) / TC_KC;
-  const uint32_t idesc = tc::idesc_tf32(TC_RT, N);
-  load_raw(0, 0);
-  cp_async_commit();
-  for (int c = 0; c < nch; ++c) {
-    cp_async_wait<0>();
-    __syncthreads();
-    if (c + 1 < nch) load_raw((c + 1) & 1, (c + 1) * TC_KC);
-    cp_async_commit();
-    if (c > 0) {  // the MMAs of chunk c-1 still read the operand tiles
-      if (tid == 0 && !tc::mbar_wait(&mbar, (c - 1) & 1, TC_WAIT_TRIES)) s_ok = 0;
-      __syncthreads();
-      if (!s_ok) break;
-      tc::fence_after_sync();
-    }
-    const float2* Ms = raw + (c & 1) * raw_elems;
-    const float2* Ts = Ms + raw_ms;
-    for (int it = tid; it < TC_RT * 16; it += TC_THREADS) {
-      const int r = it % TC_RT, p = it / TC_RT;
-      float2 g0, g1;
+    for (int d = -1; d <= 1; ++d) {
+      int off, stride = 1;
+      bool ok = true;
       if (!TRANS) {
-        g0 = Ms[r * (TC_KC + 1) + 2 * p];
-        g1 = Ms[r * (TC_KC + 1) + 2 * p + 1];
+        off = m * op.S + ((fwd ? 0 : 6) + d + 1) * q;
       } else {
-        g0 = Ms[(2 * p) * (TC_RT + 1) + r];
-        g1 = Ms[(2 * p + 1) * (TC_RT + 1) + r];
-        g0.y = -g0.y;
-        g1.y = -g1.y;
+        const int jy = nbr_y(iy, -d, ny, op.periodic);
+        ok = jy >= 0;
+        off = jy * q * op.S + ((fwd ? 6 : 0) + d + 1) * q + c;
+        stride = op.S;
       }
-      float4 h, l;
-      tc::split_tf32(g0.x, h.x, l.x);
-      tc::split_tf32(g0.y, h.y, l.y);
-      tc::split_tf32(g1.x, h.z, l.z);
-      tc::split_tf32(g1.y, h.w, l.w);
-      const uint32_t off = (uint32_t)(r >> 3) * TC_SBO + (uint32_t)p * TC_LBO + (uint32_t)(r & 7) * 16;
-      *reinterpret_cast<float4*>(A_hi + off) = h;
-      *reinterpret_cast<float4*>(A_lo + off) = l;
-    }
-    for (int it = tid; it < kp * 16; it += TC_THREADS) {
-      const int j = it % kp, p = it / kp;
-      const float2 t0 = Ts[(2 * p) * kp + j], t1 = Ts[(2 * p + 1) * kp + j];
-      float4 h0, l0, h1, l1;
-      tc::split_tf32(t0.x, h0.x, l0.x);
-      tc::split_tf32(-t0.y, h0.y, l0.y);
-      tc::split_tf32(t1.x, h0.z, l0.z);
-      tc::split_tf32(-t1.y, h0.w, l0.w);
-      h1 = make_float4(-h0.y, h0.x, -h0.w, h0.z);
-      l1 = make_float4(-l0.y, l0.x, -l0.w, l0.z);
-      const int n0 = 2 * j, n1 = 2 * j + 1;
-      const uint32_t o0 = (uint32_t)(n0 >> 3) * TC_SBO + (uint32_t)p * TC_LBO + (uint32_t)(n0 & 7) * 16;
-      const uint32_t o1 = (uint32_t)(n1 >> 3) * TC_SBO + (uint32_t)p * TC_LBO + (uint32_t)(n1 & 7) * 16;
-      *reinterpret_cast<float4*>(B_hi + o0) = h0;
-      *reinterpret_cast<float4*>(B_lo + o0) = l0;
-      *reinterpret_cast<float4*>(B_hi + o1) = h1;
-      *reinterpret_cast<float4*>(B_lo + o1) = l1;
-    }
-    tc::fence_async_smem();
-    __syncthreads();
-    if (tid == 0) {
-      tc::fence_after_sync();
-      const uint32_t a_hi = tc::smem_u32(A_hi), a_lo = tc::smem_u32(A_lo);
-      const uint32_t b_hi = tc::smem_u32(B_hi), b_lo = tc::smem_u32(B_lo);
 #pragma unroll
-      for (int prod = 0; prod < 3; ++prod) {
-        const uint32_t ab = prod == 2 ? a_lo : a_hi;
-        const uint32_t bb = prod == 1 ? b_lo : b_hi;
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-          const uint64_t ad = tc::smem_desc(ab + ks * 2 * TC_LBO, TC_LBO, TC_SBO);
-          const uint64_t bd = tc::smem_desc(bb + ks * 2 * TC_LBO, TC_LBO, TC_SBO);
-          tc::mma_tf32(tmem, ad, bd, idesc, (c > 0 || prod > 0 || ks > 0) ? 1u : 0u);
-        }
-      }
-      tc::mma_commit(&mbar);
-    }
-  }
-  cp_async_wait<0>();
-  if (s_ok) {
-    if (tid == 0 && !tc::mbar_wait(&mbar, (nch - 1) & 1, TC_WAIT_TRIES)) s_ok = 0;
-    __syncthreads();
-  }
-  tc::fence_after_sync();
-  if (s_ok && warp < 4) {
-    const int r = r0 + warp * 32 + lane;
-    for (int cc = 0; cc < N / 16; ++cc) {
-      float v[16];
-      tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(cc * 16), v);
-      if (r >= b) continue;
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const int j = cc * 8 + t;
-        if (j >= k) continue;
-        const float2 a = make_float2(v[2 * t], v[2 * t + 1]);
-        if (EPI == EPI_TMP) {
-          tmp[(size_t)f * tstride + (size_t)r * k + j] = a;
-        } else {
-          const size_t idx = (size_t)f * NK + ((size_t)ob * b + r) * k + j;
-          if (EPI == EPI_STORE) out[idx] = a;
-          else out[idx] = csub(out[idx], a);
-        }
+      for (int cp = 0; cp < 4; ++cp) {
+        const float v = ok && cp < q ? cb[off + cp * stride] : 0.f;
+        w.cf[d + 1][cp] = !TRANS && !fwd ? -v : v;
       }
     }
+  };
+  Term w;
+  const int nown = npt * q * P;
+  if (!last && (int)threadIdx.x < nown) load_term(w, threadIdx.x);
+  const float4* pf = reinterpret_cast<const float4*>(part + (size_t)f * b * k);
+  float4* xi = reinterpret_cast<float4*>(x + (size_t)f * NK + (size_t)i * b * k);
+  float4* zi = reinterpret_cast<float4*>(zh + (size_t)f * NK + (size_t)i * b * k);
+  for (int e = threadIdx.x; e < (npt + 2) * q * P; e += blockDim.x) {
+    const int lrow = e / P, jp = e - lrow * P;
+    const int lp = lrow / q, c = lrow - lp * q;
+    int y = y0 - 1 + lp;
+    const bool own = lp >= 1 && lp <= npt;
+    if (op.periodic) y = (y + ny) % ny;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (y >= 0 && y < ny) {
+      const int e0 = (y * q + c) * P + jp;
+      float4 z = v;
+      if (!TRANS && s >= nx) z = zi[e0];
+#pragma unroll 4
+      for (int t = 0; t < KS; ++t) {
+        const float4 u = pf[(size_t)t * (total >> 1) + e0];
+        v.x += u.x;
+        v.y += u.y;
+        v.z += u.z;
+        v.w += u.w;
+      }
+      if (!TRANS && s >= nx) v = make_float4(z.x - v.x, z.y - v.y, z.z - v.z, z.w - v.w);
+      if (own) {
+        if (!TRANS && s < nx) zi[e0] = v;
+        if (s >= nx - 1) xi[e0] = v;
+      }
+    }
+    o[e] = v;
   }
-  if (!s_ok && tid == 0) atomicExch(err, 1);
-  tc::fence_before_sync();
+  if (last) return;
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, ncols);
+  float4* h = reinterpret_cast<float4*>(zh + (size_t)f * NK + (size_t)i1 * b * k);
+  float4* tf = reinterpret_cast<float4*>(tbuf + (size_t)f * b * k);
+  for (int e = threadIdx.x; e < nown; e += blockDim.x) {
+    if (e != (int)threadIdx.x) load_term(w, e);
+    const int lrow = e / P, jp = e - lrow * P;
+    const int lp = lrow / q, m = (y0 + lp) * q + lrow - lp * q;
+    float4 t = w.t;
+#pragma unroll
+    for (int d = -1; d <= 1; ++d) {
+      const float4* ov = o + ((lp + 1 + (TRANS ? -d : d)) * q) * P + jp;
+#pragma unroll
+      for (int cp = 0; cp < 4; ++cp) {
+        if (cp >= q) break;
+        const float4 u = ov[cp * P];
+        const float a = w.cf[d + 1][cp];
+        t.x = fmaf(a, u.x, t.x);
+        t.y = fmaf(a, u.y, t.y);
+        t.z = fmaf(a, u.z, t.z);
+        t.w = fmaf(a, u.w, t.w);
+      }
+    }
+    if (TRANS && fwd) h[m * P + jp] = t;
+    tf[m * P + jp] = t;
+  }
 }
 
 // ---------------------------------------------------------------------------
 // Tensor-core sweep step fed by TMA, with the contraction split over KS CTAs.
 //
-// Same arithmetic as sweep_tc_kernel, on chunks of 16 complex columns.  The
-// raw 128 x 16 complex tiles of G_i (or of G_i^H) arrive by 3-D TMA (one
+// The complex product acc = op(G) t (128 rows of G per item, all k columns) is
+// one real GEMM: the interleaved rows of op(G) are the K-major A operand and the
+// right-hand side is expanded to the real matrix B~ with rows (Re t, -Im t, ...)
+// and (Im t, Re t, ...), so D = A B~^T holds (Re, Im) pairs.  FP32 accuracy
+// comes from splitting every operand (TF32 part and remainder, or BF16
+// pieces).  Chunks of 16 complex columns: the raw 128 x 16 complex tiles of G_i (or of G_i^H) arrive by 3-D TMA (one
 // tensor map over all factors, coordinate 2 = problem * nx + column), and the
 // matching 16 right-hand-side rows by a 1-D bulk copy, into a 4-stage ring
 // guarded by mbarriers.  The split into TF32 hi/lo operand tiles is
 // double-buffered so the tensor core works on chunk c while the threads
 // split chunk c+1.  CTA (row tile, part) handles the chunks
 // [part*cpp, (part+1)*cpp) and writes a partial 128 x k block;
-// sweep_combine_kernel adds the KS partials in a fixed order and applies the
-// step's epilogue.  All waits are bounded (flag *err).
+// sweep_couple_kernel adds the KS partials in a fixed order.  All waits are bounded (flag *err).
+constexpr int TC_RT = 128;                                // rows of an item
+constexpr uint32_t TC_LBO = 128;
+constexpr uint32_t TC_WAIT_TRIES = 1u << 22;
 constexpr int TC2_KC = 16;                                // complex columns per chunk
 constexpr int TC2_STAGES = 4;
-constexpr uint32_t TC2_SBO = 1024;                        // 32 reals of K per 8-row group
 constexpr uint32_t TC2_TILE_BYTES = TC_RT * TC2_KC * 8;   // 16 KB raw tile
-constexpr uint32_t TC2_A_BYTES = TC_RT * 2 * TC2_KC * 4;  // 16 KB operand tile
 
 __host__ __device__ constexpr uint32_t tc2_stage_bytes(int kp) {
   return (TC2_TILE_BYTES + (uint32_t)TC2_KC * kp * 8 + 1023u) & ~1023u;
@@ -728,31 +446,6 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
   if (warp == 0) tc::tmem_dealloc(tmem, ncols);
 }
 
-// Sum the KS partial products in a fixed order and apply the step epilogue.
-// Grid (ceil(b k / blockDim), active problems): problem f =
-// active_problem(amap, blockIdx.y).
-template <int EPI>
-__global__ void sweep_combine_kernel(int F, int b, int k, int KS, size_t NK, int ob,
-                                     const float2* __restrict__ part, float2* out, float2* tmp,
-                                     size_t tstride, const int* __restrict__ amap) {
-  const size_t total = (size_t)F * b * k;
-  const int f = active_problem(amap, blockIdx.y);
-  {
-    const int rem = blockIdx.x * blockDim.x + threadIdx.x;
-    if (rem >= b * k) return;
-    const size_t e = (size_t)f * b * k + rem;
-    float2 s = part[e];
-    for (int q = 1; q < KS; ++q) s = cadd(s, part[(size_t)q * total + e]);
-    if (EPI == EPI_TMP) {
-      tmp[(size_t)f * tstride + rem] = s;
-    } else {
-      const size_t idx = (size_t)f * NK + (size_t)ob * b * k + rem;
-      if (EPI == EPI_STORE) out[idx] = s;
-      else out[idx] = csub(out[idx], s);
-    }
-  }
-}
-
 // One launch of the TMA-fed tensor-core sweep step in the factors' operand
 // split (partial products into Pbuf).
 template <bool TRANS, int SPLIT, typename C>
@@ -786,215 +479,96 @@ bool sweep_tc2_ok(const rr_factors* fa, int k) {
 
 namespace {
 
-template <typename T> struct SweepCfg;
-template <> struct SweepCfg<float> { static constexpr int KC = 32, ST = 3; };
-template <> struct SweepCfg<double> { static constexpr int KC = 16, ST = 2; };
-
-template <typename T, bool TRANS, int EPI>
-rr_status gemm_step(rr_factors* fa, int k, int kp, int RT, int ob, int blk, const C_t<T>* Mat,
-                    size_t mstride, const C_t<T>* rhs, size_t rstride, C_t<T>* out, C_t<T>* tmp,
-                    size_t tstride) {
-  using C = C_t<T>;
-  constexpr int KC = SweepCfg<T>::KC, ST = SweepCfg<T>::ST;
-  const OpDev& d = fa->op->d;
-  const int b = d.b, F = fa->F, Fa = active_count(fa);
-  const size_t NK = (size_t)d.n * k;
-  cudaStream_t st = fa->stream;
-  if constexpr (std::is_same<T, float>::value) {
-    if (sweep_tc2_ok(fa, k)) {
-      const int nrt = (b + TC_RT - 1) / TC_RT;
-      const int nch = (b + TC2_KC - 1) / TC2_KC;
-      const int nsm = num_sms(d.device);
-      // split count: the smallest whose items fill the persistent CTAs to
-      // 85 % (each split adds a partial block to write and combine), else
-      // the best balance.  The partial buffer holds 4 F b 64 complex, so up
-      // to 256 / k splits fit; few active problems (refinement corrections)
-      // take more splits to keep the SMs busy.
-      const int ks_max = std::min(16, std::max(1, 256 / k));
-      int KS = 1;
-      double best = 0.0;
-      for (int ksc = 1; ksc <= ks_max && ksc <= nch; ++ksc) {
-        const int cppc = (nch + ksc - 1) / ksc;
-        const int ksr = (nch + cppc - 1) / cppc;
-        if (ksr > ks_max) continue;
-        const long items = (long)nrt * Fa * ksr;
-        const long waves = (items + nsm - 1) / nsm;
-        const double eff = (double)items / (double)(waves * nsm);
-        if (eff >= 0.85) {
-          KS = ksr;
-          break;
-        }
-        if (eff > best + 1e-9) { best = eff; KS = ksr; }
-      }
-      if (fa->tune_ks > 0) {  // tuned split count (at most the 4 partial buffers)
-        const int cppc = (nch + std::min(fa->tune_ks, 4) - 1) / std::min(fa->tune_ks, 4);
-        KS = (nch + cppc - 1) / cppc;
-      }
-      const int cpp = (nch + KS - 1) / KS;
-      const int nitems = nrt * Fa * KS;
-      const int grid_x = std::min(nitems, nsm);
-      const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(fa->tmap[TRANS ? 1 : 0]);
-      prof_begin(PROF_SWEEP, st);
-      rr_status ls;
-      switch (fa->prec) {
-        case RR_FP32_BF16X3:
-          ls = launch_tc2<TRANS, tc::SPLIT_BF16X3>(tm, grid_x, b, k, kp, blk, d.nx, nrt, KS, cpp,
-                                                  rhs, rstride, fa, st);
-          break;
-        case RR_FP32_BF16X6:
-          ls = launch_tc2<TRANS, tc::SPLIT_BF16X6>(tm, grid_x, b, k, kp, blk, d.nx, nrt, KS, cpp,
-                                                  rhs, rstride, fa, st);
-          break;
-        default:
-          ls = launch_tc2<TRANS, tc::SPLIT_TF32X3>(tm, grid_x, b, k, kp, blk, d.nx, nrt, KS, cpp,
-                                                  rhs, rstride, fa, st);
-      }
-      if (ls != RR_OK) return ls;
-      const dim3 cgrid((b * k + 255) / 256, Fa);
-      sweep_combine_kernel<EPI><<<cgrid, 256, 0, st>>>(
-          F, b, k, KS, NK, ob, reinterpret_cast<const float2*>(fa->Pbuf), out, tmp, tstride,
-          fa->amap);
-      prof_end(PROF_SWEEP, st);
-      prof_count(1);
-      RR_CUDA(cudaGetLastError());
-      return RR_OK;
-    }
-    if (fa->amap) {  // the active-problem list exists only on the split sweep path
-      set_error("sweep: active-problem list on a path without it");
-      return RR_ERR_ARG;
-    }
-    if (tc_prec(fa->prec) && kp <= 32) {
-      const size_t smem = tc_smem_bytes(kp, TRANS) + 1024;
-      static size_t tc_attr = 0;  // dynamic shared memory opted in so far
-      if (smem > tc_attr) {
-        RR_CUDA(cudaFuncSetAttribute(sweep_tc_kernel<TRANS, EPI>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        tc_attr = smem;
-      }
-      dim3 grid((b + TC_RT - 1) / TC_RT, F);
-      prof_begin(PROF_SWEEP, st);
-      sweep_tc_kernel<TRANS, EPI><<<grid, TC_THREADS, smem, st>>>(
-          b, k, kp, NK, ob, Mat, mstride, rhs, rstride, out, tmp, tstride, fa->flag + F);
-      prof_end(PROF_SWEEP, st);
-      cudaError_t le = cudaGetLastError();
-      if (le != cudaSuccess) {
-        cudaFuncAttributes fat;
-        cudaFuncGetAttributes(&fat, sweep_tc_kernel<TRANS, EPI>);
-        char buf[256];
-        snprintf(buf, sizeof buf,
-                 "sweep_tc launch (grid %u x %u, smem %zu, static %zu, max dyn %d, regs %d, "
-                 "max threads %d): %s",
-                 grid.x, grid.y, smem, fat.sharedSizeBytes, fat.maxDynamicSharedSizeBytes,
-                 fat.numRegs, fat.maxThreadsPerBlock, cudaGetErrorString(le));
-        set_error(buf);
-        return RR_ERR_CUDA;
-      }
-      return RR_OK;
+// Split count of a product: the smallest whose items fill the persistent CTAs to
+// 85 % (each split adds a partial block to write and sum), else the best
+// balance.  The partial buffer holds 4 F b 64 complex, so up to 256 / k splits
+// fit; few active problems (refinement corrections) take more splits to keep
+// the SMs busy.
+int split_count(const rr_factors* fa, int k, int nrt, int nch, int nsm) {
+  if (fa->tune_ks > 0) {  // tuned (at most the 4 partial buffers)
+    const int cpp = (nch + std::min(fa->tune_ks, 4) - 1) / std::min(fa->tune_ks, 4);
+    return (nch + cpp - 1) / cpp;
+  }
+  const int ks_max = std::min(16, std::max(1, 256 / k));
+  int KS = 1;
+  double best = 0.0;
+  for (int ksc = 1; ksc <= ks_max && ksc <= nch; ++ksc) {
+    const int cpp = (nch + ksc - 1) / ksc;
+    const int ksr = (nch + cpp - 1) / cpp;
+    if (ksr > ks_max) continue;
+    const long items = (long)nrt * active_count(fa) * ksr;
+    const long waves = (items + nsm - 1) / nsm;
+    const double eff = (double)items / (double)(waves * nsm);
+    if (eff >= 0.85) return ksr;
+    if (eff > best + 1e-9) {
+      best = eff;
+      KS = ksr;
     }
   }
-  static bool attr_set = false;
-  if (!attr_set) {
-    RR_CUDA(cudaFuncSetAttribute(sweep_step_kernel<T, TRANS, EPI, KC, ST>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    attr_set = true;
-  }
-  const size_t ms_elems = TRANS ? (size_t)KC * (RT + 1) : (size_t)RT * (KC + 1);
-  const size_t smem = (size_t)ST * (ms_elems + (size_t)KC * kp) * sizeof(C);
-  dim3 grid((b + RT - 1) / RT, F);
-  prof_begin(PROF_SWEEP, st);
-  sweep_step_kernel<T, TRANS, EPI, KC, ST><<<grid, SW_THREADS, smem, st>>>(
-      b, k, kp, RT, NK, ob, Mat, mstride, rhs, rstride, out, tmp, tstride);
-  prof_end(PROF_SWEEP, st);
-  return RR_OK;
+  return KS;
 }
 
-template <typename T, int MODE>
-void stage_rhs(rr_factors* fa, int i, int k, const C_t<T>* in, const C_t<T>* out, C_t<T>* tb) {
+template <bool TRANS>
+rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* zh) {
   const OpDev& d = fa->op->d;
-  const dim3 grid((d.b * k + 255) / 256, active_count(fa));
-  prof_count(1);
-  sweep_rhs_kernel<T, MODE><<<grid, 256, 0, fa->stream>>>(view(d), i, k, in, out, tb,
-                                                          (size_t)d.b * k, fa->amap);
-}
-
-template <typename T>
-rr_status solve_impl(rr_factors* fa, int k, int adjoint, const void* bv, void* xv, void* tmpv) {
-  using C = C_t<T>;
-  const OpDev& d = fa->op->d;
-  const int b = d.b, nx = d.nx, F = fa->F;
+  const int b = d.b, nx = d.nx, F = fa->F, Fa = active_count(fa);
   int kp = 8;
   while (kp < k) kp <<= 1;
-  const int RT = 2048 / kp;
-  const size_t bb = (size_t)b * b;
-  const size_t NK = (size_t)d.n * k;
-  const C* G = reinterpret_cast<const C*>(fa->G);
-  const size_t gstride = (size_t)nx * bb;
-  const C* bin = reinterpret_cast<const C*>(bv);
-  C* x = reinterpret_cast<C*>(xv);
-  C* tb = reinterpret_cast<C*>(fa->Tbuf);                     // [F][b][k]
-  C* tb2 = tb + (size_t)F * b * 64;                           // [F][b][k]
-  const size_t tstride = (size_t)b * k;
-  rr_status s;
-  if (!adjoint) {
-    for (int i = 0; i < nx; ++i) {
-      const C* rhs = bin;
-      size_t rstride = NK;
-      if (i > 0) {
-        stage_rhs<T, FWD>(fa, i, k, bin, x, tb);
-        rhs = tb;
-        rstride = tstride;
-      }
-      if ((s = gemm_step<T, false, EPI_STORE>(fa, k, kp, RT, i, i, G + i * bb, gstride, rhs, rstride,
-                                             x, nullptr, 0)) != RR_OK)
-        return s;
+  cudaStream_t st = fa->stream;
+  float2* tb = reinterpret_cast<float2*>(fa->Tbuf);  // [F][b][k]
+  const int nrt = (b + TC_RT - 1) / TC_RT, nch = (b + TC2_KC - 1) / TC2_KC;
+  const int nsm = num_sms(d.device);
+  const int KS = split_count(fa, k, nrt, nch, nsm), cpp = (nch + KS - 1) / KS;
+  const int grid_x = std::min(nrt * Fa * KS, nsm);
+  const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(fa->tmap[TRANS ? 1 : 0]);
+  const dim3 cgrid((d.ny + CPL_Y - 1) / CPL_Y, Fa);
+  const size_t csmem = (size_t)(CPL_Y + 2) * d.q * k * sizeof(float2);
+  for (int s = 0; s < 2 * nx - 1; ++s) {
+    const float2* rhs = s == 0 ? in : tb;
+    const size_t rstride = s == 0 ? (size_t)d.n * k : (size_t)b * k;
+    const int blk = sweep_col(s, nx);
+    prof_begin(PROF_SWEEP, st);
+    rr_status ls;
+    switch (fa->prec) {
+      case RR_FP32_BF16X3:
+        ls = launch_tc2<TRANS, tc::SPLIT_BF16X3>(tm, grid_x, b, k, kp, blk, nx, nrt, KS, cpp, rhs,
+                                                rstride, fa, st);
+        break;
+      case RR_FP32_BF16X6:
+        ls = launch_tc2<TRANS, tc::SPLIT_BF16X6>(tm, grid_x, b, k, kp, blk, nx, nrt, KS, cpp, rhs,
+                                                rstride, fa, st);
+        break;
+      default:
+        ls = launch_tc2<TRANS, tc::SPLIT_TF32X3>(tm, grid_x, b, k, kp, blk, nx, nrt, KS, cpp, rhs,
+                                                rstride, fa, st);
     }
-    for (int i = nx - 2; i >= 0; --i) {
-      stage_rhs<T, BWD>(fa, i, k, nullptr, x, tb);
-      if ((s = gemm_step<T, false, EPI_SUB>(fa, k, kp, RT, i, i, G + i * bb, gstride, tb, tstride, x,
-                                           nullptr, 0)) != RR_OK)
-        return s;
-    }
-  } else {
-    C* h = reinterpret_cast<C*>(tmpv);
-    if (!fa->amap) {
-      RR_CUDA(cudaMemcpyAsync(h, bin, (size_t)F * NK * sizeof(C), cudaMemcpyDeviceToDevice,
-                              fa->stream));
-    } else {
-      for (int a = 0; a < fa->Fa; ++a) {
-        const size_t o = (size_t)fa->amap_h[a] * NK;
-        RR_CUDA(cudaMemcpyAsync(h + o, bin + o, NK * sizeof(C), cudaMemcpyDeviceToDevice,
-                                fa->stream));
-      }
-    }
-    for (int i = 0; i + 1 < nx; ++i) {
-      if ((s = gemm_step<T, true, EPI_TMP>(fa, k, kp, RT, 0, i, G + i * bb, gstride,
-                                          h + (size_t)i * b * k, NK, nullptr, tb2, tstride)) !=
-          RR_OK)
-        return s;
-      prof_count(1);
-      adj_couple_kernel<T><<<dim3((b * k + 255) / 256, active_count(fa)), 256, 0, fa->stream>>>(
-          view(d), i, k, tb2, tstride, h, fa->amap);
-    }
-    for (int i = nx - 1; i >= 0; --i) {
-      const C* rhs = h + (size_t)i * b * k;
-      size_t rstride = NK;
-      if (i + 1 < nx) {
-        stage_rhs<T, ADJ_BWD>(fa, i, k, h, x, tb);
-        rhs = tb;
-        rstride = tstride;
-      }
-      if ((s = gemm_step<T, true, EPI_STORE>(fa, k, kp, RT, i, i, G + i * bb, gstride, rhs, rstride,
-                                            x, nullptr, 0)) != RR_OK)
-        return s;
-    }
+    if (ls != RR_OK) return ls;
+    sweep_couple_kernel<TRANS><<<cgrid, couple_threads(d.q, k), csmem, st>>>(
+        view(d), s, F, k, KS, reinterpret_cast<const float2*>(fa->Pbuf), in, x, zh, tb, fa->amap);
+    prof_end(PROF_SWEEP, st);
+    prof_count(1);
+    RR_CUDA(cudaGetLastError());
   }
-  RR_CUDA(cudaGetLastError());
   return RR_OK;
 }
 
 }  // namespace
 
+// FP64 factors and every FP32 shape the split tensor-core sweep does not take
+// run the whole-sweep cluster kernels.  Where both serve a shape, the one with
+// the smaller modelled time: a column step of the tensor-core sweep is two
+// launches, measured at 10 us plus the factors' bytes at 2.6 TB/s.
 rr_status launch_solve_lo(rr_factors* fa, int k, int adjoint, const void* b, void* x, void* tmp) {
-  if (fa->prec == RR_FP64) return solve_impl<double>(fa, k, adjoint, b, x, tmp);
-  return solve_impl<float>(fa, k, adjoint, b, x, tmp);
+  if (fa->prec == RR_FP64) return launch_sweep_cl64(fa, k, adjoint, b, x, tmp);
+  if (sweep_tc2_ok(fa, k)) {
+    const OpDev& d = fa->op->d;
+    const double step = 10.0 + 8.0 * active_count(fa) * d.b * d.b / 2.6e6;
+    if ((2.0 * d.nx - 1) * step < sweep_cl32_us(fa, k, adjoint))
+      return adjoint ? solve_tc2<true>(fa, k, reinterpret_cast<const float2*>(b),
+                                       reinterpret_cast<float2*>(x), reinterpret_cast<float2*>(tmp))
+                     : solve_tc2<false>(fa, k, reinterpret_cast<const float2*>(b),
+                                        reinterpret_cast<float2*>(x),
+                                        reinterpret_cast<float2*>(tmp));
+  }
+  return launch_sweep_cl32(fa, k, adjoint, b, x, tmp);
 }
