@@ -6,27 +6,27 @@
 // C_i = -L_{i,i+1} (b x b, A_i and C_i with at most 3q entries per row).  The
 // block LU is
 //     S_0 = D_0,  G_i = S_i^{-1},  X_i = G_i C_i,  S_{i+1} = D_{i+1} - A_{i+1} X_i.
-// G_i is formed explicitly by blocked Gauss-Jordan elimination with partial
-// pivoting (the block-sweep operator applied one panel of NB columns at a
-// time), so every later solve is a dense block product instead of a pair of
-// triangular solves.  Per panel K = [k0, k0+nb):
-//   panel    : pivots from an LU of the tall panel M[k0:b, K]; T = M[K,K];
-//              M[K,K] <- T^{-1};  M[I,K] <- -M[I,K] T^{-1}  (I = rows not in K)
-//   rowblock : row swaps in the other columns; B <- M[K,R] (saved);
-//              M[K,R] <- T^{-1} B
-//   update   : M[I,R] <- M[I,R] + M[I,K] B    (= D - C A^{-1} B)
-// After the last panel M = (P S)^{-1}; S^{-1} is M with its columns permuted.
+// G_i is formed explicitly, so every later solve is a dense block product
+// instead of a pair of triangular solves.  This file holds the Schur update and
+// the Gauss-Jordan inversion used for FP64 factors and for the FP32 shapes that
+// the slab form (factor_w.cu) does not take; both pivot implicitly (rows never
+// move; rowpiv[r] is the column row r pivoted for, pivslot[c] the row that
+// pivoted column c).  Per panel K of 16 columns:
+//   panel  : one cluster of CTAs per problem applies the previous panel's
+//            transformation to K and runs the 16 eliminations
+//            (gjp_panel_kernel);
+//   gather : B = M[P, :], P the panel's pivot rows, saved before they change;
+//   update : M[r, m] += M[r, K] B[:, m] (r not in P), M[P, m] = M[P, K] B[:, m]
+//            for the columns m outside K and the next panel, on all SMs beside
+//            the next panel (gjp_update_kernel).
 #include <cuda.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "rr_internal.cuh"
 #include "tc.cuh"
 
 namespace {
-
-constexpr int PANEL_THREADS = 512;
 
 __device__ __forceinline__ int slotx(int dx, int dy) { return (dx + 1) * 3 + (dy + 1); }
 
@@ -124,714 +124,343 @@ schur_kernel(OpView op, const double2* __restrict__ shifts, int i,
   }
 }
 
-// argmax reduction helper: larger value wins, lower index on ties
+// ------------------------------------------------------------------- panel
+constexpr int GP_NB = 16;       // panel width
+constexpr int GP_LPR = 4;       // lanes of a row
+constexpr int GP_CPL = GP_NB / GP_LPR;
+constexpr int GP_MAXW = 16;     // warps of a CTA: 8 rows each
+constexpr int GP_CLMAX = 8;
+
+// 16-byte pieces of a candidate row and of 1 / pivot
+template <typename T> __host__ __device__ constexpr int gp_pieces() { return GP_NB * (int)sizeof(C_t<T>) / 16; }
+// a candidate slot: the row, then 1 / pivot in one 16-byte piece
+template <typename T> __host__ __device__ constexpr int gp_slot() { return (gp_pieces<T>() + 1) * 16; }
+
+// pivot magnitude as an integer that orders like it (without its lowest five
+// bits): |x|^2 in FP32, the larger of |re| and |im| in FP64, whose high words
+// need no FP64 arithmetic (its rate is a sixty-fourth of the integer rate)
+__device__ __forceinline__ unsigned gp_mag(float2 x) {
+  return __float_as_uint(x.x * x.x + x.y * x.y) & ~31u;
+}
+__device__ __forceinline__ unsigned gp_mag(double2 x) {
+  return max((unsigned)__double2hiint(x.x) & 0x7fffffffu, (unsigned)__double2hiint(x.y) & 0x7fffffffu) &
+         ~31u;
+}
+// a magnitude above this is not a number
+template <typename T> __device__ __forceinline__ constexpr unsigned gp_inf() {
+  return sizeof(T) == 8 ? 0x7ff00000u : 0x7f800000u;
+}
+__device__ __forceinline__ float2 gp_shfl(float2 v, int src) {
+  return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+__device__ __forceinline__ double2 gp_shfl(double2 v, int src) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+
+struct PanelArgs {
+  int b, k0, nbk, kp0, rpc, CL, F;
+  int* rowpiv;    // [F][b]
+  int* pivslot;   // [F][b]
+  int* flag;      // [F] singular flags, [F] = wait timeout
+  uint32_t tries;
+};
+
 template <typename T>
-__device__ __forceinline__ void amax_merge(T& v, int& i, T v2, int i2) {
-  if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
+constexpr size_t panel_smem(int rpc, int CL) {
+  return (size_t)2 * CL * gp_slot<T>() + (size_t)2 * GP_MAXW * gp_slot<T>() +
+         (size_t)rpc * (GP_NB + 1) * sizeof(C_t<T>) + (size_t)GP_NB * GP_NB * sizeof(C_t<T>);
 }
 
-// Pivoted panel step.  The tall panel M[:, K] sits in shared memory by
-// original row ("slot"); the LU with partial pivoting over slots >= k0 never
-// moves data: each step picks the largest remaining |.|^2 of column j (lowest
-// slot on ties), marks that slot as the j-th pivot and eliminates column j
-// from the other remaining slots, with one block barrier per step (every
-// warp reduces the per-warp candidates itself).  Warp 0 then replays the
-// choices as the equivalent sequence of row interchanges (ipiv, as the row
-// block kernel applies them to the other columns) and the final position of
-// every slot, and the transformed panel is written back in that order:
-//   pivot rows  -> T^{-1} = U11^{-1} L11^{-1}
-//   rows above  -> -row T^{-1}
-//   other rows  -> -(their multipliers) L11^{-1}   (= -M[I,K] T^{-1})
-template <typename T, int NB>
-__global__ void __launch_bounds__(PANEL_THREADS)
-gj_panel_kernel(int b, int k0, int nbk, C_t<T>* __restrict__ Mall, int* __restrict__ ipiv_all,
-                int* __restrict__ perm_all, int* __restrict__ flag) {
+// Eliminates the columns K = [k0, k0 + nbk) of every row of M; CTA rank r of the
+// problem's cluster holds the rows r, r + CL, ... with four columns of K per
+// lane.  When kp0 >= 0 the panel [kp0, kp0 + 16) was factored last and its
+// transformation has reached every column but its own and K; it is applied to K
+// first, x += M[r, Kp] B (x = M[r, Kp] B in its pivot rows).  Per step: the CTA's
+// best eligible row (warp reductions and a barrier), whose warp forms 1 / pivot;
+// it goes to every CTA of the cluster (st.async, see gjw_slab_kernel for the
+// buffers' reuse); each warp picks the best of the CL candidates and eliminates.
+// Outputs: the columns K of M, rowpiv of the rows pivoted here, pivslot.
+// Bound (FP64): 20 FP64 instructions per warp and step at 64 cycles of its
+// quarter of the SM, and the step's chain.  192 rows, four problems: 1.5 us a
+// step; one CTA per problem took 243 us a panel.
+template <typename T>
+__global__ void __launch_bounds__(GP_MAXW * 32) gjp_panel_kernel(PanelArgs g, C_t<T>* __restrict__ Mall) {
   using C = C_t<T>;
-  constexpr int PS = NB + 1;  // padded row stride: column walks hit distinct banks
-  constexpr int NW = PANEL_THREADS / 32;
-  constexpr int MAXOWN = (1024 + PANEL_THREADS - 1) / PANEL_THREADS;
+  constexpr int NB = GP_NB, LPR = GP_LPR, CPL = GP_CPL, NP = gp_pieces<T>(), SLOT = gp_slot<T>();
+  constexpr int CS = sizeof(C), PPL = CPL * CS / 16;  // pieces of a lane
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* P = reinterpret_cast<C*>(smem_raw);  // [b][PS] by slot
-  __shared__ C Ui[NB][NB + 1], Li[NB][NB + 1], Ti[NB][NB + 1];
-  __shared__ T red_v[2][NW];  // per-step candidates, double buffered by step parity
-  __shared__ int red_i[2][NW];
-  __shared__ int chosen[NB];
-  __shared__ int sigK[NB];            // slot that ends at position k0 + j
-  __shared__ int nkPos[32], nkSlot[32];
-  __shared__ int s_nk;
-  __shared__ unsigned touched[32];    // positions outside K that receive another slot
-  const int tid = threadIdx.x, nt = PANEL_THREADS;
-  const int lane = tid & 31, warp = tid >> 5;
-  const int f = blockIdx.x;
+  __shared__ uint64_t mbar[2];
+  __shared__ unsigned wkey[2][32];
+  const int CL = g.CL, b = g.b, nbk = g.nbk;
+  unsigned char* cand = smem_raw;                       // [2][CL][SLOT], slot CL - 1 - rank
+  unsigned char* wst = cand + (size_t)2 * CL * SLOT;    // [2][GP_MAXW][SLOT], slot 15 - warp
+  C* As = reinterpret_cast<C*>(wst + (size_t)2 * GP_MAXW * SLOT);  // [rpc][NB + 1]
+  C* Bp = As + (size_t)g.rpc * (NB + 1);                // [NB][NB]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x;
+  const int rank = (int)tc::cluster_rank();
+  const int f = blockIdx.x / CL;
+  const int nrows = max(0, (b - rank + CL - 1) / CL);
   C* M = Mall + (size_t)f * b * b;
-  int* perm = perm_all + (size_t)f * b;
-  int* ipiv = ipiv_all + f * 32;
+  int* rowpiv = g.rowpiv + (size_t)f * b;
+  const int* pivslot = g.pivslot + (size_t)f * b;
+  const int prow = tid / LPR, cg = (tid % LPR) * CPL;
+  const bool live = prow < nrows;
+  const int grow = prow * CL + rank;
 
-  for (int e = tid; e < b * nbk; e += nt) {
-    int r = e / nbk, c = e - r * nbk;
-    P[r * PS + c] = M[(size_t)r * b + k0 + c];
+  if (tid < 2) tc::mbar_init(&mbar[tid], 1);
+  for (int e = tid; e < 64; e += nthr) wkey[e >> 5][e & 31] = 0u;  // (a CTA may be one warp)
+  const int rp = live && g.k0 > 0 ? rowpiv[grow] : -1;
+  const bool prevpiv = g.kp0 >= 0 && rp >= g.kp0 && rp < g.kp0 + NB;
+  C x[CPL];
+#pragma unroll
+  for (int c = 0; c < CPL; ++c)
+    x[c] = live && !prevpiv && cg + c < nbk ? M[(size_t)grow * b + g.k0 + cg + c] : czero<C>();
+  if (g.kp0 >= 0) {
+    for (int e = tid; e < nrows * NB; e += nthr) {
+      const int r = e / NB, j = e - r * NB;
+      As[r * (NB + 1) + j] = M[(size_t)(r * CL + rank) * b + g.kp0 + j];
+    }
+    for (int e = tid; e < NB * NB; e += nthr) {
+      const int j = e / NB, c = e - j * NB;
+      Bp[e] = c < nbk ? M[(size_t)pivslot[g.kp0 + j] * b + g.k0 + c] : czero<C>();
+    }
   }
-  if (tid < 32) touched[tid] = 0u;
-  unsigned done = 0u;  // bit t: slot k0 + tid + t*nt already pivoted
-  __syncthreads();
+  // barriers initialised, and every CTA's reads of M done before any CTA writes
+  tc::cluster_sync();
+  if (g.kp0 >= 0 && live) {
+#pragma unroll 4
+    for (int j = 0; j < NB; ++j) {
+      const C a = As[prow * (NB + 1) + j];
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) x[c] = cfma(a, Bp[j * NB + cg + c], x[c]);
+    }
+  }
+  bool elig = live && rp < 0;
+  int mypiv = -1;
+  bool singular = false, ok = true;
 
-  for (int j = 0; j < nbk; ++j) {
-    T bv = (T)-1;
-    int bi = b;
+  // the CTA's candidate: warp w sends its pieces to the CTAs w, w + W, ...
+  const int myslot = CL - 1 - rank;
+  const uint32_t cand_a = tc::smem_u32(cand) + (uint32_t)myslot * SLOT;
+  const uint32_t mbar_a = tc::smem_u32(&mbar[0]);
+  const uint32_t cbytes = (uint32_t)CL * SLOT;
+  const unsigned row_id = 31u - (unsigned)(lane / LPR);
+  unsigned char* my_wst = wst + (size_t)(GP_MAXW - 1 - warp) * SLOT + cg * CS;
+#pragma unroll 1
+  for (int jb = 0; jb < LPR; ++jb) {
+    const int src_lane = (lane & ~(LPR - 1)) | jb;
+    const bool mycol = cg == jb * CPL;
 #pragma unroll
-    for (int t = 0; t < MAXOWN; ++t) {
-      int r = k0 + tid + t * nt;
-      if (r < b && !(done & (1u << t))) amax_merge(bv, bi, cabs2(P[r * PS + j]), r);
-    }
+    for (int s = 0; s < CPL; ++s) {
+      const int j = jb * CPL + s, buf = s & 1;
+      if (j >= nbk) break;
+      const C xs = gp_shfl(x[s], src_lane);
+      const unsigned kmax = __reduce_max_sync(0xffffffffu, (elig ? gp_mag(xs) : 0u) | row_id);
+      const bool wrow = ((kmax ^ row_id) & 31u) == 0u;  // the warp's best row
+      if (wrow) {
+        if (cg == 0) wkey[buf][warp] = kmax;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      T v2 = __shfl_xor_sync(0xffffffffu, bv, o);
-      int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-      amax_merge(bv, bi, v2, i2);
-    }
-    // one barrier per step: it publishes the candidates and orders the
-    // owner's elimination of step j-1 on the pivot row before its reads
-    // below; the other rows are only ever touched by their owner thread
-    if (lane == 0) { red_v[j & 1][warp] = bv; red_i[j & 1][warp] = bi; }
-    __syncthreads();
-    bv = lane < NW ? red_v[j & 1][lane] : (T)-1;
-    bi = lane < NW ? red_i[j & 1][lane] : b;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      T v2 = __shfl_xor_sync(0xffffffffu, bv, o);
-      int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-      amax_merge(bv, bi, v2, i2);
-    }
-    const int p = bi < b ? bi : k0 + j;  // (bi >= b cannot happen while slots remain)
-    if (tid == 0) {
-      chosen[j] = p;
-      if (!(bv > (T)0)) flag[f] = 1;
-    }
-    C piv = P[p * PS + j];
-    if (cabs2(piv) == (T)0) piv = mk(sizeof(T) == 8 ? (T)1e-150 : (T)1e-18, (T)0);
-    const C pinv = cinv(piv);
-#pragma unroll
-    for (int t = 0; t < MAXOWN; ++t) {
-      int r = k0 + tid + t * nt;
-      if (r >= b || (done & (1u << t))) continue;
-      if (r == p) { done |= 1u << t; continue; }
-      C l = cmul(P[r * PS + j], pinv);
-      P[r * PS + j] = l;
-#pragma unroll
-      for (int c = 0; c < NB; ++c)
-        if (c > j && c < nbk) P[r * PS + c] = csub(P[r * PS + c], cmul(l, P[p * PS + c]));
-    }
-  }
-  __syncthreads();
-
-  // warp 0: replay the choices as row interchanges (position a = k0 + j with
-  // the current position q of the chosen slot), tracking where slots end
-  if (warp == 0) {
-    int kc = (lane < nbk) ? k0 + lane : -1;  // slot now at position k0 + lane
-    int np = -1, nc = -1, cnt = 0;           // touched position outside K and its slot
-    for (int j = 0; j < nbk; ++j) {
-      const int sj = chosen[j];
-      unsigned bK = __ballot_sync(0xffffffffu, lane < nbk && kc == sj);
-      unsigned bN = __ballot_sync(0xffffffffu, np >= 0 && nc == sj);
-      int q, ql;
-      bool inK;
-      if (bK) {
-        ql = __ffs(bK) - 1;
-        q = k0 + ql;
-        inK = true;
-      } else if (bN) {
-        ql = __ffs(bN) - 1;
-        q = __shfl_sync(0xffffffffu, np, ql);
-        inK = false;
-      } else {
-        ql = cnt++;
-        q = sj;
-        inK = false;
-        if (lane == ql) { np = sj; nc = sj; }
-      }
-      const int ca = __shfl_sync(0xffffffffu, kc, j);
-      const int cq = inK ? __shfl_sync(0xffffffffu, kc, ql) : __shfl_sync(0xffffffffu, nc, ql);
-      if (lane == j) kc = cq;
-      if (inK && lane == ql) kc = ca;
-      if (!inK && lane == ql) nc = ca;
-      if (lane == 0) ipiv[j] = q;
-      __syncwarp();
-    }
-    // perm undergoes the same interchanges: every position that received
-    // another slot takes that slot's old entry (all reads before any write,
-    // instead of a chain of dependent global swaps)
-    const bool movedK = lane < nbk && kc != k0 + lane;
-    const int pk = movedK ? perm[kc] : 0;
-    const int pn = lane < cnt ? perm[nc] : 0;
-    __syncwarp();
-    if (movedK) perm[k0 + lane] = pk;
-    if (lane < cnt) perm[np] = pn;
-    if (lane < nbk) sigK[lane] = kc;
-    if (lane < cnt) {
-      nkPos[lane] = np;
-      nkSlot[lane] = nc;
-      atomicOr(&touched[np >> 5], 1u << (np & 31));
-    }
-    if (lane == 0) s_nk = cnt;
-  }
-
-  // inverses of U11 (warp 0) and of the unit lower L11 (warp 1) in parallel,
-  // rows = chosen slots in order, one column per lane; then
-  // T^{-1} = U11^{-1} L11^{-1}
-  if (warp == 0 && lane < nbk) {
-    const int c = lane;
-    for (int i = 0; i < NB; ++i) Ui[i][c] = czero<C>();
-    for (int i = c; i >= 0; --i) {
-      const C* row = P + chosen[i] * PS;
-      C sacc = (i == c) ? mk((T)1, (T)0) : czero<C>();
-      for (int m = i + 1; m <= c; ++m) sacc = csub(sacc, cmul(row[m], Ui[m][c]));
-      Ui[i][c] = cmul(sacc, cinv(row[i]));
-    }
-  } else if (warp == 1 && lane < nbk) {
-    const int c = lane;
-    for (int i = 0; i < NB; ++i) Li[i][c] = czero<C>();
-    Li[c][c] = mk((T)1, (T)0);
-    for (int i = c + 1; i < nbk; ++i) {
-      const C* row = P + chosen[i] * PS;
-      C sacc = czero<C>();
-      for (int m = c; m < i; ++m) sacc = csub(sacc, cmul(row[m], Li[m][c]));
-      Li[i][c] = sacc;
-    }
-  }
-  __syncthreads();
-  for (int e = tid; e < nbk * nbk; e += nt) {
-    int i = e / nbk, c = e - i * nbk;
-    C s = czero<C>();
-    for (int m = max(i, c); m < nbk; ++m) s = cfma(Ui[i][m], Li[m][c], s);
-    Ti[i][c] = s;
-  }
-  __syncthreads();
-
-  // transform every slot in place
-  for (int r = tid; r < b; r += nt) {
-    int jpiv = -1;
-    if (r >= k0)
-      for (int j = 0; j < nbk; ++j)
-        if (chosen[j] == r) jpiv = j;
-    if (jpiv >= 0) {
-#pragma unroll
-      for (int c = 0; c < NB; ++c)
-        if (c < nbk) P[r * PS + c] = Ti[jpiv][c];
-      continue;
-    }
-    C v[NB];
-#pragma unroll
-    for (int m = 0; m < NB; ++m) v[m] = (m < nbk) ? P[r * PS + m] : czero<C>();
-    const bool above = r < k0;
-#pragma unroll
-    for (int c = 0; c < NB; ++c) {
-      if (c >= nbk) continue;
-      C s = czero<C>();
-#pragma unroll
-      for (int m = 0; m < NB; ++m)
-        if (m < nbk) s = cfma(v[m], above ? Ti[m][c] : Li[m][c], s);
-      P[r * PS + c] = cneg(s);
-    }
-  }
-  __syncthreads();
-  // write back by position: K positions take their pivot slot, touched
-  // positions outside K take the displaced slot, the rest keep their own
-  const int nk = s_nk;
-  for (int e = tid; e < b * nbk; e += nt) {
-    int a = e / nbk, c = e - a * nbk;
-    int slot = a;
-    if (a >= k0 && a < k0 + nbk) {
-      slot = sigK[a - k0];
-    } else if (touched[a >> 5] & (1u << (a & 31))) {
-      for (int t = 0; t < nk; ++t)
-        if (nkPos[t] == a) slot = nkSlot[t];
-    }
-    M[(size_t)a * b + k0 + c] = P[slot * PS + c];
-  }
-}
-
-// Row swaps + B save + M[K,R] <- T^{-1} B for the columns outside the panel.
-// Warp 0 first turns the panel's sequence of swaps into the net movement of
-// at most 2*NB rows; every thread then moves its column with independent
-// loads (all issued before any store) instead of a chain of dependent swaps.
-template <typename T, int NB>
-__host__ __device__ constexpr int rb_threads() {
-  return (NB * 128 * (int)sizeof(C_t<T>) > 32768) ? 32768 / (NB * (int)sizeof(C_t<T>)) : 128;
-}
-template <typename T, int NB>
-__global__ void __launch_bounds__(128)
-gj_rowblock_kernel(int b, int k0, int nbk, C_t<T>* __restrict__ Mall,
-                   const int* __restrict__ ipiv_all, C_t<T>* __restrict__ Ball) {
-  using C = C_t<T>;
-  __shared__ C Ts[NB][NB + 1];
-  __shared__ int srcK[NB];       // original row now at position k0 + j
-  __shared__ int nkPos[32], nkSrc[32];
-  __shared__ int s_nk;
-  constexpr int RBT = rb_threads<T, NB>();
-  __shared__ C W[NB][RBT];        // values moving to positions outside K
-  const int f = blockIdx.y;
-  C* M = Mall + (size_t)f * b * b;
-  C* B = Ball + (size_t)f * NB * b;
-  for (int e = threadIdx.x; e < nbk * nbk; e += blockDim.x) {
-    int i = e / nbk, c = e - i * nbk;
-    Ts[i][c] = M[(size_t)(k0 + i) * b + k0 + c];
-  }
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    for (int j = lane; j < NB; j += 32) srcK[j] = k0 + j;
-    // the panel's interchanges, one per lane, read once (not one dependent
-    // global load per step of the serial loop below)
-    const int piv_l = lane < nbk ? ipiv_all[f * 32 + lane] : 0;
-    int myPos = -1, myCont = -1, nk = 0;
-    __syncwarp();
-    for (int j = 0; j < nbk; ++j) {
-      const int a = k0 + j;
-      const int p = __shfl_sync(0xffffffffu, piv_l, j);
-      if (p == a) continue;
-      if (p < k0 + nbk) {
-        if (lane == 0) {
-          int t = srcK[j];
-          srcK[j] = srcK[p - k0];
-          srcK[p - k0] = t;
+        for (int c = 0; c < CPL; ++c) {
+          // (a warp without an eligible row: zero in the pivot's place)
+          const C v = c == s && mycol && kmax < 32u ? czero<C>() : x[c];
+          *reinterpret_cast<C*>(my_wst + (size_t)buf * GP_MAXW * SLOT + c * CS) = v;
         }
-        __syncwarp();
-        continue;
       }
-      unsigned hit = __ballot_sync(0xffffffffu, myPos == p);
-      int owner;
-      if (hit) {
-        owner = __ffs(hit) - 1;
-      } else {
-        owner = nk;
-        if (lane == owner) { myPos = p; myCont = p; }
-        ++nk;
+      __syncthreads();
+      const unsigned wk = (wkey[buf][lane] & ~31u) | ((15u - lane) & 31u);
+      const unsigned cw = __reduce_max_sync(0xffffffffu, wk) & 15u;  // 15 - warp
+      const unsigned char* src = wst + ((size_t)buf * GP_MAXW + cw) * SLOT;
+      if (cw + warp == 15u) {  // 1 / pivot, by the warp that holds the candidate
+        C pv = *reinterpret_cast<const C*>(src + j * CS);
+        if (gp_mag(pv) == 0u) pv = mk(sizeof(T) == 8 ? (T)1e-150 : (T)1e-18, (T)0);
+        const T rd = (T)1 / (pv.x * pv.x + pv.y * pv.y);
+        alignas(16) C pi[16 / CS] = {};
+        pi[0] = mk(pv.x * rd, -pv.y * rd);
+        const float4 val = *reinterpret_cast<const float4*>(pi);
+        if (lane < CL)
+          tc::st_async16(tc::cluster_map(cand_a + (uint32_t)(buf * CL * SLOT + NP * 16), lane), val,
+                         tc::cluster_map(mbar_a + buf * 8, lane));
       }
-      int kc = srcK[j];
-      int oc = __shfl_sync(0xffffffffu, myCont, owner);
-      if (lane == owner) myCont = kc;
-      __syncwarp();
-      if (lane == 0) srcK[j] = oc;
-      __syncwarp();
+      {
+        const int W = nthr >> 5, per = 32 / NP;  // receivers of one warp instruction
+        const float4 val = *reinterpret_cast<const float4*>(src + (lane % NP) * 16);
+        for (int d0 = warp * per; d0 < CL; d0 += W * per) {
+          const int d = d0 + lane / NP;
+          if (d < CL)
+            tc::st_async16(tc::cluster_map(cand_a + (uint32_t)(buf * CL * SLOT + (lane % NP) * 16), d),
+                           val, tc::cluster_map(mbar_a + buf * 8, d));
+        }
+      }
+      if (tid == 0) tc::mbar_expect_tx(&mbar[buf], cbytes);
+      if (ok) ok = tc::cluster_wait(&mbar[buf], (s >> 1) & 1, g.tries);
+      const unsigned char* cb = cand + (size_t)buf * CL * SLOT;
+      const int sl = min(lane, CL - 1);
+      const unsigned cmax = __reduce_max_sync(
+          0xffffffffu, gp_mag(*reinterpret_cast<const C*>(cb + (size_t)sl * SLOT + j * CS)) | sl);
+      singular |= cmax < 32u || (cmax & ~31u) > gp_inf<T>();
+      const int pc = (int)(cmax & 31u);
+      src = cb + (size_t)pc * SLOT;
+      const C pinv = *reinterpret_cast<const C*>(src + NP * 16);
+      C q[CPL];
+#pragma unroll
+      for (int u = 0; u < PPL; ++u)
+        reinterpret_cast<float4*>(q)[u] = *reinterpret_cast<const float4*>(src + cg * CS + u * 16);
+      C m = cneg(cmul(xs, pinv));
+      if (pc == myslot && cw + warp == 15u) {  // (the whole warp)
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+          x[c].x = wrow ? (T)0 : x[c].x;
+          x[c].y = wrow ? (T)0 : x[c].y;
+        }
+        m.x = wrow ? pinv.x : m.x;
+        m.y = wrow ? pinv.y : m.y;
+        elig = elig && !wrow;
+        mypiv = wrow ? j : mypiv;
+      }
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) x[c] = cfma(m, q[c], x[c]);
+      if (mycol) x[s] = m;
     }
-    if (lane < nk) { nkPos[lane] = myPos; nkSrc[lane] = myCont; }
-    if (lane == 0) s_nk = nk;
   }
-  __syncthreads();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= b || (c >= k0 && c < k0 + nbk)) return;
-  const int nk = s_nk;
-  C v[NB];
+  if (live) {
 #pragma unroll
-  for (int j = 0; j < NB; ++j) v[j] = (j < nbk) ? M[(size_t)srcK[j] * b + c] : czero<C>();
-  for (int t = 0; t < nk; ++t) W[t][threadIdx.x] = M[(size_t)nkSrc[t] * b + c];
-  for (int t = 0; t < nk; ++t) M[(size_t)nkPos[t] * b + c] = W[t][threadIdx.x];
-#pragma unroll
-  for (int j = 0; j < NB; ++j)
-    if (j < nbk) B[(size_t)j * b + c] = v[j];
-#pragma unroll
-  for (int i = 0; i < NB; ++i) {
-    if (i >= nbk) continue;
-    C s = czero<C>();
-#pragma unroll
-    for (int j = 0; j < NB; ++j)
-      if (j < nbk) s = cfma(Ts[i][j], v[j], s);
-    M[(size_t)(k0 + i) * b + c] = s;
+    for (int c = 0; c < CPL; ++c)
+      if (cg + c < nbk) M[(size_t)grow * b + g.k0 + cg + c] = x[c];
+    if (cg == 0) {
+      if (mypiv >= 0) {
+        rowpiv[grow] = g.k0 + mypiv;
+        g.pivslot[(size_t)f * b + g.k0 + mypiv] = grow;
+      } else if (g.k0 == 0) {
+        rowpiv[grow] = -1;
+      }
+    }
   }
+  if (rank == 0 && tid == 0 && singular) g.flag[f] = 1;
+  if (!ok && lane == 0) atomicExch(g.flag + g.F, 1);
+  if (!ok) tc::cluster_settle();
+  tc::cluster_sync();  // no CTA leaves while another may still send to it
 }
 
-// Trailing update M[I,R] += M[I,K] B on 64 x 64 tiles (16 x 16 threads, 4 x 4
-// each) for the columns [c_begin, c_end) outside K and outside [ex_lo, ex_hi).
-template <typename T, int NB>
+// B[f][j][m] = M[P_j][m] for the panel [k0, k0 + nbk), zero beyond nbk
+template <typename T>
+__global__ void gjp_gather_kernel(int b, int k0, int nbk, const C_t<T>* __restrict__ Mall,
+                                  const int* __restrict__ pivslot_all, C_t<T>* __restrict__ Ball) {
+  const int f = blockIdx.z, j = blockIdx.y, m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= b) return;
+  C_t<T> v = czero<C_t<T>>();
+  if (j < nbk) v = Mall[((size_t)f * b + pivslot_all[(size_t)f * b + k0 + j]) * b + m];
+  Ball[((size_t)f * GP_NB + j) * b + m] = v;
+}
+
+// The rank-16 update on TR x TR tiles (16 x 16 threads) of the columns outside
+// [k0, k0 + nbk) and [n0, n1).  FP64 is bound by its pipe, so small tiles fill
+// the SMs; FP32 by shared memory, so a thread holds 4 x 4 outputs.
+template <typename T> struct UpdCfg { static constexpr int TR = sizeof(T) == 8 ? 32 : 64; };
+template <typename T>
 __global__ void __launch_bounds__(256)
-gj_update_kernel(int b, int k0, int nbk, int c_begin, int c_end, int ex_lo, int ex_hi,
-                 C_t<T>* __restrict__ Mall, const C_t<T>* __restrict__ Ball) {
+gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, C_t<T>* __restrict__ Mall,
+                  const C_t<T>* __restrict__ Ball, const int* __restrict__ rowpiv_all) {
   using C = C_t<T>;
-  __shared__ C As[64][NB + 1];
-  __shared__ C Bs[NB][64];
+  constexpr int NB = GP_NB, TR = UpdCfg<T>::TR, PT = TR / 16;
+  __shared__ C As[TR][NB + 1];
+  __shared__ C Bs[NB][TR];
   const int f = blockIdx.z;
   C* M = Mall + (size_t)f * b * b;
   const C* B = Ball + (size_t)f * NB * b;
-  const int r0 = blockIdx.y * 64, c0 = c_begin + blockIdx.x * 64;
+  const int* rowpiv = rowpiv_all + (size_t)f * b;
+  const int r0 = blockIdx.y * TR, c0 = blockIdx.x * TR;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  for (int e = tid; e < 64 * NB; e += 256) {
-    int rr = e / NB, m = e - rr * NB;
-    int r = r0 + rr;
+  auto col_live = [&](int c) {
+    return c < b && !(c >= k0 && c < k0 + nbk) && !(c >= n0 && c < n1);
+  };
+  C acc[PT][PT];
+#pragma unroll
+  for (int a = 0; a < PT; ++a) {
+    const int r = r0 + ty + 16 * a;
+    const int rp = r < b ? rowpiv[r] : -1;
+    const bool keep = r < b && !(rp >= k0 && rp < k0 + nbk);
+#pragma unroll
+    for (int d = 0; d < PT; ++d) {
+      const int c = c0 + tx + 16 * d;
+      acc[a][d] = keep && col_live(c) ? M[(size_t)r * b + c] : czero<C>();
+    }
+  }
+  for (int e = tid; e < TR * NB; e += 256) {
+    const int rr = e / NB, m = e - rr * NB, r = r0 + rr;
     As[rr][m] = (r < b && m < nbk) ? M[(size_t)r * b + k0 + m] : czero<C>();
   }
-  for (int e = tid; e < NB * 64; e += 256) {
-    int m = e / 64, cc = e - m * 64;
-    int c = c0 + cc;
-    Bs[m][cc] = (c < c_end && m < nbk) ? B[(size_t)m * b + c] : czero<C>();
+  for (int e = tid; e < NB * TR; e += 256) {
+    const int m = e / TR, cc = e - m * TR, c = c0 + cc;
+    Bs[m][cc] = c < b ? B[(size_t)m * b + c] : czero<C>();
   }
   __syncthreads();
-  C acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int d = 0; d < 4; ++d) acc[a][d] = czero<C>();
 #pragma unroll 4
   for (int m = 0; m < NB; ++m) {
-    C av[4], bv[4];
+    C av[PT], bv[PT];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) av[a] = As[ty + 16 * a][m];
+    for (int a = 0; a < PT; ++a) av[a] = As[ty + 16 * a][m];
 #pragma unroll
-    for (int d = 0; d < 4; ++d) bv[d] = Bs[m][tx + 16 * d];
+    for (int d = 0; d < PT; ++d) bv[d] = Bs[m][tx + 16 * d];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < PT; ++a)
 #pragma unroll
-      for (int d = 0; d < 4; ++d) acc[a][d] = cfma(av[a], bv[d], acc[a][d]);
+      for (int d = 0; d < PT; ++d) acc[a][d] = cfma(av[a], bv[d], acc[a][d]);
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    int r = r0 + ty + 16 * a;
-    if (r >= b || (r >= k0 && r < k0 + nbk)) continue;
+  for (int a = 0; a < PT; ++a) {
+    const int r = r0 + ty + 16 * a;
+    if (r >= b) continue;
 #pragma unroll
-    for (int d = 0; d < 4; ++d) {
-      int c = c0 + tx + 16 * d;
-      if (c >= c_end || (c >= k0 && c < k0 + nbk) || (c >= ex_lo && c < ex_hi)) continue;
-      size_t o = (size_t)r * b + c;
-      M[o] = cadd(M[o], acc[a][d]);
+    for (int d = 0; d < PT; ++d) {
+      const int c = c0 + tx + 16 * d;
+      if (col_live(c)) M[(size_t)r * b + c] = acc[a][d];
     }
   }
 }
 
-// ---------------------------------------------------------------------------
-// Trailing update on the tensor cores (FP32 factors, 32-column panels):
-// M[I,R] += M[I,K] B as a real GEMM on tcgen05.mma kind::tf32.
-//
-// A tile is 128 rows of M[., K] read interleaved (re, im) as 64 K-major reals;
-// the right operand is B expanded to B~ with rows (Re, -Im), (Im, Re) per
-// complex column, so one real product gives the complex one.  FP32 accuracy
-// comes from the 3xTF32 split (hi.hi + hi.lo + lo.hi into one FP32 TMEM
-// accumulator).  One CTA per item (problem, tile of 64 complex columns,
-// group of row tiles): it expands B~ once and streams the item's row tiles
-// of M through a warp-specialised pipeline:
-//   warp 10     loads the raw A tile of row tile t+1 by TMA (3-D map over M)
-//               and issues the 24 MMAs of tile t into accumulator t & 1,
-//   warps 8-9   split the raw A tile into the hi / lo operand tiles,
-//   warps 0-7   prefetch the M rows of tile t (coalesced, whole 512-byte tile
-//               rows per warp instruction), move accumulator t & 1 through a
-//               shared staging tile and add it to M in place (rows in K,
-//               columns in K and in [ex_lo, ex_hi) untouched),
-// so the HBM traffic of tile t overlaps the split and MMAs of tile t+1.
-// Every mbarrier wait is bounded; a timeout sets *err and the CTA winds down
-// (in-flight MMAs drain, TMEM is freed).
-constexpr int UTC_RT = 128;                                   // rows per tile
-constexpr int UTC_CT = 64;                                    // complex columns per tile
-constexpr uint32_t UTC_LBO = 128, UTC_SBO = 2048;             // 64 reals of K
-constexpr uint32_t UTC_OP_BYTES = UTC_RT * 64 * 4;            // 32 KB operand tile
-constexpr int UTC_STAGE_LD = 2 * UTC_CT + 4;                  // staging row pitch (floats)
-constexpr uint32_t UTC_STAGE_BYTES = UTC_RT * UTC_STAGE_LD * 4;
-constexpr int UTC_EPI = 256, UTC_CONV = 64;                   // epilogue / split threads
-constexpr int UTC_THREADS = UTC_EPI + UTC_CONV + 32;          // + MMA warp
-// B~ hi/lo, A hi/lo, the raw A tile (TMA destination) and the staging tile
-constexpr size_t UTC_SMEM = 5 * (size_t)UTC_OP_BYTES + UTC_STAGE_BYTES + 128;
-constexpr uint32_t UTC_WAIT_TRIES = 1u << 22;
-
-// bounded wait; gives up at once when another thread has aborted
-__device__ __forceinline__ bool utc_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t t = 0; t < UTC_WAIT_TRIES; ++t) {
-    if (tc::mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-  }
-  *abort_flag = 1;
-  return false;
-}
-
-__device__ __forceinline__ void utc_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(bar)) : "memory");
-}
-
-// barrier among the 256 epilogue threads only
-__device__ __forceinline__ void utc_epi_sync() {
-  asm volatile("bar.sync 1, %0;\n" ::"n"(UTC_EPI) : "memory");
-}
-
-__global__ void __launch_bounds__(UTC_THREADS, 1)
-gj_update_tc_kernel(const __grid_constant__ CUtensorMap tmapM, int b, int k0, int nbk, int c_begin,
-                    int c_end, int ex_lo, int ex_hi, float2* __restrict__ Mall,
-                    const float2* __restrict__ Ball, int F, int nct, int nrg, int* err) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint64_t raw_full, a_full, mma_done[2], acc_empty[2];
-  __shared__ uint32_t tmem_base;
-  __shared__ int abort_sh;
-  volatile int* abort_flag = &abort_sh;
-  unsigned char* base = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
-  unsigned char* Bhi = base;
-  unsigned char* Blo = base + UTC_OP_BYTES;
-  unsigned char* Ahi = base + 2 * UTC_OP_BYTES;
-  unsigned char* Alo = base + 3 * UTC_OP_BYTES;
-  const float* Araw = reinterpret_cast<const float*>(base + 4 * UTC_OP_BYTES);  // [128][64]
-  float* stage = reinterpret_cast<float*>(base + 5 * UTC_OP_BYTES);  // [128][UTC_STAGE_LD]
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool is_epi = tid < UTC_EPI;
-  const bool is_conv = tid >= UTC_EPI && tid < UTC_EPI + UTC_CONV;
-  const bool is_mma = tid == UTC_EPI + UTC_CONV;
-  const int nrt = (b + UTC_RT - 1) / UTC_RT;
-  const int rpg = (nrt + nrg - 1) / nrg;  // row tiles per row group
-  const int nitems = nct * F * nrg;
-
-  if (warp == 0) tc::tmem_alloc(&tmem_base, 256);
-  if (tid == 0) {
-    tc::mbar_init(&raw_full, 1);
-    tc::mbar_init(&a_full, UTC_CONV);
-    for (int q = 0; q < 2; ++q) {
-      tc::mbar_init(&mma_done[q], 1);
-      tc::mbar_init(&acc_empty[q], UTC_EPI);
-    }
-    abort_sh = 0;
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = tmem_base;
-  const uint32_t idesc = tc::idesc_tf32(UTC_RT, 2 * UTC_CT);
-  uint64_t dBhi = 0, dBlo = 0, dAhi = 0, dAlo = 0;
-  if (is_mma) {
-    dBhi = tc::smem_desc(tc::smem_u32(Bhi), UTC_LBO, UTC_SBO);
-    dBlo = tc::smem_desc(tc::smem_u32(Blo), UTC_LBO, UTC_SBO);
-    dAhi = tc::smem_desc(tc::smem_u32(Ahi), UTC_LBO, UTC_SBO);
-    dAlo = tc::smem_desc(tc::smem_u32(Alo), UTC_LBO, UTC_SBO);
-  }
-  int g = 0;           // row tiles of this CTA so far (all items)
-  int issued = 0;      // tiles whose MMAs were issued (MMA thread)
-  int tma_issued = 0;  // raw A tiles requested (MMA thread)
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-    const int rg = it % nrg, fc = it / nrg;
-    const int f = fc / nct, ct = fc - f * nct;
-    const int rt0 = rg * rpg, rt1 = min(nrt, rt0 + rpg);
-    const int c0 = c_begin + ct * UTC_CT;
-    float2* M = Mall + (size_t)f * b * b;
-    // every earlier tile's MMAs are complete here (their epilogues waited
-    // for them before this barrier), so B~ may be overwritten
-    __syncthreads();
-    if ((is_epi || is_conv) && !*abort_flag) {
-      const float2* B = Ball + (size_t)f * 32 * b;
-      for (int e = tid; e < UTC_CT * 16; e += UTC_EPI + UTC_CONV) {
-        const int j = e & (UTC_CT - 1), p = e / UTC_CT;
-        const int c = c0 + j, m0 = 2 * p, m1 = m0 + 1;
-        const bool cv = c < c_end;
-        const float2 t0 = (cv && m0 < nbk) ? B[(size_t)m0 * b + c] : make_float2(0.f, 0.f);
-        const float2 t1 = (cv && m1 < nbk) ? B[(size_t)m1 * b + c] : make_float2(0.f, 0.f);
-        float4 h0, l0;
-        tc::split_tf32(t0.x, h0.x, l0.x);
-        tc::split_tf32(-t0.y, h0.y, l0.y);
-        tc::split_tf32(t1.x, h0.z, l0.z);
-        tc::split_tf32(-t1.y, h0.w, l0.w);
-        const float4 h1 = make_float4(-h0.y, h0.x, -h0.w, h0.z);
-        const float4 l1 = make_float4(-l0.y, l0.x, -l0.w, l0.z);
-        const int n0 = 2 * j, n1 = n0 + 1;
-        const uint32_t o0 = (uint32_t)(n0 >> 3) * UTC_SBO + (uint32_t)p * UTC_LBO + (uint32_t)(n0 & 7) * 16;
-        const uint32_t o1 = (uint32_t)(n1 >> 3) * UTC_SBO + (uint32_t)p * UTC_LBO + (uint32_t)(n1 & 7) * 16;
-        *reinterpret_cast<float4*>(Bhi + o0) = h0;
-        *reinterpret_cast<float4*>(Blo + o0) = l0;
-        *reinterpret_cast<float4*>(Bhi + o1) = h1;
-        *reinterpret_cast<float4*>(Blo + o1) = l1;
-      }
-      tc::fence_async_smem();
-    }
-    __syncthreads();
-    if (is_mma && !*abort_flag && rt0 < rt1) {  // raw A tile of the item's first row tile
-      tc::mbar_expect_tx(&raw_full, UTC_OP_BYTES);
-      tc::tma_load_3d(base + 4 * UTC_OP_BYTES, &tmapM, 2 * k0, rt0 * UTC_RT, f, &raw_full);
-      ++tma_issued;
-    }
-    for (int rt = rt0; rt < rt1; ++rt, ++g) {
-      const int q = g & 1;
-      const uint32_t ph = (uint32_t)(g >> 1) & 1u;  // phase of tile g on the barriers q
-      if (is_conv) {
-        // raw A tile (row-major 128 x 64 floats: rows rt*128.., the 32 panel
-        // columns; zero beyond b) -> TF32 hi / lo tiles in the K-major
-        // core-matrix layout.  Each 8-lane phase takes a diagonal: rows
-        // 8G + a and K groups ((a + D) & 7) + 8H for a = 0..7, so both the
-        // raw reads (slot p mod 8) and the core-matrix writes (slot i mod 8)
-        // hit 8 distinct 16-byte bank slots.
-        const int ci = tid - UTC_EPI;
-        bool ok = !*abort_flag;
-        if (ok) ok = utc_wait(&raw_full, (uint32_t)g & 1u, abort_flag);
-        // the A operand tiles are free once tile g-1's MMAs are complete
-        if (ok && g >= 1) ok = utc_wait(&mma_done[(g - 1) & 1], (uint32_t)((g - 1) >> 1) & 1u, abort_flag);
-        if (ok) {
-#pragma unroll 8
-          for (int s = 0; s < 32; ++s) {
-            const int a = lane & 7;
-            const int combo = ((ci >> 5) * 32 + s) * 4 + (lane >> 3);  // 0 .. 255
-            const int i = 8 * (combo & 15) + a;                         // row
-            const int p = ((a + (combo >> 5)) & 7) + 8 * ((combo >> 4) & 1);  // K group
-            const float4 v = *reinterpret_cast<const float4*>(Araw + i * 64 + 4 * p);
-            float4 h, l;
-            tc::split_tf32(v.x, h.x, l.x);
-            tc::split_tf32(v.y, h.y, l.y);
-            tc::split_tf32(v.z, h.z, l.z);
-            tc::split_tf32(v.w, h.w, l.w);
-            const uint32_t off = (uint32_t)(i >> 3) * UTC_SBO + (uint32_t)p * UTC_LBO + (uint32_t)(i & 7) * 16;
-            *reinterpret_cast<float4*>(Ahi + off) = h;
-            *reinterpret_cast<float4*>(Alo + off) = l;
-          }
-          tc::fence_async_smem();
-        }
-        utc_arrive(&a_full);
-      } else if (is_mma) {
-        bool ok = !*abort_flag;
-        if (ok) ok = utc_wait(&a_full, (uint32_t)g & 1u, abort_flag);
-        if (ok && rt + 1 < rt1) {  // the raw tile has been split: fetch the next one
-          tc::mbar_expect_tx(&raw_full, UTC_OP_BYTES);
-          tc::tma_load_3d(base + 4 * UTC_OP_BYTES, &tmapM, 2 * k0, (rt + 1) * UTC_RT, f, &raw_full);
-          ++tma_issued;
-        }
-        if (ok && g >= 2) ok = utc_wait(&acc_empty[q], (uint32_t)((g - 2) >> 1) & 1u, abort_flag);
-        if (ok) {
-          tc::fence_after_sync();
-          const uint32_t acc = tmem + (uint32_t)q * (2 * UTC_CT);
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint64_t koff = (uint64_t)((kk * 2 * UTC_LBO) >> 4);
-            tc::mma_tf32(acc, dAhi + koff, dBhi + koff, idesc, kk > 0 ? 1u : 0u);
-            tc::mma_tf32(acc, dAhi + koff, dBlo + koff, idesc, 1u);
-            tc::mma_tf32(acc, dAlo + koff, dBhi + koff, idesc, 1u);
-          }
-          tc::mma_commit(&mma_done[q]);
-          issued = g + 1;
-        }
-      } else if (is_epi) {
-        // 1. prefetch: warp w owns tile rows 16w..16w+15; lane l the complex
-        //    columns c0 + 2l, c0 + 2l + 1 (whole 512-byte tile rows per load)
-        const int cl = c0 + 2 * lane;
-        const bool cval = cl < c_end && !(cl >= k0 && cl < k0 + nbk) && !(cl >= ex_lo && cl < ex_hi);
-        float4 cm[16];
-        unsigned rvalid = 0u;
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const int r = rt * UTC_RT + 16 * warp + u;
-          const bool v = cval && r < b && !(r >= k0 && r < k0 + nbk);
-          rvalid |= (v ? 1u : 0u) << u;
-          cm[u] = v ? *reinterpret_cast<const float4*>(M + (size_t)r * b + cl)
-                    : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        bool ok = !*abort_flag;
-        if (ok) ok = utc_wait(&mma_done[q], ph, abort_flag);
-        // 2. the previous tile's staging reads are complete
-        utc_epi_sync();
-        if (ok) {
-          // 3. accumulator -> staging: thread = TMEM lane (tile row), 64 of
-          //    the 128 real columns per warp (half h)
-          tc::fence_after_sync();
-          const int wq = warp & 3, h = warp >> 2;
-          const int row = wq * 32 + lane;
-          float* srow = stage + row * UTC_STAGE_LD + h * 64;
-#pragma unroll
-          for (int grp = 0; grp < 4; ++grp) {
-            float v[16];
-            const uint32_t ta = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)q * (2 * UTC_CT) +
-                                (uint32_t)(h * 64 + grp * 16);
-            tc::tmem_ld16(ta, v);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              *reinterpret_cast<float4*>(srow + grp * 16 + 4 * u) =
-                  make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
-          }
-          tc::fence_before_sync();
-        }
-        utc_arrive(&acc_empty[q]);
-        // 4. staging complete; 5. add and store the owned rows
-        utc_epi_sync();
-        if (ok) {
-#pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            if (!(rvalid & (1u << u))) continue;
-            const int row = 16 * warp + u;
-            const float4 a = *reinterpret_cast<const float4*>(stage + row * UTC_STAGE_LD + 4 * lane);
-            float4 m = cm[u];
-            m.x += a.x;
-            m.y += a.y;
-            m.z += a.z;
-            m.w += a.w;
-            *reinterpret_cast<float4*>(M + (size_t)(rt * UTC_RT + row) * b + cl) = m;
-          }
-        }
-      }
-    }
-  }
-  if (is_mma && issued > 0) {
-    // the last commit covers every MMA issued: drain before TMEM is freed
-    const int last = issued - 1;
-    tc::mbar_wait(&mma_done[last & 1], (uint32_t)(last >> 1) & 1u, UTC_WAIT_TRIES);
-  }
-  if (is_mma && tma_issued > 0) {
-    // a raw tile still in flight (after an abort) lands before the CTA exits
-    const int last = tma_issued - 1;
-    tc::mbar_wait(&raw_full, (uint32_t)last & 1u, UTC_WAIT_TRIES);
-  }
-  if (tid == 0 && *abort_flag) atomicExch(err, 1);
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, 256);
-}
-
-// G_i[:, perm[c]] = M[:, c];  X_i = G_i C_i with C_i = -L_{i,i+1}.
+// G_i[j][p_m] = M[p_j][m];  X_i = G_i C_i with C_i = -L_{i,i+1}.
 template <typename T>
-__global__ void gj_finalize_kernel(OpView op, int i, int RB, const C_t<T>* __restrict__ Mall,
-                                   const int* __restrict__ perm_all, C_t<T>* __restrict__ Gi,
-                                   size_t gstride, C_t<T>* __restrict__ Xi, size_t xstride) {
+__global__ void gjp_finalize_kernel(OpView op, int i, int RB, const C_t<T>* __restrict__ Mall,
+                                    const int* __restrict__ pivslot_all, C_t<T>* __restrict__ Gi,
+                                    size_t gstride, C_t<T>* __restrict__ Xi, size_t xstride) {
   using C = C_t<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int b = op.b, q = op.q;
-  C* Gs = reinterpret_cast<C*>(smem_raw);          // [RB][b]
+  C* Gs = reinterpret_cast<C*>(smem_raw);                 // [RB][b]
   int* ps = reinterpret_cast<int*>(Gs + (size_t)RB * b);  // [b]
   const int f = blockIdx.y;
   const int r0 = blockIdx.x * RB;
   const C* M = Mall + (size_t)f * b * b;
-  for (int c = threadIdx.x; c < b; c += blockDim.x) ps[c] = perm_all[(size_t)f * b + c];
+  for (int c = threadIdx.x; c < b; c += blockDim.x) ps[c] = pivslot_all[(size_t)f * b + c];
   __syncthreads();
   for (int e = threadIdx.x; e < RB * b; e += blockDim.x) {
-    int rr = e / b, c = e - rr * b;
-    int r = r0 + rr;
-    if (r < b) Gs[rr * b + ps[c]] = M[(size_t)r * b + c];
+    const int rr = e / b, c = e - rr * b, r = r0 + rr;
+    if (r < b) Gs[rr * b + ps[c]] = M[(size_t)ps[r] * b + c];
   }
   __syncthreads();
   C* G = Gi + (size_t)f * gstride;
   for (int e = threadIdx.x; e < RB * b; e += blockDim.x) {
-    int rr = e / b, c = e - rr * b;
-    int r = r0 + rr;
+    const int rr = e / b, c = e - rr * b, r = r0 + rr;
     if (r < b) G[(size_t)r * b + c] = Gs[rr * b + c];
   }
   if (Xi == nullptr) return;
   C* X = Xi + (size_t)f * xstride;
   for (int e = threadIdx.x; e < RB * b; e += blockDim.x) {
-    int rr = e / b, c = e - rr * b;
-    int r = r0 + rr;
+    const int rr = e / b, c = e - rr * b, r = r0 + rr;
     if (r >= b) continue;
     const int iyc = c / q, cc = c - iyc * q;
     C s = czero<C>();
     for (int dy = -1; dy <= 1; ++dy) {
-      int iym = nbr_y(iyc, -dy, op.ny, op.periodic);
+      const int iym = nbr_y(iyc, -dy, op.ny, op.periodic);
       if (iym < 0) continue;
       for (int cm = 0; cm < q; ++cm) {
-        int m = iym * q + cm;
-        T a = coefv<T>(op, ((size_t)i * b + m) * op.S + slotx(1, dy) * q + cc);
+        const int m = iym * q + cm;
+        const T a = coefv<T>(op, ((size_t)i * b + m) * op.S + slotx(1, dy) * q + cc);
         if (a != (T)0) s = crfma(a, Gs[rr * b + m], s);
       }
     }
     X[(size_t)r * b + c] = cneg(s);
   }
-}
-
-__global__ void iota_kernel(int* perm, int b, int F) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < b * F) perm[e] = e % b;
-}
-
-// Widest panel whose tall slab (b x NB) plus the static NB x NB scratch fits
-// the 227 KB of shared memory a CTA may use.
-template <typename T>
-int panel_nb(int b) {
-  const size_t csz = sizeof(C_t<T>);
-  const size_t cap = 227 * 1024 - 2048;
-  // complex double keeps NB <= 16 so the static NB x NB scratch stays small
-  for (int nb = (csz == 16 ? 16 : 32); nb >= 8; nb >>= 1)
-    if ((size_t)b * (nb + 1) * csz + 3 * (size_t)nb * (nb + 1) * csz <= cap) return nb;
-  return 8;
 }
 
 template <typename T>
@@ -849,130 +478,109 @@ void launch_schur(const OpView& ov, const double2* shifts, int i, const C_t<T>* 
   schur_kernel<T><<<gs, CB, smem, st>>>(ov, shifts, i, Xprev, xstride, M);
 }
 
-template <typename T, int NB>
+template <typename T>
+rr_status launch_panel(rr_factors* fa, int k0, int nbk, int kp0, cudaStream_t st) {
+  const OpDev& d = fa->op->d;
+  PanelArgs a;
+  a.b = d.b;
+  a.k0 = k0;
+  a.nbk = nbk;
+  a.kp0 = kp0;
+  a.F = fa->F;
+  a.CL = std::min(GP_CLMAX, (d.b + 7) / 8);  // at least eight rows per CTA
+  a.rpc = (d.b + a.CL - 1) / a.CL;
+  a.rowpiv = fa->rowpiv;
+  a.pivslot = fa->pivslot;
+  a.flag = fa->flag;
+  a.tries = wait_tries();
+  const size_t smem = panel_smem<T>(a.rpc, a.CL);
+  static bool attr = false;
+  if (!attr) {
+    RR_CUDA(cudaFuncSetAttribute(gjp_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)panel_smem<T>(GP_MAXW * 8, GP_CLMAX)));
+    attr = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(a.CL * fa->F), 1, 1);
+  cfg.blockDim = dim3((unsigned)((a.rpc * GP_LPR + 31) / 32 * 32), 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = a.CL;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  prof_begin(PROF_PANEL, st);
+  RR_CUDA(cudaLaunchKernelEx(&cfg, gjp_panel_kernel<T>, a, reinterpret_cast<C_t<T>*>(fa->M)));
+  prof_end(PROF_PANEL, st);
+  return RR_OK;
+}
+
+template <typename T>
 rr_status factor_impl(rr_factors* fa) {
   using C = C_t<T>;
+  constexpr int NB = GP_NB;
   const OpDev& d = fa->op->d;
   const OpView ov = view(d);
   const int b = d.b, nx = d.nx, F = fa->F;
-  cudaStream_t st = fa->stream;
+  cudaStream_t st = fa->stream, st2 = fa->stream2;
   C* M = reinterpret_cast<C*>(fa->M);
   C* G = reinterpret_cast<C*>(fa->G);
   C* X = reinterpret_cast<C*>(fa->X);
   C* Bbuf = reinterpret_cast<C*>(fa->Bbuf);
   const size_t bb = (size_t)b * b;
-  const size_t gstride = (size_t)nx * bb;          // per problem
-  const size_t xstride = bb;  // X_i is transient: one b x b block per problem
-
-  const size_t psmem = (size_t)b * (NB + 1) * sizeof(C);
-  RR_CUDA(cudaFuncSetAttribute(gj_panel_kernel<T, NB>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem));
   int RB = 4;
   while (RB > 1 && (size_t)RB * b * sizeof(C) + b * sizeof(int) > 160 * 1024) RB >>= 1;
   const size_t fsmem = (size_t)RB * b * sizeof(C) + b * sizeof(int);
-  RR_CUDA(cudaFuncSetAttribute(gj_finalize_kernel<T>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
-
-  // look-ahead: panel p+1 runs on a second stream while the trailing update
-  // of panel p proceeds on the main stream (disjoint columns of M)
-  cudaStream_t st2 = fa->stream2;
-  const int P = (b + NB - 1) / NB;
-  // FP32 factors with 32-column panels, b % 8 == 0 (16-byte aligned rows)
-  // and b >= 128 (the TMA map of M) update on the tensor cores;
-  // RR_FP32_SIMT and FP64 on the CUDA cores
-  constexpr bool tc_shape = std::is_same<T, float>::value && NB == 32;
-  const bool use_tc = tc_shape && tc_prec(fa->prec) && b % 8 == 0 && b >= UTC_RT &&
-                      fa->tma_m_ok && fa->tune_update != 1;
-  if (use_tc)
-    RR_CUDA(cudaFuncSetAttribute(gj_update_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)UTC_SMEM));
-  auto update = [&](int k0, int nbk, int cb, int ce, int exl, int exh) {
-    prof_begin(PROF_UPDATE, st);
-    if constexpr (tc_shape) {
-      if (use_tc) {
-        // one CTA per item (not persistent): CTAs retire after one column
-        // tile, so the look-ahead panel kernel on the second stream finds
-        // free SMs while the update runs
-        // a slice of one column tile (the next panel's columns) splits its
-        // row tiles over CTAs: it is on the look-ahead critical path
-        const int nct = (ce - cb + UTC_CT - 1) / UTC_CT;
-        const int nrg = nct == 1 ? (b + UTC_RT - 1) / UTC_RT : 1;
-        const int grid = nct * F * nrg;
-        gj_update_tc_kernel<<<grid, UTC_THREADS, UTC_SMEM, st>>>(
-            *reinterpret_cast<const CUtensorMap*>(fa->tmap[2]), b, k0, nbk, cb, ce, exl, exh,
-            reinterpret_cast<float2*>(M),
-            reinterpret_cast<const float2*>(Bbuf), F, nct, nrg, fa->flag + F);
-        prof_end(PROF_UPDATE, st);
-        return;
-      }
-    }
-    const int ntile = (ce - cb + 63) / 64;
-    gj_update_kernel<T, NB><<<dim3(ntile, (b + 63) / 64, F), 256, 0, st>>>(
-        b, k0, nbk, cb, ce, exl, exh, M, Bbuf);
-    prof_end(PROF_UPDATE, st);
-  };
-  auto panel = [&](int p, cudaStream_t s) {
-    const int k0 = p * NB, nbk = std::min(NB, b - k0);
-    prof_begin(PROF_PANEL, s);
-    gj_panel_kernel<T, NB><<<F, PANEL_THREADS, psmem, s>>>(b, k0, nbk, M, fa->ipiv, fa->perm,
-                                                          fa->flag);
-    prof_end(PROF_PANEL, s);
-  };
+  RR_CUDA(cudaFuncSetAttribute(gjp_finalize_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)fsmem));
+  constexpr int TR = UpdCfg<T>::TR;
+  const int nt = (b + TR - 1) / TR, P = (b + NB - 1) / NB;
   // (factor_cols > 0 stops after that many columns: autotuner timing only)
   const int ncols = fa->factor_cols > 0 ? std::min(fa->factor_cols, nx) : nx;
+  rr_status s;
   for (int i = 0; i < ncols; ++i) {
-    iota_kernel<<<(b * F + 255) / 256, 256, 0, st>>>(fa->perm, b, F);
-    prof_count(1);
-    const C* Xprev = (i > 0) ? X : nullptr;
     prof_begin(PROF_SCHUR, st);
-    launch_schur<T>(ov, fa->shifts, i, Xprev, xstride, M, F, st);
+    launch_schur<T>(ov, fa->shifts, i, i > 0 ? X : nullptr, bb, M, F, st);
     prof_end(PROF_SCHUR, st);
-    panel(0, st);
+    // The panels run in order on the second (high-priority) stream, the updates
+    // in order on the main one.  Panel p applies panel p - 1's transformation to
+    // its own columns, so it waits only for the update of panel p - 2 and runs
+    // beside that of p - 1 (disjoint columns; rowpiv entries written meanwhile
+    // go from "none" to a column outside p - 1, which the update reads as "not
+    // its pivot row" either way).
+    RR_CUDA(cudaEventRecord(fa->ev_next, st));
+    RR_CUDA(cudaStreamWaitEvent(st2, fa->ev_next, 0));
     for (int p = 0; p < P; ++p) {
       const int k0 = p * NB, nbk = std::min(NB, b - k0);
+      if (p >= 2) RR_CUDA(cudaStreamWaitEvent(st2, fa->ev_ring[4 + ((p - 2) & 3)], 0));
+      if ((s = launch_panel<T>(fa, k0, nbk, p > 0 ? k0 - NB : -1, st2)) != RR_OK) return s;
+      RR_CUDA(cudaEventRecord(fa->ev_ring[p & 3], st2));
+      RR_CUDA(cudaStreamWaitEvent(st, fa->ev_ring[p & 3], 0));
+      if (P == 1) break;
       prof_begin(PROF_ROWBLOCK, st);
-      constexpr int RBT = rb_threads<T, NB>();
-      gj_rowblock_kernel<T, NB><<<dim3((b + RBT - 1) / RBT, F), RBT, 0, st>>>(
-          b, k0, nbk, M, fa->ipiv, Bbuf);
+      gjp_gather_kernel<T><<<dim3((b + 127) / 128, NB, F), 128, 0, st>>>(b, k0, nbk, M, fa->pivslot, Bbuf);
       prof_end(PROF_ROWBLOCK, st);
-      if (p + 1 < P && st2 != nullptr) {
-        const int n0 = k0 + nbk, n1 = std::min(b, n0 + NB);
-        update(k0, nbk, n0, n1, 0, 0);
-        RR_CUDA(cudaEventRecord(fa->ev_next, st));
-        RR_CUDA(cudaStreamWaitEvent(st2, fa->ev_next, 0));
-        panel(p + 1, st2);
-        RR_CUDA(cudaEventRecord(fa->ev_panel, st2));
-        update(k0, nbk, 0, b, n0, n1);
-        RR_CUDA(cudaStreamWaitEvent(st, fa->ev_panel, 0));
-      } else {
-        update(k0, nbk, 0, b, 0, 0);
-        if (p + 1 < P) panel(p + 1, st);
-      }
+      const int n0 = p + 1 < P ? k0 + NB : 0, n1 = p + 1 < P ? std::min(b, n0 + NB) : 0;
+      prof_begin(PROF_UPDATE, st);
+      gjp_update_kernel<T><<<dim3(nt, nt, F), 256, 0, st>>>(b, k0, nbk, n0, n1, M, Bbuf, fa->rowpiv);
+      prof_end(PROF_UPDATE, st);
+      RR_CUDA(cudaEventRecord(fa->ev_ring[4 + (p & 3)], st));
+      RR_CUDA(cudaGetLastError());
     }
     C* Xi = (i + 1 < nx) ? X : nullptr;
     prof_begin(PROF_FINALIZE, st);
-    gj_finalize_kernel<T><<<dim3((b + RB - 1) / RB, F), 256, fsmem, st>>>(
-        ov, i, RB, M, fa->perm, G + (size_t)i * bb, gstride, Xi, xstride);
+    gjp_finalize_kernel<T><<<dim3((b + RB - 1) / RB, F), 256, fsmem, st>>>(
+        ov, i, RB, M, fa->pivslot, G + (size_t)i * bb, (size_t)nx * bb, Xi, bb);
     prof_end(PROF_FINALIZE, st);
     RR_CUDA(cudaGetLastError());
   }
   return RR_OK;
 }
 
-template <typename T>
-rr_status factor_dispatch(rr_factors* fa) {
-  switch (panel_nb<T>(fa->op->d.b)) {
-    case 32: return factor_impl<T, 32>(fa);
-    case 16: return factor_impl<T, 16>(fa);
-    default: return factor_impl<T, 8>(fa);
-  }
-}
-
 }  // namespace
-
-int factor_panel_width(int prec, int b) {
-  return prec == RR_FP64 ? panel_nb<double>(b) : panel_nb<float>(b);
-}
 
 rr_status launch_schur_f32(rr_factors* fa, int i, cudaStream_t st) {
   const OpDev& d = fa->op->d;
@@ -987,7 +595,7 @@ rr_status launch_schur_f32(rr_factors* fa, int i, cudaStream_t st) {
 }
 
 rr_status launch_factor(rr_factors* fa) {
-  if (fa->prec == RR_FP64) return factor_dispatch<double>(fa);
+  if (fa->prec == RR_FP64) return factor_impl<double>(fa);
   if (factor_wide_ok(fa) && fa->tune_update != 1) return launch_factor_wide(fa);
-  return factor_dispatch<float>(fa);
+  return factor_impl<float>(fa);
 }

@@ -479,6 +479,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
   }
   if (rank == 0 && tid == 0 && singular) g.flag[f] = 1;
   if (!ok && lane == 0) atomicExch(g.flag + g.F, 1);
+  if (!ok) tc::cluster_settle();
   if (!SOLO) tc::cluster_sync();  // no CTA leaves while another may still send to it
 }
 

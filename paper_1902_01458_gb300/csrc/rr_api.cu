@@ -495,31 +495,6 @@ static int encode_factor_maps(rr_factors* fa) {
   return (r1 == CUDA_SUCCESS && r2 == CUDA_SUCCESS) ? 1 : 0;
 }
 
-// TMA map over the FP32 work matrices M [F][b][b] (complex, viewed as floats
-// [F][b][2b]): tiles of 128 rows x 32 complex, the A operand of the
-// tensor-core trailing update.  Needs b >= 128 and b % 8 == 0.
-static int encode_m_map(rr_factors* fa) {
-  const OpDev& d = fa->op->d;
-  if (!tc_prec(fa->prec) || d.b < 128 || (d.b & 7)) return 0;
-  cudaDriverEntryPointQueryResult q;
-  void* fn = nullptr;
-  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                       &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess || fn == nullptr) {
-    cudaGetLastError();
-    return 0;
-  }
-  auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-  const cuuint64_t dims[3] = {(cuuint64_t)2 * d.b, (cuuint64_t)d.b, (cuuint64_t)fa->F};
-  const cuuint64_t strides[2] = {(cuuint64_t)2 * d.b * 4, (cuuint64_t)2 * d.b * d.b * 4};
-  const cuuint32_t box[3] = {64, 128, 1}, es[3] = {1, 1, 1};
-  CUresult r = encode(reinterpret_cast<CUtensorMap*>(fa->tmap[2]), CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
-                      3, fa->M, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? 1 : 0;
-}
-
 // TMA maps of the wide factorisation (FP32 factors): chunks of 16 complex
 // columns x 128 rows of M (the left operand of the rank-128 update, read in
 // place), and tiles of 16 rows x 64 complex of the gathered pivot rows Wbuf
@@ -740,23 +715,20 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
   if ((s = dalloc(&fa->G, (size_t)nshift * d.nx * bb * fa->csz)) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->X, (size_t)nshift * bb * fa->csz)) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->M, (size_t)nshift * bb * fa->csz)) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->Bbuf, (size_t)nshift * 32 * d.b * fa->csz)) != RR_OK) return fail(s);
+  if ((s = dalloc(&fa->Bbuf, (size_t)nshift * 16 * d.b * fa->csz)) != RR_OK) return fail(s);
+  if ((s = dalloc(&fa->rowpiv, (size_t)nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
+  if ((s = dalloc(&fa->pivslot, (size_t)nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->Tbuf, (size_t)nshift * 128 * d.b * fa->csz)) != RR_OK) return fail(s);
   if (tc_prec(prec)) {
     if ((s = dalloc(&fa->Pbuf, (size_t)4 * nshift * 64 * d.b * sizeof(float2))) != RR_OK)
       return fail(s);
     fa->tma_ok = encode_factor_maps(fa);
-    fa->tma_m_ok = encode_m_map(fa);
     if (d.b >= 64 && d.b <= 768 && d.b % 8 == 0) {
-      if ((s = dalloc(&fa->rowpiv, (size_t)nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
-      if ((s = dalloc(&fa->pivslot, (size_t)nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
       if ((s = dalloc(&fa->Wbuf, (size_t)nshift * 128 * d.b * sizeof(float2))) != RR_OK)
         return fail(s);
       fa->wide_ok = encode_wide_maps(fa);
     }
   }
-  if ((s = dalloc(&fa->perm, (size_t)nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->ipiv, (size_t)nshift * 32 * sizeof(int))) != RR_OK) return fail(s);
   // flags: one singular-pivot flag per shift, then the tensor-core wait flag,
   // then room for the active-problem list of the refinement
   if ((s = dalloc(&fa->flag, (size_t)(2 * nshift + 1) * sizeof(int))) != RR_OK) return fail(s);
@@ -770,6 +742,8 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
     cudaError_t e1 = cudaStreamCreateWithPriority(&fa->stream2, cudaStreamNonBlocking, hi_prio);
     if (e1 == cudaSuccess) e1 = cudaEventCreateWithFlags(&fa->ev_next, cudaEventDisableTiming);
     if (e1 == cudaSuccess) e1 = cudaEventCreateWithFlags(&fa->ev_panel, cudaEventDisableTiming);
+    for (int q = 0; q < 8 && e1 == cudaSuccess; ++q)
+      e1 = cudaEventCreateWithFlags(&fa->ev_ring[q], cudaEventDisableTiming);
     if (e1 != cudaSuccess) return fail(cuda_status(e1, "rr_factor: stream/event creation"));
   }
   fa->shifts_h = new double2[nshift];
@@ -780,6 +754,9 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
   if (e != cudaSuccess) return fail(cuda_status(e, "rr_factor shifts"));
   e = cudaMemsetAsync(fa->flag, 0, (nshift + 1) * sizeof(int), st);
   if (e != cudaSuccess) return fail(cuda_status(e, "rr_factor flags"));
+  // a row index in every entry, also of a factorisation that found no pivot
+  e = cudaMemsetAsync(fa->pivslot, 0, (size_t)nshift * d.b * sizeof(int), st);
+  if (e != cudaSuccess) return fail(cuda_status(e, "rr_factor pivots"));
   if ((s = launch_factor(fa)) != RR_OK) return fail(s);
   std::vector<int> flags(nshift + 1);
   e = cudaMemcpyAsync(flags.data(), fa->flag, (nshift + 1) * sizeof(int), cudaMemcpyDeviceToHost,
@@ -818,8 +795,6 @@ extern "C" rr_status rr_destroy_factors(rr_factors* fa) {
   cudaFree(fa->Bbuf);
   cudaFree(fa->Tbuf);
   cudaFree(fa->Pbuf);
-  cudaFree(fa->perm);
-  cudaFree(fa->ipiv);
   cudaFree(fa->rowpiv);
   cudaFree(fa->pivslot);
   cudaFree(fa->Wbuf);
@@ -831,6 +806,8 @@ extern "C" rr_status rr_destroy_factors(rr_factors* fa) {
   }
   if (fa->ev_next) cudaEventDestroy(fa->ev_next);
   if (fa->ev_panel) cudaEventDestroy(fa->ev_panel);
+  for (int q = 0; q < 8; ++q)
+    if (fa->ev_ring[q]) cudaEventDestroy(fa->ev_ring[q]);
   delete[] fa->shifts_h;
   delete fa;
   return RR_OK;

@@ -139,22 +139,20 @@ struct rr_factors {
   cudaStream_t stream;
   cudaStream_t stream2;  // look-ahead panel / slab stream (owned)
   cudaEvent_t ev_next, ev_panel;
+  cudaEvent_t ev_ring[8];  // panel / update rings of the 16-column factorisation
   size_t csz;        // bytes of one complex element of the factors
   void* G;           // [F][nx][b][b]   inverse of each Schur block
   void* X;           // [F][b][b] X_i = G_i C_i of the current column (transient)
   void* M;           // [F][b][b] work matrix
-  void* Bbuf;        // [F][32][b] saved pivot rows of the current panel
+  void* Bbuf;        // [F][16][b] saved pivot rows of the current panel
   void* Tbuf;        // [2][F][b][64] staging blocks of one sweep step
   void* Pbuf;        // [4][F][b][64] partial products of the split tensor-core sweep
-  alignas(64) unsigned char tmap[3][128];  // TMA maps: G tiles, G^H tiles, M row tiles (FP32)
+  alignas(64) unsigned char tmap[2][128];  // TMA maps: G tiles, G^H tiles (FP32)
   int tma_ok;        // 1 if the maps of G were encoded
-  int tma_m_ok;      // 1 if the map of M was encoded
-  int* perm;         // [F][b]
-  int* ipiv;         // [F][32]
-  // wide (two-level, implicitly pivoted) factorisation of FP32 factors
-  int wide_ok;       // 1 if the buffers and TMA maps below exist
   int* rowpiv;       // [F][b] pivot column of each row (-1: not yet pivoted)
   int* pivslot;      // [F][b] pivot row of each column
+  // slab (two-level) factorisation of FP32 factors
+  int wide_ok;       // 1 if the buffers and TMA maps below exist
   void* Wbuf;        // [F][128][b] gathered pivot rows of a slab (outer update)
   alignas(64) unsigned char wmap[2][128];  // TMA maps: A chunks of M, Wbuf rows
   int* flag;         // [F] singular-pivot flags
@@ -239,7 +237,6 @@ rr_status time_solve(rr_factors* fa, int k, float* ms);
 
 // factor.cu
 rr_status launch_factor(rr_factors* f);
-int factor_panel_width(int prec, int b);
 // M = D_i - A_i X_{i-1} for FP32 factors (the Schur update of column i)
 rr_status launch_schur_f32(rr_factors* f, int i, cudaStream_t st);
 // factor_w.cu: the wide FP32 factorisation (TF32 or BF16 operand splits)

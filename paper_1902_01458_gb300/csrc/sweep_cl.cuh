@@ -396,6 +396,7 @@ __global__ void __launch_bounds__(MAXW * 32, 1) sweep_cl_kernel(Args<T> a) {
     }
   }
   if (!ok && tid == 0) atomicExch(a.err, 1);
+  if (!ok) tc::cluster_settle();
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   tc::cluster_sync();  // no CTA leaves while another may still send to it
 }

@@ -139,6 +139,11 @@ __device__ __forceinline__ void st_async16(uint32_t addr, float4 v, uint32_t mba
       "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(mbar)
       : "memory");
 }
+// After a wait has given up: time for the data still on its way between CTAs to
+// land before any of them exits (a sent 16 bytes takes well under a microsecond)
+__device__ __forceinline__ void cluster_settle() {
+  for (int t = 0; t < 50; ++t) __nanosleep(1000);
+}
 // bounded wait that acquires data sent from other CTAs of the cluster
 __device__ __forceinline__ bool cluster_wait(uint64_t* bar, uint32_t parity, uint32_t tries) {
   for (uint32_t t = 0; t < tries; ++t) {
