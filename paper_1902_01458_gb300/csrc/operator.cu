@@ -204,89 +204,37 @@ __global__ void assemble_kernel(AsmParams p, const double* __restrict__ flow,
   }
 }
 
-// y = (s I - L)^H x, optionally r = b - that (the forward product uses the
-// ELL kernel below).  Block (blockIdx.y = problem f) of rows x columns: a
-// group of tpr threads shares one row n and covers its k columns (coalesced
-// [n][k] accesses, the stencil entries read once per group through L1); all
-// index arithmetic is 32-bit and done once per row; Q (unknowns per point) is
-// a template parameter so the 9 x Q stencil loop unrolls and its loads issue
-// together.  (L^T x)[n] sums over the rows r whose stencil reaches n: row r
-// at point (ix - dx, iy - dy) reaches n through its slot (dx, dy).
-template <bool RESID, int Q>
-__global__ void __launch_bounds__(256)
-apply_adjoint_kernel(OpView op, const double2* __restrict__ shifts, int k,
-                     const double2* __restrict__ bvec, const double2* __restrict__ x,
-                     double2* __restrict__ y, const int* __restrict__ amap) {
-  const int f = amap ? amap[blockIdx.y] : (int)blockIdx.y;
-  const int tpr = k < (int)blockDim.x ? k : (int)blockDim.x;
-  const int rows_per = blockDim.x / tpr;
-  const int rsub = threadIdx.x / tpr, jt = threadIdx.x - rsub * tpr;
-  if (rsub >= rows_per) return;
-  const size_t NK = (size_t)op.n * k;
-  const double2* xf = x + (size_t)f * NK;
-  double2* yf = y + (size_t)f * NK;
-  const double2* bf = RESID ? bvec + (size_t)f * NK : nullptr;
-  const double2 s = make_double2(shifts[f].x, -shifts[f].y);
-  constexpr int q = Q, S = 9 * Q;
-  for (int n = blockIdx.x * rows_per + rsub; n < op.n; n += gridDim.x * rows_per) {
-    const int pt = n / q, c = n - pt * q;
-    const int ix = pt / op.ny, iy = pt - ix * op.ny;
-    // bases of the points whose stencils reach n (-1: Dirichlet ghost)
-    int nb[9];
-#pragma unroll
-    for (int dx = -1; dx <= 1; ++dx)
-#pragma unroll
-      for (int dy = -1; dy <= 1; ++dy) {
-        const int jx = ix - dx;
-        const int jy = nbr_y(iy, -dy, op.ny, op.periodic);
-        nb[(dx + 1) * 3 + (dy + 1)] =
-            (jx >= 0 && jx < op.nx && jy >= 0) ? (jx * op.ny + jy) * q : -1;
-      }
-    for (int j = jt; j < k; j += tpr) {
-      double2 acc = cmul(s, xf[(size_t)n * k + j]);
-#pragma unroll
-      for (int sl = 0; sl < 9; ++sl) {
-        const int base = nb[sl];
-        if (base < 0) continue;
-#pragma unroll
-        for (int cr = 0; cr < q; ++cr) {
-          const double a = op.coef[(size_t)(base + cr) * S + sl * q + c];
-          acc = crfma(-a, xf[(size_t)(base + cr) * k + j], acc);
-        }
-      }
-      if (RESID) {
-        const double2 bb = bf[(size_t)n * k + j];
-        acc = mk(bb.x - acc.x, bb.y - acc.y);
-      }
-      yf[(size_t)n * k + j] = acc;
-    }
-  }
-}
-
-// y = (s I - L) x (or r = b - that) from the ELL copy of the stencil: a
-// row's nonzero entries in slot order, the same sum as over all 9q slots
-// (the skipped terms are zero).  The width WT is a compile-time constant so
-// the loop runs exactly WT multiply-adds per entry: the kernel is bound by
-// the FP64 pipe, and the Navier-Stokes rows have at most 13 of their 27
-// slots nonzero.  Threads as in apply_adjoint_kernel.
+// y = (s I - L) x or (s I - L)^H x = (conj(s) I - L^T) x, optionally
+// r = b - that, from the diagonal and an ELL copy of the off-diagonal entries of
+// L or L^T in slot order (the skipped terms are zero).  Block (blockIdx.y =
+// problem f) of rows x columns: a group of tpr threads shares one row n and
+// covers its k columns (coalesced [n][k] accesses, the entries read once per
+// group through L1); all index arithmetic is 32-bit and done once per row.
+// Bound: the FP64 pipe, so the width WT is a compile-time constant (exactly WT
+// real by complex multiply-adds) and the diagonal is folded into the shift:
+// 28 FP64 operations per entry of a Navier-Stokes row (12 off-diagonal
+// entries), 12 of advection-diffusion.  256 x 128, eight shifts, 16 columns:
+// adjoint 1.36 ms over all 27 slots of a row before.
 template <bool RESID, int WT>
 __global__ void __launch_bounds__(256)
-apply_ell_kernel(OpView op, const double2* __restrict__ shifts, int k,
-                 const double2* __restrict__ bvec, const double2* __restrict__ x,
+apply_ell_kernel(int N, const double* __restrict__ diag, const double* __restrict__ val,
+                 const int* __restrict__ col, const double2* __restrict__ shifts, double sign,
+                 int k, const double2* __restrict__ bvec, const double2* __restrict__ x,
                  double2* __restrict__ y, const int* __restrict__ amap) {
   const int f = amap ? amap[blockIdx.y] : (int)blockIdx.y;
   const int tpr = k < (int)blockDim.x ? k : (int)blockDim.x;
   const int rows_per = blockDim.x / tpr;
   const int rsub = threadIdx.x / tpr, jt = threadIdx.x - rsub * tpr;
   if (rsub >= rows_per) return;
-  const size_t NK = (size_t)op.n * k;
+  const size_t NK = (size_t)N * k;
   const double2* xf = x + (size_t)f * NK;
   double2* yf = y + (size_t)f * NK;
   const double2* bf = RESID ? bvec + (size_t)f * NK : nullptr;
-  const double2 s = shifts[f];
-  for (int n = blockIdx.x * rows_per + rsub; n < op.n; n += gridDim.x * rows_per) {
-    const double* ev = op.ell_val + (size_t)n * WT;
-    const int* ec = op.ell_col + (size_t)n * WT;
+  const double sr = shifts[f].x, si = sign * shifts[f].y;
+  for (int n = blockIdx.x * rows_per + rsub; n < N; n += gridDim.x * rows_per) {
+    const double* ev = val + (size_t)n * WT;
+    const int* ec = col + (size_t)n * WT;
+    const double2 s = make_double2(sr - diag[n], si);
     double a[WT];
     int m[WT];
 #pragma unroll
@@ -308,46 +256,57 @@ apply_ell_kernel(OpView op, const double2* __restrict__ shifts, int k,
 }
 
 // Widths the ELL apply kernel is compiled for; a row set is padded to the
-// smallest one that holds its widest row.
-constexpr int kEllWidths[] = {4, 6, 8, 10, 13, 16, 20, 27};
+// smallest one that holds its widest row (at most 9 q - 1 entries).
+constexpr int kEllWidths[] = {4, 6, 8, 10, 12, 13, 15, 16, 20, 27, 35};
 
-// ELL copy of the stencil: the widest row, then every row's nonzero entries
-// in slot order, padded with zero entries on the row itself.  Both kernels
-// walk the entries of a row with the same rule (in-grid neighbour, nonzero
-// coefficient), so the counted width always holds the filled row; a row that
-// would not fit anyway sets *overflow instead of losing entries.
-template <typename Visit>
-__device__ __forceinline__ void ell_row_entries(const OpView& op, int n, Visit&& visit) {
-  const int q = op.q, pt = n / q;
+// Visits the off-diagonal nonzero entries of row n of L (TRANS: of L^T: the
+// rows r at the points (ix - dx, iy - dy) reach n through their slot (dx, dy)),
+// in slot order; returns the diagonal entry.  The count and the fill walk the
+// entries with this one rule, so the counted width always holds the filled
+// row; a row that would not fit anyway sets *overflow instead of losing entries.
+template <bool TRANS, typename Visit>
+__device__ __forceinline__ double ell_row_entries(const OpView& op, int n, Visit&& visit) {
+  const int q = op.q, pt = n / q, c = n - pt * q;
   const int ix = pt / op.ny, iy = pt - ix * op.ny;
-  const double* cf = op.coef + (size_t)n * op.S;
+  double diag = 0.0;
   for (int sl = 0; sl < 9; ++sl) {
-    const int jx = ix + sl / 3 - 1;
-    const int jy = nbr_y(iy, sl % 3 - 1, op.ny, op.periodic);
+    const int dx = sl / 3 - 1, dy = sl % 3 - 1;
+    const int jx = TRANS ? ix - dx : ix + dx;
+    const int jy = nbr_y(iy, TRANS ? -dy : dy, op.ny, op.periodic);
     if (jx < 0 || jx >= op.nx || jy < 0) continue;
     for (int cp = 0; cp < q; ++cp) {
-      const double a = cf[sl * q + cp];
-      if (a != 0.0) visit(a, (jx * op.ny + jy) * q + cp);
+      const int m = (jx * op.ny + jy) * q + cp;
+      const double a = TRANS ? op.coef[(size_t)m * op.S + sl * q + c]
+                             : op.coef[(size_t)n * op.S + sl * q + cp];
+      if (m == n) diag = a;
+      else if (a != 0.0) visit(a, m);
     }
+  }
+  return diag;
+}
+
+// wmax[t]: widest row of L (t = 0) and L^T (t = 1)
+__global__ void ell_count_kernel(OpView op, int* wmax) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  int c0 = 0, c1 = 0;
+  if (n < op.n) {
+    ell_row_entries<false>(op, n, [&](double, int) { ++c0; });
+    ell_row_entries<true>(op, n, [&](double, int) { ++c1; });
+  }
+  const int m0 = __reduce_max_sync(0xffffffffu, c0), m1 = __reduce_max_sync(0xffffffffu, c1);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(wmax, m0);
+    atomicMax(wmax + 1, m1);
   }
 }
 
-__global__ void ell_count_kernel(OpView op, int* wmax) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= op.n) return;
-  int cnt = 0;
-  ell_row_entries(op, n, [&](double, int) { ++cnt; });
-  atomicMax(wmax, cnt);
-}
-
-__global__ void ell_fill_kernel(OpView op, int W, double* __restrict__ val, int* __restrict__ col,
-                                int* overflow) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= op.n) return;
+template <bool TRANS>
+__device__ __forceinline__ void ell_fill_row(const OpView& op, int n, int W, double* val, int* col,
+                                             double* diag, int* overflow) {
   double* v = val + (size_t)n * W;
   int* c = col + (size_t)n * W;
   int t = 0;
-  ell_row_entries(op, n, [&](double a, int m) {
+  const double d = ell_row_entries<TRANS>(op, n, [&](double a, int m) {
     if (t < W) {
       v[t] = a;
       c[t] = m;
@@ -359,6 +318,16 @@ __global__ void ell_fill_kernel(OpView op, int W, double* __restrict__ val, int*
     v[t] = 0.0;
     c[t] = n;
   }
+  if (!TRANS) diag[n] = d;
+}
+
+__global__ void ell_fill_kernel(OpView op, int W0, int W1, double* __restrict__ val0,
+                                int* __restrict__ col0, double* __restrict__ val1,
+                                int* __restrict__ col1, double* __restrict__ diag, int* overflow) {
+  const int n = blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= op.n) return;
+  ell_fill_row<false>(op, n, W0, val0, col0, diag, overflow);
+  ell_fill_row<true>(op, n, W1, val1, col1, diag, overflow);
 }
 
 __global__ void phi_kernel(const double* __restrict__ flow, int nx, int ny, int periodic,
@@ -384,41 +353,45 @@ __global__ void round_coef_kernel(const double* __restrict__ in, float* __restri
 static dim3 apply_grid(const OpDev& d, int F, int k);
 
 rr_status build_ell(OpDev& d) {
-  int* wdev = nullptr;  // [0] widest row, [1] overflow flag of the fill
-  RR_CUDA(cudaMalloc(&wdev, 2 * sizeof(int)));
+  int* wdev = nullptr;  // [0..1] widest rows of L and L^T, [2] overflow flag of the fill
+  RR_CUDA(cudaMalloc(&wdev, 3 * sizeof(int)));
   const int blocks = (d.n + 255) / 256;
-  int W = 0;
-  cudaError_t e = cudaMemset(wdev, 0, 2 * sizeof(int));
+  int W[2] = {0, 0};
+  cudaError_t e = cudaMemset(wdev, 0, 3 * sizeof(int));
   if (e == cudaSuccess) {
     prof_count(1);
     ell_count_kernel<<<blocks, 256>>>(view(d), wdev);
-    e = cudaMemcpy(&W, wdev, sizeof(int), cudaMemcpyDeviceToHost);
+    e = cudaMemcpy(W, wdev, 2 * sizeof(int), cudaMemcpyDeviceToHost);
   }
   if (e != cudaSuccess) {
     cudaFree(wdev);
     return cuda_status(e, "ELL stencil width");
   }
   constexpr int kWidest = kEllWidths[sizeof(kEllWidths) / sizeof(int) - 1];
-  if (W > kWidest) {
+  if (W[0] > kWidest || W[1] > kWidest) {
     cudaFree(wdev);
     set_error("ELL stencil row wider than the widest compiled apply kernel");
     return RR_ERR_ARG;
   }
-  d.ell_w = kWidest;
-  for (int w : kEllWidths)
-    if (w >= W) {
-      d.ell_w = w;
-      break;
-    }
-  e = cudaMalloc(&d.ell_val, (size_t)d.n * d.ell_w * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&d.ell_col, (size_t)d.n * d.ell_w * sizeof(int));
+  e = cudaMalloc(&d.diag, (size_t)d.n * sizeof(double));
+  for (int t = 0; t < 2 && e == cudaSuccess; ++t) {
+    d.ell_w[t] = kWidest;
+    for (int w : kEllWidths)
+      if (w >= W[t]) {
+        d.ell_w[t] = w;
+        break;
+      }
+    e = cudaMalloc(&d.ell_val[t], (size_t)d.n * d.ell_w[t] * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&d.ell_col[t], (size_t)d.n * d.ell_w[t] * sizeof(int));
+  }
   int overflow = 0;
   if (e == cudaSuccess) {
     prof_count(1);
-    ell_fill_kernel<<<blocks, 256>>>(view(d), d.ell_w, d.ell_val, d.ell_col, wdev + 1);
+    ell_fill_kernel<<<blocks, 256>>>(view(d), d.ell_w[0], d.ell_w[1], d.ell_val[0], d.ell_col[0],
+                                     d.ell_val[1], d.ell_col[1], d.diag, wdev + 2);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpy(&overflow, wdev + 1, sizeof(int), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(&overflow, wdev + 2, sizeof(int), cudaMemcpyDeviceToHost);
   cudaFree(wdev);
   if (e != cudaSuccess) return cuda_status(e, "ELL stencil copy");
   if (overflow) {
@@ -428,24 +401,25 @@ rr_status build_ell(OpDev& d) {
   return RR_OK;
 }
 
-// Forward operator application (adjoint == 0) on the ELL copy, by width.
+// Operator application (or residual) on the ELL copies, by width.
 template <bool RESID>
-static rr_status launch_ell(const OpDev& d, int F, const double2* shifts, int k,
+static rr_status launch_ell(const OpDev& d, int F, const double2* shifts, int k, int adjoint,
                             const double2* b, const double2* x, double2* y, cudaStream_t st,
                             const int* amap) {
   const dim3 grid = apply_grid(d, F, k);
-  const OpView v = view(d);
-  switch (d.ell_w) {
-    case 4: apply_ell_kernel<RESID, 4><<<grid, 256, 0, st>>>(v, shifts, k, b, x, y, amap); break;
-    case 6: apply_ell_kernel<RESID, 6><<<grid, 256, 0, st>>>(v, shifts, k, b, x, y, amap); break;
-    case 8: apply_ell_kernel<RESID, 8><<<grid, 256, 0, st>>>(v, shifts, k, b, x, y, amap); break;
-    case 10: apply_ell_kernel<RESID, 10><<<grid, 256, 0, st>>>(v, shifts, k, b, x, y, amap); break;
-    case 13: apply_ell_kernel<RESID, 13><<<grid, 256, 0, st>>>(v, shifts, k, b, x, y, amap); break;
-    case 16: apply_ell_kernel<RESID, 16><<<grid, 256, 0, st>>>(v, shifts, k, b, x, y, amap); break;
-    case 20: apply_ell_kernel<RESID, 20><<<grid, 256, 0, st>>>(v, shifts, k, b, x, y, amap); break;
-    case 27: apply_ell_kernel<RESID, 27><<<grid, 256, 0, st>>>(v, shifts, k, b, x, y, amap); break;
+  const int t = adjoint ? 1 : 0;
+  const double sign = adjoint ? -1.0 : 1.0;
+#define RR_ELL(W)                                                                               \
+  case W:                                                                                       \
+    apply_ell_kernel<RESID, W><<<grid, 256, 0, st>>>(d.n, d.diag, d.ell_val[t], d.ell_col[t],   \
+                                                     shifts, sign, k, b, x, y, amap);           \
+    break;
+  switch (d.ell_w[t]) {
+    RR_ELL(4) RR_ELL(6) RR_ELL(8) RR_ELL(10) RR_ELL(12) RR_ELL(13) RR_ELL(15) RR_ELL(16)
+    RR_ELL(20) RR_ELL(27) RR_ELL(35)
     default: set_error("ELL width without a compiled kernel"); return RR_ERR_ARG;
   }
+#undef RR_ELL
   RR_CUDA(cudaGetLastError());
   return RR_OK;
 }
@@ -484,18 +458,7 @@ static dim3 apply_grid(const OpDev& d, int F, int k) {
 rr_status launch_apply(const OpDev& d, int F, const double2* shifts, int k, int adjoint,
                        const double2* x, double2* y, cudaStream_t st) {
   prof_count(1);
-  if (!adjoint) return launch_ell<false>(d, F, shifts, k, nullptr, x, y, st, nullptr);
-  if (d.q == 4)
-    apply_adjoint_kernel<false, 4><<<apply_grid(d, F, k), 256, 0, st>>>(view(d), shifts, k,
-                                                                        nullptr, x, y, nullptr);
-  else if (d.q == 3)
-    apply_adjoint_kernel<false, 3><<<apply_grid(d, F, k), 256, 0, st>>>(view(d), shifts, k,
-                                                                        nullptr, x, y, nullptr);
-  else
-    apply_adjoint_kernel<false, 1><<<apply_grid(d, F, k), 256, 0, st>>>(view(d), shifts, k,
-                                                                        nullptr, x, y, nullptr);
-  RR_CUDA(cudaGetLastError());
-  return RR_OK;
+  return launch_ell<false>(d, F, shifts, k, adjoint, nullptr, x, y, st, nullptr);
 }
 
 // ----------------------------------------------------------------------------
@@ -591,23 +554,9 @@ rr_status launch_residual(const OpDev& d, int F, const double2* shifts, int k, i
                           const double2* b, const double2* x, double2* r, cudaStream_t st,
                           const int* amap) {
   prof_begin(PROF_RESIDUAL, st);
-  if (!adjoint) {
-    rr_status s = launch_ell<true>(d, F, shifts, k, b, x, r, st, amap);
-    prof_end(PROF_RESIDUAL, st);
-    return s;
-  }
-  if (d.q == 4)
-    apply_adjoint_kernel<true, 4><<<apply_grid(d, F, k), 256, 0, st>>>(view(d), shifts, k, b, x,
-                                                                       r, amap);
-  else if (d.q == 3)
-    apply_adjoint_kernel<true, 3><<<apply_grid(d, F, k), 256, 0, st>>>(view(d), shifts, k, b, x,
-                                                                       r, amap);
-  else
-    apply_adjoint_kernel<true, 1><<<apply_grid(d, F, k), 256, 0, st>>>(view(d), shifts, k, b, x,
-                                                                       r, amap);
+  const rr_status s = launch_ell<true>(d, F, shifts, k, adjoint, b, x, r, st, amap);
   prof_end(PROF_RESIDUAL, st);
-  RR_CUDA(cudaGetLastError());
-  return RR_OK;
+  return s;
 }
 
 rr_status launch_phi(const OpDev& d, double* phi, cudaStream_t st) {

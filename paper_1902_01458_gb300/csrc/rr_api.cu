@@ -577,11 +577,13 @@ extern "C" rr_status rr_create_operator(const rr_grid* g, const rr_baseflow* fl,
   d.dy = d.periodic ? (g->y1 - g->y0) / g->ny : (g->y1 - g->y0) / (g->ny + 1);
   d.device = device;
   d.coef = nullptr; d.coef32 = nullptr; d.wsqrt = nullptr; d.wisqrt = nullptr; d.flow = nullptr;
-  d.ell_val = nullptr; d.ell_col = nullptr; d.ell_w = 0;
+  d.diag = nullptr;
+  for (int t = 0; t < 2; ++t) { d.ell_val[t] = nullptr; d.ell_col[t] = nullptr; d.ell_w[t] = 0; }
   rr_status s;
   auto fail = [&](rr_status st) {
     cudaFree(d.coef); cudaFree(d.coef32); cudaFree(d.wsqrt); cudaFree(d.wisqrt); cudaFree(d.flow);
-    cudaFree(d.ell_val); cudaFree(d.ell_col);
+    cudaFree(d.diag);
+    for (int t = 0; t < 2; ++t) { cudaFree(d.ell_val[t]); cudaFree(d.ell_col[t]); }
     delete op;
     return st;
   };
@@ -622,8 +624,11 @@ extern "C" rr_status rr_destroy_operator(rr_operator* op) {
   DeviceGuard guard(op->d.device);
   cudaFree(op->d.coef);
   cudaFree(op->d.coef32);
-  cudaFree(op->d.ell_val);
-  cudaFree(op->d.ell_col);
+  cudaFree(op->d.diag);
+  for (int t = 0; t < 2; ++t) {
+    cudaFree(op->d.ell_val[t]);
+    cudaFree(op->d.ell_col[t]);
+  }
   cudaFree(op->d.wsqrt);
   cudaFree(op->d.wisqrt);
   cudaFree(op->d.flow);
