@@ -3,9 +3,11 @@
 // of the small k x N matrix B via its k x k R factor (fifth step), and the
 // recovery of sigma_j and u_j by column norms (Eq. 8, seventh and eighth
 // steps), plus the sorting and phase normalisation of the outputs.
+#include <algorithm>
 #include <cmath>
 
 #include "rr_internal.cuh"
+#include "tc.cuh"
 
 namespace {
 
@@ -213,19 +215,28 @@ __global__ void gram_part_kernel(int N, int k, int nblk, const double2* __restri
   }
 }
 
+// G[f] = sum of the partials, a fixed order: part t of 8 adds the blocks t, t + 8,
+// ..., then the parts in order (a thread per element waited for up to 304
+// dependent loads, 78 us)
 __global__ void gram_reduce_kernel(int F, int k, int nblk, const double2* __restrict__ part,
                                    double2* __restrict__ G) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  int kk = k * k;
-  if (e >= F * kk) return;
-  int f = e / kk, p = e % kk;
+  __shared__ double2 ps[8][32];
+  const int kk = k * k, le = threadIdx.x & 31, t = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + le;
+  const int f = e / kk, p = e - f * kk;
   const int a = p / k, c = p - a * k;
   // only the upper triangle was formed: G[c][a] = conj(G[a][c])
   const int src = a <= c ? p : c * k + a;
   double2 s = make_double2(0.0, 0.0);
-  for (int b = 0; b < nblk; ++b) s = cadd(s, part[((size_t)f * nblk + b) * kk + src]);
-  if (a > c) s.y = -s.y;
-  G[e] = s;
+  if (e < F * kk)
+    for (int b = t; b < nblk; b += 8) s = cadd(s, part[((size_t)f * nblk + b) * kk + src]);
+  ps[t][le] = s;
+  __syncthreads();
+  if (t == 0 && e < F * kk) {
+    for (int u = 1; u < 8; ++u) s = cadd(s, ps[u][le]);
+    if (a > c) s.y = -s.y;
+    G[e] = s;
+  }
 }
 
 // Cholesky G (+ shift) = R^H R (R upper) and R^{-1}; one CTA per problem.
@@ -280,19 +291,33 @@ __global__ void cholesky_kernel(int k, const double2* __restrict__ Gall, double2
     int i = e / k, c = e % k;
     R[e] = (c >= i) ? A[e] : make_double2(0.0, 0.0);
   }
-  // R^{-1}: thread per column, back substitution
+  // R^{-1}: four lanes per column share the sums of the back substitution
+  // (a thread per column left most of the FP64 pipe idle)
   double2* Ri = Riall + (size_t)f * kk;
-  if (threadIdx.x < k) {
-    const int c = threadIdx.x;
-    for (int i = k - 1; i >= 0; --i) {
-      double2 s = (i == c) ? make_double2(1.0, 0.0) : make_double2(0.0, 0.0);
-      if (i <= c)
-        for (int m = i + 1; m <= c; ++m) s = csub(s, cmul(A[i * k + m], Ri[m * k + c]));
-      else
-        s = make_double2(0.0, 0.0);
-      Ri[i * k + c] = (i <= c) ? make_double2(s.x / A[i * k + i].x, s.y / A[i * k + i].x)
-                               : make_double2(0.0, 0.0);
+  double2* I = A + kk;  // [k][k], column c by its four lanes
+  for (int c0 = 0; c0 < k; c0 += blockDim.x / 4) {
+    const int c = c0 + (threadIdx.x >> 2), h = threadIdx.x & 3;
+    // the lanes of a warp run as many rows as its last column
+    const int top = min(k - 1, c0 + (int)(threadIdx.x >> 5) * 8 + 7);
+    for (int i = top; i >= 0; --i) {
+      double2 s = make_double2(0.0, 0.0);
+      if (c < k && i < c)
+        for (int m = i + 1 + h; m <= c; m += 4) s = cfma(A[i * k + m], I[m * k + c], s);
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, 1);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, 1);
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, 2);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, 2);
+      if (c < k && i <= c && h == 0) {
+        const double d = A[i * k + i].x;
+        I[i * k + c] = i == c ? make_double2(1.0 / d, 0.0) : make_double2(-s.x / d, -s.y / d);
+      }
+      __syncwarp();
     }
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < kk; e += blockDim.x) {
+    const int i = e / k, c = e - i * k;
+    Ri[e] = i <= c ? I[e] : make_double2(0.0, 0.0);
   }
   if (threadIdx.x == 0) {
     double mx = 0.0, mn = 1e300;
@@ -354,21 +379,33 @@ __global__ void right_mul_upper_kernel(int N, int k, int RB, const double2* Y,
     for (int e = threadIdx.x; e < rows * kh; e += blockDim.x) {
       const int r = e / kh, j1 = e - r * kh, j2 = k - 1 - j1;
       const double2* yr = Yr + r * k;
-      double2 s1 = make_double2(0.0, 0.0), s2 = make_double2(0.0, 0.0);
-      for (int m = 0; m <= j1; ++m) s1 = cfma(yr[m], S[m * k + j1], s1);
-      of[(size_t)(n0 + r) * k + j1] = s1;
-      if (j2 != j1) {
-        for (int m = 0; m <= j2; ++m) s2 = cfma(yr[m], S[m * k + j2], s2);
-        of[(size_t)(n0 + r) * k + j2] = s2;
+      // one loop over both columns, so that lanes with a short first column
+      // are already in their second one
+      double2 s = make_double2(0.0, 0.0), s1 = s;
+      const double2* sp = S + j1;
+      int m = 0;
+      for (int t = 0; t <= k; ++t) {
+        s = cfma(yr[m], sp[m * k], s);
+        if (++m > j1 && sp == S + j1) {
+          s1 = s;
+          s = make_double2(0.0, 0.0);
+          sp = S + j2;
+          m = 0;
+        }
+        if (j2 == j1 && t == j1) break;
       }
+      of[(size_t)(n0 + r) * k + j1] = s1;
+      if (j2 != j1) of[(size_t)(n0 + r) * k + j2] = s;
     }
   }
 }
 
+// C = A B per problem (blockIdx.x), rows spread over blockIdx.y: FP64-bound, so
+// one CTA per problem left the other SMs idle (286 us at k = 64)
 __global__ void small_mul_kernel(int k, const double2* __restrict__ A, const double2* __restrict__ B,
                                  double2* __restrict__ C) {
   const int f = blockIdx.x, kk = k * k;
-  for (int e = threadIdx.x; e < kk; e += blockDim.x) {
+  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < kk; e += gridDim.y * blockDim.x) {
     int i = e / k, j = e % k;
     double2 s = make_double2(0.0, 0.0);
     for (int m = 0; m < k; ++m) s = cfma(A[(size_t)f * kk + i * k + m], B[(size_t)f * kk + m * k + j], s);
@@ -377,101 +414,185 @@ __global__ void small_mul_kernel(int k, const double2* __restrict__ A, const dou
 }
 
 // One-sided Jacobi SVD of a k x k matrix R = Ul diag(sigma) Vr^H, applied to
-// the columns of M = R^H (M J = Vr Sigma with J = Ul).  One warp per column
-// pair, round-robin ordering, one CTA per problem; sigma sorted descending.
-__global__ void jacobi_svd_kernel(int k, int kp, const double2* __restrict__ Rall,
-                                  double* __restrict__ sig_out, double2* __restrict__ Ul_out,
-                                  double2* __restrict__ Vr_out, int* __restrict__ sweeps_out) {
+// the columns of M = R^H (M J = Vr Sigma with J = Ul); sigma sorted descending.
+// A cluster of CL CTAs per problem: column c of M and J lives in CTA c % CL, one
+// warp per column pair (round-robin ordering) reads its two columns from their
+// CTAs, rotates them in registers and writes them back; a cluster barrier ends
+// a round.  Bound: the FP64 pipe (a warp's instruction takes 64 cycles of its
+// quarter of an SM), so the pairs are spread over SMs, four warps each: k = 64
+// took 24.4 ms with the 32 warps on one SM.
+constexpr int JAC_CLMAX = 8;
+inline int jac_cluster(int kp) { return std::max(1, std::min(JAC_CLMAX, kp / 8)); }
+inline int jac_warps(int kp, int CL) { return (kp / 2 + CL - 1) / CL; }
+
+__device__ __forceinline__ double2 ld_cluster_c(uint32_t addr) {
+  double2 v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];\n" : "=d"(v.x), "=d"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_cluster_c(uint32_t addr, double2 v) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};\n" ::"r"(addr), "d"(v.x), "d"(v.y) : "memory");
+}
+
+// sums of four values over the warp, all four in every lane: the first two
+// exchanges halve the values a lane carries, so a lane adds 6 times, not 20
+__device__ __forceinline__ void warp_sum4(double& a, double& b, double& c, double& d) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const bool h1 = lane & 1, h2 = lane & 2;
+  // after step 1: even lanes carry (a, b), odd lanes (c, d)
+  double s0 = h1 ? a : c, s1 = h1 ? b : d, k0 = h1 ? c : a, k1 = h1 ? d : b;
+  k0 += __shfl_xor_sync(full, s0, 1);
+  k1 += __shfl_xor_sync(full, s1, 1);
+  // after step 2: one value per lane, by lane % 4: a, c, b, d
+  double s = h2 ? k0 : k1, k = h2 ? k1 : k0;
+  k += __shfl_xor_sync(full, s, 2);
+  k += __shfl_xor_sync(full, k, 4);
+  k += __shfl_xor_sync(full, k, 8);
+  k += __shfl_xor_sync(full, k, 16);
+  a = __shfl_sync(full, k, 0);
+  c = __shfl_sync(full, k, 1);
+  b = __shfl_sync(full, k, 2);
+  d = __shfl_sync(full, k, 3);
+}
+
+__global__ void __launch_bounds__(256)
+jacobi_svd_kernel(int k, int kp, int CL, const double2* __restrict__ Rall,
+                  double* __restrict__ sig_out, double2* __restrict__ Ul_out,
+                  double2* __restrict__ Vr_out, int* __restrict__ sweeps_out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double2* A = reinterpret_cast<double2*>(smem_raw);  // column-major [kp cols][kp rows]
-  double2* J = A + kp * kp;                            // column-major
-  double* nrm = reinterpret_cast<double*>(J + kp * kp);  // [kp]
-  int* order = reinterpret_cast<int*>(nrm + kp);        // [kp]
-  __shared__ int s_rot;
-  const int f = blockIdx.x, kk = k * k;
+  const int ncol = (kp + CL - 1) / CL;                 // columns of a CTA
+  double2* A = reinterpret_cast<double2*>(smem_raw);   // [ncol][kp]
+  double2* J = A + ncol * kp;                          // [ncol][kp]
+  __shared__ double nrm[64];
+  __shared__ int rank_of[64];
+  __shared__ int rot[2];
+  const int rank = (int)tc::cluster_rank();
+  const int f = blockIdx.x / CL, kk = k * k;
   const double2* R = Rall + (size_t)f * kk;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int npair = kp / 2;
-  // M = R^H: M[row i][col c] = conj(R[c][i]); column c of M stored at A[c*kp + i]
-  for (int e = threadIdx.x; e < kp * kp; e += blockDim.x) {
-    int c = e / kp, i = e % kp;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nthr = blockDim.x;
+  const int npair = kp / 2, pair = warp * CL + rank;
+  // column c of M = R^H: M[i][c] = conj(R[c][i])
+  for (int e = threadIdx.x; e < ncol * kp; e += nthr) {
+    const int c = (e / kp) * CL + rank, i = e - (e / kp) * kp;
     A[e] = (c < k && i < k) ? cconj(R[c * k + i]) : make_double2(0.0, 0.0);
     J[e] = (c == i) ? make_double2(1.0, 0.0) : make_double2(0.0, 0.0);
   }
-  __syncthreads();
+  if (threadIdx.x < 2) rot[threadIdx.x] = 0;
+  const uint32_t A_a = tc::smem_u32(A), J_a = tc::smem_u32(J), rot_a = tc::smem_u32(rot);
+  tc::cluster_sync();
   int sweep = 0;
   for (; sweep < 60; ++sweep) {
-    if (threadIdx.x == 0) s_rot = 0;
-    __syncthreads();
+    const int sp = sweep & 1;
     for (int step = 0; step < kp - 1; ++step) {
-      if (warp < npair) {
+      if (pair < npair) {
         int p, q;
-        if (warp == 0) { p = kp - 1; q = step; }
-        else {
-          p = (step + warp) % (kp - 1);
-          q = (step - warp + (kp - 1)) % (kp - 1);
+        if (pair == 0) {
+          p = kp - 1;
+          q = step;
+        } else {
+          p = (step + pair) % (kp - 1);
+          q = (step - pair + (kp - 1)) % (kp - 1);
         }
-        if (p > q) { int t = p; p = q; q = t; }
+        if (p > q) {
+          const int t = p;
+          p = q;
+          q = t;
+        }
+        const uint32_t op = (uint32_t)((p / CL) * kp * 16), oq = (uint32_t)((q / CL) * kp * 16);
+        const uint32_t ap = tc::cluster_map(A_a + op, p % CL), aq = tc::cluster_map(A_a + oq, q % CL);
+        double2 x[2], y[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int i = lane + 32 * u;
+          x[u] = i < kp ? ld_cluster_c(ap + i * 16) : make_double2(0.0, 0.0);
+          y[u] = i < kp ? ld_cluster_c(aq + i * 16) : make_double2(0.0, 0.0);
+        }
         double al = 0.0, be = 0.0;
         double2 ga = make_double2(0.0, 0.0);
-        for (int i = lane; i < kp; i += 32) {
-          double2 x = A[p * kp + i], y = A[q * kp + i];
-          al += x.x * x.x + x.y * x.y;
-          be += y.x * y.x + y.y * y.y;
-          ga = cfmac(x, y, ga);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if (u == 1 && kp <= 32) break;
+          al += x[u].x * x[u].x + x[u].y * x[u].y;
+          be += y[u].x * y[u].x + y[u].y * y[u].y;
+          ga = cfmac(x[u], y[u], ga);
         }
-        for (int o = 16; o > 0; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o);
-          ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
-        }
-        double g = sqrt(ga.x * ga.x + ga.y * ga.y);
+        warp_sum4(al, be, ga.x, ga.y);
+        const double g = sqrt(ga.x * ga.x + ga.y * ga.y);
         if (g > 1e-15 * sqrt(al * be) && g > 1e-300) {
-          double zeta = (be - al) / (2.0 * g);
-          double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-          double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-          double2 ph = make_double2(ga.x / g, -ga.y / g);  // e^{-i phi}
-          for (int i = lane; i < kp; i += 32) {
-            double2 x = A[p * kp + i], y = cmul(ph, A[q * kp + i]);
-            A[p * kp + i] = make_double2(c * x.x - s * y.x, c * x.y - s * y.y);
-            A[q * kp + i] = make_double2(s * x.x + c * y.x, s * x.y + c * y.y);
-            double2 u = J[p * kp + i], v = cmul(ph, J[q * kp + i]);
-            J[p * kp + i] = make_double2(c * u.x - s * v.x, c * u.y - s * v.y);
-            J[q * kp + i] = make_double2(s * u.x + c * v.x, s * u.y + c * v.y);
+          const uint32_t jp = tc::cluster_map(J_a + op, p % CL), jq = tc::cluster_map(J_a + oq, q % CL);
+          double2 u2[2], v2[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int i = lane + 32 * u;
+            u2[u] = i < kp ? ld_cluster_c(jp + i * 16) : make_double2(0.0, 0.0);
+            v2[u] = i < kp ? ld_cluster_c(jq + i * 16) : make_double2(0.0, 0.0);
           }
-          if (lane == 0) atomicAdd(&s_rot, 1);
+          const double zeta = (be - al) / (2.0 * g);
+          const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+          const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
+          const double2 ph = make_double2(ga.x / g, -ga.y / g);  // e^{-i phi}
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int i = lane + 32 * u;
+            if (i >= kp) continue;
+            const double2 yy = cmul(ph, y[u]), vv = cmul(ph, v2[u]);
+            st_cluster_c(ap + i * 16, make_double2(c * x[u].x - s * yy.x, c * x[u].y - s * yy.y));
+            st_cluster_c(aq + i * 16, make_double2(s * x[u].x + c * yy.x, s * x[u].y + c * yy.y));
+            st_cluster_c(jp + i * 16, make_double2(c * u2[u].x - s * vv.x, c * u2[u].y - s * vv.y));
+            st_cluster_c(jq + i * 16, make_double2(s * u2[u].x + c * vv.x, s * u2[u].y + c * vv.y));
+          }
+          if (lane == 0) rot[sp] = 1;
         }
       }
-      __syncthreads();
+      tc::cluster_sync();
     }
-    if (s_rot == 0) break;
-    __syncthreads();
+    // rotations of this sweep in any CTA; the other parity's flag is read by
+    // no one until the next sweep ends
+    int any = 0;
+    for (int r = 0; r < CL; ++r) {
+      int v;
+      asm volatile("ld.shared::cluster.s32 %0, [%1];\n" : "=r"(v) : "r"(tc::cluster_map(rot_a + sp * 4, r)) : "memory");
+      any |= v;
+    }
+    if (threadIdx.x == 0) rot[sp ^ 1] = 0;
+    tc::cluster_sync();
+    if (!any) break;
   }
-  // column norms and descending order (stable by index)
-  for (int c = threadIdx.x; c < kp; c += blockDim.x) {
+  // column norms (to every CTA) and descending order (stable by index)
+  for (int lc = warp; lc < ncol; lc += nthr >> 5) {
+    const int c = lc * CL + rank;
+    if (c >= kp) continue;
     double s = 0.0;
-    for (int i = 0; i < kp; ++i) s += cabs2(A[c * kp + i]);
-    nrm[c] = (c < k) ? sqrt(s) : -1.0;
+    for (int i = lane; i < kp; i += 32) s += cabs2(A[lc * kp + i]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const double nv = c < k ? sqrt(s) : -1.0;
+    if (lane < CL)
+      asm volatile("st.shared::cluster.f64 [%0], %1;\n" ::"r"(
+                       tc::cluster_map(tc::smem_u32(&nrm[c]), lane)),
+                   "d"(nv)
+                   : "memory");
   }
-  __syncthreads();
-  for (int c = threadIdx.x; c < k; c += blockDim.x) {
-    int rank = 0;
+  tc::cluster_sync();
+  for (int c = threadIdx.x; c < k; c += nthr) {
+    int rk = 0;
     for (int m = 0; m < k; ++m)
-      if (nrm[m] > nrm[c] || (nrm[m] == nrm[c] && m < c)) ++rank;
-    order[rank] = c;
+      if (nrm[m] > nrm[c] || (nrm[m] == nrm[c] && m < c)) ++rk;
+    rank_of[c] = rk;
+    if (rank == 0) sig_out[(size_t)f * k + rk] = nrm[c];
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < kk; e += blockDim.x) {
-    int i = e / k, jn = e % k;  // output row i, output column jn
-    int c = order[jn];
-    double sg = nrm[c];
-    Ul_out[(size_t)f * kk + e] = J[c * kp + i];
-    double2 a = A[c * kp + i];
-    Vr_out[(size_t)f * kk + e] = (sg > 0.0) ? make_double2(a.x / sg, a.y / sg) : make_double2(0.0, 0.0);
+  for (int e = threadIdx.x; e < ncol * kp; e += nthr) {
+    const int lc = e / kp, c = lc * CL + rank, i = e - lc * kp;
+    if (c >= k || i >= k) continue;
+    const int jn = rank_of[c];
+    const double sg = nrm[c];
+    Ul_out[(size_t)f * kk + (size_t)i * k + jn] = J[e];
+    const double2 a = A[e];
+    Vr_out[(size_t)f * kk + (size_t)i * k + jn] =
+        (sg > 0.0) ? make_double2(a.x / sg, a.y / sg) : make_double2(0.0, 0.0);
   }
-  for (int jn = threadIdx.x; jn < k; jn += blockDim.x) sig_out[(size_t)f * k + jn] = nrm[order[jn]];
-  if (threadIdx.x == 0 && sweeps_out) sweeps_out[f] = sweep;
+  if (rank == 0 && threadIdx.x == 0 && sweeps_out) sweeps_out[f] = sweep;
 }
 
 __global__ void col_scale_kernel(int F, int N, int k, const double2* __restrict__ in,
@@ -659,18 +780,18 @@ rr_status launch_gram(int F, int N, int k, const double2* Y, double2* part, int 
   gram_part_kernel<<<dim3(nblk, F), 256, smem, st>>>(N, k, nblk, Y, part);
   prof_end(PROF_GRAM, st);
   prof_count(1);
-  gram_reduce_kernel<<<(F * k * k + 127) / 128, 128, 0, st>>>(F, k, nblk, part, G);
+  gram_reduce_kernel<<<(F * k * k + 31) / 32, 256, 0, st>>>(F, k, nblk, part, G);
   RR_CUDA(cudaGetLastError());
   return RR_OK;
 }
 
 rr_status launch_cholesky(int F, int k, const double2* G, double2* R, double2* Rinv, int* bad,
                           double shift_rel, double* cond, cudaStream_t st) {
-  size_t smem = (size_t)k * k * sizeof(double2);
+  size_t smem = (size_t)2 * k * k * sizeof(double2);
   static bool attr = false;
   if (!attr) {
     RR_CUDA(cudaFuncSetAttribute(cholesky_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 96 * 1024));
+                                 2 * 64 * 64 * (int)sizeof(double2)));
     attr = true;
   }
   prof_begin(PROF_SMALL, st);
@@ -707,7 +828,7 @@ rr_status launch_right_mul(int F, int N, int k, const double2* Y, const double2*
 rr_status launch_small_mul(int F, int k, const double2* A, const double2* B, double2* C,
                            cudaStream_t st) {
   prof_count(1);
-  small_mul_kernel<<<F, 256, 0, st>>>(k, A, B, C);
+  small_mul_kernel<<<dim3(F, (k * k + 127) / 128), 128, 0, st>>>(k, A, B, C);
   RR_CUDA(cudaGetLastError());
   return RR_OK;
 }
@@ -716,17 +837,22 @@ rr_status launch_jacobi_svd(int F, int k, const double2* R, double* sigma, doubl
                             double2* Vr, int* sweeps, cudaStream_t st) {
   int kp = (k + 1) & ~1;
   if (kp < 2) kp = 2;
-  size_t smem = 2 * (size_t)kp * kp * sizeof(double2) + kp * (sizeof(double) + sizeof(int));
-  static bool attr = false;
-  if (!attr) {
-    RR_CUDA(cudaFuncSetAttribute(jacobi_svd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 160 * 1024));
-    attr = true;
-  }
-  int threads = 32 * (kp / 2);
-  if (threads < 64) threads = 64;
+  const int CL = jac_cluster(kp);
+  const size_t smem = 2 * (size_t)((kp + CL - 1) / CL) * kp * sizeof(double2);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(F * CL), 1, 1);
+  cfg.blockDim = dim3((unsigned)(32 * jac_warps(kp, CL)), 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CL;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   prof_begin(PROF_SMALL, st);
-  jacobi_svd_kernel<<<F, threads, smem, st>>>(k, kp, R, sigma, Ul, Vr, sweeps);
+  RR_CUDA(cudaLaunchKernelEx(&cfg, jacobi_svd_kernel, k, kp, CL, R, sigma, Ul, Vr, sweeps));
   prof_end(PROF_SMALL, st);
   RR_CUDA(cudaGetLastError());
   return RR_OK;

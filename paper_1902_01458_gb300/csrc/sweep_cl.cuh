@@ -77,10 +77,15 @@ __device__ __forceinline__ void cp_async(uint32_t dst, const void* src, int byte
                  : "memory");
 }
 
+// Warps of a CTA: large lane tiles need more than the 128 registers that sixteen
+// warps leave them
+template <typename T, int CPL, int RPL>
+constexpr int max_warps() { return sizeof(T) == 4 && CPL * RPL >= 20 ? 8 : MAXW; }
+
 // LR = 32 / LC lanes over rows x LC over columns; a lane holds RPL rows (LR
 // apart) x CPL adjacent columns
 template <typename T, bool TRANS, int LC, int CPL, int RPL>
-__global__ void __launch_bounds__(MAXW * 32, 1) sweep_cl_kernel(Args<T> a) {
+__global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_kernel(Args<T> a) {
   using C = C_t<T>;
   constexpr int CS = sizeof(C);
   constexpr int KC = 64 / CS;            // contraction columns of a chunk
@@ -410,13 +415,13 @@ struct Plan {
 // Microseconds of a column step: the chain of a step plus a part that grows
 // with the block and the lane tile.  Measured (two problems, FP32, CPL = 2):
 // blocks of 192 rows 2.9 us with clusters of eight (RPL 2), 3.6 of four (RPL 3),
-// 6.0 of two (RPL 6); 384 rows 5.8 and 10.7; 768 rows 21 to 23; CPL = 4 takes
-// 3.6 / 4.9 / 10 to 13 at 192 rows and 8.1 at 384 (RPL 3).  FP64, a lane tile of
+// 6.0 of two (RPL 6); 384 rows 5.8 and 10.7; 768 rows 18 to 22; CPL = 4 takes
+// 3.6 / 4.9 / 8.3 at 192 rows and 7.9 at 384 (RPL 3).  FP64, a lane tile of
 // one row and column: 10.3 us at 192 rows (arithmetic).
 inline double step_us(bool dp, int b, int rpl, int cpl) {
   if (dp) return 3.0 + 0.037 * b * rpl * cpl;
-  const double two[10] = {0, 5, 6.8, 11, 15, 20, 25, 32, 40, 46};
-  const double four[10] = {0, 6, 11, 17, 26, 38, 55, 68, 80, 92};
+  const double two[10] = {0, 5, 6.8, 11, 15, 24, 24, 32, 40, 46};
+  const double four[10] = {0, 6, 11, 17, 24, 36, 36, 60, 60, 70};
   return 1.6 + 1e-3 * b * (cpl == 2 ? two[rpl] : four[rpl]);
 }
 
@@ -426,11 +431,11 @@ template <typename T>
 Plan make_plan(const OpDev& d, int Fa, int k, int trans) {
   constexpr bool DP = sizeof(T) == 8;
   constexpr int KC = 64 / sizeof(C_t<T>);
-  const int lr = DP ? 32 : 16, rplmax = DP ? 5 : 9;
-  const int kcs[3] = {DP ? 1 : 4, DP ? 2 : 8, DP ? 4 : 8};
+  const int kcs[3] = {DP ? 1 : 4, DP ? 2 : 8, 4};
   Plan best{0, 0, 0, 0, 0, -1.0};
+  const int lr = DP ? 32 : 16, rplmax = DP ? 5 : 9;
   for (int ki = 0; ki < (DP ? 3 : 2); ++ki) {
-    const int kc = kcs[ki], ng = (k + kc - 1) / kc;
+    const int kc = kcs[ki], ng = (k + kc - 1) / kc, cpl = DP ? kc : kc / 2;
     for (int cl0 = CLMAX; cl0 >= 1; --cl0) {
       const int npt = (d.ny + cl0 - 1) / cl0, CL = (d.ny + npt - 1) / npt;
       if (CL != cl0) continue;
@@ -439,7 +444,8 @@ Plan make_plan(const OpDev& d, int Fa, int k, int trans) {
       const int nch = (d.b + KC - 1) / KC;
       const int upr = kc * (int)sizeof(C_t<T>) / 16, units = rmax * upr;
       int W = 0;
-      for (int w = std::min(MAXW, nch); w >= 1; --w) {
+      const int wmax = !DP && cpl * (rpl == 5 ? 6 : rpl) >= 20 ? 8 : MAXW;
+      for (int w = std::min(wmax, nch); w >= 1; --w) {
         const int rounds = (nch + w - 1) / w, wb = (nch + rounds - 1) / rounds;
         const size_t sm = trans ? smem_bytes<T, true>(d.b, rmax, d.q, kc, wb)
                                 : smem_bytes<T, false>(d.b, rmax, d.q, kc, wb);
@@ -451,7 +457,7 @@ Plan make_plan(const OpDev& d, int Fa, int k, int trans) {
       if (W == 0) continue;
       const int slots = cluster_slots(d.device, CL);
       const int waves = (int)(((long)Fa * ng + slots - 1) / slots);
-      const double us = waves * (2.0 * d.nx - 1) * step_us(DP, d.b, rpl, DP ? kc : kc / 2);
+      const double us = waves * (2.0 * d.nx - 1) * step_us(DP, d.b, rpl, cpl);
       if (best.us < 0 || us < best.us) best = Plan{kc, CL, npt, W, rpl, us};
     }
   }
