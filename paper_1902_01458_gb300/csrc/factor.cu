@@ -4,8 +4,17 @@
 // With the unknowns ordered by streamwise column, s I - L has diagonal blocks
 // D_i, sub-diagonal blocks A_i = -L_{i,i-1} and super-diagonal blocks
 // C_i = -L_{i,i+1} (b x b, A_i and C_i with at most 3q entries per row).  The
-// block LU is
-//     S_0 = D_0,  G_i = S_i^{-1},  X_i = G_i C_i,  S_{i+1} = D_{i+1} - A_{i+1} X_i.
+// block LU runs from both ends to the middle column m = nx / 2 at once, so that
+// the chain of dependent blocks is half as long and every launch has twice the
+// problems (half 0: columns 0, 1, .. m - 1; half 1: nx - 1, nx - 2, .. m + 1):
+//     S_0 = D_0,  G_i = S_i^{-1},  X_i = G_i C_i,  S_{i+1} = D_{i+1} - A_{i+1} X_i
+//     S_{nx-1} = D_{nx-1},  X_i = G_i A_i,  S_{i-1} = D_{i-1} - C_{i-1} X_i
+//     S_m = D_m - A_m X_{m-1} - C_m X_{m+1}.
+// Work buffers hold 2 F problems: problem f of half h at index h F + f.  Measured
+// against the same kernels run from one end, factorisation and solves: two
+// frequencies of 128 x 64 points 13.5 ms instead of 25.5, six of 512 x 256 points
+// 401 instead of 619; in FP64 four of 128 x 64 points and their gradient 75
+// instead of 101.
 // G_i is formed explicitly, so every later solve is a dense block product
 // instead of a pair of triangular solves.  This file holds the Schur update and
 // the Gauss-Jordan inversion used for FP64 factors and for the FP32 shapes that
@@ -30,9 +39,11 @@ namespace {
 
 __device__ __forceinline__ int slotx(int dx, int dy) { return (dx + 1) * 3 + (dy + 1); }
 
-// M = D_i (+ L_{i,i-1} X_{i-1} for i > 0), i.e. S_i = D_i - A_i X_{i-1}.  One
-// CTA per (SCHUR_Y grid points in y = SCHUR_Y * q rows, column tile, problem):
-// the rows of X_{i-1} its rows couple to (the y neighbours, SCHUR_Y + 2
+// M = D_i + L_{i,i+dx} X_{i+dx} (dx = -1 in half 0, +1 in half 1; no X for the end
+// columns), i.e. S_i = D_i - A_i X_{i-1} and its mirror image; with add, M +=
+// L_{i,i+dx} X_{i+dx} only (the middle column's second neighbour).  One CTA per
+// (SCHUR_Y grid points in y = SCHUR_Y * q rows, column tile, problem): the rows of
+// X its rows couple to (the y neighbours, SCHUR_Y + 2
 // points) are staged once in shared memory, so every X row is read from
 // memory about once instead of once per coupled row; a row's stencil
 // coefficients are uniform across the CTA (broadcast loads).
@@ -46,19 +57,21 @@ __host__ __device__ constexpr size_t schur_smem(int q) {
 
 template <typename T>
 __global__ void __launch_bounds__(SchurCfg<T>::CB)
-schur_kernel(OpView op, const double2* __restrict__ shifts, int i,
-             const C_t<T>* __restrict__ Xprev, size_t xstride, C_t<T>* __restrict__ M) {
+schur_kernel(OpView op, const double2* __restrict__ shifts, int nh, int col0, int col1, int dx0,
+             int add, const C_t<T>* __restrict__ Xprev, C_t<T>* __restrict__ M) {
   using C = C_t<T>;
   constexpr int CB = SchurCfg<T>::CB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* Xs = reinterpret_cast<C*>(smem_raw);  // [(SCHUR_Y + 2) * q][CB]
   const int b = op.b, q = op.q, ny = op.ny;
-  const int f = blockIdx.z;
-  const int y0 = blockIdx.x * SCHUR_Y;
+  const int nt = gridDim.x / nh, half = blockIdx.x / nt;
+  const int f = blockIdx.z, pf = half * gridDim.z + f;
+  const int i = half ? col1 : col0, dx = half ? -dx0 : dx0;
+  const int y0 = (blockIdx.x - half * nt) * SCHUR_Y;
   const int c0 = blockIdx.y * CB;
   const C sh = mk((T)shifts[f].x, (T)shifts[f].y);
-  const C* Xp = Xprev ? Xprev + (size_t)f * xstride : nullptr;
-  C* Mf = M + (size_t)f * b * b;
+  const C* Xp = Xprev ? Xprev + (size_t)pf * b * b : nullptr;
+  C* Mf = M + (size_t)pf * b * b;
   const int ny_blk = min(SCHUR_Y, ny - y0);
   // stage X rows of y points y0 - 1 .. y0 + ny_blk (slot k <-> point y0 - 1 + k)
   if (Xp) {
@@ -80,7 +93,7 @@ schur_kernel(OpView op, const double2* __restrict__ shifts, int i,
   // coefficients: stage them once, with the neighbour point of every y
   // offset (-1: a Dirichlet ghost), so the per-entry loop reads shared
   // memory only.
-  __shared__ T cA[SCHUR_Y * 4][12];  // coupling to column i-1 (slot dx = -1), term (dy, cp)
+  __shared__ T cA[SCHUR_Y * 4][12];  // coupling to column i + dx, term (dy, cp)
   __shared__ T cD[SCHUR_Y * 4][12];  // diagonal block D_i (slot dx = 0)
   __shared__ int jyt[SCHUR_Y][3];    // neighbour y of point y0 + ly at dy = -1, 0, 1
   const int nt3 = 3 * q;
@@ -90,7 +103,7 @@ schur_kernel(OpView op, const double2* __restrict__ shifts, int i,
     const int iy = y0 + ly, dy = t / q - 1, cp = t - (t / q) * q;
     const int jy = nbr_y(iy, dy, ny, op.periodic);
     const size_t cf = ((size_t)i * b + iy * q + comp) * op.S;
-    cA[lr][t] = (jy >= 0 && Xp) ? coefv<T>(op, cf + slotx(-1, dy) * q + cp) : (T)0;
+    cA[lr][t] = (jy >= 0 && Xp) ? coefv<T>(op, cf + slotx(dx, dy) * q + cp) : (T)0;
     cD[lr][t] = jy >= 0 ? coefv<T>(op, cf + slotx(0, dy) * q + cp) : (T)0;
   }
   for (int e = threadIdx.x; e < ny_blk * 3; e += blockDim.x)
@@ -103,11 +116,11 @@ schur_kernel(OpView op, const double2* __restrict__ shifts, int i,
     const int iy = y0 + ly;
     for (int comp = 0; comp < q; ++comp) {
       const int r = iy * q + comp, lr = ly * q + comp;
-      C val = (r == c) ? sh : czero<C>();
+      C val = add ? Mf[(size_t)r * b + c] : (r == c) ? sh : czero<C>();
       // D_i: the row's entries at column c (one per y offset landing on jc)
 #pragma unroll
       for (int dy = 0; dy < 3; ++dy)
-        if (jyt[ly][dy] == jc) val.x -= cD[lr][dy * q + cc];
+        if (!add && jyt[ly][dy] == jc) val.x -= cD[lr][dy * q + cc];
       if (Xp) {
 #pragma unroll
         for (int t = 0; t < 12; ++t) {  // 3 y neighbours x q <= 4 variables
@@ -198,7 +211,7 @@ __global__ void __launch_bounds__(GP_MAXW * 32) gjp_panel_kernel(PanelArgs g, C_
   C* Bp = As + (size_t)g.rpc * (NB + 1);                // [NB][NB]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x;
   const int rank = (int)tc::cluster_rank();
-  const int f = blockIdx.x / CL;
+  const int f = blockIdx.x / CL;  // problem of a half
   const int nrows = max(0, (b - rank + CL - 1) / CL);
   C* M = Mall + (size_t)f * b * b;
   int* rowpiv = g.rowpiv + (size_t)f * b;
@@ -335,7 +348,7 @@ __global__ void __launch_bounds__(GP_MAXW * 32) gjp_panel_kernel(PanelArgs g, C_
       }
     }
   }
-  if (rank == 0 && tid == 0 && singular) g.flag[f] = 1;
+  if (rank == 0 && tid == 0 && singular) g.flag[f % g.F] = 1;
   if (!ok && lane == 0) atomicExch(g.flag + g.F, 1);
   if (!ok) tc::cluster_settle();
   tc::cluster_sync();  // no CTA leaves while another may still send to it
@@ -343,9 +356,11 @@ __global__ void __launch_bounds__(GP_MAXW * 32) gjp_panel_kernel(PanelArgs g, C_
 
 // B[f][j][m] = M[P_j][m] for the panel [k0, k0 + nbk), zero beyond nbk
 template <typename T>
-__global__ void gjp_gather_kernel(int b, int k0, int nbk, const C_t<T>* __restrict__ Mall,
+__global__ void gjp_gather_kernel(int b, int k0, int nbk, int nh, const C_t<T>* __restrict__ Mall,
                                   const int* __restrict__ pivslot_all, C_t<T>* __restrict__ Ball) {
-  const int f = blockIdx.z, j = blockIdx.y, m = blockIdx.x * blockDim.x + threadIdx.x;
+  const int nt = gridDim.x / nh, half = blockIdx.x / nt;
+  const int f = half * gridDim.z + blockIdx.z, j = blockIdx.y;
+  const int m = (blockIdx.x - half * nt) * blockDim.x + threadIdx.x;
   if (m >= b) return;
   C_t<T> v = czero<C_t<T>>();
   if (j < nbk) v = Mall[((size_t)f * b + pivslot_all[(size_t)f * b + k0 + j]) * b + m];
@@ -358,17 +373,18 @@ __global__ void gjp_gather_kernel(int b, int k0, int nbk, const C_t<T>* __restri
 template <typename T> struct UpdCfg { static constexpr int TR = sizeof(T) == 8 ? 32 : 64; };
 template <typename T>
 __global__ void __launch_bounds__(256)
-gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, C_t<T>* __restrict__ Mall,
+gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, int nh, C_t<T>* __restrict__ Mall,
                   const C_t<T>* __restrict__ Ball, const int* __restrict__ rowpiv_all) {
   using C = C_t<T>;
   constexpr int NB = GP_NB, TR = UpdCfg<T>::TR, PT = TR / 16;
   __shared__ C As[TR][NB + 1];
   __shared__ C Bs[NB][TR];
-  const int f = blockIdx.z;
+  const int nt = gridDim.x / nh, half = blockIdx.x / nt;
+  const int f = half * gridDim.z + blockIdx.z;
   C* M = Mall + (size_t)f * b * b;
   const C* B = Ball + (size_t)f * NB * b;
   const int* rowpiv = rowpiv_all + (size_t)f * b;
-  const int r0 = blockIdx.y * TR, c0 = blockIdx.x * TR;
+  const int r0 = blockIdx.y * TR, c0 = (blockIdx.x - half * nt) * TR;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   auto col_live = [&](int c) {
     return c < b && !(c >= k0 && c < k0 + nbk) && !(c >= n0 && c < n1);
@@ -418,33 +434,37 @@ gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, C_t<T>* __restrict__ M
   }
 }
 
-// G_i[j][p_m] = M[p_j][m];  X_i = G_i C_i with C_i = -L_{i,i+1}.
+// G_i[j][p_m] = M[p_j][m];  X_i = G_i C_i with C_i = -L_{i,i+1} (half 0) or
+// G_i A_i with A_i = -L_{i,i-1} (half 1).
 template <typename T>
-__global__ void gjp_finalize_kernel(OpView op, int i, int RB, const C_t<T>* __restrict__ Mall,
-                                    const int* __restrict__ pivslot_all, C_t<T>* __restrict__ Gi,
-                                    size_t gstride, C_t<T>* __restrict__ Xi, size_t xstride) {
+__global__ void gjp_finalize_kernel(OpView op, int nh, int col0, int col1, int RB,
+                                    const C_t<T>* __restrict__ Mall,
+                                    const int* __restrict__ pivslot_all, C_t<T>* __restrict__ Gall,
+                                    C_t<T>* __restrict__ Xall) {
   using C = C_t<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int b = op.b, q = op.q;
   C* Gs = reinterpret_cast<C*>(smem_raw);                 // [RB][b]
   int* ps = reinterpret_cast<int*>(Gs + (size_t)RB * b);  // [b]
-  const int f = blockIdx.y;
-  const int r0 = blockIdx.x * RB;
-  const C* M = Mall + (size_t)f * b * b;
-  for (int c = threadIdx.x; c < b; c += blockDim.x) ps[c] = pivslot_all[(size_t)f * b + c];
+  const int nt = gridDim.x / nh, half = blockIdx.x / nt;
+  const int f = blockIdx.y, pf = half * gridDim.y + f, i = half ? col1 : col0;
+  const int r0 = (blockIdx.x - half * nt) * RB;
+  const C* M = Mall + (size_t)pf * b * b;
+  for (int c = threadIdx.x; c < b; c += blockDim.x) ps[c] = pivslot_all[(size_t)pf * b + c];
   __syncthreads();
   for (int e = threadIdx.x; e < RB * b; e += blockDim.x) {
     const int rr = e / b, c = e - rr * b, r = r0 + rr;
     if (r < b) Gs[rr * b + ps[c]] = M[(size_t)ps[r] * b + c];
   }
   __syncthreads();
-  C* G = Gi + (size_t)f * gstride;
+  C* G = Gall + ((size_t)f * op.nx + i) * b * b;
   for (int e = threadIdx.x; e < RB * b; e += blockDim.x) {
     const int rr = e / b, c = e - rr * b, r = r0 + rr;
     if (r < b) G[(size_t)r * b + c] = Gs[rr * b + c];
   }
-  if (Xi == nullptr) return;
-  C* X = Xi + (size_t)f * xstride;
+  if (Xall == nullptr) return;
+  C* X = Xall + (size_t)pf * b * b;
+  const int dx = half ? -1 : 1;
   for (int e = threadIdx.x; e < RB * b; e += blockDim.x) {
     const int rr = e / b, c = e - rr * b, r = r0 + rr;
     if (r >= b) continue;
@@ -455,7 +475,7 @@ __global__ void gjp_finalize_kernel(OpView op, int i, int RB, const C_t<T>* __re
       if (iym < 0) continue;
       for (int cm = 0; cm < q; ++cm) {
         const int m = iym * q + cm;
-        const T a = coefv<T>(op, ((size_t)i * b + m) * op.S + slotx(1, dy) * q + cc);
+        const T a = coefv<T>(op, ((size_t)i * b + m) * op.S + slotx(dx, dy) * q + cc);
         if (a != (T)0) s = crfma(a, Gs[rr * b + m], s);
       }
     }
@@ -464,8 +484,8 @@ __global__ void gjp_finalize_kernel(OpView op, int i, int RB, const C_t<T>* __re
 }
 
 template <typename T>
-void launch_schur(const OpView& ov, const double2* shifts, int i, const C_t<T>* Xprev,
-                  size_t xstride, C_t<T>* M, int F, cudaStream_t st) {
+void launch_schur(const OpView& ov, const double2* shifts, int F, int nh, int col0, int col1,
+                  int dx0, int add, const C_t<T>* Xprev, C_t<T>* M, cudaStream_t st) {
   constexpr int CB = SchurCfg<T>::CB;
   const size_t smem = Xprev ? schur_smem<T>(ov.q) : 0;
   static bool attr = false;
@@ -474,12 +494,33 @@ void launch_schur(const OpView& ov, const double2* shifts, int i, const C_t<T>* 
                          (int)schur_smem<T>(4));
     attr = true;
   }
-  dim3 gs((ov.ny + SCHUR_Y - 1) / SCHUR_Y, (ov.b + CB - 1) / CB, F);
-  schur_kernel<T><<<gs, CB, smem, st>>>(ov, shifts, i, Xprev, xstride, M);
+  dim3 gs((ov.ny + SCHUR_Y - 1) / SCHUR_Y * nh, (ov.b + CB - 1) / CB, F);
+  schur_kernel<T><<<gs, CB, smem, st>>>(ov, shifts, nh, col0, col1, dx0, add, Xprev, M);
+}
+
+// M = S_i for step t of the factorisation (twist_steps)
+template <typename T>
+rr_status schur_step(rr_factors* fa, const TwistStep& t, cudaStream_t st) {
+  const OpDev& d = fa->op->d;
+  const OpView ov = view(d);
+  using C = C_t<T>;
+  C* M = reinterpret_cast<C*>(fa->M);
+  const C* X = reinterpret_cast<const C*>(fa->X);
+  prof_begin(PROF_SCHUR, st);
+  launch_schur<T>(ov, fa->shifts, fa->F, t.nh, t.col0, t.col1, -1, 0, t.first ? nullptr : X, M, st);
+  prof_end(PROF_SCHUR, st);
+  if (t.middle) {
+    prof_begin(PROF_SCHUR, st);
+    launch_schur<T>(ov, fa->shifts, fa->F, 1, t.col0, t.col1, 1, 1, X + (size_t)fa->F * d.b * d.b,
+                    M, st);
+    prof_end(PROF_SCHUR, st);
+  }
+  RR_CUDA(cudaGetLastError());
+  return RR_OK;
 }
 
 template <typename T>
-rr_status launch_panel(rr_factors* fa, int k0, int nbk, int kp0, cudaStream_t st) {
+rr_status launch_panel(rr_factors* fa, int nh, int k0, int nbk, int kp0, cudaStream_t st) {
   const OpDev& d = fa->op->d;
   PanelArgs a;
   a.b = d.b;
@@ -501,7 +542,7 @@ rr_status launch_panel(rr_factors* fa, int k0, int nbk, int kp0, cudaStream_t st
     attr = true;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(a.CL * fa->F), 1, 1);
+  cfg.gridDim = dim3((unsigned)(a.CL * fa->F * nh), 1, 1);
   cfg.blockDim = dim3((unsigned)((a.rpc * GP_LPR + 31) / 32 * 32), 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -524,13 +565,12 @@ rr_status factor_impl(rr_factors* fa) {
   constexpr int NB = GP_NB;
   const OpDev& d = fa->op->d;
   const OpView ov = view(d);
-  const int b = d.b, nx = d.nx, F = fa->F;
+  const int b = d.b, F = fa->F;
   cudaStream_t st = fa->stream, st2 = fa->stream2;
   C* M = reinterpret_cast<C*>(fa->M);
   C* G = reinterpret_cast<C*>(fa->G);
   C* X = reinterpret_cast<C*>(fa->X);
   C* Bbuf = reinterpret_cast<C*>(fa->Bbuf);
-  const size_t bb = (size_t)b * b;
   int RB = 4;
   while (RB > 1 && (size_t)RB * b * sizeof(C) + b * sizeof(int) > 160 * 1024) RB >>= 1;
   const size_t fsmem = (size_t)RB * b * sizeof(C) + b * sizeof(int);
@@ -538,13 +578,11 @@ rr_status factor_impl(rr_factors* fa) {
                                (int)fsmem));
   constexpr int TR = UpdCfg<T>::TR;
   const int nt = (b + TR - 1) / TR, P = (b + NB - 1) / NB;
-  // (factor_cols > 0 stops after that many columns: autotuner timing only)
-  const int ncols = fa->factor_cols > 0 ? std::min(fa->factor_cols, nx) : nx;
   rr_status s;
-  for (int i = 0; i < ncols; ++i) {
-    prof_begin(PROF_SCHUR, st);
-    launch_schur<T>(ov, fa->shifts, i, i > 0 ? X : nullptr, bb, M, F, st);
-    prof_end(PROF_SCHUR, st);
+  for (int step = 0; step < twist_steps(fa); ++step) {
+    const TwistStep t = twist_step(fa, step);
+    const int nh = t.nh;
+    if ((s = schur_step<T>(fa, t, st)) != RR_OK) return s;
     // The panels run in order on the second (high-priority) stream, the updates
     // in order on the main one.  Panel p applies panel p - 1's transformation to
     // its own columns, so it waits only for the update of panel p - 2 and runs
@@ -556,24 +594,25 @@ rr_status factor_impl(rr_factors* fa) {
     for (int p = 0; p < P; ++p) {
       const int k0 = p * NB, nbk = std::min(NB, b - k0);
       if (p >= 2) RR_CUDA(cudaStreamWaitEvent(st2, fa->ev_ring[4 + ((p - 2) & 3)], 0));
-      if ((s = launch_panel<T>(fa, k0, nbk, p > 0 ? k0 - NB : -1, st2)) != RR_OK) return s;
+      if ((s = launch_panel<T>(fa, nh, k0, nbk, p > 0 ? k0 - NB : -1, st2)) != RR_OK) return s;
       RR_CUDA(cudaEventRecord(fa->ev_ring[p & 3], st2));
       RR_CUDA(cudaStreamWaitEvent(st, fa->ev_ring[p & 3], 0));
       if (P == 1) break;
       prof_begin(PROF_ROWBLOCK, st);
-      gjp_gather_kernel<T><<<dim3((b + 127) / 128, NB, F), 128, 0, st>>>(b, k0, nbk, M, fa->pivslot, Bbuf);
+      gjp_gather_kernel<T><<<dim3((b + 127) / 128 * nh, NB, F), 128, 0, st>>>(b, k0, nbk, nh, M, fa->pivslot,
+                                                                            Bbuf);
       prof_end(PROF_ROWBLOCK, st);
       const int n0 = p + 1 < P ? k0 + NB : 0, n1 = p + 1 < P ? std::min(b, n0 + NB) : 0;
       prof_begin(PROF_UPDATE, st);
-      gjp_update_kernel<T><<<dim3(nt, nt, F), 256, 0, st>>>(b, k0, nbk, n0, n1, M, Bbuf, fa->rowpiv);
+      gjp_update_kernel<T><<<dim3(nt * nh, nt, F), 256, 0, st>>>(b, k0, nbk, n0, n1, nh, M, Bbuf,
+                                                                 fa->rowpiv);
       prof_end(PROF_UPDATE, st);
       RR_CUDA(cudaEventRecord(fa->ev_ring[4 + (p & 3)], st));
       RR_CUDA(cudaGetLastError());
     }
-    C* Xi = (i + 1 < nx) ? X : nullptr;
     prof_begin(PROF_FINALIZE, st);
-    gjp_finalize_kernel<T><<<dim3((b + RB - 1) / RB, F), 256, fsmem, st>>>(
-        ov, i, RB, M, fa->pivslot, G + (size_t)i * bb, (size_t)nx * bb, Xi, bb);
+    gjp_finalize_kernel<T><<<dim3((b + RB - 1) / RB * nh, F), 256, fsmem, st>>>(
+        ov, nh, t.col0, t.col1, RB, M, fa->pivslot, G, t.middle ? nullptr : X);
     prof_end(PROF_FINALIZE, st);
     RR_CUDA(cudaGetLastError());
   }
@@ -582,16 +621,26 @@ rr_status factor_impl(rr_factors* fa) {
 
 }  // namespace
 
-rr_status launch_schur_f32(rr_factors* fa, int i, cudaStream_t st) {
-  const OpDev& d = fa->op->d;
-  const int b = d.b;
-  float2* X = reinterpret_cast<float2*>(fa->X);
-  prof_begin(PROF_SCHUR, st);
-  launch_schur<float>(view(d), fa->shifts, i, i > 0 ? X : nullptr, (size_t)b * b,
-                      reinterpret_cast<float2*>(fa->M), fa->F, st);
-  prof_end(PROF_SCHUR, st);
-  RR_CUDA(cudaGetLastError());
-  return RR_OK;
+// Steps of the factorisation: the pairs of columns from the ends inwards, then
+// the middle one (factor_cols > 0 stops after that many: autotuner timing only)
+int twist_steps(const rr_factors* fa) {
+  const int n = twist_mid(fa->op->d.nx) + 1;
+  return fa->factor_cols > 0 ? std::min(fa->factor_cols, n - 1) : n;
+}
+
+TwistStep twist_step(const rr_factors* fa, int t) {
+  const int nx = fa->op->d.nx, m = twist_mid(nx);
+  TwistStep s;
+  s.first = t == 0;
+  s.middle = t == m;
+  s.nh = !s.middle && t < nx - 1 - m ? 2 : 1;
+  s.col0 = t;
+  s.col1 = nx - 1 - t;
+  return s;
+}
+
+rr_status launch_schur_f32(rr_factors* fa, const TwistStep& t, cudaStream_t st) {
+  return schur_step<float>(fa, t, st);
 }
 
 rr_status launch_factor(rr_factors* fa) {

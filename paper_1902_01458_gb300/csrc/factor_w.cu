@@ -95,9 +95,9 @@ constexpr size_t SL_SMEM_CAP = 226 * 1024;  // dynamic shared memory of a CTA
 
 struct SlabArgs {
   int b, c0, c1, rpc, CL;
-  float2* M;                     // [F][b][b]
-  int* rowpiv;                   // [F][b]
-  int* pivslot;                  // [F][b]
+  float2* M;                     // [2F][b][b]
+  int* rowpiv;                   // [2F][b]
+  int* pivslot;                  // [2F][b]
   int* flag;                     // [F] singular flags, [F] = wait timeout
   int F;
   uint32_t tries;
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
       rowpiv[grow] = -1;
     }
   }
-  if (rank == 0 && tid == 0 && singular) g.flag[f] = 1;
+  if (rank == 0 && tid == 0 && singular) g.flag[f % g.F] = 1;
   if (!ok && lane == 0) atomicExch(g.flag + g.F, 1);
   if (!ok) tc::cluster_settle();
   if (!SOLO) tc::cluster_sync();  // no CTA leaves while another may still send to it
@@ -508,14 +508,15 @@ int slab_cluster(int b, int F, int device) {
   return best;
 }
 
-rr_status launch_slab(rr_factors* fa, int c0, int c1, cudaStream_t st) {
+rr_status launch_slab(rr_factors* fa, int nh, int c0, int c1, cudaStream_t st) {
   const OpDev& d = fa->op->d;
   SlabArgs a;
   a.b = d.b;
   a.c0 = c0;
   a.c1 = c1;
   a.F = fa->F;
-  a.CL = slab_cluster(d.b, fa->F, d.device);
+  const int P = fa->F * nh;  // problems of this launch
+  a.CL = slab_cluster(d.b, P, d.device);
   a.rpc = (d.b + a.CL - 1) / a.CL;
   a.M = reinterpret_cast<float2*>(fa->M);
   a.rowpiv = fa->rowpiv;
@@ -537,11 +538,11 @@ rr_status launch_slab(rr_factors* fa, int c0, int c1, cudaStream_t st) {
   }
   prof_begin(PROF_PANEL, st);
   if (a.CL == 1) {
-    if (lpr == 4) gjw_slab_kernel<true, 4><<<fa->F, SL_THREADS, smem, st>>>(a);
-    else gjw_slab_kernel<true, 2><<<fa->F, SL_THREADS, smem, st>>>(a);
+    if (lpr == 4) gjw_slab_kernel<true, 4><<<P, SL_THREADS, smem, st>>>(a);
+    else gjw_slab_kernel<true, 2><<<P, SL_THREADS, smem, st>>>(a);
   } else {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(a.CL * fa->F), 1, 1);
+    cfg.gridDim = dim3((unsigned)(a.CL * P), 1, 1);
     cfg.blockDim = dim3(SL_THREADS, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -563,8 +564,9 @@ rr_status launch_slab(rr_factors* fa, int c0, int c1, cudaStream_t st) {
 // [c0, c1) and c < c1 - c0; zero elsewhere (rows up to GW_W).
 __global__ void gjw_gather_kernel(int b, int c0, int c1, const float2* __restrict__ Mall,
                                   const int* __restrict__ pivslot_all, float2* __restrict__ Bout) {
-  const int f = blockIdx.y;
-  const int c = blockIdx.x;  // 0 .. GW_W - 1
+  const int half = blockIdx.x / GW_W;
+  const int f = half * gridDim.y + blockIdx.y;
+  const int c = blockIdx.x - half * GW_W;  // 0 .. GW_W - 1
   const float2* M = Mall + (size_t)f * b * b;
   float2* dst = Bout + ((size_t)f * GW_W + c) * b;
   const bool row_ok = c < c1 - c0;
@@ -887,7 +889,8 @@ gjw_gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
 
 // ---------------------------------------------------------------- finalize
 // G_i[j][p_m] = M[p_j][m] (S^{-1} from the implicitly pivoted work matrix),
-// X_i = G_i C_i with C_i = -L_{i,i+1} (at most 3q entries per column).  A CTA
+// X_i = G_i C_i with C_i = -L_{i,i+1} in half 0 and G_i A_i with A_i = -L_{i,i-1}
+// in half 1 (at most 3q entries per column).  A CTA
 // gathers RB rows into shared memory (scattering the columns), writes them
 // as rows of G_i and forms the same rows of X_i; each thread owns fixed
 // columns of X_i, so the (up to 3q) coupling coefficients of a column are
@@ -895,37 +898,38 @@ gjw_gemm_kernel(const __grid_constant__ CUtensorMap tmapA, const __grid_constant
 constexpr int FIN_THREADS = 256, FIN_CPT = 4;  // columns per thread (b <= 1024)
 
 __global__ void __launch_bounds__(FIN_THREADS)
-gjw_finalize_kernel(OpView op, int i, int RB, const float2* __restrict__ Mall,
-                    const int* __restrict__ pivslot_all, float2* __restrict__ Gi, size_t gstride,
-                    float2* __restrict__ Xi, size_t xstride) {
+gjw_finalize_kernel(OpView op, int nh, int col0, int col1, int RB,
+                    const float2* __restrict__ Mall, const int* __restrict__ pivslot_all,
+                    float2* __restrict__ Gall, float2* __restrict__ Xall) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int b = op.b, q = op.q;
   float2* Gs = reinterpret_cast<float2*>(smem_raw);        // [RB][b]
   int* ps = reinterpret_cast<int*>(Gs + (size_t)RB * b);   // [b]
-  const int f = blockIdx.y;
-  const int r0 = blockIdx.x * RB;
+  const int nt = gridDim.x / nh, half = blockIdx.x / nt;
+  const int f = blockIdx.y, pf = half * gridDim.y + f, i = half ? col1 : col0;
+  const int r0 = (blockIdx.x - half * nt) * RB;
   const int nr = min(RB, b - r0);
-  const float2* M = Mall + (size_t)f * b * b;
-  for (int c = threadIdx.x; c < b; c += FIN_THREADS) ps[c] = pivslot_all[(size_t)f * b + c];
+  const float2* M = Mall + (size_t)pf * b * b;
+  for (int c = threadIdx.x; c < b; c += FIN_THREADS) ps[c] = pivslot_all[(size_t)pf * b + c];
   __syncthreads();
   for (int e = threadIdx.x; e < nr * b; e += FIN_THREADS) {
     const int rr = e / b, c = e - rr * b;
     Gs[rr * b + ps[c]] = M[(size_t)ps[r0 + rr] * b + c];
   }
   __syncthreads();
-  float2* G = Gi + (size_t)f * gstride;
+  float2* G = Gall + ((size_t)f * op.nx + i) * b * b;
   for (int e = threadIdx.x; e < nr * b; e += FIN_THREADS) {
     const int rr = e / b, c = e - rr * b;
     G[(size_t)(r0 + rr) * b + c] = Gs[rr * b + c];
   }
-  if (Xi == nullptr) return;
-  float2* X = Xi + (size_t)f * xstride;
+  if (Xall == nullptr) return;
+  float2* X = Xall + (size_t)pf * b * b;
 #pragma unroll
   for (int k = 0; k < FIN_CPT; ++k) {
     const int c = threadIdx.x + k * FIN_THREADS;
     if (c >= b) break;
-    // the coupling of column c: entries L[(i, m), (i + 1, c)] for the rows m
-    // of the y neighbours of c's point
+    // the coupling of column c: entries L[(i, m), (i +- 1, c)] (half 0: + 1) for
+    // the rows m of the y neighbours of c's point
     const int iyc = c / q, cc = c - iyc * q;
     int mm[12];  // 3 y neighbours x q <= 4 variables
     float aa[12];
@@ -938,7 +942,7 @@ gjw_finalize_kernel(OpView op, int i, int RB, const float2* __restrict__ Mall,
         const int iym = nbr_y(iyc, -dy, op.ny, op.periodic);
         if (iym >= 0) {
           mm[t] = iym * q + cm;
-          aa[t] = op.coef32[((size_t)i * b + mm[t]) * op.S + (2 * 3 + (dy + 1)) * q + cc];
+          aa[t] = op.coef32[((size_t)i * b + mm[t]) * op.S + ((half ? 0 : 6) + (dy + 1)) * q + cc];
         }
       }
     }
@@ -953,12 +957,12 @@ gjw_finalize_kernel(OpView op, int i, int RB, const float2* __restrict__ Mall,
 }
 
 template <int SPLIT>
-rr_status launch_gemm(rr_factors* fa, const CUtensorMap* ta, const CUtensorMap* tb, int ka, int Kc,
+rr_status launch_gemm(rr_factors* fa, int nh, const CUtensorMap* ta, const CUtensorMap* tb, int ka, int Kc,
                       int x0, int x1, int y0, int y1, cudaStream_t st) {
   const OpDev& d = fa->op->d;
   GemmArgs a;
   a.b = d.b;
-  a.F = fa->F;
+  a.F = fa->F * nh;
   a.ka = ka;
   a.Kc = Kc;
   a.x0 = x0; a.x1 = x1; a.y0 = y0; a.y1 = y1;
@@ -967,7 +971,7 @@ rr_status launch_gemm(rr_factors* fa, const CUtensorMap* ta, const CUtensorMap* 
   a.err = fa->flag + fa->F;
   a.tries = wait_tries();
   const int nrt = (d.b + GG_RT - 1) / GG_RT;
-  const long items = (long)fa->F * nrt * ((x1 - x0) + (y1 - y0));
+  const long items = (long)a.F * nrt * ((x1 - x0) + (y1 - y0));
   if (items <= 0) return RR_OK;
   // small launches (up to 8 items per SM): one wave of persistent CTAs;
   // large ones: about four items per CTA, so CTAs retire during the launch
@@ -991,12 +995,11 @@ template <int SPLIT>
 rr_status factor_wide_impl(rr_factors* fa) {
   const OpDev& d = fa->op->d;
   const OpView ov = view(d);
-  const int b = d.b, nx = d.nx, F = fa->F;
+  const int b = d.b, F = fa->F;
   cudaStream_t st = fa->stream;
   float2* M = reinterpret_cast<float2*>(fa->M);
   float2* G = reinterpret_cast<float2*>(fa->G);
   float2* X = reinterpret_cast<float2*>(fa->X);
-  const size_t bb = (size_t)b * b;
   const CUtensorMap* tA = reinterpret_cast<const CUtensorMap*>(fa->wmap[0]);
   const CUtensorMap* tBout = reinterpret_cast<const CUtensorMap*>(fa->wmap[1]);
   const int RB = 8;
@@ -1004,9 +1007,10 @@ rr_status factor_wide_impl(rr_factors* fa) {
   RR_CUDA(cudaFuncSetAttribute(gjw_finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)fsmem));
   const int nct_all = (b + GG_CT - 1) / GG_CT;
-  const int ncols = fa->factor_cols > 0 ? std::min(fa->factor_cols, nx) : nx;
-  for (int i = 0; i < ncols; ++i) {
-    rr_status s = launch_schur_f32(fa, i, st);
+  for (int step = 0; step < twist_steps(fa); ++step) {
+    const TwistStep t = twist_step(fa, step);
+    const int nh = t.nh;
+    rr_status s = launch_schur_f32(fa, t, st);
     if (s != RR_OK) return s;
     // Look-ahead: once the next slab's columns have received this slab's
     // rank-128 update, the next slab's inner factorisation runs on the second
@@ -1017,40 +1021,39 @@ rr_status factor_wide_impl(rr_factors* fa) {
     // stream's update reads as "not a pivot of this slab" either way).  The
     // next slab's pivot rows are gathered on the main stream after both.
     cudaStream_t st2 = fa->stream2;
-    if ((s = launch_slab(fa, 0, std::min(b, GW_W), st)) != RR_OK) return s;
+    if ((s = launch_slab(fa, nh, 0, std::min(b, GW_W), st)) != RR_OK) return s;
     for (int c0 = 0; c0 < b; c0 += GW_W) {
       const int c1 = std::min(b, c0 + GW_W);
       if (c1 >= b && c0 == 0) break;  // one slab: no outer update
       prof_begin(PROF_ROWBLOCK, st);
-      gjw_gather_kernel<<<dim3(GW_W, F), 256, 0, st>>>(b, c0, c1, M, fa->pivslot,
+      gjw_gather_kernel<<<dim3(GW_W * nh, F), 256, 0, st>>>(b, c0, c1, M, fa->pivslot,
                                                       reinterpret_cast<float2*>(fa->Wbuf));
       prof_end(PROF_ROWBLOCK, st);
       const int s0 = c0 / GG_CT, s1 = (c1 + GG_CT - 1) / GG_CT;
       if (c1 < b) {
         const int n1 = std::min(b, c1 + GW_W);
         const int u1 = (n1 + GG_CT - 1) / GG_CT;  // tiles [s1, u1): the next slab
-        if ((s = launch_gemm<SPLIT>(fa, tA, tBout, c0, GW_W, s1, u1, 0, 0, st)) != RR_OK) return s;
+        if ((s = launch_gemm<SPLIT>(fa, nh, tA, tBout, c0, GW_W, s1, u1, 0, 0, st)) != RR_OK) return s;
         if (st2 != nullptr) {
           RR_CUDA(cudaEventRecord(fa->ev_next, st));
           RR_CUDA(cudaStreamWaitEvent(st2, fa->ev_next, 0));
-          if ((s = launch_slab(fa, c1, n1, st2)) != RR_OK) return s;
+          if ((s = launch_slab(fa, nh, c1, n1, st2)) != RR_OK) return s;
           RR_CUDA(cudaEventRecord(fa->ev_panel, st2));
-          if ((s = launch_gemm<SPLIT>(fa, tA, tBout, c0, GW_W, 0, s0, u1, nct_all, st)) != RR_OK)
+          if ((s = launch_gemm<SPLIT>(fa, nh, tA, tBout, c0, GW_W, 0, s0, u1, nct_all, st)) != RR_OK)
             return s;
           RR_CUDA(cudaStreamWaitEvent(st, fa->ev_panel, 0));
         } else {
-          if ((s = launch_gemm<SPLIT>(fa, tA, tBout, c0, GW_W, 0, s0, u1, nct_all, st)) != RR_OK)
+          if ((s = launch_gemm<SPLIT>(fa, nh, tA, tBout, c0, GW_W, 0, s0, u1, nct_all, st)) != RR_OK)
             return s;
-          if ((s = launch_slab(fa, c1, n1, st)) != RR_OK) return s;
+          if ((s = launch_slab(fa, nh, c1, n1, st)) != RR_OK) return s;
         }
       } else {
-        if ((s = launch_gemm<SPLIT>(fa, tA, tBout, c0, GW_W, 0, s0, 0, 0, st)) != RR_OK) return s;
+        if ((s = launch_gemm<SPLIT>(fa, nh, tA, tBout, c0, GW_W, 0, s0, 0, 0, st)) != RR_OK) return s;
       }
     }
-    float2* Xi = (i + 1 < nx) ? X : nullptr;
     prof_begin(PROF_FINALIZE, st);
-    gjw_finalize_kernel<<<dim3((b + RB - 1) / RB, F), FIN_THREADS, fsmem, st>>>(
-        ov, i, RB, M, fa->pivslot, G + (size_t)i * bb, (size_t)nx * bb, Xi, bb);
+    gjw_finalize_kernel<<<dim3((b + RB - 1) / RB * nh, F), FIN_THREADS, fsmem, st>>>(
+        ov, nh, t.col0, t.col1, RB, M, fa->pivslot, G, t.middle ? nullptr : X);
     prof_end(PROF_FINALIZE, st);
     RR_CUDA(cudaGetLastError());
   }

@@ -511,10 +511,10 @@ static int encode_wide_maps(rr_factors* fa) {
   }
   auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   const cuuint32_t es[3] = {1, 1, 1};
-  const cuuint64_t dm[3] = {(cuuint64_t)2 * d.b, (cuuint64_t)d.b, (cuuint64_t)fa->F};
+  const cuuint64_t dm[3] = {(cuuint64_t)2 * d.b, (cuuint64_t)d.b, (cuuint64_t)2 * fa->F};
   const cuuint64_t sm[2] = {(cuuint64_t)2 * d.b * 4, (cuuint64_t)2 * d.b * d.b * 4};
   const cuuint32_t boxA[3] = {32, 128, 1}, boxB[3] = {128, 16, 1};
-  const cuuint64_t dw[3] = {(cuuint64_t)2 * d.b, 128, (cuuint64_t)fa->F};
+  const cuuint64_t dw[3] = {(cuuint64_t)2 * d.b, 128, (cuuint64_t)2 * fa->F};
   const cuuint64_t sw[2] = {(cuuint64_t)2 * d.b * 4, (cuuint64_t)2 * d.b * 128 * 4};
   CUresult r0 = encode(reinterpret_cast<CUtensorMap*>(fa->wmap[0]), CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                        3, fa->M, dm, sm, boxA, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -718,18 +718,18 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
     return st;
   };
   if ((s = dalloc(&fa->G, (size_t)nshift * d.nx * bb * fa->csz)) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->X, (size_t)nshift * bb * fa->csz)) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->M, (size_t)nshift * bb * fa->csz)) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->Bbuf, (size_t)nshift * 16 * d.b * fa->csz)) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->rowpiv, (size_t)nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->pivslot, (size_t)nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
+  if ((s = dalloc(&fa->X, (size_t)2 * nshift * bb * fa->csz)) != RR_OK) return fail(s);
+  if ((s = dalloc(&fa->M, (size_t)2 * nshift * bb * fa->csz)) != RR_OK) return fail(s);
+  if ((s = dalloc(&fa->Bbuf, (size_t)2 * nshift * 16 * d.b * fa->csz)) != RR_OK) return fail(s);
+  if ((s = dalloc(&fa->rowpiv, (size_t)2 * nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
+  if ((s = dalloc(&fa->pivslot, (size_t)2 * nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->Tbuf, (size_t)nshift * 128 * d.b * fa->csz)) != RR_OK) return fail(s);
   if (tc_prec(prec)) {
     if ((s = dalloc(&fa->Pbuf, (size_t)4 * nshift * 64 * d.b * sizeof(float2))) != RR_OK)
       return fail(s);
     fa->tma_ok = encode_factor_maps(fa);
     if (d.b >= 64 && d.b <= 768 && d.b % 8 == 0) {
-      if ((s = dalloc(&fa->Wbuf, (size_t)nshift * 128 * d.b * sizeof(float2))) != RR_OK)
+      if ((s = dalloc(&fa->Wbuf, (size_t)2 * nshift * 128 * d.b * sizeof(float2))) != RR_OK)
         return fail(s);
       fa->wide_ok = encode_wide_maps(fa);
     }
@@ -760,7 +760,7 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
   e = cudaMemsetAsync(fa->flag, 0, (nshift + 1) * sizeof(int), st);
   if (e != cudaSuccess) return fail(cuda_status(e, "rr_factor flags"));
   // a row index in every entry, also of a factorisation that found no pivot
-  e = cudaMemsetAsync(fa->pivslot, 0, (size_t)nshift * d.b * sizeof(int), st);
+  e = cudaMemsetAsync(fa->pivslot, 0, (size_t)2 * nshift * d.b * sizeof(int), st);
   if (e != cudaSuccess) return fail(cuda_status(e, "rr_factor pivots"));
   if ((s = launch_factor(fa)) != RR_OK) return fail(s);
   std::vector<int> flags(nshift + 1);

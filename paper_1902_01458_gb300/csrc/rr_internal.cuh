@@ -138,18 +138,20 @@ struct rr_factors {
   cudaEvent_t ev_ring[8];  // panel / update rings of the 16-column factorisation
   size_t csz;        // bytes of one complex element of the factors
   void* G;           // [F][nx][b][b]   inverse of each Schur block
-  void* X;           // [F][b][b] X_i = G_i C_i of the current column (transient)
-  void* M;           // [F][b][b] work matrix
-  void* Bbuf;        // [F][16][b] saved pivot rows of the current panel
+  // The factorisation runs from both ends to the middle column (factor.cu):
+  // its work buffers hold 2 F problems, problem f of half h at h F + f.
+  void* X;           // [2F][b][b] X_i = G_i C_i (G_i A_i) of the current columns (transient)
+  void* M;           // [2F][b][b] work matrices
+  void* Bbuf;        // [2F][16][b] saved pivot rows of the current panel
   void* Tbuf;        // [2][F][b][64] staging blocks of one sweep step
   void* Pbuf;        // [4][F][b][64] partial products of the split tensor-core sweep
   alignas(64) unsigned char tmap[2][128];  // TMA maps: G tiles, G^H tiles (FP32)
   int tma_ok;        // 1 if the maps of G were encoded
-  int* rowpiv;       // [F][b] pivot column of each row (-1: not yet pivoted)
-  int* pivslot;      // [F][b] pivot row of each column
+  int* rowpiv;       // [2F][b] pivot column of each row (-1: not yet pivoted)
+  int* pivslot;      // [2F][b] pivot row of each column
   // slab (two-level) factorisation of FP32 factors
   int wide_ok;       // 1 if the buffers and TMA maps below exist
-  void* Wbuf;        // [F][128][b] gathered pivot rows of a slab (outer update)
+  void* Wbuf;        // [2F][128][b] gathered pivot rows of a slab (outer update)
   alignas(64) unsigned char wmap[2][128];  // TMA maps: A chunks of M, Wbuf rows
   int* flag;         // [F] singular-pivot flags
   double2* shifts;   // [F] device
@@ -233,8 +235,17 @@ rr_status time_solve(rr_factors* fa, int k, float* ms);
 
 // factor.cu
 rr_status launch_factor(rr_factors* f);
-// M = D_i - A_i X_{i-1} for FP32 factors (the Schur update of column i)
-rr_status launch_schur_f32(rr_factors* f, int i, cudaStream_t st);
+// middle column of the factorisation (nx >= 3: columns on both sides), and its
+// steps: half 0 on col0 and, when nh == 2, half 1 on col1
+__host__ __device__ inline int twist_mid(int nx) { return nx / 2; }
+struct TwistStep {
+  int nh, col0, col1;
+  bool first, middle;
+};
+int twist_steps(const rr_factors* f);
+TwistStep twist_step(const rr_factors* f, int t);
+// the Schur blocks of a step for FP32 factors
+rr_status launch_schur_f32(rr_factors* f, const TwistStep& t, cudaStream_t st);
 // factor_w.cu: the wide FP32 factorisation (TF32 or BF16 operand splits)
 bool factor_wide_ok(const rr_factors* f);
 rr_status launch_factor_wide(rr_factors* f);

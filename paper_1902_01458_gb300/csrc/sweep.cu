@@ -3,15 +3,21 @@
 // one factorisation of s I - L (Sec. III.A).
 //
 // With G_i = S_i^{-1} and C_i = -L_{i,i+1} (at most 3q entries per row):
+// and the factorisation run from both ends to the middle column m (factor.cu), a
+// solve goes inwards in both halves, through the middle, and outwards (written
+// for the left half, i < m; the right one is the mirror image):
 // Normal solve (s I - L) y = f:
-//   forward  z_0 = G_0 f_0,      z_i = G_i (f_i + L_{i,i-1} z_{i-1})
-//   backward y_{n-1} = z_{n-1},  y_i = z_i - G_i (C_i y_{i+1})
+//   inward   z_0 = G_0 f_0,      z_i = G_i (f_i + L_{i,i-1} z_{i-1})
+//   middle   y_m = G_m (f_m + L_{m,m-1} z_{m-1} + L_{m,m+1} z_{m+1})
+//   outward  y_i = z_i - G_i (C_i y_{i+1})
 // Adjoint solve (s I - L)^H w = g:
-//   forward  h_0 = g_0,          h_{i+1} = g_{i+1} - C_i^H (G_i^H h_i)
-//   backward w_{n-1} = G^H h,    w_i = G_i^H (h_i + L_{i+1,i}^T w_{i+1})
-// Only G_i is stored.  Two forms: one launch per solve with a cluster of CTAs
-// per problem (sweep_cl.cuh), or, for large blocks and batches, two launches
-// per streamwise column for all problems of the batch: the dense (b x b) x
+//   inward   h_0 = g_0,          h_{i+1} = g_{i+1} - C_i^H (G_i^H h_i)
+//   middle   h_m from both sides, w_m = G_m^H h_m
+//   outward  w_i = G_i^H (h_i + L_{i+1,i}^T w_{i+1})
+// The chain is nx + 1 products instead of the 2 nx - 1 of a sweep from one end.
+// Only G_i is stored.  Two forms: two launches per solve with a cluster of CTAs
+// per problem and half (sweep_cl.cuh), or, for large blocks and batches, two
+// launches per pair of streamwise columns for all problems of the batch: the dense (b x b) x
 // (b x k) product on the tensor cores, its contraction split over CTAs
 // (sweep_tc2_kernel), and the sum of the partial blocks with the sparse
 // coupling that forms the next column's right-hand side (sweep_couple_kernel).
@@ -25,17 +31,31 @@
 
 namespace {
 
-// Step s of a solve works on column sweep_col(s): forward, then back.
-__host__ __device__ __forceinline__ int sweep_col(int s, int nx) { return s < nx ? s : 2 * nx - 2 - s; }
+// A step of the tensor-core sweeps: for half 0 and, when nh == 2, half 1 (the
+// mirror image), a column of the inward sweep, the middle one, or one of the
+// outward sweep.  Half h has its `own` columns h == 0: 0 .. mid - 1,
+// h == 1: nx - 1 .. mid + 1.
+enum { SW_IN = 0, SW_MID = 1, SW_OUT = 2 };
+struct SweepStep {
+  int phase, t, nh;  // t: columns from the end (SW_IN) or from the middle (SW_OUT)
+};
+__host__ __device__ __forceinline__ int half_cols(int half, int nx) {
+  return half ? nx - 1 - twist_mid(nx) : twist_mid(nx);
+}
+__host__ __device__ __forceinline__ int step_col(const SweepStep& s, int half, int nx) {
+  if (s.phase == SW_IN) return half ? nx - 1 - s.t : s.t;
+  return half ? twist_mid(nx) + s.t : twist_mid(nx) - s.t;
+}
 
-// Result of step s and right-hand side of step s + 1.  Per problem and tile of
+// Result of a step and right-hand side of the next.  Per problem, half and tile of
 // CPL_Y grid points: o = the sum of the KS partial products in a fixed order
-// (back sweep: z_i minus it), of the tile's rows and of one point on either
-// side (recomputed, not exchanged), kept in shared memory; then
-//   t = in + L_{i,i-1} o (forward), -L_{i,i+1} o (back),
-//   t = in + L_{i-1,i}^T o (adjoint forward, stored as h too),
-//   t = h + L_{i+1,i}^T o (adjoint back)
-// for the next column i.  z goes to zh in the forward sweep, so the back sweep's
+// (outward: z_i minus it), of the tile's rows and of one point on either
+// side (recomputed, not exchanged), kept in shared memory; then, with i the
+// column before of the half,
+//   t = in + L_{i',i} o (inward), -L_{i',i} o (outward),
+//   t = in + L_{i,i'}^T o (adjoint inward, stored as h too),
+//   t = h + L_{i,i'}^T o (adjoint outward)
+// for the next column i'.  z goes to zh in the inward sweep, so the outward one's
 // results (x) never overwrite a value a neighbouring tile still needs.
 // Bound: L2 latency (the partials were just written), so the coefficients and
 // inputs of the coupling are requested before the partials are summed, and a
@@ -47,22 +67,28 @@ inline int couple_threads(int q, int k) {
 
 template <bool TRANS>
 __global__ void __launch_bounds__(CPL_MAXTHR)
-sweep_couple_kernel(OpView op, int s, int F, int k, int KS, const float2* __restrict__ part,
-                    const float2* __restrict__ in, float2* x, float2* zh,
-                    float2* __restrict__ tbuf, const int* __restrict__ amap) {
+sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
+                    const float2* __restrict__ part, const float2* __restrict__ in, float2* x,
+                    float2* zh, float2* __restrict__ tbuf, const int* __restrict__ amap) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* o = reinterpret_cast<float4*>(smem_raw);  // [(CPL_Y + 2) q][k / 2]
   const int b = op.b, q = op.q, ny = op.ny, nx = op.nx, P = k >> 1;
-  const int f = active_problem(amap, blockIdx.y);
+  const int half = blockIdx.y / Fa, f = active_problem(amap, blockIdx.y - half * Fa);
   const int y0 = blockIdx.x * CPL_Y, npt = min(CPL_Y, ny - y0);
-  const size_t NK = (size_t)op.n * k, total = (size_t)F * b * k;
-  const int i = sweep_col(s, nx);
-  const bool last = s == 2 * nx - 2, fwd = s + 1 < nx;
-  const int i1 = last ? i : sweep_col(s + 1, nx);
-  const float* cb = op.coef32 + (size_t)(!TRANS ? i1 : fwd ? i1 - 1 : i1 + 1) * b * op.S;
-  // (h_0 is the input itself: no forward step stores it)
-  const float4* src = reinterpret_cast<const float4*>((fwd || i1 == 0 ? in : zh) + (size_t)f * NK +
-                                                      (size_t)i1 * b * k);
+  const size_t NK = (size_t)op.n * k, total = (size_t)s.nh * F * b * k;
+  const int i = step_col(s, half, nx);
+  const bool inw = s.phase == SW_IN, outw = s.phase == SW_OUT;
+  const int dcol = (half != 0) == inw ? -1 : 1;  // to the next column
+  // (the middle's right-hand side needs both halves: sweep_middle_kernel)
+  const bool last = s.phase != SW_MID && s.t + (inw ? 1 : 0) == half_cols(half, nx);
+  const int i1 = last ? i : i + dcol;
+  // L[(i1, .), (i, .)]: slots dx = -dcol of the rows of i1; transposed, dx = dcol of
+  // those of i
+  const float* cb = op.coef32 + (size_t)(!TRANS ? i1 : i) * b * op.S;
+  const int slot = (!TRANS ? 1 - dcol : 1 + dcol) * 3;
+  // (h of the end columns is the input itself: no step stores it)
+  const float4* src = reinterpret_cast<const float4*>(
+      (inw || i1 == 0 || i1 == nx - 1 ? in : zh) + (size_t)f * NK + (size_t)i1 * b * k);
   struct Term {
     float cf[3][4];
     float4 t;
@@ -70,30 +96,32 @@ sweep_couple_kernel(OpView op, int s, int F, int k, int KS, const float2* __rest
   auto load_term = [&](Term& w, int e) {
     const int lrow = e / P, jp = e - lrow * P;
     const int lp = lrow / q, c = lrow - lp * q, iy = y0 + lp, m = iy * q + c;
-    w.t = TRANS || fwd ? src[m * P + jp] : make_float4(0.f, 0.f, 0.f, 0.f);
+    w.t = TRANS || inw ? src[m * P + jp] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int d = -1; d <= 1; ++d) {
       int off, stride = 1;
       bool ok = true;
       if (!TRANS) {
-        off = m * op.S + ((fwd ? 0 : 6) + d + 1) * q;
+        off = m * op.S + (slot + d + 1) * q;
       } else {
         const int jy = nbr_y(iy, -d, ny, op.periodic);
         ok = jy >= 0;
-        off = jy * q * op.S + ((fwd ? 6 : 0) + d + 1) * q + c;
+        off = jy * q * op.S + (slot + d + 1) * q + c;
         stride = op.S;
       }
 #pragma unroll
       for (int cp = 0; cp < 4; ++cp) {
         const float v = ok && cp < q ? cb[off + cp * stride] : 0.f;
-        w.cf[d + 1][cp] = !TRANS && !fwd ? -v : v;
+        w.cf[d + 1][cp] = !TRANS && !inw ? -v : v;
       }
     }
   };
   Term w;
   const int nown = npt * q * P;
   if (!last && (int)threadIdx.x < nown) load_term(w, threadIdx.x);
-  const float4* pf = reinterpret_cast<const float4*>(part + (size_t)f * b * k);
+  // (the middle's partials are the first half's)
+  const size_t pidx = s.phase == SW_MID ? f : (size_t)half * F + f;
+  const float4* pf = reinterpret_cast<const float4*>(part + pidx * b * k);
   float4* xi = reinterpret_cast<float4*>(x + (size_t)f * NK + (size_t)i * b * k);
   float4* zi = reinterpret_cast<float4*>(zh + (size_t)f * NK + (size_t)i * b * k);
   for (int e = threadIdx.x; e < (npt + 2) * q * P; e += blockDim.x) {
@@ -106,7 +134,7 @@ sweep_couple_kernel(OpView op, int s, int F, int k, int KS, const float2* __rest
     if (y >= 0 && y < ny) {
       const int e0 = (y * q + c) * P + jp;
       float4 z = v;
-      if (!TRANS && s >= nx) z = zi[e0];
+      if (!TRANS && outw) z = zi[e0];
 #pragma unroll 4
       for (int t = 0; t < KS; ++t) {
         const float4 u = pf[(size_t)t * (total >> 1) + e0];
@@ -115,10 +143,11 @@ sweep_couple_kernel(OpView op, int s, int F, int k, int KS, const float2* __rest
         v.z += u.z;
         v.w += u.w;
       }
-      if (!TRANS && s >= nx) v = make_float4(z.x - v.x, z.y - v.y, z.z - v.z, z.w - v.w);
+      if (!TRANS && outw) v = make_float4(z.x - v.x, z.y - v.y, z.z - v.z, z.w - v.w);
       if (own) {
-        if (!TRANS && s < nx) zi[e0] = v;
-        if (s >= nx - 1) xi[e0] = v;
+        if (!TRANS && inw) zi[e0] = v;
+        // x; the adjoint's last inward result waits there for the middle
+        if (outw || (s.phase == SW_MID && half == 0) || (TRANS && inw && last)) xi[e0] = v;
       }
     }
     o[e] = v;
@@ -126,7 +155,7 @@ sweep_couple_kernel(OpView op, int s, int F, int k, int KS, const float2* __rest
   if (last) return;
   __syncthreads();
   float4* h = reinterpret_cast<float4*>(zh + (size_t)f * NK + (size_t)i1 * b * k);
-  float4* tf = reinterpret_cast<float4*>(tbuf + (size_t)f * b * k);
+  float4* tf = reinterpret_cast<float4*>(tbuf + ((size_t)half * F + f) * b * k);
   for (int e = threadIdx.x; e < nown; e += blockDim.x) {
     if (e != (int)threadIdx.x) load_term(w, e);
     const int lrow = e / P, jp = e - lrow * P;
@@ -146,9 +175,47 @@ sweep_couple_kernel(OpView op, int s, int F, int k, int KS, const float2* __rest
         t.w = fmaf(a, u.w, t.w);
       }
     }
-    if (TRANS && fwd) h[m * P + jp] = t;
+    if (TRANS && inw) h[m * P + jp] = t;
     tf[m * P + jp] = t;
   }
+}
+
+// Right-hand side of the middle column: in + the couplings of both halves' last
+// inward results (z in zh, adjoint p in x), one thread per row and two columns;
+// a few microseconds of L2 latency, once per solve.
+template <bool TRANS>
+__global__ void sweep_middle_kernel(OpView op, int k, const float2* __restrict__ in,
+                                    const float2* __restrict__ src, float2* __restrict__ tbuf,
+                                    const int* __restrict__ amap) {
+  const int b = op.b, q = op.q, mid = twist_mid(op.nx), P = k >> 1;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= b * P) return;
+  const int f = active_problem(amap, blockIdx.y);
+  const int m = e / P, jp = e - m * P, iy = m / q, c = m - iy * q;
+  const size_t NK = (size_t)op.n * k;
+  float4 t = reinterpret_cast<const float4*>(in + f * NK + (size_t)mid * b * k)[e];
+  for (int dx = -1; dx <= 1; dx += 2) {
+    const float4* o = reinterpret_cast<const float4*>(src + f * NK + (size_t)(mid + dx) * b * k);
+    const float* cb = op.coef32 + (size_t)(TRANS ? mid + dx : mid) * b * op.S;
+#pragma unroll
+    for (int d = -1; d <= 1; ++d) {
+      const int jy = nbr_y(iy, TRANS ? -d : d, op.ny, op.periodic);
+      if (jy < 0) continue;
+#pragma unroll
+      for (int cp = 0; cp < 4; ++cp) {
+        if (cp >= q) break;
+        const int r = jy * q + cp;
+        const float a = TRANS ? cb[r * op.S + ((1 - dx) * 3 + d + 1) * q + c]
+                              : cb[m * op.S + ((1 + dx) * 3 + d + 1) * q + cp];
+        const float4 u = o[r * P + jp];
+        t.x = fmaf(a, u.x, t.x);
+        t.y = fmaf(a, u.y, t.y);
+        t.z = fmaf(a, u.z, t.z);
+        t.w = fmaf(a, u.w, t.w);
+      }
+    }
+  }
+  reinterpret_cast<float4*>(tbuf + (size_t)f * b * k)[e] = t;
 }
 
 // ---------------------------------------------------------------------------
@@ -202,9 +269,9 @@ constexpr int TC2_THREADS = TC2_CONV + 32;    // + control warp 16 (TMA producer
 
 template <bool TRANS, int SPLIT>
 __global__ void __launch_bounds__(TC2_THREADS, 1)
-sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp, int blk,
+sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp, SweepStep step,
                  int nx, int nrt, int KS, int cpp, const float2* rhs, size_t rstride,
-                 float2* __restrict__ part, int F, int Fa, const int* __restrict__ amap, int* err,
+                 size_t hstride, float2* __restrict__ part, int F, int Fa, const int* __restrict__ amap, int* err,
                  uint32_t tries, int stall) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t full_bar[TC2_STAGES];
@@ -223,7 +290,7 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool ctrl = (tid == TC2_CONV);  // the one thread that feeds TMA and the tensor core
   const int nch = (b + TC2_KC - 1) / TC2_KC;
-  const int nitems = nrt * KS * Fa;  // over the active problems
+  const int nitems = nrt * KS * Fa * step.nh;  // over the active problems of both halves
   const int my_items = nitems > (int)blockIdx.x
                            ? (nitems - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x
                            : 0;
@@ -236,12 +303,14 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
   // MMAs into one set of 6N columns: p0 x [q0 | q1 | q2], p1 x [q0 | q1], p2 x q0.
   const uint32_t ncols = X6 ? (6 * N <= 128 ? 128u : 6 * N <= 256 ? 256u : 512u)
                             : ((N <= 32) ? 256u : 512u);
-  // work item t of this CTA -> (problem, row tile, contraction part)
-  auto item = [&](int t, int& f, int& rt, int& ks) {
+  // work item t of this CTA -> (half, problem, row tile, contraction part)
+  auto item = [&](int t, int& half, int& f, int& rt, int& ks) {
     const int it = (int)blockIdx.x + t * (int)gridDim.x;
     rt = it % nrt;
     ks = (it / nrt) % KS;
-    f = active_problem(amap, it / (nrt * KS));
+    const int p = it / (nrt * KS);
+    half = p >= Fa;
+    f = active_problem(amap, half ? p - Fa : p);
   };
   auto item_len = [&](int ks) { return min(nch, ks * cpp + cpp) - ks * cpp; };
 
@@ -263,10 +332,10 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
   // stall set (a diagnostic of the bounded waits) the first CTA issues
   // nothing at all, so its first wait runs out with no copy or MMA in flight.
   const bool stalled = stall && blockIdx.x == 0;
-  int p_item = 0, p_lc = 0, issued = 0, p_f = 0, p_rt = 0, p_ks = 0, p_len = 0;
+  int p_item = 0, p_lc = 0, issued = 0, p_h = 0, p_f = 0, p_rt = 0, p_ks = 0, p_len = 0;
   int committed = 0;  // chunks whose MMAs have been committed (control thread)
   if (ctrl && my_items > 0) {
-    item(0, p_f, p_rt, p_ks);
+    item(0, p_h, p_f, p_rt, p_ks);
     p_len = item_len(p_ks);
   }
   auto issue_next = [&]() {
@@ -275,17 +344,17 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
     const int s = issued % TC2_STAGES;
     const uint32_t rhs_bytes = (uint32_t)(min(TC2_KC, b - m0) * k * 8);
     unsigned char* st = raw + s * stage_bytes;
-    const int zblk = p_f * nx + blk;
+    const int zblk = p_f * nx + step_col(step, p_h, nx);
     tc::mbar_expect_tx(&full_bar[s], TC2_TILE_BYTES + rhs_bytes);
     if (!TRANS) tc::tma_load_3d(st, &tmap, 2 * m0, p_rt * TC_RT, zblk, &full_bar[s]);
     else tc::tma_load_3d(st, &tmap, 2 * p_rt * TC_RT, m0, zblk, &full_bar[s]);
-    tc::bulk_load(st + TC2_TILE_BYTES, rhs + (size_t)p_f * rstride + (size_t)m0 * k, rhs_bytes,
-                  &full_bar[s]);
+    tc::bulk_load(st + TC2_TILE_BYTES, rhs + p_h * hstride + p_f * rstride + (size_t)m0 * k,
+                  rhs_bytes, &full_bar[s]);
     ++issued;
     if (++p_lc == p_len) {
       p_lc = 0;
       if (++p_item < my_items) {
-        item(p_item, p_f, p_rt, p_ks);
+        item(p_item, p_h, p_f, p_rt, p_ks);
         p_len = item_len(p_ks);
       }
     }
@@ -313,8 +382,8 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
   int g = 0;  // chunks consumed so far (global over this CTA's items)
   bool failed = false;
   for (int t = 0; t < my_items && !failed; ++t) {
-    int f, rt, ks;
-    item(t, f, rt, ks);
+    int half, f, rt, ks;
+    item(t, half, f, rt, ks);
     const int nl = item_len(ks);
     for (int lc = 0; lc < nl; ++lc, ++g) {
       const int s = g % TC2_STAGES, q = g & 1;
@@ -397,7 +466,7 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
       // columns 4 r + t % 4, so four consecutive threads write 32 contiguous
       // bytes of a row (whole sectors)
       const int lq = warp & 3, sb = (warp >> 2) & 1;
-      float2* pf = part + ((size_t)ks * F + f) * (size_t)b * k;
+      float2* pf = part + (((size_t)ks * step.nh + half) * F + f) * (size_t)b * k;
       for (int hh = warp >> 3; hh < (N + 31) / 32; hh += 2) {
         float v[16], w[16];
         const uint32_t ta =
@@ -449,9 +518,9 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
 // One launch of the TMA-fed tensor-core sweep step in the factors' operand
 // split (partial products into Pbuf).
 template <bool TRANS, int SPLIT, typename C>
-rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp, int blk, int nx,
-                     int nrt, int KS, int cpp, const C* rhs, size_t rstride, rr_factors* fa,
-                     cudaStream_t st) {
+rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
+                     const SweepStep& step, int nx, int nrt, int KS, int cpp, const C* rhs,
+                     size_t rstride, size_t hstride, rr_factors* fa, cudaStream_t st) {
   const size_t smem = tc2_smem_bytes<SPLIT>(kp) + 1024;
   static size_t attr = 0;  // dynamic shared memory opted in so far
   if (smem > attr) {
@@ -460,7 +529,7 @@ rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp, in
     attr = smem;
   }
   sweep_tc2_kernel<TRANS, SPLIT><<<grid_x, TC2_THREADS, smem, st>>>(
-      *tm, b, k, kp, blk, nx, nrt, KS, cpp, reinterpret_cast<const float2*>(rhs), rstride,
+      *tm, b, k, kp, step, nx, nrt, KS, cpp, reinterpret_cast<const float2*>(rhs), rstride, hstride,
       reinterpret_cast<float2*>(fa->Pbuf), fa->F, active_count(fa), fa->amap, fa->flag + fa->F,
       wait_tries(), take_stall());
   return RR_OK;
@@ -482,21 +551,22 @@ namespace {
 // Split count of a product: the smallest whose items fill the persistent CTAs to
 // 85 % (each split adds a partial block to write and sum), else the best
 // balance.  The partial buffer holds 4 F b 64 complex, so up to 256 / k splits
-// fit; few active problems (refinement corrections) take more splits to keep
+// of one half's problems fit; few active problems (refinement corrections) take more splits to keep
 // the SMs busy.
-int split_count(const rr_factors* fa, int k, int nrt, int nch, int nsm) {
-  if (fa->tune_ks > 0) {  // tuned (at most the 4 partial buffers)
-    const int cpp = (nch + std::min(fa->tune_ks, 4) - 1) / std::min(fa->tune_ks, 4);
+int split_count(const rr_factors* fa, int k, int nh, int nrt, int nch, int nsm) {
+  const int ks_max = std::min(16, std::max(1, 256 / (k * nh)));
+  if (fa->tune_ks > 0) {  // tuned (as far as the partial buffer goes)
+    const int ksc = std::min(fa->tune_ks, ks_max);
+    const int cpp = (nch + ksc - 1) / ksc;
     return (nch + cpp - 1) / cpp;
   }
-  const int ks_max = std::min(16, std::max(1, 256 / k));
   int KS = 1;
   double best = 0.0;
   for (int ksc = 1; ksc <= ks_max && ksc <= nch; ++ksc) {
     const int cpp = (nch + ksc - 1) / ksc;
     const int ksr = (nch + cpp - 1) / cpp;
     if (ksr > ks_max) continue;
-    const long items = (long)nrt * active_count(fa) * ksr;
+    const long items = (long)nrt * active_count(fa) * nh * ksr;
     const long waves = (items + nsm - 1) / nsm;
     const double eff = (double)items / (double)(waves * nsm);
     if (eff >= 0.85) return ksr;
@@ -515,36 +585,51 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
   int kp = 8;
   while (kp < k) kp <<= 1;
   cudaStream_t st = fa->stream;
-  float2* tb = reinterpret_cast<float2*>(fa->Tbuf);  // [F][b][k]
+  float2* tb = reinterpret_cast<float2*>(fa->Tbuf);  // [2][F][b][k]
   const int nrt = (b + TC_RT - 1) / TC_RT, nch = (b + TC2_KC - 1) / TC2_KC;
   const int nsm = num_sms(d.device);
-  const int KS = split_count(fa, k, nrt, nch, nsm), cpp = (nch + KS - 1) / KS;
-  const int grid_x = std::min(nrt * Fa * KS, nsm);
   const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(fa->tmap[TRANS ? 1 : 0]);
-  const dim3 cgrid((d.ny + CPL_Y - 1) / CPL_Y, Fa);
   const size_t csmem = (size_t)(CPL_Y + 2) * d.q * k * sizeof(float2);
-  for (int s = 0; s < 2 * nx - 1; ++s) {
+  const int n0 = half_cols(0, nx), n1 = half_cols(1, nx);  // n1 is n0 or n0 - 1
+  for (int s = 0; s <= 2 * n0; ++s) {
+    SweepStep step;
+    step.phase = s < n0 ? SW_IN : s == n0 ? SW_MID : SW_OUT;
+    step.t = s < n0 ? s : s - n0;
+    step.nh = step.phase == SW_IN ? (step.t < n1 ? 2 : 1) : step.phase == SW_MID ? 1
+              : step.t <= n1 ? 2 : 1;
     const float2* rhs = s == 0 ? in : tb;
     const size_t rstride = s == 0 ? (size_t)d.n * k : (size_t)b * k;
-    const int blk = sweep_col(s, nx);
+    const size_t hstride = s == 0 ? (size_t)(nx - 1) * b * k : (size_t)F * b * k;
+    const int KS = split_count(fa, k, step.nh, nrt, nch, nsm), cpp = (nch + KS - 1) / KS;
+    const int grid_x = std::min(nrt * Fa * step.nh * KS, nsm);
+    if (step.phase == SW_MID) {
+      prof_begin(PROF_SWEEP, st);
+      sweep_middle_kernel<TRANS><<<dim3((b * (k / 2) + 255) / 256, Fa), 256, 0, st>>>(
+          view(d), k, in, TRANS ? x : zh, tb, fa->amap);
+      prof_end(PROF_SWEEP, st);
+    }
     prof_begin(PROF_SWEEP, st);
     rr_status ls;
     switch (fa->prec) {
       case RR_FP32_BF16X3:
-        ls = launch_tc2<TRANS, tc::SPLIT_BF16X3>(tm, grid_x, b, k, kp, blk, nx, nrt, KS, cpp, rhs,
-                                                rstride, fa, st);
+        ls = launch_tc2<TRANS, tc::SPLIT_BF16X3>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
+                                                rstride, hstride, fa, st);
         break;
       case RR_FP32_BF16X6:
-        ls = launch_tc2<TRANS, tc::SPLIT_BF16X6>(tm, grid_x, b, k, kp, blk, nx, nrt, KS, cpp, rhs,
-                                                rstride, fa, st);
+        ls = launch_tc2<TRANS, tc::SPLIT_BF16X6>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
+                                                rstride, hstride, fa, st);
         break;
       default:
-        ls = launch_tc2<TRANS, tc::SPLIT_TF32X3>(tm, grid_x, b, k, kp, blk, nx, nrt, KS, cpp, rhs,
-                                                rstride, fa, st);
+        ls = launch_tc2<TRANS, tc::SPLIT_TF32X3>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
+                                                rstride, hstride, fa, st);
     }
     if (ls != RR_OK) return ls;
-    sweep_couple_kernel<TRANS><<<cgrid, couple_threads(d.q, k), csmem, st>>>(
-        view(d), s, F, k, KS, reinterpret_cast<const float2*>(fa->Pbuf), in, x, zh, tb, fa->amap);
+    // (the middle's result starts both halves' outward sweeps)
+    const int ch = step.phase == SW_MID ? 2 : step.nh;
+    sweep_couple_kernel<TRANS><<<dim3((d.ny + CPL_Y - 1) / CPL_Y, ch * Fa), couple_threads(d.q, k),
+                                 csmem, st>>>(view(d), step, F, Fa, k, KS,
+                                              reinterpret_cast<const float2*>(fa->Pbuf), in, x, zh,
+                                              tb, fa->amap);
     prof_end(PROF_SWEEP, st);
     prof_count(1);
     RR_CUDA(cudaGetLastError());
@@ -562,8 +647,8 @@ rr_status launch_solve_lo(rr_factors* fa, int k, int adjoint, const void* b, voi
   if (fa->prec == RR_FP64) return launch_sweep_cl64(fa, k, adjoint, b, x, tmp);
   if (sweep_tc2_ok(fa, k)) {
     const OpDev& d = fa->op->d;
-    const double step = 10.0 + 8.0 * active_count(fa) * d.b * d.b / 2.6e6;
-    if ((2.0 * d.nx - 1) * step < sweep_cl32_us(fa, k, adjoint))
+    const double step = 10.0 + 16.0 * active_count(fa) * d.b * d.b / 2.6e6;
+    if ((d.nx + 1.0) * step < sweep_cl32_us(fa, k, adjoint))
       return adjoint ? solve_tc2<true>(fa, k, reinterpret_cast<const float2*>(b),
                                        reinterpret_cast<float2*>(x), reinterpret_cast<float2*>(tmp))
                      : solve_tc2<false>(fa, k, reinterpret_cast<const float2*>(b),

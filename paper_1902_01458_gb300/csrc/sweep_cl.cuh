@@ -1,6 +1,10 @@
-// Whole block sweeps in one launch: the forward and back sweep of a solve (see
-// sweep.cu for the recurrences) run by one thread-block cluster per problem and
-// group of right-hand-side columns, in FP32 or FP64 on the CUDA cores.
+// Whole block sweeps in two launches: the sweeps of a solve from both ends to the
+// middle column and back out (see sweep.cu for the recurrences), each run by one
+// thread-block cluster per problem, half and group of right-hand-side columns,
+// in FP32 or FP64 on the CUDA cores.  The halves meet between the launches: the
+// inward one leaves each half's last result in an edge buffer, from which both
+// halves of the outward one form the middle column's right-hand side (and both
+// multiply it: cheaper than an exchange between clusters).
 //
 // CTA `rank` of a cluster owns the grid points [rank npt, (rank + 1) npt) of
 // every streamwise column (npt q rows).  Step s of a solve multiplies one G_i
@@ -45,6 +49,8 @@ struct Args {
   const C_t<T>* in;    // [F][N][k]
   C_t<T>* x;           // [F][N][k]
   C_t<T>* h;           // [F][N][k] scratch (adjoint)
+  C_t<T>* edge;        // [2][F][b][k] last inward result of each half
+  int F, out;          // problems; inward (0) or outward (1) launch
   int k, ng, npt, CL;
   const int* amap;
   int* err;
@@ -101,8 +107,8 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
   const int W = blockDim.x >> 5, nthr = blockDim.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = (int)tc::cluster_rank();
-  const int cl = blockIdx.x / CL, f = active_problem(a.amap, cl / a.ng);
-  const int j0 = (cl % a.ng) * NC;
+  const int cl = blockIdx.x / CL, half = cl & 1, f = active_problem(a.amap, (cl >> 1) / a.ng);
+  const int j0 = ((cl >> 1) % a.ng) * NC;
   const int rmax = npt * q, bp = (b + KC - 1) / KC * KC, nch = bp / KC;
   const int pts = max(0, min(npt, ny - rank * npt)), rows = pts * q, row0 = rank * rmax;
   const size_t SB = stage_bytes<T, KC, TRANS>(rmax);
@@ -117,8 +123,14 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
   C* x = a.x + (size_t)f * NK;
   C* h = TRANS ? a.h + (size_t)f * NK : nullptr;
   const int k = a.k;
-  const int nstep = 2 * nx - 1;
-  auto step_col = [&](int s) { return s < nx ? s : 2 * nx - 2 - s; };
+  // columns of the half: step s of the inward launch is column s (nx - 1 - s), of
+  // the outward one column mid - s (mid + s), the middle first
+  const bool outw = a.out != 0;
+  const int mid = twist_mid(nx);
+  const int nstep = (half ? nx - 1 - mid : mid) + (outw ? 1 : 0);
+  const int dcol = (half != 0) == outw ? 1 : -1;      // column of step s + 1 minus that of s
+  const int col0 = outw ? mid : half ? nx - 1 : 0;
+  auto step_col = [&](int s) { return col0 + s * dcol; };
 
   if (tid < 2) {
     tc::mbar_init(&mT[tid], 1);
@@ -185,39 +197,62 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
   auto load_unit = [&](Unit& w, int e, int s) {
     const int r = e / UPR, j = j0 + (e - r * UPR) * VEC, m = row0 + r;
     const int i = step_col(s), iy = m / q, c = m - iy * q;
-    const bool fwd = s < nx;
-    // !TRANS: L[(i, m), (i -+ 1, ...)], slots dx = -1 (forward) or +1 of the row;
-    // TRANS: L[(i -+ 1, r), (i, m)], rows r of the points whose stencil reaches m
-    const T* cb = coef + (size_t)(!TRANS ? i : fwd ? i - 1 : i + 1) * b * op.S;
+    // the column before, i - dcol, couples in.  !TRANS: L[(i, m), (i - dcol, ...)],
+    // slots dx = -dcol of the row; TRANS: L[(i - dcol, r), (i, m)], rows r of the
+    // points whose stencil reaches m
+    const T* cb = coef + (size_t)(!TRANS ? i : s > 0 ? i - dcol : i) * b * op.S;
+    const int slot = (!TRANS ? 1 - dcol : 1 + dcol) * 3;
 #pragma unroll
     for (int d = -1; d <= 1; ++d) {
       int off = 0, stride = 1;
       bool ok = s > 0;
       if (!TRANS) {
-        off = m * op.S + ((fwd ? 0 : 6) + d + 1) * q;
+        off = m * op.S + (slot + d + 1) * q;
       } else {
         const int jy = nbr_y(iy, -d, ny, op.periodic);
         ok = ok && jy >= 0;
-        off = jy * q * op.S + ((fwd ? 6 : 0) + d + 1) * q + c;
+        off = jy * q * op.S + (slot + d + 1) * q + c;
         stride = op.S;
       }
 #pragma unroll
       for (int cp = 0; cp < 4; ++cp) {
         T v = (T)0;
         if (ok && cp < q) v = cb[off + cp * stride];
-        w.cf[d + 1][cp] = !TRANS && !fwd ? -v : v;
+        w.cf[d + 1][cp] = !TRANS && outw ? -v : v;
       }
     }
-    // right-hand side: in (forward), nothing (back), the stored h (adjoint back)
+    // right-hand side: in (inward, middle), nothing (outward), the stored h
+    // (adjoint outward)
 #pragma unroll
     for (int v = 0; v < VEC; ++v) {
       C z = czero<C>();
       const size_t g = ((size_t)i * b + m) * k + j + v;
       if (j + v < k) {
-        if (fwd) z = in[g];
+        if (!outw || s == 0) z = in[g];
         else if (TRANS) z = h[g];
       }
       w.in[v] = z;
+    }
+  };
+  // the middle column's: both neighbours' last inward results
+  auto load_middle = [&](Unit& w, int e) {
+    const int r = e / UPR, j = j0 + (e - r * UPR) * VEC, m = row0 + r;
+    const int iy = m / q, c = m - iy * q;
+    for (int side = 0; side < 2; ++side) {
+      const int dx = side ? 1 : -1;
+      const C* E = a.edge + ((size_t)side * a.F + f) * (size_t)b * k;
+      for (int d = -1; d <= 1; ++d) {
+        const int jy = nbr_y(iy, TRANS ? -d : d, ny, op.periodic);
+        if (jy < 0) continue;
+        for (int cp = 0; cp < q; ++cp) {
+          const T v = TRANS ? coef[((size_t)(mid + dx) * b + jy * q + cp) * op.S +
+                                   ((1 - dx) * 3 + d + 1) * q + c]
+                            : coef[((size_t)mid * b + m) * op.S + ((1 + dx) * 3 + d + 1) * q + cp];
+#pragma unroll
+          for (int u = 0; u < VEC; ++u)
+            if (j + u < k) w.in[u] = crfma(v, E[(size_t)(jy * q + cp) * k + j + u], w.in[u]);
+        }
+      }
     }
   };
   const uint32_t tb_a = tc::smem_u32(tb), mT_a = tc::smem_u32(&mT[0]);
@@ -241,7 +276,7 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
         }
       }
     }
-    if (TRANS && s < nx) {  // h_i for the back sweep (own rows only)
+    if (TRANS && !outw) {  // h_i for the outward sweep (own rows only)
 #pragma unroll
       for (int v = 0; v < VEC; ++v)
         if (j + v < k) h[((size_t)i * b + m) * k + j + v] = t[v];
@@ -264,6 +299,7 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
   if (tid == 0) tc::mbar_expect_tx(&mT[0], t_bytes);
   for (int e = tid; e < units; e += nthr) {
     load_unit(un[0], e, 0);
+    if (outw) load_middle(un[0], e);
     couple_unit(un[0], e, 0);
   }
   const int lr = lane / LC, lc = (lane % LC) * CPL;
@@ -331,7 +367,7 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
       const int e = tid + p * nthr;
       if (e >= units) break;
       if (!last) load_unit(un[p], e, s + 1);
-      if (!TRANS && s >= nx) {
+      if (!TRANS && outw && s > 0) {
         const int r = e / UPR, j = j0 + (e - r * UPR) * VEC;
 #pragma unroll
         for (int v = 0; v < VEC; ++v)
@@ -365,14 +401,21 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
 #pragma unroll
         for (int v = 0; v < VEC; ++v) o[v] = cadd(o[v], pv[v]);
       }
-      if (!TRANS && s >= nx) {
+      if (!TRANS && outw && s > 0) {
 #pragma unroll
         for (int v = 0; v < VEC; ++v) o[v] = csub(xo[p][v], o[v]);
       }
-      if (!TRANS || s >= nx - 1) {
+      // (the middle column's result is half 0's to store)
+      if (outw ? s > 0 || half == 0 : !TRANS) {
 #pragma unroll
         for (int v = 0; v < VEC; ++v)
           if (j + v < k) x[((size_t)i * b + row0 + r) * k + j + v] = o[v];
+      }
+      if (!outw && last) {
+        C* E = a.edge + ((size_t)half * a.F + f) * (size_t)b * k;
+#pragma unroll
+        for (int v = 0; v < VEC; ++v)
+          if (j + v < k) E[(size_t)(row0 + r) * k + j + v] = o[v];
       }
       const float4 val = *reinterpret_cast<const float4*>(o);
       *reinterpret_cast<float4*>(ob + (size_t)(q + r) * NC + cu * VEC) = val;
@@ -456,8 +499,8 @@ Plan make_plan(const OpDev& d, int Fa, int k, int trans) {
       }
       if (W == 0) continue;
       const int slots = cluster_slots(d.device, CL);
-      const int waves = (int)(((long)Fa * ng + slots - 1) / slots);
-      const double us = waves * (2.0 * d.nx - 1) * step_us(DP, d.b, rpl, cpl);
+      const int waves = (int)((2L * Fa * ng + slots - 1) / slots);
+      const double us = waves * (d.nx + 1.0) * step_us(DP, d.b, rpl, cpl);
       if (best.us < 0 || us < best.us) best = Plan{kc, CL, npt, W, rpl, us};
     }
   }
@@ -516,6 +559,8 @@ rr_status launch_plan(rr_factors* fa, const Plan& p, int k, const void* in, void
   a.in = reinterpret_cast<const C_t<T>*>(in);
   a.x = reinterpret_cast<C_t<T>*>(x);
   a.h = reinterpret_cast<C_t<T>*>(h);
+  a.edge = reinterpret_cast<C_t<T>*>(fa->Tbuf);
+  a.F = fa->F;
   a.k = k;
   a.ng = (k + p.kc - 1) / p.kc;
   a.npt = p.npt;
@@ -523,22 +568,25 @@ rr_status launch_plan(rr_factors* fa, const Plan& p, int k, const void* in, void
   a.amap = fa->amap;
   a.err = fa->flag + fa->F;
   a.tries = wait_tries();
-  a.stall = take_stall();
-  const int clusters = active_count(fa) * a.ng;
+  const int clusters = 2 * active_count(fa) * a.ng;
   const size_t smem = smem_bytes<T, TRANS>(d.b, p.npt * d.q, d.q, p.kc, p.W);
   cudaStream_t st = fa->stream;
-  prof_begin(PROF_SWEEP, st);
-  rr_status s;
-  if constexpr (sizeof(T) == 8) {
-    if (p.kc == 1) s = launch_rpl<T, TRANS, 1, 1>(a, p.rpl, clusters, smem, p.W, st);
-    else if (p.kc == 2) s = launch_rpl<T, TRANS, 1, 2>(a, p.rpl, clusters, smem, p.W, st);
-    else s = launch_rpl<T, TRANS, 1, 4>(a, p.rpl, clusters, smem, p.W, st);
-  } else {
-    if (p.kc == 4) s = launch_rpl<T, TRANS, 2, 2>(a, p.rpl, clusters, smem, p.W, st);
-    else s = launch_rpl<T, TRANS, 2, 4>(a, p.rpl, clusters, smem, p.W, st);
+  for (a.out = 0; a.out < 2; ++a.out) {
+    a.stall = take_stall();
+    prof_begin(PROF_SWEEP, st);
+    rr_status s;
+    if constexpr (sizeof(T) == 8) {
+      if (p.kc == 1) s = launch_rpl<T, TRANS, 1, 1>(a, p.rpl, clusters, smem, p.W, st);
+      else if (p.kc == 2) s = launch_rpl<T, TRANS, 1, 2>(a, p.rpl, clusters, smem, p.W, st);
+      else s = launch_rpl<T, TRANS, 1, 4>(a, p.rpl, clusters, smem, p.W, st);
+    } else {
+      if (p.kc == 4) s = launch_rpl<T, TRANS, 2, 2>(a, p.rpl, clusters, smem, p.W, st);
+      else s = launch_rpl<T, TRANS, 2, 4>(a, p.rpl, clusters, smem, p.W, st);
+    }
+    prof_end(PROF_SWEEP, st);
+    if (s != RR_OK) return s;
   }
-  prof_end(PROF_SWEEP, st);
-  return s;
+  return RR_OK;
 }
 
 }  // namespace sweepcl
