@@ -464,7 +464,8 @@ rr_status cholqr2(rr_factors* fa, int k, double2* Y, double2* Rout, Work& w, rr_
 
 // TMA tensor maps over all FP32 factors G [F][nx][b][b] (complex, viewed as
 // floats [F*nx][b][2b]): tiles of 128 rows x 16 complex (G) and of 16 rows x
-// 128 complex (for G^H).  Used only when b >= 128 and the row pitch is a
+// 128 complex (for G^H).  The rows of the former are 128 bytes and each thread
+// reads one, so they arrive swizzled.  Used only when b >= 128 and the row pitch is a
 // multiple of 16 bytes (b even); otherwise the sweeps use cp.async kernels.
 static int encode_factor_maps(rr_factors* fa) {
   const OpDev& d = fa->op->d;
@@ -486,7 +487,7 @@ static int encode_factor_maps(rr_factors* fa) {
   const cuuint32_t boxN[3] = {32, 128, 1}, boxT[3] = {256, 16, 1}, es[3] = {1, 1, 1};
   CUresult r1 = encode(reinterpret_cast<CUtensorMap*>(fa->tmap[0]), CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                        3, fa->G, dims, strides, boxN, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                       CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                       CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   CUresult r2 = encode(reinterpret_cast<CUtensorMap*>(fa->tmap[1]), CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                        3, fa->G, dims, strides, boxT, es, CU_TENSOR_MAP_INTERLEAVE_NONE,

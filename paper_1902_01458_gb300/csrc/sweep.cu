@@ -121,6 +121,8 @@ sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
   if (!last && (int)threadIdx.x < nown) load_term(w, threadIdx.x);
   // (the middle's partials are the first half's)
   const size_t pidx = s.phase == SW_MID ? f : (size_t)half * F + f;
+  tc::grid_wait();  // (above: what kernels before the product's wrote, and constants)
+  tc::grid_trigger();
   const float4* pf = reinterpret_cast<const float4*>(part + pidx * b * k);
   float4* xi = reinterpret_cast<float4*>(x + (size_t)f * NK + (size_t)i * b * k);
   float4* zi = reinterpret_cast<float4*>(zh + (size_t)f * NK + (size_t)i * b * k);
@@ -226,38 +228,68 @@ __global__ void sweep_middle_kernel(OpView op, int k, const float2* __restrict__
 // right-hand side is expanded to the real matrix B~ with rows (Re t, -Im t, ...)
 // and (Im t, Re t, ...), so D = A B~^T holds (Re, Im) pairs.  FP32 accuracy
 // comes from splitting every operand (TF32 part and remainder, or BF16
-// pieces).  Chunks of 16 complex columns: the raw 128 x 16 complex tiles of G_i (or of G_i^H) arrive by 3-D TMA (one
-// tensor map over all factors, coordinate 2 = problem * nx + column), and the
-// matching 16 right-hand-side rows by a 1-D bulk copy, into a 4-stage ring
-// guarded by mbarriers.  The split into TF32 hi/lo operand tiles is
-// double-buffered so the tensor core works on chunk c while the threads
-// split chunk c+1.  CTA (row tile, part) handles the chunks
-// [part*cpp, (part+1)*cpp) and writes a partial 128 x k block;
-// sweep_couple_kernel adds the KS partials in a fixed order.  All waits are bounded (flag *err).
+// pieces).  Chunks of 16 complex columns: the raw 128 x 16 complex tiles of G_i
+// (or of G_i^H) arrive by 3-D TMA (one tensor map over all factors, coordinate 2
+// = problem * nx + column), and the matching 16 right-hand-side rows by a 1-D
+// bulk copy, into a ring of tc2_stages guarded by mbarriers.  The pieces of A go
+// straight to TMEM (a thread has one row of the tile and half of its columns),
+// those of B~ to shared memory, into one of tc2_bufs operand buffers.  Roles:
+// two groups of eight warps, each splitting every other chunk (splitting one is
+// a chain of latencies, about 1000 cycles, with 420 cycles of MMAs); one thread
+// that issues the MMAs of a chunk when its group has arrived on conv_bar; one
+// that refills a stage when its group has read it (free_bar).  The launches of a
+// solve follow each other by programmatic dependence: set-up and the first tiles
+// of G do not wait for the coupling before.
+// Bound: splitting and MMAs, which share shared memory (with neither, the same
+// loop takes the time of the tiles from memory).  Measured, 12 blocks of 768 x 768
+// by 32 columns: 17 us a launch, 23 with both operands staged in shared memory and
+// one barrier a chunk, 8 for G's bytes; the step with its coupling and gaps 20 us
+// instead of 27 before the dependent launches.  32 blocks: 34 instead of 59.
+// CTA (row tile, part) handles the chunks [part*cpp, (part+1)*cpp) and writes a
+// partial 128 x k block; sweep_couple_kernel adds the KS partials in a fixed
+// order.  All waits are bounded (flag *err).
 constexpr int TC_RT = 128;                                // rows of an item
 constexpr uint32_t TC_LBO = 128;
 constexpr uint32_t TC_WAIT_TRIES = 1u << 22;
 constexpr int TC2_KC = 16;                                // complex columns per chunk
-constexpr int TC2_STAGES = 4;
+constexpr int TC2_MAXSTAGES = 8;
+constexpr int TC2_MAXBUFS = 4;
+__host__ __device__ constexpr int tc2_stages(int kp) { return kp > 32 ? 6 : TC2_MAXSTAGES; }
 constexpr uint32_t TC2_TILE_BYTES = TC_RT * TC2_KC * 8;   // 16 KB raw tile
 
 __host__ __device__ constexpr uint32_t tc2_stage_bytes(int kp) {
   return (TC2_TILE_BYTES + (uint32_t)TC2_KC * kp * 8 + 1023u) & ~1023u;
 }
-// one operand piece: A is 128 rows, B~ is 2 kp rows, of 32 reals of K
+// one operand piece of a chunk (32 reals of K): A, TMEM columns of 128 rows; B~,
+// shared memory of 2 kp rows
 template <int SPLIT>
-__host__ __device__ constexpr uint32_t tc2_a_piece() { return (TC_RT / 8) * tc::sbo32<SPLIT>(); }
+__host__ __device__ constexpr uint32_t tc2_a_cols() { return 8u * tc::SplitCfg<SPLIT>::ESZ; }
 template <int SPLIT>
 __host__ __device__ constexpr uint32_t tc2_b_piece(int kp) {
   return (uint32_t)(2 * kp / 8) * tc::sbo32<SPLIT>();
 }
 template <int SPLIT>
 __host__ __device__ constexpr uint32_t tc2_buf_bytes(int kp) {
-  return tc::SplitCfg<SPLIT>::PIECES * (tc2_a_piece<SPLIT>() + tc2_b_piece<SPLIT>(kp));
+  return tc::SplitCfg<SPLIT>::PIECES * tc2_b_piece<SPLIT>(kp);
+}
+// TMEM columns: the accumulator, then the buffers of A pieces
+template <int SPLIT>
+__host__ __device__ constexpr uint32_t tc2_acc_cols(int kp) {
+  return ((uint32_t)tc::SplitCfg<SPLIT>::NPROD * 2 * kp + 31u) & ~31u;
+}
+template <int SPLIT>
+__host__ __device__ constexpr uint32_t tc2_tmem_cols(int kp, int bufs) {
+  return tc2_acc_cols<SPLIT>(kp) + bufs * tc::SplitCfg<SPLIT>::PIECES * tc2_a_cols<SPLIT>();
+}
+// operand buffers: two for each group of warps where TMEM has the room
+template <int SPLIT>
+__host__ __device__ constexpr int tc2_bufs(int kp) {
+  return tc2_tmem_cols<SPLIT>(kp, TC2_MAXBUFS) <= 512 ? TC2_MAXBUFS : 2;
 }
 template <int SPLIT>
 __host__ __device__ constexpr size_t tc2_smem_bytes(int kp) {
-  return 2 * (size_t)tc2_buf_bytes<SPLIT>(kp) + (size_t)TC2_STAGES * tc2_stage_bytes(kp);
+  return tc2_bufs<SPLIT>(kp) * (size_t)tc2_buf_bytes<SPLIT>(kp) +
+         (size_t)tc2_stages(kp) * tc2_stage_bytes(kp);
 }
 
 __device__ __forceinline__ bool tc_poll(uint64_t* bar, uint32_t parity, uint32_t tries) {
@@ -265,7 +297,8 @@ __device__ __forceinline__ bool tc_poll(uint64_t* bar, uint32_t parity, uint32_t
 }
 
 constexpr int TC2_CONV = 512;                 // converter threads (warps 0-15)
-constexpr int TC2_THREADS = TC2_CONV + 32;    // + control warp 16 (TMA producer, MMA issuer)
+constexpr int TC2_GROUP = TC2_CONV / 2;       // threads of a group
+constexpr int TC2_THREADS = TC2_CONV + 64;    // + warp 16, issues the MMAs, and 17, the copies
 
 template <bool TRANS, int SPLIT>
 __global__ void __launch_bounds__(TC2_THREADS, 1)
@@ -274,35 +307,36 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
                  size_t hstride, float2* __restrict__ part, int F, int Fa, const int* __restrict__ amap, int* err,
                  uint32_t tries, int stall) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint64_t full_bar[TC2_STAGES];
-  __shared__ uint64_t mma_bar[2];
+  __shared__ uint64_t full_bar[TC2_MAXSTAGES], free_bar[TC2_MAXSTAGES];  // raw stage in, read
+  __shared__ uint64_t conv_bar[TC2_MAXBUFS], mma_bar[TC2_MAXBUFS];     // buffer split, used
+  __shared__ uint64_t item_bar, acc_bar;                               // accumulator done, read
   __shared__ uint32_t tmem_base;
+  __shared__ int sfail;
   constexpr int PIECES = tc::SplitCfg<SPLIT>::PIECES;
   constexpr bool X6 = SPLIT == tc::SPLIT_BF16X6;
   const int N = 2 * kp;
-  const uint32_t a_piece = tc2_a_piece<SPLIT>();
+  constexpr uint32_t AC = tc2_a_cols<SPLIT>();
   const uint32_t bt_bytes = tc2_b_piece<SPLIT>(kp);
-  const uint32_t buf_bytes = tc2_buf_bytes<SPLIT>(kp);  // pieces of A and B of one chunk
+  const uint32_t buf_bytes = tc2_buf_bytes<SPLIT>(kp);  // pieces of B~ of one chunk
   unsigned char* ops = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  unsigned char* raw = ops + 2 * buf_bytes;  // TC2_STAGES stages, 1 KB aligned
+  const int stages = tc2_stages(kp), NB = tc2_bufs<SPLIT>(kp), nbs = NB == 4 ? 2 : 1;
+  unsigned char* raw = ops + NB * buf_bytes;  // stages, 1 KB aligned
   const uint32_t stage_bytes = tc2_stage_bytes(kp);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool ctrl = (tid == TC2_CONV);  // the one thread that feeds TMA and the tensor core
+  const bool ctrl = (tid == TC2_CONV);       // the one thread that feeds the tensor core
+  const bool prod = (tid == TC2_CONV + 32);  // the one that feeds TMA
   const int nch = (b + TC2_KC - 1) / TC2_KC;
   const int nitems = nrt * KS * Fa * step.nh;  // over the active problems of both halves
   const int my_items = nitems > (int)blockIdx.x
                            ? (nitems - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x
                            : 0;
   // x3 splits, per K step two MMAs: A_hi x [B_hi | B_lo] (N = 2 * 2k, both
-  // hi products in one pass over A_hi) and A_lo x B_hi.  Up to 32 columns
-  // (3N <= 256) two accumulator sets (even and odd K steps) keep consecutive
-  // MMAs independent and the epilogue adds six partial sums; with 64 columns
-  // one set of 3N = 384 columns takes every K step.  Set layout: [hi.hi |
-  // hi.lo | lo.hi], 3N columns.  BF16 x6 (up to 32 columns), per K step three
-  // MMAs into one set of 6N columns: p0 x [q0 | q1 | q2], p1 x [q0 | q1], p2 x q0.
-  const uint32_t ncols = X6 ? (6 * N <= 128 ? 128u : 6 * N <= 256 ? 256u : 512u)
-                            : ((N <= 32) ? 256u : 512u);
+  // hi products in one pass over A_hi) and A_lo x B_hi, into the 3N columns
+  // [hi.hi | hi.lo | lo.hi].  BF16 x6 (up to 32 columns), per K step three
+  // MMAs into 6N columns: p0 x [q0 | q1 | q2], p1 x [q0 | q1], p2 x q0.
+  constexpr int NPROD = tc::SplitCfg<SPLIT>::NPROD;  // partial sums the epilogue adds
+  const uint32_t ncols = tc2_tmem_cols<SPLIT>(kp, NB) <= 256 ? 256u : 512u;
   // work item t of this CTA -> (half, problem, row tile, contraction part)
   auto item = [&](int t, int& half, int& f, int& rt, int& ks) {
     const int it = (int)blockIdx.x + t * (int)gridDim.x;
@@ -316,40 +350,55 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
 
   if (warp == 0) tc::tmem_alloc(&tmem_base, ncols);
   if (tid == 0) {
-    for (int s = 0; s < TC2_STAGES; ++s) tc::mbar_init(&full_bar[s], 1);
-    tc::mbar_init(&mma_bar[0], 1);
-    tc::mbar_init(&mma_bar[1], 1);
+    for (int s = 0; s < stages; ++s) {
+      tc::mbar_init(&full_bar[s], 1);
+      tc::mbar_init(&free_bar[s], TC2_GROUP / 32);
+    }
+    for (int q = 0; q < NB; ++q) {
+      tc::mbar_init(&conv_bar[q], TC2_GROUP / 32);
+      tc::mbar_init(&mma_bar[q], 1);
+    }
+    tc::mbar_init(&item_bar, 1);
+    tc::mbar_init(&acc_bar, TC2_CONV / 32);
+    sfail = 0;
   }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_base;
-  const uint32_t set_cols = (uint32_t)(3 * N <= 128 ? 128 : 256);  // one accumulator set
-  const bool two_sets = !X6 && 3 * N <= 256;
-  const int nprod = (X6 || two_sets) ? 6 : 3;  // partial sums the epilogue adds
+  const uint32_t abuf = tmem + tc2_acc_cols<SPLIT>(kp);
 
-  // control thread: the stream of chunks of all this CTA's items.  With
+  // the stream of chunks of all this CTA's items.  With
   // stall set (a diagnostic of the bounded waits) the first CTA issues
   // nothing at all, so its first wait runs out with no copy or MMA in flight.
   const bool stalled = stall && blockIdx.x == 0;
-  int p_item = 0, p_lc = 0, issued = 0, p_h = 0, p_f = 0, p_rt = 0, p_ks = 0, p_len = 0;
-  int committed = 0;  // chunks whose MMAs have been committed (control thread)
-  if (ctrl && my_items > 0) {
+  int p_item = 0, p_lc = 0, issued = 0, p_h = 0, p_f = 0, p_rt = 0, p_ks = 0, p_len = 0, p_s = 0;
+  int committed = 0;  // chunks whose MMAs this thread has committed
+  if (prod && my_items > 0) {
     item(0, p_h, p_f, p_rt, p_ks);
     p_len = item_len(p_ks);
   }
-  auto issue_next = [&]() {
-    if (stalled || p_item >= my_items) return;
+  struct Rhs {
+    unsigned char* dst;
+    const float2* src;
+    uint32_t bytes;
+    uint64_t* bar;
+  };
+  // the tile of the next chunk; its right-hand side is left to the caller
+  auto issue_tile = [&]() {
+    Rhs w{nullptr, nullptr, 0, nullptr};
+    if (stalled || p_item >= my_items) return w;
     const int m0 = (p_ks * cpp + p_lc) * TC2_KC;
-    const int s = issued % TC2_STAGES;
+    const int s = p_s;
+    if (++p_s == stages) p_s = 0;
     const uint32_t rhs_bytes = (uint32_t)(min(TC2_KC, b - m0) * k * 8);
     unsigned char* st = raw + s * stage_bytes;
     const int zblk = p_f * nx + step_col(step, p_h, nx);
     tc::mbar_expect_tx(&full_bar[s], TC2_TILE_BYTES + rhs_bytes);
     if (!TRANS) tc::tma_load_3d(st, &tmap, 2 * m0, p_rt * TC_RT, zblk, &full_bar[s]);
     else tc::tma_load_3d(st, &tmap, 2 * p_rt * TC_RT, m0, zblk, &full_bar[s]);
-    tc::bulk_load(st + TC2_TILE_BYTES, rhs + p_h * hstride + p_f * rstride + (size_t)m0 * k,
-                  rhs_bytes, &full_bar[s]);
+    w = Rhs{st + TC2_TILE_BYTES, rhs + p_h * hstride + p_f * rstride + (size_t)m0 * k, rhs_bytes,
+            &full_bar[s]};
     ++issued;
     if (++p_lc == p_len) {
       p_lc = 0;
@@ -358,108 +407,186 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
         p_len = item_len(p_ks);
       }
     }
+    return w;
   };
-  if (ctrl)
-    for (int q = 0; q < TC2_STAGES; ++q) issue_next();
-  // operand descriptors of both buffers (piece 0 of A and the pieces of A
-  // and of the stacked B~); a K step (32 bytes) advances 256 bytes
+  auto issue_next = [&]() {
+    const Rhs w = issue_tile();
+    if (w.bytes) tc::bulk_load(w.dst, w.src, w.bytes, w.bar);
+  };
+  if (prod) {
+    Rhs first[TC2_MAXSTAGES];
+#pragma unroll
+    for (int q = 0; q < TC2_MAXSTAGES; ++q)
+      first[q] = q < stages ? issue_tile() : Rhs{nullptr, nullptr, 0, nullptr};
+    tc::grid_wait();
+    tc::grid_trigger();
+#pragma unroll
+    for (int q = 0; q < TC2_MAXSTAGES; ++q)
+      if (first[q].bytes) tc::bulk_load(first[q].dst, first[q].src, first[q].bytes, first[q].bar);
+  }
+  // operand addresses of both buffers; a K step (32 bytes) advances 8 TMEM
+  // columns of A and 256 bytes of B~
   constexpr uint32_t SBO = tc::sbo32<SPLIT>();
-  uint64_t dA[2][3], dB[2];
-  if (ctrl)
-    for (int q = 0; q < 2; ++q) {
-      const uint32_t a0 = tc::smem_u32(ops + q * buf_bytes);
-      for (int pc = 0; pc < PIECES; ++pc) dA[q][pc] = tc::smem_desc(a0 + pc * a_piece, TC_LBO, SBO);
-      dB[q] = tc::smem_desc(a0 + PIECES * a_piece, TC_LBO, SBO);
-    }
   auto idesc = [](int n) {
     return SPLIT == tc::SPLIT_TF32X3 ? tc::idesc_tf32(TC_RT, n) : tc::idesc_bf16(TC_RT, n);
   };
   const uint32_t id1 = idesc(N), id2 = idesc(2 * N), id3 = idesc(3 * N);
-  auto mma = [](uint32_t d, uint64_t a, uint64_t bb, uint32_t id, uint32_t acc) {
-    if (SPLIT == tc::SPLIT_TF32X3) tc::mma_tf32(d, a, bb, id, acc);
-    else tc::mma_bf16(d, a, bb, id, acc);
+  auto mma = [](uint32_t d, uint32_t a, uint64_t bb, uint32_t id, uint32_t acc) {
+    if (SPLIT == tc::SPLIT_TF32X3) tc::mma_tf32_ta(d, a, bb, id, acc);
+    else tc::mma_bf16_ta(d, a, bb, id, acc);
   };
-  int g = 0;  // chunks consumed so far (global over this CTA's items)
+  int g = 0;  // chunk of this CTA, over all its items
   bool failed = false;
-  for (int t = 0; t < my_items && !failed; ++t) {
-    int half, f, rt, ks;
-    item(t, half, f, rt, ks);
-    const int nl = item_len(ks);
-    for (int lc = 0; lc < nl; ++lc, ++g) {
-      const int s = g % TC2_STAGES, q = g & 1;
-      bool ok = true;
-      if (tid < TC2_CONV) {
-        ok = tc_poll(&full_bar[s], (g / TC2_STAGES) & 1, tries);
-        if (ok && g >= 2) ok = tc_poll(&mma_bar[q], ((g - 2) >> 1) & 1, tries);  // buffer q is free
-        tc::fence_after_sync();
-        unsigned char* ob = ops + q * buf_bytes;
-        unsigned char* ap[3] = {ob, ob + a_piece, ob + 2 * a_piece};
-        unsigned char* bp[3] = {ob + PIECES * a_piece, ob + PIECES * a_piece + bt_bytes,
-                                ob + PIECES * a_piece + 2 * bt_bytes};
-        const float* R = reinterpret_cast<const float*>(raw + s * stage_bytes);
-        const float2* Rt = reinterpret_cast<const float2*>(raw + s * stage_bytes + TC2_TILE_BYTES);
-        if (ok) {
-          // rotated item order keeps the 16-byte reads and writes conflict-free
-          for (int it = tid; it < TC_RT * 8; it += TC2_CONV) {
-            const int r = (it & 7) + 8 * (it >> 6);
-            const int p = (((it >> 3) & 7) + r) & 7;
-            float4 gv;
-            if (!TRANS) {
-              gv = *reinterpret_cast<const float4*>(R + r * 32 + 4 * p);
-            } else {
-              const float2 a = *reinterpret_cast<const float2*>(R + (2 * p) * 256 + 2 * r);
-              const float2 c = *reinterpret_cast<const float2*>(R + (2 * p + 1) * 256 + 2 * r);
-              gv = make_float4(a.x, -a.y, c.x, -c.y);
-            }
-            tc::store_split<SPLIT>(gv, ap, tc::kmajor_off32<SPLIT>(r, 4 * p));
-          }
-          // B~ rows 2j (x_r, -x_i) and 2j + 1 (x_i, x_r) of column j: consecutive
-          // threads take consecutive rows, so each 8-thread phase of the
-          // 16-byte stores covers the eight row slots of a core matrix
-          const int m0 = (ks * cpp + lc) * TC2_KC;
-          for (int it = tid; it < 2 * kp * 8; it += TC2_CONV) {
-            const int row = it % (2 * kp), p = it / (2 * kp), j = row >> 1;
-            const int ma = m0 + 2 * p, mb = ma + 1;
-            const float2 t0 = (j < k && ma < b) ? Rt[(2 * p) * k + j] : make_float2(0.f, 0.f);
-            const float2 t1 = (j < k && mb < b) ? Rt[(2 * p + 1) * k + j] : make_float2(0.f, 0.f);
-            const float4 v = (row & 1) ? make_float4(t0.y, t0.x, t1.y, t1.x)
-                                       : make_float4(t0.x, -t0.y, t1.x, -t1.y);
-            tc::store_split<SPLIT>(v, bp, tc::kmajor_off32<SPLIT>(row, 4 * p));
-          }
+  if (tid >= TC2_CONV + 32) {
+    // ---- refills
+    if (prod) {
+      int s = 0;
+      uint32_t sp = 0;
+      while (!stalled && p_item < my_items) {
+        if (!tc_poll(&free_bar[s], sp, tries)) {
+          failed = true;
+          break;
         }
-        tc::fence_async_smem();
+        issue_next();
+        if (++s == stages) {
+          s = 0;
+          sp ^= 1u;
+        }
       }
-      failed = __syncthreads_or(ok ? 0 : 1) != 0;
-      if (failed) break;
-      if (ctrl) {
+    }
+  } else if (tid >= TC2_CONV) {
+    // ---- MMAs of the split chunks
+    for (int t = 0; ctrl && t < my_items && !failed; ++t) {
+      int half, f, rt, ks;
+      item(t, half, f, rt, ks);
+      const int nl = item_len(ks);
+      if (t > 0 && !tc_poll(&acc_bar, (uint32_t)(t - 1) & 1u, tries)) {
+        failed = true;
+        break;
+      }
+      for (int lc = 0; lc < nl; ++lc, ++g) {
+        const int q = g & (NB - 1);
+        if (!tc_poll(&conv_bar[q], (uint32_t)(g >> nbs) & 1u, tries)) {
+          failed = true;
+          break;
+        }
         tc::fence_after_sync();
-        issue_next();  // stage s has been split: refill it
+        const uint64_t dB = tc::smem_desc(tc::smem_u32(ops + q * buf_bytes), TC_LBO, SBO);
+        const uint32_t aq = abuf + (uint32_t)(q * PIECES) * AC;
 #pragma unroll
         for (int kk = 0; kk < tc::ksteps32<SPLIT>(); ++kk) {
-          const uint64_t koff = (uint64_t)(kk * 2 * TC_LBO >> 4);
+          const uint64_t bk = dB + (uint64_t)(kk * 2 * TC_LBO >> 4);
+          const uint32_t ak = aq + (uint32_t)kk * 8;
+          const uint32_t acc = (lc > 0 || kk > 0) ? 1u : 0u;
           if (X6) {
-            const uint32_t acc = (lc > 0 || kk > 0) ? 1u : 0u;
-            mma(tmem, dA[q][0] + koff, dB[q] + koff, id3, acc);
-            mma(tmem + 3 * N, dA[q][1] + koff, dB[q] + koff, id2, acc);
-            mma(tmem + 5 * N, dA[q][2] + koff, dB[q] + koff, id1, acc);
+            mma(tmem, ak, bk, id3, acc);
+            mma(tmem + 3 * N, ak + AC, bk, id2, acc);
+            mma(tmem + 5 * N, ak + 2 * AC, bk, id1, acc);
           } else {
-            const uint32_t set = tmem + (two_sets ? (uint32_t)(kk & 1) * set_cols : 0u);
-            const uint32_t acc = (lc > 0 || kk > (two_sets ? 1 : 0)) ? 1u : 0u;
-            mma(set, dA[q][0] + koff, dB[q] + koff, id2, acc);
-            mma(set + 2 * N, dA[q][1] + koff, dB[q] + koff, id1, acc);
+            mma(tmem, ak, bk, id2, acc);
+            mma(tmem + 2 * N, ak + AC, bk, id1, acc);
           }
         }
         tc::mma_commit(&mma_bar[q]);
+        if (lc == nl - 1) tc::mma_commit(&item_bar);
         ++committed;
       }
     }
-    if (failed) break;
-    // item done: wait for its last MMAs, then move the accumulator to its slot
-    bool ok = (tid < TC2_CONV) ? tc_poll(&mma_bar[(g - 1) & 1], ((g - 1) >> 1) & 1, tries) : true;
-    failed = __syncthreads_or(ok ? 0 : 1) != 0;
-    if (failed) break;
-    tc::fence_after_sync();
-    if (tid < TC2_CONV) {
+  } else {
+    // ---- converters: group gi splits the chunks g with g % 2 == gi
+    const int gi = warp >> 3, gt = tid & (TC2_GROUP - 1);
+    const int r = (warp & 3) * 32 + lane, kh = (warp >> 2) & 1;  // row and K half of A
+    const int lkp = 31 - __clz(kp), j = gt & (kp - 1), p0 = gt >> lkp, pstep = TC2_GROUP >> lkp;
+    const int first = (j >> 2) & 1;
+    const uint32_t alane = abuf + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)kh * (AC / 2);
+    int s = gi;
+    uint32_t sp = 0;  // stage of the group's next chunk, and its parity
+    for (int t = 0; t < my_items && !failed; ++t) {
+      int half, f, rt, ks;
+      item(t, half, f, rt, ks);
+      const int nl = item_len(ks);
+      for (int lc = 0; lc < nl; ++lc, ++g) {
+        if ((g & 1) != gi) continue;
+        const int q = g & (NB - 1);
+        bool ok = tc_poll(&full_bar[s], sp, tries);
+        if (ok && g >= NB) ok = tc_poll(&mma_bar[q], (uint32_t)((g >> nbs) - 1) & 1u, tries);
+        ok = __all_sync(0xffffffffu, ok);  // the stores to TMEM are a warp's
+        if (!ok) {
+          failed = true;
+          break;
+        }
+        tc::fence_after_sync();
+        const float* R = reinterpret_cast<const float*>(raw + s * stage_bytes);
+        const float2* Rt = reinterpret_cast<const float2*>(raw + s * stage_bytes + TC2_TILE_BYTES);
+        // A: the lane's row, reals 16 kh ..; the 16-byte units of a swizzled row are
+        // exchanged by its number mod 8
+        float v[2][8];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if (!TRANS) {
+#pragma unroll
+            for (int h2 = 0; h2 < 2; ++h2) {
+              const float4 g4 = *reinterpret_cast<const float4*>(
+                  R + r * 32 + 4 * ((4 * kh + 2 * u + h2) ^ (r & 7)));
+              v[u][4 * h2] = g4.x;
+              v[u][4 * h2 + 1] = g4.y;
+              v[u][4 * h2 + 2] = g4.z;
+              v[u][4 * h2 + 3] = g4.w;
+            }
+          } else {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              const float2 c =
+                  *reinterpret_cast<const float2*>(R + (8 * kh + 4 * u + m) * 256 + 2 * r);
+              v[u][2 * m] = c.x;
+              v[u][2 * m + 1] = -c.y;
+            }
+          }
+        }
+        const int m0 = (ks * cpp + lc) * TC2_KC;
+        // B~ rows 2j (x_r, -x_i) and 2j + 1 (x_i, x_r) of column j: both by one
+        // thread, in the order that gives each 8-thread phase of the 16-byte
+        // stores the eight row slots of a core matrix
+        unsigned char* ob = ops + q * buf_bytes;
+        unsigned char* bp[3] = {ob, ob + bt_bytes, ob + 2 * bt_bytes};
+        for (int p = p0; p < 8; p += pstep) {
+          const int ma = m0 + 2 * p, mb = ma + 1;
+          const float2 t0 = (j < k && ma < b) ? Rt[(2 * p) * k + j] : make_float2(0.f, 0.f);
+          const float2 t1 = (j < k && mb < b) ? Rt[(2 * p + 1) * k + j] : make_float2(0.f, 0.f);
+#pragma unroll
+          for (int h2 = 0; h2 < 2; ++h2) {
+            const int odd = first ^ h2;
+            const float4 w = odd ? make_float4(t0.y, t0.x, t1.y, t1.x)
+                                 : make_float4(t0.x, -t0.y, t1.x, -t1.y);
+            tc::store_split<SPLIT>(w, bp, tc::kmajor_off32<SPLIT>(2 * j + odd, 4 * p));
+          }
+        }
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&free_bar[s]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          tc::tmem_store_split<SPLIT>(v[u], alane + (uint32_t)(q * PIECES) * AC + u * (AC / 4), AC);
+        tc::fence_async_smem();
+        tc::tmem_wait_st();
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&conv_bar[q]);
+        s += 2;
+        if (s >= stages) {
+          s -= stages;
+          sp ^= 1u;
+        }
+      }
+      if (failed) break;
+      // item done: wait for its last MMAs, then move the accumulator to its slot
+      // (item_bar: a group does not follow the other one's buffers phase by phase)
+      const bool ok = tc_poll(&item_bar, (uint32_t)t & 1u, tries);
+      if (!__all_sync(0xffffffffu, ok)) {
+        failed = true;
+        break;
+      }
+      tc::fence_after_sync();
+      tc::grid_wait();  // the partials are the coupling's before, until it is done
       // 16x256b fragments: warp w reads lanes 32 (w % 4) + 16 sb + [0, 16)
       // (sb = (w / 4) & 1) and float columns 32 hh + [0, 32) (hh = w / 8) of
       // each partial product; thread t holds rows t/4 and t/4 + 8 and complex
@@ -473,14 +600,8 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
             tmem + ((uint32_t)(lq * 32 + 16 * sb) << 16) + (uint32_t)(hh * 32);
         tc::tmem_ld_16x256b_x4(ta, v);
 #pragma unroll
-        for (int a = 1; a < 6; ++a) {  // the partial products
-          // x3: sets 0/1 x {hi.hi, hi.lo, lo.hi} (one set: a < 3); x6:
-          // p0.q0..2, p1.q0..1, p2.q0
-          if (a >= nprod) break;
-          const uint32_t col = (X6 || !two_sets)
-                                   ? (uint32_t)(a * N)
-                                   : (uint32_t)(a / 3) * set_cols + (uint32_t)(a % 3) * N;
-          tc::tmem_ld_16x256b_x4(ta + col, w);
+        for (int a = 1; a < NPROD; ++a) {  // the partial products
+          tc::tmem_ld_16x256b_x4(ta + (uint32_t)(a * N), w);
 #pragma unroll
           for (int tt = 0; tt < 16; ++tt) v[tt] += w[tt];
         }
@@ -496,23 +617,47 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
           }
         }
       }
-    }
-    tc::fence_before_sync();  // accumulator reads complete before the next item's MMAs
-  }
-  if (failed && ctrl) {
-    atomicExch(err, 1);
-    // drain the copies still in flight before the CTA's shared memory goes,
-    // and the last committed MMAs before their tensor memory is freed
-    for (int qq = g; qq < issued; ++qq)
-      tc::mbar_wait(&full_bar[qq % TC2_STAGES], (qq / TC2_STAGES) & 1, TC_WAIT_TRIES);
-    if (committed > 0) {
-      const int last = committed - 1;
-      tc::mbar_wait(&mma_bar[last & 1], (uint32_t)(last >> 1) & 1u, TC_WAIT_TRIES);
+      tc::fence_before_sync();  // accumulator reads complete before the next item's MMAs
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&acc_bar);
     }
   }
+  if (failed) sfail = 1;
   tc::fence_before_sync();
   __syncthreads();
+  if (sfail) {
+    // the copies in flight land before the CTA's shared memory goes, the MMAs
+    // committed complete before their tensor memory is freed (the uses before of
+    // these stages and buffers were waited for)
+    if (prod)
+      for (int qq = max(0, issued - stages); qq < issued; ++qq)
+        tc::mbar_wait(&full_bar[qq % stages], (uint32_t)(qq / stages) & 1u, TC_WAIT_TRIES);
+    if (ctrl) {
+      atomicExch(err, 1);
+      if (committed > 0) {
+        const int last = committed - 1;
+        tc::mbar_wait(&mma_bar[last & (NB - 1)], (uint32_t)(last >> nbs) & 1u, TC_WAIT_TRIES);
+      }
+    }
+    __syncthreads();
+  }
   if (warp == 0) tc::tmem_dealloc(tmem, ncols);
+}
+
+// Launch that may start before its predecessor in the stream has finished; the
+// kernel orders itself by grid_wait
+cudaLaunchConfig_t dependent_launch(dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                    cudaLaunchAttribute* at, bool dependent) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cfg;
 }
 
 // One launch of the TMA-fed tensor-core sweep step in the factors' operand
@@ -520,7 +665,7 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
 template <bool TRANS, int SPLIT, typename C>
 rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
                      const SweepStep& step, int nx, int nrt, int KS, int cpp, const C* rhs,
-                     size_t rstride, size_t hstride, rr_factors* fa, cudaStream_t st) {
+                     size_t rstride, size_t hstride, bool first, rr_factors* fa, cudaStream_t st) {
   const size_t smem = tc2_smem_bytes<SPLIT>(kp) + 1024;
   static size_t attr = 0;  // dynamic shared memory opted in so far
   if (smem > attr) {
@@ -528,10 +673,13 @@ rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr = smem;
   }
-  sweep_tc2_kernel<TRANS, SPLIT><<<grid_x, TC2_THREADS, smem, st>>>(
-      *tm, b, k, kp, step, nx, nrt, KS, cpp, reinterpret_cast<const float2*>(rhs), rstride, hstride,
-      reinterpret_cast<float2*>(fa->Pbuf), fa->F, active_count(fa), fa->amap, fa->flag + fa->F,
-      wait_tries(), take_stall());
+  // dependent launch, but for the first: its predecessor is not of this solve
+  cudaLaunchAttribute at[1];
+  const cudaLaunchConfig_t cfg = dependent_launch(dim3(grid_x), TC2_THREADS, smem, st, at, !first);
+  RR_CUDA(cudaLaunchKernelEx(
+      &cfg, sweep_tc2_kernel<TRANS, SPLIT>, *tm, b, k, kp, step, nx, nrt, KS, cpp, reinterpret_cast<const float2*>(rhs), rstride, hstride,
+      reinterpret_cast<float2*>(fa->Pbuf), fa->F, active_count(fa), (const int*)fa->amap, fa->flag + fa->F,
+      wait_tries(), take_stall()));
   return RR_OK;
 }
 
@@ -613,23 +761,26 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
     switch (fa->prec) {
       case RR_FP32_BF16X3:
         ls = launch_tc2<TRANS, tc::SPLIT_BF16X3>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
-                                                rstride, hstride, fa, st);
+                                                rstride, hstride, s == 0, fa, st);
         break;
       case RR_FP32_BF16X6:
         ls = launch_tc2<TRANS, tc::SPLIT_BF16X6>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
-                                                rstride, hstride, fa, st);
+                                                rstride, hstride, s == 0, fa, st);
         break;
       default:
         ls = launch_tc2<TRANS, tc::SPLIT_TF32X3>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
-                                                rstride, hstride, fa, st);
+                                                rstride, hstride, s == 0, fa, st);
     }
     if (ls != RR_OK) return ls;
     // (the middle's result starts both halves' outward sweeps)
     const int ch = step.phase == SW_MID ? 2 : step.nh;
-    sweep_couple_kernel<TRANS><<<dim3((d.ny + CPL_Y - 1) / CPL_Y, ch * Fa), couple_threads(d.q, k),
-                                 csmem, st>>>(view(d), step, F, Fa, k, KS,
-                                              reinterpret_cast<const float2*>(fa->Pbuf), in, x, zh,
-                                              tb, fa->amap);
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg =
+        dependent_launch(dim3((d.ny + CPL_Y - 1) / CPL_Y, ch * Fa), couple_threads(d.q, k), csmem, st,
+                         at, true);
+    RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_couple_kernel<TRANS>, view(d), step, F, Fa, k, KS,
+                               reinterpret_cast<const float2*>(fa->Pbuf), in, x, zh, tb,
+                               (const int*)fa->amap));
     prof_end(PROF_SWEEP, st);
     prof_count(1);
     RR_CUDA(cudaGetLastError());
@@ -641,13 +792,19 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
 
 // FP64 factors and every FP32 shape the split tensor-core sweep does not take
 // run the whole-sweep cluster kernels.  Where both serve a shape, the one with
-// the smaller modelled time: a column step of the tensor-core sweep is two
-// launches, measured at 10 us plus the factors' bytes at 2.6 TB/s.
+// the smaller modelled time: a pair of columns in the tensor-core sweep takes 6.5
+// us + 0.04 us a column of the right-hand side + the factors' bytes at 4.5 TB/s.
+// Measured, cluster and tensor-core form, us per pair in a solve with its
+// residual check: blocks of 192 rows, 16 columns, 4 / 8 / 16 problems 6.9, 9.2,
+// 14.9 and 10.3, 12.7, 16.8; 64 columns, 4 / 8 problems 14.8, 27.8 and 17.6,
+// 22.9; 384 rows, 16 columns, 2 / 4 / 8 / 16 problems 11.8, 20.4, 22.9, 43.9 and
+// 11.2, 14.3, 18.6, 30.0; 768 rows, 32 columns, 1 / 6 problems 70.9, 248 and
+// 18.0, 38.9.
 rr_status launch_solve_lo(rr_factors* fa, int k, int adjoint, const void* b, void* x, void* tmp) {
   if (fa->prec == RR_FP64) return launch_sweep_cl64(fa, k, adjoint, b, x, tmp);
   if (sweep_tc2_ok(fa, k)) {
     const OpDev& d = fa->op->d;
-    const double step = 10.0 + 16.0 * active_count(fa) * d.b * d.b / 2.6e6;
+    const double step = 6.5 + 0.04 * k + 16.0 * active_count(fa) * d.b * d.b / 4.5e6;
     if ((d.nx + 1.0) * step < sweep_cl32_us(fa, k, adjoint))
       return adjoint ? solve_tc2<true>(fa, k, reinterpret_cast<const float2*>(b),
                                        reinterpret_cast<float2*>(x), reinterpret_cast<float2*>(tmp))

@@ -54,14 +54,14 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "r"(ncols));
 }
 __device__ __forceinline__ void fence_before_sync() {
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::);
+  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
 }
 __device__ __forceinline__ void fence_after_sync() {
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
+  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
 // generic-proxy shared-memory writes -> visible to the tensor core (async proxy)
 __device__ __forceinline__ void fence_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;\n" ::);
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
 }
 
 // ---- MMA: D[tmem] (+)= A[smem] * B[smem]^T, issued by one thread -----------
@@ -71,6 +71,21 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+// the same with A in TMEM (lane = row; one 32-bit column per TF32 or two BF16)
+__device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
+                                            uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+__device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
+                                            uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
 // kind::f16 MMA (BF16 operands per the instruction descriptor), FP32 accumulate
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
@@ -84,7 +99,8 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
 __device__ __forceinline__ void mma_commit(uint64_t* mbar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-          smem_u32(mbar)));
+          smem_u32(mbar))
+      : "memory");
 }
 
 // ---- mbarrier -------------------------------------------------------------
@@ -98,7 +114,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* mbar, uint32_t parity) {
       "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
       " selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(ok)
-      : "r"(smem_u32(mbar)), "r"(parity));
+      : "r"(smem_u32(mbar)), "r"(parity)
+      : "memory");
   return ok != 0;
 }
 // Bounded wait: returns false after max_tries unsuccessful polls.
@@ -108,11 +125,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint3
   return false;
 }
 
+__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(mbar)) : "memory");
+}
 // arrive on an mbarrier and announce `bytes` of incoming TMA traffic
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* mbar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(mbar)),
                "r"(bytes)
                : "memory");
+}
+
+// ---- programmatic dependent launch ------------------------------------------
+// until the kernel this one depends on has finished and its writes are visible
+// (at once in an ordinary launch)
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+// the dependent kernel may start once every CTA has come here (or exited).  After
+// grid_wait only: then what ran before this kernel's predecessor is complete
+// when the dependent starts
+__device__ __forceinline__ void grid_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
 // ---- thread-block clusters: distributed shared memory ----------------------
@@ -177,6 +210,23 @@ __device__ __forceinline__ void bulk_load(void* smem_dst, const void* gsrc, uint
           "r"(smem_u32(smem_dst)),
       "l"(gsrc), "r"(bytes), "r"(smem_u32(mbar))
       : "memory");
+}
+
+// ---- registers -> TMEM: 8 (4) consecutive 32-bit columns of this warp's lanes --
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"r"(
+                   taddr),
+               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),
+               "r"(r[7])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&r)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};\n" ::"r"(taddr),
+               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() {
+  asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
 }
 
 // ---- TMEM -> registers: 32 lanes x 16 consecutive 32-bit columns ----------
@@ -319,6 +369,40 @@ __device__ __forceinline__ void store_split(float4 v, unsigned char* const* piec
       r[1] -= f0.y;
       r[2] -= f1.x;
       r[3] -= f1.y;
+    }
+  }
+}
+
+
+// Split 8 consecutive reals of this lane's row and store them in TMEM: per piece
+// (piece_cols apart) 8 columns (TF32) or 4 (BF16 pairs) from taddr.
+template <int SPLIT>
+__device__ __forceinline__ void tmem_store_split(float (&v)[8], uint32_t taddr,
+                                                 uint32_t piece_cols) {
+  if constexpr (SPLIT == SPLIT_TF32X3) {
+    uint32_t h[8], l[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float hi, lo;
+      split_tf32(v[i], hi, lo);
+      h[i] = __float_as_uint(hi);
+      l[i] = __float_as_uint(lo);
+    }
+    tmem_st8(taddr, h);
+    tmem_st8(taddr + piece_cols, l);
+  } else {
+#pragma unroll
+    for (int p = 0; p < SplitCfg<SPLIT>::PIECES; ++p) {
+      uint32_t u[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        __nv_bfloat162 pk = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+        u[i] = *reinterpret_cast<uint32_t*>(&pk);
+        const float2 f = __bfloat1622float2(pk);
+        v[2 * i] -= f.x;
+        v[2 * i + 1] -= f.y;
+      }
+      tmem_st4(taddr + p * piece_cols, u);
     }
   }
 }
