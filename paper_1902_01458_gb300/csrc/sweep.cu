@@ -272,23 +272,38 @@ template <int SPLIT>
 __host__ __device__ constexpr uint32_t tc2_buf_bytes(int kp) {
   return tc::SplitCfg<SPLIT>::PIECES * tc2_b_piece<SPLIT>(kp);
 }
-// TMEM columns: the accumulator, then the buffers of A pieces
+// TMEM: accumulator sets, then the buffers of A pieces.  A set sums the piece
+// products by order (x3: hi.hi | hi.lo + lo.hi; x6: three orders), N = 2 kp
+// columns each; consecutive K steps go to different sets, because the tensor
+// core's accumulation rounds towards zero (one set instead of two at 32 columns:
+// 35 % more error in a solve).  The small orders need no such care.
+template <int SPLIT>
+__host__ __device__ constexpr int tc2_orders() { return SPLIT == tc::SPLIT_BF16X6 ? 3 : 2; }
+template <int SPLIT>
+__host__ __device__ constexpr int tc2_sets(int kp) {
+  const int fit = 256 / (tc2_orders<SPLIT>() * 2 * kp);
+  return fit < 1 ? 1 : fit < tc::ksteps32<SPLIT>() ? fit : tc::ksteps32<SPLIT>();
+}
 template <int SPLIT>
 __host__ __device__ constexpr uint32_t tc2_acc_cols(int kp) {
-  return ((uint32_t)tc::SplitCfg<SPLIT>::NPROD * 2 * kp + 31u) & ~31u;
+  return (uint32_t)(tc2_sets<SPLIT>(kp) * tc2_orders<SPLIT>() * 2 * kp + 31) & ~31u;
 }
+// operand buffers: two for each group of warps where shared memory has the room
+__host__ __device__ constexpr int tc2_bufs(int kp) { return kp > 32 ? 2 : TC2_MAXBUFS; }
 template <int SPLIT>
-__host__ __device__ constexpr uint32_t tc2_tmem_cols(int kp, int bufs) {
-  return tc2_acc_cols<SPLIT>(kp) + bufs * tc::SplitCfg<SPLIT>::PIECES * tc2_a_cols<SPLIT>();
+__host__ __device__ constexpr uint32_t tc2_tmem_cols(int kp) {
+  return tc2_acc_cols<SPLIT>(kp) +
+         tc2_bufs(kp) * tc::SplitCfg<SPLIT>::PIECES * tc2_a_cols<SPLIT>();
 }
-// operand buffers: two for each group of warps where TMEM has the room
-template <int SPLIT>
-__host__ __device__ constexpr int tc2_bufs(int kp) {
-  return tc2_tmem_cols<SPLIT>(kp, TC2_MAXBUFS) <= 512 ? TC2_MAXBUFS : 2;
-}
+static_assert(tc2_tmem_cols<tc::SPLIT_TF32X3>(32) <= 512 &&
+                  tc2_tmem_cols<tc::SPLIT_TF32X3>(64) <= 512 &&
+                  tc2_tmem_cols<tc::SPLIT_TF32X3>(16) <= 512 &&
+                  tc2_tmem_cols<tc::SPLIT_BF16X3>(64) <= 512 &&
+                  tc2_tmem_cols<tc::SPLIT_BF16X6>(32) <= 512,
+              "tensor memory of a CTA");
 template <int SPLIT>
 __host__ __device__ constexpr size_t tc2_smem_bytes(int kp) {
-  return tc2_bufs<SPLIT>(kp) * (size_t)tc2_buf_bytes<SPLIT>(kp) +
+  return tc2_bufs(kp) * (size_t)tc2_buf_bytes<SPLIT>(kp) +
          (size_t)tc2_stages(kp) * tc2_stage_bytes(kp);
 }
 
@@ -320,7 +335,7 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
   const uint32_t buf_bytes = tc2_buf_bytes<SPLIT>(kp);  // pieces of B~ of one chunk
   unsigned char* ops = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int stages = tc2_stages(kp), NB = tc2_bufs<SPLIT>(kp), nbs = NB == 4 ? 2 : 1;
+  const int stages = tc2_stages(kp), NB = tc2_bufs(kp), nbs = NB == 4 ? 2 : 1;
   unsigned char* raw = ops + NB * buf_bytes;  // stages, 1 KB aligned
   const uint32_t stage_bytes = tc2_stage_bytes(kp);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -331,12 +346,13 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
   const int my_items = nitems > (int)blockIdx.x
                            ? (nitems - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x
                            : 0;
-  // x3 splits, per K step two MMAs: A_hi x [B_hi | B_lo] (N = 2 * 2k, both
-  // hi products in one pass over A_hi) and A_lo x B_hi, into the 3N columns
-  // [hi.hi | hi.lo | lo.hi].  BF16 x6 (up to 32 columns), per K step three
-  // MMAs into 6N columns: p0 x [q0 | q1 | q2], p1 x [q0 | q1], p2 x q0.
-  constexpr int NPROD = tc::SplitCfg<SPLIT>::NPROD;  // partial sums the epilogue adds
-  const uint32_t ncols = tc2_tmem_cols<SPLIT>(kp, NB) <= 256 ? 256u : 512u;
+  // x3 splits, per K step two MMAs: A_hi x [B_hi | B_lo] into [hi.hi | cross] and
+  // A_lo x B_hi into cross.  BF16 x6 (up to 32 columns), three: p0 x [q0 | q1 | q2],
+  // p1 x [q0 | q1], p2 x q0.
+  constexpr int ORDERS = tc2_orders<SPLIT>();
+  const int SETS = tc2_sets<SPLIT>(kp);
+  const uint32_t set_cols = (uint32_t)(ORDERS * N);
+  const uint32_t ncols = tc2_tmem_cols<SPLIT>(kp) <= 256 ? 256u : 512u;
   // work item t of this CTA -> (half, problem, row tile, contraction part)
   auto item = [&](int t, int& half, int& f, int& rt, int& ks) {
     const int it = (int)blockIdx.x + t * (int)gridDim.x;
@@ -477,14 +493,14 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
         for (int kk = 0; kk < tc::ksteps32<SPLIT>(); ++kk) {
           const uint64_t bk = dB + (uint64_t)(kk * 2 * TC_LBO >> 4);
           const uint32_t ak = aq + (uint32_t)kk * 8;
-          const uint32_t acc = (lc > 0 || kk > 0) ? 1u : 0u;
+          const uint32_t set = tmem + (uint32_t)(kk & (SETS - 1)) * set_cols;
+          const uint32_t acc = (lc > 0 || kk >= SETS) ? 1u : 0u;
+          mma(set, ak, bk, X6 ? id3 : id2, acc);
           if (X6) {
-            mma(tmem, ak, bk, id3, acc);
-            mma(tmem + 3 * N, ak + AC, bk, id2, acc);
-            mma(tmem + 5 * N, ak + 2 * AC, bk, id1, acc);
+            mma(set + N, ak + AC, bk, id2, 1u);
+            mma(set + 2 * N, ak + 2 * AC, bk, id1, 1u);
           } else {
-            mma(tmem, ak, bk, id2, acc);
-            mma(tmem + 2 * N, ak + AC, bk, id1, acc);
+            mma(set + N, ak + AC, bk, id1, 1u);
           }
         }
         tc::mma_commit(&mma_bar[q]);
@@ -600,7 +616,7 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
             tmem + ((uint32_t)(lq * 32 + 16 * sb) << 16) + (uint32_t)(hh * 32);
         tc::tmem_ld_16x256b_x4(ta, v);
 #pragma unroll
-        for (int a = 1; a < NPROD; ++a) {  // the partial products
+        for (int a = 1; a < SETS * ORDERS; ++a) {  // the partial sums
           tc::tmem_ld_16x256b_x4(ta + (uint32_t)(a * N), w);
 #pragma unroll
           for (int tt = 0; tt < 16; ++tt) v[tt] += w[tt];
