@@ -40,8 +40,7 @@ BF16_PEAK_TFLOPS = 1900.0   # fallback burst figure
 # capture of the current kernels (profiles/), or None when the kernel changed
 # since the counters were taken.
 UPDATE_TRAFFIC = None
-# sweep_tc2_kernel, one launch over all 64 frequencies (profiles/sweep_tc2_ns2d-8x256-k32_batch64.md)
-SWEEP_TRAFFIC = 310.0e6 + 18.3e6
+SWEEP_TRAFFIC = None
 PRECISIONS = ("fp32", "fp32_bf16x3", "fp32_bf16x6")
 # tensor-core MMAs per FP32-level product of each operand split
 SPLIT_MMAS = {"fp32": ("tf32", 3), "fp32_bf16x3": ("bf16", 3), "fp32_bf16x6": ("bf16", 6)}
@@ -194,7 +193,7 @@ def batch_for(step, rank, world, F, omegas, seed0):
 def wide_gemm_work(b):
     """Algorithmic work of the updates of one Schur-block inverse (block b) in
     the wide factorisation.  Per 128-column slab: the rank-16 updates of the
-    slab's other columns (inner: FP32 CUDA cores) and the rank-128 update of
+    slab's other columns (inner: FP32 CUDA cores, inside the slab kernel) and the rank-128 update of
     the columns outside it (outer: tensor cores).  Returns
     {"inner": (flops, bytes), "outer": (flops, bytes)} -- 8 real flops per
     complex multiply-add; bytes = one read and one write of every updated
@@ -431,19 +430,18 @@ def run_ours(args):
     ms_sw, n_sw = cls_read["sweep"]
     if n_sw > 0 and ms_sw > 0:
         # every block solve of one problem streams G_i of each streamwise
-        # column once forward and once backward (2 nx - 1 column steps) plus
+        # column once inward and once outward (the middle one once) plus
         # its right-hand side, result and the K-split partial blocks
         tot_s = ms_sw / 1e3
         work = solves_timed * (2 * nx - 1) * (b * b * 8 + 3 * b * k * 8)
         ach = work / tot_s / 1e9
         rooflines["sweep"] = {
-            "kernel": "sweep_tc2_kernel + sweep_combine_kernel (one streamwise column step "
+            "kernel": "sweep_tc2_kernel + sweep_couple_kernel (one pair of streamwise columns "
                       "of the active frequencies, tcgen05)",
             "bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
             "traffic": SWEEP_TRAFFIC, "peak_source": src,
-            "traffic_note": "ncu DRAM read + write of one launch over all F frequencies "
-                            "(the refinement's launches cover only the active ones)",
-            "algorithmic_full_launch": F * (b * b * 8 + 3 * b * k * 8),
+            "traffic_note": "DRAM counters of the current kernel not taken",
+            "algorithmic_full_launch": 2 * F * (b * b * 8 + 3 * b * k * 8),
             "algorithmic_per_launch": work / n_sw, "launches": n_sw,
             "avg_launch_us": tot_s / n_sw * 1e6,
             "algorithmic_note": "per block solve of one problem: (2 nx - 1) x (b^2 x 8 B of "

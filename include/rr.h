@@ -54,11 +54,11 @@ typedef enum {
 
 /* Arithmetic of the block factorisation and the block sweeps.  FP64 runs
  * everything in complex double.  FP32 stores the factors in complex float,
- * runs the factorisation's rank-128 updates and the sweep products on the
- * tensor cores (tcgen05 kind::tf32 with each operand split into a TF32 part
+ * runs the factorisation's rank-128 updates and the sweep products of large
+ * blocks and batches on the tensor cores (tcgen05 kind::tf32 with each operand split into a TF32 part
  * and its remainder, hi.hi + hi.lo + lo.hi: FP32-level products, FP32
- * accumulation; the pivoted panels and the rank-16 updates inside a
- * 128-column slab run in FP32 on the CUDA cores) and wins accuracy back by
+ * accumulation; the pivoted 128-column slabs and the sweeps of small blocks
+ * run in FP32 on the CUDA cores) and wins accuracy back by
  * iterative refinement against an FP64 residual.
  * FP32_BF16X3 and FP32_BF16X6 are the same with the operands split into
  * BF16 pieces on tcgen05 kind::f16: two pieces and three products (about 16
@@ -215,10 +215,10 @@ rr_status rr_destroy_factors(rr_factors* f);
  * iterative refinement x <- x + solve(b - A x) with the residual in FP64
  * (FP64 factors too, when refine_tol > 0): it stops once every column's
  * ||b - A x|| / ||b|| <= refine_tol or a correction removes less than a
- * tenth of the residual.  With FP32 factors on the tensor-core sweep (even
- * k <= 32, even block >= 128) each problem is refined on its own and leaves
- * the set of corrected problems when it stops.  info may be NULL.  Errors:
- * RR_ERR_ARG, RR_ERR_NOCONV (x still written), RR_ERR_CUDA. */
+ * tenth of the residual.  With FP32 factors on the tensor cores, an even block
+ * of at least 128 and an even k of at most 64 (32: FP32_BF16X6), each problem
+ * is refined on its own and leaves the set of corrected problems when it
+ * stops.  info may be NULL.  Errors: RR_ERR_ARG, RR_ERR_NOCONV (x still written), RR_ERR_CUDA. */
 rr_status rr_solve(rr_factors* f, int k, int adjoint, const void* b, void* x,
                    double refine_tol, int max_refine, rr_info* info);
 
@@ -429,7 +429,7 @@ rr_status rr_batch_destroy(rr_batch* b);
  * launching stream.  Classes: 0 Schur update, 1 pivoted panel, 2 row block,
  * 3 trailing update (tensor cores), 4 finalize (inverse + X), 5 block sweep
  * step, 6 FP64 residual, 7 Gram, 8 right multiply, 9 small k x k kernels,
- * 10 inner slab update of the wide factorisation (CUDA cores).
+ * 10 unused (the slab's inner update is part of the pivoted panel, class 1).
  * rr_profile_read(cls): summed event time (ms) and launches of a class. */
 long long rr_launch_count(void);
 rr_status rr_profile_start(unsigned mask);
@@ -441,8 +441,8 @@ rr_status rr_profile_read(int cls, double* ms, long long* launches);
  * 2^22) before the kernel records a timeout, drains what it has in flight,
  * frees its tensor memory and returns; the call that launched it then
  * returns RR_ERR_TIMEOUT.  stall_launches > 0 makes that many of the next
- * tensor-core sweep launches stall on purpose: the control thread of their
- * first CTA issues no copy and no MMA, so that CTA's first wait runs out with
+ * tensor-core sweep launches stall on purpose: the first CTA of
+ * each issues no copy and no MMA, so that CTA's first wait runs out with
  * nothing in flight.  Process-wide, not thread-safe; for tests only. */
 rr_status rr_debug_waits(unsigned tries, int stall_launches);
 
