@@ -143,7 +143,7 @@ struct rr_factors {
   void* X;           // [2F][b][b] X_i = G_i C_i (G_i A_i) of the current columns (transient)
   void* M;           // [2F][b][b] work matrices
   void* Bbuf;        // [2F][16][b] saved pivot rows of the current panel
-  void* Tbuf;        // [2][F][b][64] staging blocks of one sweep step
+  void* Tbuf;        // [2][F][b][64] right-hand sides (or edge blocks) of both halves
   void* Pbuf;        // [4][F][b][64] partial products of the split tensor-core sweep
   alignas(64) unsigned char tmap[2][128];  // TMA maps: G tiles, G^H tiles (FP32)
   int tma_ok;        // 1 if the maps of G were encoded
