@@ -429,13 +429,15 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
       asm volatile("bar.sync 2, %0;\n" ::"r"(nuw * 32) : "memory");
       const uint32_t mb = tc::smem_u32(&mbarB);
       for (int j = uw; j < NB; j += nuw) {
-        int lr = j < nbk ? -1 : -2;
+        // (a row beyond a ragged panel's columns waits for the last pivot: with one
+        // buffer the panel warps read B, the panel before's, until their first step)
+        int lr = -1;
         for (uint32_t t = 0; lr == -1 && t < g.tries; ++t) {
-          lr = own[p & 1][j];
+          lr = own[p & 1][min(j, nbk - 1)];
           if (lr == -1) __nanosleep(400);
         }
         if (lr == -1) ok = false;
-        if (lr < 0) {
+        if (lr < 0 || j >= nbk) {
           // (rows beyond a ragged panel's columns multiply zeros; keep them finite)
           if (j >= nbk)
             for (int c = lane; c < GW_W; c += 32) Bp[j * GW_W + c] = make_float2(0.f, 0.f);
