@@ -57,6 +57,8 @@ __host__ __device__ __forceinline__ int step_col(const SweepStep& s, int half, i
 //   t = h + L_{i,i'}^T o (adjoint outward)
 // for the next column i'.  z goes to zh in the inward sweep, so the outward one's
 // results (x) never overwrite a value a neighbouring tile still needs.
+// (part is not __restrict__: the product writes it while this kernel already runs,
+// until grid_wait, so no load of it may go through the read-only path or move up.)
 // Bound: L2 latency (the partials were just written), so the coefficients and
 // inputs of the coupling are requested before the partials are summed, and a
 // thread has one element (two columns) of each phase at k <= 32.
@@ -68,8 +70,7 @@ inline int couple_threads(int q, int k) {
 template <bool TRANS>
 __global__ void __launch_bounds__(CPL_MAXTHR)
 sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
-                    const float2* __restrict__ part, const float2* __restrict__ in, float2* x,
-                    float2* zh, float2* __restrict__ tbuf, const int* __restrict__ amap) {
+                    const float2* part, const float2* __restrict__ in, float2* x, float2* zh, float2* __restrict__ tbuf, const int* __restrict__ amap) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* o = reinterpret_cast<float4*>(smem_raw);  // [(CPL_Y + 2) q][k / 2]
   const int b = op.b, q = op.q, ny = op.ny, nx = op.nx, P = k >> 1;
