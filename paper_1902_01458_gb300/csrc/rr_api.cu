@@ -182,6 +182,20 @@ void info_reset(rr_info* info) {
   info->problem_solves = 0;
 }
 
+// RR_ERR_TIMEOUT when a wait of the sweeps launched so far gave up (synchronises).
+// Reported once: the flag is cleared so the factors serve later solves.
+rr_status sweep_status(rr_factors* fa) {
+  int tc_err = 0;
+  cudaStream_t st = fa->stream;
+  RR_CUDA(cudaMemcpyAsync(&tc_err, fa->flag + fa->F, sizeof(int), cudaMemcpyDeviceToHost, st));
+  RR_CUDA(cudaStreamSynchronize(st));
+  if (!tc_err) return RR_OK;
+  RR_CUDA(cudaMemsetAsync(fa->flag + fa->F, 0, sizeof(int), st));
+  RR_CUDA(cudaStreamSynchronize(st));
+  g_err = "a sweep kernel timed out in a bounded wait";
+  return RR_ERR_TIMEOUT;
+}
+
 // x = A^{-1} b (or A^{-H} b) in FP64 [F][N][k], b != x, with FP64 iterative
 // refinement: x <- x + solve(b - A x) until every column's relative residual
 // is at most tol (tol <= 0: one solve, residual reported only when info).
@@ -203,7 +217,7 @@ rr_status solve_refined(rr_factors* fa, int k, int adjoint, const double2* b, do
   }
   if (info) info->problem_solves += F;
   const bool check = lo || info != nullptr || tol > 0.0 || fa->sched_mode != SCHED_EAGER;
-  if (!check) return RR_OK;
+  if (!check) return sweep_status(fa);
   if ((s = launch_colnorm2(F, d.n, k, b, w.dpart, w.nblk_col, w.bn, st)) != RR_OK) return s;
   if (fa->sched_mode == SCHED_REPLAY) {
     // the recorded number of corrections, no host reads; the final residual
@@ -271,16 +285,7 @@ rr_status solve_refined(rr_factors* fa, int k, int adjoint, const double2* b, do
     if ((s = launch_colnorm2(nres, d.n, k, w.R64, w.dpart, w.nblk_col, w.rn, st, amap)) != RR_OK)
       return s;
     RR_CUDA(cudaMemcpyAsync(rn.data(), w.rn, rn.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-    int tc_err = 0;
-    RR_CUDA(cudaMemcpyAsync(&tc_err, fa->flag + F, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RR_CUDA(cudaStreamSynchronize(st));
-    if (tc_err) {
-      // reported once: the flag is cleared so the factors serve later solves
-      RR_CUDA(cudaMemsetAsync(fa->flag + F, 0, sizeof(int), st));
-      RR_CUDA(cudaStreamSynchronize(st));
-      g_err = "a tensor-core sweep kernel timed out in a bounded wait";
-      return RR_ERR_TIMEOUT;
-    }
+    if ((s = sweep_status(fa)) != RR_OK) return s;
     rel = 0.0;
     for (int f = 0; f < F; ++f) {
       if (!subset || active[f]) {

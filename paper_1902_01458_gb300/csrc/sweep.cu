@@ -70,7 +70,8 @@ inline int couple_threads(int q, int k) {
 template <bool TRANS>
 __global__ void __launch_bounds__(CPL_MAXTHR)
 sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
-                    const float2* part, const float2* __restrict__ in, float2* x, float2* zh, float2* __restrict__ tbuf, const int* __restrict__ amap) {
+                    const float2* part, const float2* __restrict__ in, float2* x, float2* zh,
+                    float2* __restrict__ tbuf, const int* __restrict__ amap) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* o = reinterpret_cast<float4*>(smem_raw);  // [(CPL_Y + 2) q][k / 2]
   const int b = op.b, q = op.q, ny = op.ny, nx = op.nx, P = k >> 1;
