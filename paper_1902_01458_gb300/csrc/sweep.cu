@@ -57,6 +57,7 @@ __host__ __device__ __forceinline__ int step_col(const SweepStep& s, int half, i
 //   t = h + L_{i,i'}^T o (adjoint outward)
 // for the next column i'.  z goes to zh in the inward sweep, so the outward one's
 // results (x) never overwrite a value a neighbouring tile still needs.
+// One grid dimension: two halves of 65,535 problems exceed the second one's limit.
 // (part is not __restrict__: the product writes it while this kernel already runs,
 // until grid_wait, so no load of it may go through the read-only path or move up.)
 // Bound: L2 latency (the partials were just written), so the coefficients and
@@ -75,8 +76,9 @@ sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* o = reinterpret_cast<float4*>(smem_raw);  // [(CPL_Y + 2) q][k / 2]
   const int b = op.b, q = op.q, ny = op.ny, nx = op.nx, P = k >> 1;
-  const int half = blockIdx.y / Fa, f = active_problem(amap, blockIdx.y - half * Fa);
-  const int y0 = blockIdx.x * CPL_Y, npt = min(CPL_Y, ny - y0);
+  const int nty = (ny + CPL_Y - 1) / CPL_Y, p = blockIdx.x / nty;
+  const int half = p / Fa, f = active_problem(amap, p - half * Fa);
+  const int y0 = (blockIdx.x - p * nty) * CPL_Y, npt = min(CPL_Y, ny - y0);
   const size_t NK = (size_t)op.n * k, total = (size_t)s.nh * F * b * k;
   const int i = step_col(s, half, nx);
   const bool inw = s.phase == SW_IN, outw = s.phase == SW_OUT;
@@ -794,8 +796,8 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
     const int ch = step.phase == SW_MID ? 2 : step.nh;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg =
-        dependent_launch(dim3((d.ny + CPL_Y - 1) / CPL_Y, ch * Fa), couple_threads(d.q, k), csmem, st,
-                         at, true);
+        dependent_launch(dim3((d.ny + CPL_Y - 1) / CPL_Y * ch * Fa), couple_threads(d.q, k), csmem,
+                         st, at, true);
     RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_couple_kernel<TRANS>, view(d), step, F, Fa, k, KS,
                                reinterpret_cast<const float2*>(fa->Pbuf), in, x, zh, tb,
                                (const int*)fa->amap));
