@@ -241,12 +241,17 @@ __global__ void __launch_bounds__(GP_MAXW * 32) gjp_panel_kernel(PanelArgs g, C_
   // barriers initialised, and every CTA's reads of M done before any CTA writes
   tc::cluster_sync();
   if (g.kp0 >= 0 && live) {
+    C u[CPL];  // summed on its own: one rounding against x (gjp_update_kernel)
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) u[c] = czero<C>();
 #pragma unroll 4
     for (int j = 0; j < NB; ++j) {
       const C a = As[prow * (NB + 1) + j];
 #pragma unroll
-      for (int c = 0; c < CPL; ++c) x[c] = cfma(a, Bp[j * NB + cg + c], x[c]);
+      for (int c = 0; c < CPL; ++c) u[c] = cfma(a, Bp[j * NB + cg + c], u[c]);
     }
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) x[c] = cadd(x[c], u[c]);
   }
   bool elig = live && rp < 0;
   int mypiv = -1;
@@ -367,6 +372,9 @@ __global__ void gjp_gather_kernel(int b, int k0, int nbk, int nh, const C_t<T>* 
   Ball[((size_t)f * GP_NB + j) * b + m] = v;
 }
 
+// (Summing onto the matrix entries instead rounds them sixteen times a panel: the
+// unrefined residual of a 384-row FP64 adjoint solve was 6.3e-14 instead of 3.0e-14,
+// of a 768-row FP32 one 8.6e-5 instead of 2.3e-5, at the same speed.)
 // The rank-16 update on TR x TR tiles (16 x 16 threads) of the columns outside
 // [k0, k0 + nbk) and [n0, n1).  FP64 is bound by its pipe, so small tiles fill
 // the SMs; FP32 by shared memory, so a thread holds 4 x 4 outputs.
@@ -389,7 +397,9 @@ gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, int nh, C_t<T>* __rest
   auto col_live = [&](int c) {
     return c < b && !(c >= k0 && c < k0 + nbk) && !(c >= n0 && c < n1);
   };
-  C acc[PT][PT];
+  // the old values are requested first and added last: the sixteen products are
+  // summed on their own, one rounding a panel against the matrix entry
+  C acc[PT][PT], old[PT][PT];
 #pragma unroll
   for (int a = 0; a < PT; ++a) {
     const int r = r0 + ty + 16 * a;
@@ -398,7 +408,8 @@ gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, int nh, C_t<T>* __rest
 #pragma unroll
     for (int d = 0; d < PT; ++d) {
       const int c = c0 + tx + 16 * d;
-      acc[a][d] = keep && col_live(c) ? M[(size_t)r * b + c] : czero<C>();
+      acc[a][d] = czero<C>();
+      old[a][d] = keep && col_live(c) ? M[(size_t)r * b + c] : czero<C>();
     }
   }
   for (int e = tid; e < TR * NB; e += 256) {
@@ -429,7 +440,7 @@ gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, int nh, C_t<T>* __rest
 #pragma unroll
     for (int d = 0; d < PT; ++d) {
       const int c = c0 + tx + 16 * d;
-      if (col_live(c)) M[(size_t)r * b + c] = acc[a][d];
+      if (col_live(c)) M[(size_t)r * b + c] = cadd(old[a][d], acc[a][d]);
     }
   }
 }
