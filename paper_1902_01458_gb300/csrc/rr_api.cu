@@ -196,6 +196,13 @@ rr_status sweep_status(rr_factors* fa) {
   return RR_ERR_TIMEOUT;
 }
 
+// Solves whose problems are refined one by one (rr_solve in rr.h)
+bool per_problem_refinement(const rr_factors* fa, int k) {
+  const int b = fa->op->d.b;
+  return tc_prec(fa->prec) && b >= 128 && b % 2 == 0 && k % 2 == 0 &&
+         k <= (fa->prec == RR_FP32_BF16X6 ? 32 : 64);
+}
+
 // x = A^{-1} b (or A^{-H} b) in FP64 [F][N][k], b != x, with FP64 iterative
 // refinement: x <- x + solve(b - A x) until every column's relative residual
 // is at most tol (tol <= 0: one solve, residual reported only when info).
@@ -255,13 +262,12 @@ rr_status solve_refined(rr_factors* fa, int k, int adjoint, const double2* b, do
   if (fa->sched_mode == SCHED_RECORD) fa->chk_need += 2 * (size_t)F * k * sizeof(double);
   std::vector<double> bn((size_t)F * k), rn((size_t)F * k);
   RR_CUDA(cudaMemcpyAsync(bn.data(), w.bn, bn.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-  // Eager solves on the split tensor-core sweep refine each problem on its
-  // own: a problem leaves the active set once its residual meets tol or a
-  // correction no longer halves it, and the corrections and residuals that
-  // follow run on the active problems only.  Elsewhere (and when recording a
-  // schedule) all problems take every correction until the largest residual
-  // meets tol or stops halving.
-  const bool per_problem = fa->sched_mode == SCHED_EAGER && lo && sweep_tc2_ok(fa, k);
+  // Eager solves of these shapes refine each problem on its own: a problem leaves
+  // the active set once its residual meets tol or a correction removes less than a
+  // tenth of it, and the corrections and residuals that follow run on the active
+  // problems only.  Elsewhere (and when recording a schedule) all problems take
+  // every correction until the largest residual meets tol or stops falling.
+  const bool per_problem = fa->sched_mode == SCHED_EAGER && per_problem_refinement(fa, k);
   struct MapReset {  // the solve path never keeps a subset past this call
     rr_factors* fa;
     ~MapReset() {

@@ -259,8 +259,8 @@ rr_status launch_sweep_cl32(rr_factors* f, int k, int adjoint, const void* b, vo
 rr_status launch_sweep_cl64(rr_factors* f, int k, int adjoint, const void* b, void* x, void* tmp);
 double sweep_cl32_us(const rr_factors* f, int k, int adjoint);
 double sweep_cl64_us(const rr_factors* f, int k, int adjoint);
-// true when the solves of k columns take the split tensor-core sweep, the
-// one path that can run on a subset of the problems (rr_factors::amap)
+// true when solves of k columns may take the split tensor-core sweep (both forms
+// run on a subset of the problems, rr_factors::amap)
 bool sweep_tc2_ok(const rr_factors* f, int k);
 
 // dense.cu

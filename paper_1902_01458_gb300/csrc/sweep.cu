@@ -63,19 +63,41 @@ __host__ __device__ __forceinline__ int step_col(const SweepStep& s, int half, i
 // Bound: L2 latency (the partials were just written), so the coefficients and
 // inputs of the coupling are requested before the partials are summed, and a
 // thread has one element (two columns) of each phase at k <= 32.
+// V is a unit of a row: two columns (float4) where k is even, else one (float2).
+// (Odd k on the cluster form instead, 768 rows, 31 columns, 16 problems, 16 columns of
+// the grid: 10.2 ms forward and 5.8 adjoint; here 1.9 both.)
 constexpr int CPL_Y = 4, CPL_MAXTHR = 512;
-inline int couple_threads(int q, int k) {
-  return std::min(CPL_MAXTHR, ((CPL_Y + 2) * q * (k / 2) + 31) & ~31);
+inline int couple_threads(int q, int units) {
+  return std::min(CPL_MAXTHR, ((CPL_Y + 2) * q * units + 31) & ~31);
+}
+__device__ __forceinline__ float4 vadd(float4 a, float4 b) {
+  return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) {
+  return make_float2(a.x + b.x, a.y + b.y);
+}
+__device__ __forceinline__ float4 vsub(float4 a, float4 b) {
+  return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) {
+  return make_float2(a.x - b.x, a.y - b.y);
+}
+__device__ __forceinline__ float4 vfma(float a, float4 u, float4 t) {
+  return make_float4(fmaf(a, u.x, t.x), fmaf(a, u.y, t.y), fmaf(a, u.z, t.z), fmaf(a, u.w, t.w));
+}
+__device__ __forceinline__ float2 vfma(float a, float2 u, float2 t) {
+  return make_float2(fmaf(a, u.x, t.x), fmaf(a, u.y, t.y));
 }
 
-template <bool TRANS>
+template <bool TRANS, typename V>
 __global__ void __launch_bounds__(CPL_MAXTHR)
 sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
                     const float2* part, const float2* __restrict__ in, float2* x, float2* zh,
                     float2* __restrict__ tbuf, const int* __restrict__ amap) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4* o = reinterpret_cast<float4*>(smem_raw);  // [(CPL_Y + 2) q][k / 2]
-  const int b = op.b, q = op.q, ny = op.ny, nx = op.nx, P = k >> 1;
+  constexpr int VW = sizeof(V) / sizeof(float2);  // columns of a unit
+  V* o = reinterpret_cast<V*>(smem_raw);           // [(CPL_Y + 2) q][P]
+  const int b = op.b, q = op.q, ny = op.ny, nx = op.nx, P = k / VW;
   const int nty = (ny + CPL_Y - 1) / CPL_Y, p = blockIdx.x / nty;
   const int half = p / Fa, f = active_problem(amap, p - half * Fa);
   const int y0 = (blockIdx.x - p * nty) * CPL_Y, npt = min(CPL_Y, ny - y0);
@@ -91,16 +113,16 @@ sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
   const float* cb = op.coef32 + (size_t)(!TRANS ? i1 : i) * b * op.S;
   const int slot = (!TRANS ? 1 - dcol : 1 + dcol) * 3;
   // (h of the end columns is the input itself: no step stores it)
-  const float4* src = reinterpret_cast<const float4*>(
+  const V* src = reinterpret_cast<const V*>(
       (inw || i1 == 0 || i1 == nx - 1 ? in : zh) + (size_t)f * NK + (size_t)i1 * b * k);
   struct Term {
     float cf[3][4];
-    float4 t;
+    V t;
   };
   auto load_term = [&](Term& w, int e) {
     const int lrow = e / P, jp = e - lrow * P;
     const int lp = lrow / q, c = lrow - lp * q, iy = y0 + lp, m = iy * q + c;
-    w.t = TRANS || inw ? src[m * P + jp] : make_float4(0.f, 0.f, 0.f, 0.f);
+    w.t = TRANS || inw ? src[m * P + jp] : V{};
 #pragma unroll
     for (int d = -1; d <= 1; ++d) {
       int off, stride = 1;
@@ -127,29 +149,23 @@ sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
   const size_t pidx = s.phase == SW_MID ? f : (size_t)half * F + f;
   tc::grid_wait();  // (above: what kernels before the product's wrote, and constants)
   tc::grid_trigger();
-  const float4* pf = reinterpret_cast<const float4*>(part + pidx * b * k);
-  float4* xi = reinterpret_cast<float4*>(x + (size_t)f * NK + (size_t)i * b * k);
-  float4* zi = reinterpret_cast<float4*>(zh + (size_t)f * NK + (size_t)i * b * k);
+  const V* pf = reinterpret_cast<const V*>(part + pidx * b * k);
+  V* xi = reinterpret_cast<V*>(x + (size_t)f * NK + (size_t)i * b * k);
+  V* zi = reinterpret_cast<V*>(zh + (size_t)f * NK + (size_t)i * b * k);
   for (int e = threadIdx.x; e < (npt + 2) * q * P; e += blockDim.x) {
     const int lrow = e / P, jp = e - lrow * P;
     const int lp = lrow / q, c = lrow - lp * q;
     int y = y0 - 1 + lp;
     const bool own = lp >= 1 && lp <= npt;
     if (op.periodic) y = (y + ny) % ny;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    V v = V{};
     if (y >= 0 && y < ny) {
       const int e0 = (y * q + c) * P + jp;
-      float4 z = v;
+      V z = v;
       if (!TRANS && outw) z = zi[e0];
 #pragma unroll 4
-      for (int t = 0; t < KS; ++t) {
-        const float4 u = pf[(size_t)t * (total >> 1) + e0];
-        v.x += u.x;
-        v.y += u.y;
-        v.z += u.z;
-        v.w += u.w;
-      }
-      if (!TRANS && outw) v = make_float4(z.x - v.x, z.y - v.y, z.z - v.z, z.w - v.w);
+      for (int t = 0; t < KS; ++t) v = vadd(v, pf[(size_t)t * (total / VW) + e0]);
+      if (!TRANS && outw) v = vsub(z, v);
       if (own) {
         if (!TRANS && inw) zi[e0] = v;
         // x; the adjoint's last inward result waits there for the middle
@@ -160,25 +176,20 @@ sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
   }
   if (last) return;
   __syncthreads();
-  float4* h = reinterpret_cast<float4*>(zh + (size_t)f * NK + (size_t)i1 * b * k);
-  float4* tf = reinterpret_cast<float4*>(tbuf + ((size_t)half * F + f) * b * k);
+  V* h = reinterpret_cast<V*>(zh + (size_t)f * NK + (size_t)i1 * b * k);
+  V* tf = reinterpret_cast<V*>(tbuf + ((size_t)half * F + f) * b * k);
   for (int e = threadIdx.x; e < nown; e += blockDim.x) {
     if (e != (int)threadIdx.x) load_term(w, e);
     const int lrow = e / P, jp = e - lrow * P;
     const int lp = lrow / q, m = (y0 + lp) * q + lrow - lp * q;
-    float4 t = w.t;
+    V t = w.t;
 #pragma unroll
     for (int d = -1; d <= 1; ++d) {
-      const float4* ov = o + ((lp + 1 + (TRANS ? -d : d)) * q) * P + jp;
+      const V* ov = o + ((lp + 1 + (TRANS ? -d : d)) * q) * P + jp;
 #pragma unroll
       for (int cp = 0; cp < 4; ++cp) {
         if (cp >= q) break;
-        const float4 u = ov[cp * P];
-        const float a = w.cf[d + 1][cp];
-        t.x = fmaf(a, u.x, t.x);
-        t.y = fmaf(a, u.y, t.y);
-        t.z = fmaf(a, u.z, t.z);
-        t.w = fmaf(a, u.w, t.w);
+        t = vfma(w.cf[d + 1][cp], ov[cp * P], t);
       }
     }
     if (TRANS && inw) h[m * P + jp] = t;
@@ -187,21 +198,22 @@ sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
 }
 
 // Right-hand side of the middle column: in + the couplings of both halves' last
-// inward results (z in zh, adjoint p in x), one thread per row and two columns;
+// inward results (z in zh, adjoint p in x), one thread per row and unit of columns;
 // a few microseconds of L2 latency, once per solve.
-template <bool TRANS>
+template <bool TRANS, typename V>
 __global__ void sweep_middle_kernel(OpView op, int k, const float2* __restrict__ in,
                                     const float2* __restrict__ src, float2* __restrict__ tbuf,
                                     const int* __restrict__ amap) {
-  const int b = op.b, q = op.q, mid = twist_mid(op.nx), P = k >> 1;
+  const int b = op.b, q = op.q, mid = twist_mid(op.nx);
+  const int P = k / (int)(sizeof(V) / sizeof(float2));
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= b * P) return;
   const int f = active_problem(amap, blockIdx.y);
   const int m = e / P, jp = e - m * P, iy = m / q, c = m - iy * q;
   const size_t NK = (size_t)op.n * k;
-  float4 t = reinterpret_cast<const float4*>(in + f * NK + (size_t)mid * b * k)[e];
+  V t = reinterpret_cast<const V*>(in + f * NK + (size_t)mid * b * k)[e];
   for (int dx = -1; dx <= 1; dx += 2) {
-    const float4* o = reinterpret_cast<const float4*>(src + f * NK + (size_t)(mid + dx) * b * k);
+    const V* o = reinterpret_cast<const V*>(src + f * NK + (size_t)(mid + dx) * b * k);
     const float* cb = op.coef32 + (size_t)(TRANS ? mid + dx : mid) * b * op.S;
 #pragma unroll
     for (int d = -1; d <= 1; ++d) {
@@ -213,15 +225,11 @@ __global__ void sweep_middle_kernel(OpView op, int k, const float2* __restrict__
         const int r = jy * q + cp;
         const float a = TRANS ? cb[r * op.S + ((1 - dx) * 3 + d + 1) * q + c]
                               : cb[m * op.S + ((1 + dx) * 3 + d + 1) * q + cp];
-        const float4 u = o[r * P + jp];
-        t.x = fmaf(a, u.x, t.x);
-        t.y = fmaf(a, u.y, t.y);
-        t.z = fmaf(a, u.z, t.z);
-        t.w = fmaf(a, u.w, t.w);
+        t = vfma(a, o[r * P + jp], t);
       }
     }
   }
-  reinterpret_cast<float4*>(tbuf + (size_t)f * b * k)[e] = t;
+  reinterpret_cast<V*>(tbuf + (size_t)f * b * k)[e] = t;
 }
 
 // ---------------------------------------------------------------------------
@@ -706,12 +714,10 @@ rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
 }  // namespace
 
 // The split tensor-core sweep (sweep_tc2_kernel) serves FP32 factors with an
-// even block of at least 128 and an even k of at most 64 columns (32 for the
-// BF16 x6 split, whose six products need 6N accumulator columns); only this
-// path runs on a subset of the problems.
+// even block of at least 128 and at most 64 columns (32 for the BF16 x6 split,
+// whose three orders need 6N accumulator columns).
 bool sweep_tc2_ok(const rr_factors* fa, int k) {
-  const int kmax = fa->prec == RR_FP32_BF16X6 ? 32 : 64;
-  return tc_prec(fa->prec) && k <= kmax && fa->tma_ok && (k % 2) == 0;
+  return tc_prec(fa->prec) && k <= (fa->prec == RR_FP32_BF16X6 ? 32 : 64) && fa->tma_ok;
 }
 
 namespace {
@@ -746,10 +752,11 @@ int split_count(const rr_factors* fa, int k, int nh, int nrt, int nch, int nsm) 
   return KS;
 }
 
-template <bool TRANS>
+template <bool TRANS, typename V>
 rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* zh) {
   const OpDev& d = fa->op->d;
   const int b = d.b, nx = d.nx, F = fa->F, Fa = active_count(fa);
+  const int units = k / (int)(sizeof(V) / sizeof(float2));  // of a row
   int kp = 8;
   while (kp < k) kp <<= 1;
   cudaStream_t st = fa->stream;
@@ -772,7 +779,7 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
     const int grid_x = std::min(nrt * Fa * step.nh * KS, nsm);
     if (step.phase == SW_MID) {
       prof_begin(PROF_SWEEP, st);
-      sweep_middle_kernel<TRANS><<<dim3((b * (k / 2) + 255) / 256, Fa), 256, 0, st>>>(
+      sweep_middle_kernel<TRANS, V><<<dim3((b * units + 255) / 256, Fa), 256, 0, st>>>(
           view(d), k, in, TRANS ? x : zh, tb, fa->amap);
       prof_end(PROF_SWEEP, st);
     }
@@ -796,9 +803,9 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
     const int ch = step.phase == SW_MID ? 2 : step.nh;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg =
-        dependent_launch(dim3((d.ny + CPL_Y - 1) / CPL_Y * ch * Fa), couple_threads(d.q, k), csmem,
+        dependent_launch(dim3((d.ny + CPL_Y - 1) / CPL_Y * ch * Fa), couple_threads(d.q, units), csmem,
                          st, at, true);
-    RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_couple_kernel<TRANS>, view(d), step, F, Fa, k, KS,
+    RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_couple_kernel<TRANS, V>, view(d), step, F, Fa, k, KS,
                                reinterpret_cast<const float2*>(fa->Pbuf), in, x, zh, tb,
                                (const int*)fa->amap));
     prof_end(PROF_SWEEP, st);
@@ -825,12 +832,15 @@ rr_status launch_solve_lo(rr_factors* fa, int k, int adjoint, const void* b, voi
   if (sweep_tc2_ok(fa, k)) {
     const OpDev& d = fa->op->d;
     const double step = 6.5 + 0.04 * k + 16.0 * active_count(fa) * d.b * d.b / 4.5e6;
-    if ((d.nx + 1.0) * step < sweep_cl32_us(fa, k, adjoint))
-      return adjoint ? solve_tc2<true>(fa, k, reinterpret_cast<const float2*>(b),
-                                       reinterpret_cast<float2*>(x), reinterpret_cast<float2*>(tmp))
-                     : solve_tc2<false>(fa, k, reinterpret_cast<const float2*>(b),
-                                        reinterpret_cast<float2*>(x),
-                                        reinterpret_cast<float2*>(tmp));
+    if ((d.nx + 1.0) * step < sweep_cl32_us(fa, k, adjoint)) {
+      const float2* in = reinterpret_cast<const float2*>(b);
+      float2 *xo = reinterpret_cast<float2*>(x), *zh = reinterpret_cast<float2*>(tmp);
+      if (k % 2)
+        return adjoint ? solve_tc2<true, float2>(fa, k, in, xo, zh)
+                       : solve_tc2<false, float2>(fa, k, in, xo, zh);
+      return adjoint ? solve_tc2<true, float4>(fa, k, in, xo, zh)
+                     : solve_tc2<false, float4>(fa, k, in, xo, zh);
+    }
   }
   return launch_sweep_cl32(fa, k, adjoint, b, x, tmp);
 }

@@ -1,0 +1,71 @@
+"""GPU parity of the tensor-core form of the sweeps over what it serves: odd numbers of
+right-hand sides, every operand split, tiles cut by the edge, both directions.  Each
+case is a batch that takes this form (its launches are counted: one per column
+pair and direction, where the cluster form has two in all).
+
+Checked against the oracle's dense LU solve: the refined solve to 1e-9, and the
+unrefined one to the bars of the factors, 1e-4 (BF16x3, 16 bits a product: 1e-2).
+"""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import operator as op
+from tests.gpu_util import lib, rel_err, to_dev, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def check(kind, nx, ny, k, F, precision, periodic=False, adjoint=False):
+    torch = torch_cuda()
+    rr = lib()
+    from paper_1902_01458_gb300 import _lib
+    if kind == "kz":
+        g = W.kz_grid(nx, ny, 0.8)
+    elif kind == "ns":
+        g = W.ns_grid(nx, ny)
+    else:
+        g = W.Grid(kind=W.KIND_ADVDIFF, nx=nx, ny=ny, x0=0, x1=10, y0=-5, y1=5, re=20.0)
+    if periodic:
+        g = dataclasses.replace(g, periodic_y=True, sponge_max=0.0)
+    flow = W.smooth_random_flow(g, 32)
+    L = op.assemble(g, flow)
+    o = rr.Operator(g, flow)
+    shifts = 0.05 + 1j * np.linspace(0.4, 2.5, F)
+    fa = o.factor(shifts, precision)
+    rng = np.random.default_rng(ny * 10 + k)
+    b = rng.standard_normal((F, o.n, k)) + 1j * rng.standard_normal((F, o.n, k))
+    bd = to_dev(b, torch)
+    _lib.rr_profile_start(["sweep"])
+    x0, _ = fa.solve(bd, adjoint, refine_tol=0.0, max_refine=0, check=False)
+    launches = _lib.rr_profile_read("sweep")[1]
+    _lib.rr_profile_start([])
+    assert launches == 2 * (nx // 2) + 2  # the products and the middle column's
+    x, _ = fa.solve(bd, adjoint)
+    for f in sorted({0, F // 2, F - 1}):
+        A = op.shifted(L, shifts[f]).toarray()
+        want = np.linalg.solve(A.conj().T if adjoint else A, b[f])
+        assert rel_err(x0[f].cpu().numpy(), want) < (1e-2 if precision.endswith("x3") else 1e-4)
+        assert rel_err(x[f].cpu().numpy(), want) < 1e-9
+    fa.close()
+    o.close()
+
+
+@pytest.mark.parametrize("kind,ny,k,F,precision,periodic",
+                         [("ns", 128, 15, 32, "fp32", False), ("ns", 256, 1, 16, "fp32", False),
+                          ("ns", 64, 63, 24, "fp32", True), ("kz", 40, 33, 24, "fp32", True),
+                          ("ns", 128, 31, 32, "fp32_bf16x3", False),
+                          ("ns", 86, 7, 64, "fp32_bf16x6", True)])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_odd_columns(kind, ny, k, F, precision, periodic, adjoint):
+    check(kind, 5, ny, k, F, precision, periodic, adjoint)
+
+
+@pytest.mark.parametrize("kind,ny,k,F", [("ns", 128, 16, 40), ("ns", 130, 32, 24),
+                                         ("ad", 130, 6, 200)])
+@pytest.mark.parametrize("precision", ["fp32", "fp32_bf16x3", "fp32_bf16x6"])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_operand_splits(kind, ny, k, F, precision, adjoint):
+    check(kind, 5, ny, k, F, precision, False, adjoint)
