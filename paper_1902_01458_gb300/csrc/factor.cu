@@ -448,7 +448,7 @@ gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, int nh, C_t<T>* __rest
 // G_i[j][p_m] = M[p_j][m];  X_i = G_i C_i with C_i = -L_{i,i+1} (half 0) or
 // G_i A_i with A_i = -L_{i,i-1} (half 1).
 template <typename T>
-__global__ void gjp_finalize_kernel(OpView op, int nh, int col0, int col1, int RB,
+__global__ void gjp_finalize_kernel(OpView op, int ldg, int nh, int col0, int col1, int RB,
                                     const C_t<T>* __restrict__ Mall,
                                     const int* __restrict__ pivslot_all, C_t<T>* __restrict__ Gall,
                                     C_t<T>* __restrict__ Xall) {
@@ -468,10 +468,10 @@ __global__ void gjp_finalize_kernel(OpView op, int nh, int col0, int col1, int R
     if (r < b) Gs[rr * b + ps[c]] = M[(size_t)ps[r] * b + c];
   }
   __syncthreads();
-  C* G = Gall + ((size_t)f * op.nx + i) * b * b;
+  C* G = Gall + ((size_t)f * op.nx + i) * b * ldg;
   for (int e = threadIdx.x; e < RB * b; e += blockDim.x) {
     const int rr = e / b, c = e - rr * b, r = r0 + rr;
-    if (r < b) G[(size_t)r * b + c] = Gs[rr * b + c];
+    if (r < b) G[(size_t)r * ldg + c] = Gs[rr * b + c];
   }
   if (Xall == nullptr) return;
   C* X = Xall + (size_t)pf * b * b;
@@ -623,7 +623,7 @@ rr_status factor_impl(rr_factors* fa) {
     }
     prof_begin(PROF_FINALIZE, st);
     gjp_finalize_kernel<T><<<dim3((b + RB - 1) / RB * nh, F), 256, fsmem, st>>>(
-        ov, nh, t.col0, t.col1, RB, M, fa->pivslot, G, t.middle ? nullptr : X);
+        ov, fa->ldg, nh, t.col0, t.col1, RB, M, fa->pivslot, G, t.middle ? nullptr : X);
     prof_end(PROF_FINALIZE, st);
     RR_CUDA(cudaGetLastError());
   }

@@ -919,7 +919,7 @@ gjw_finalize_kernel(OpView op, int nh, int col0, int col1, int RB,
     Gs[rr * b + ps[c]] = M[(size_t)ps[r0 + rr] * b + c];
   }
   __syncthreads();
-  float2* G = Gall + ((size_t)f * op.nx + i) * b * b;
+  float2* G = Gall + ((size_t)f * op.nx + i) * b * b;  // (b % 8 == 0: ldg is b)
   for (int e = threadIdx.x; e < nr * b; e += FIN_THREADS) {
     const int rr = e / b, c = e - rr * b;
     G[(size_t)(r0 + rr) * b + c] = Gs[rr * b + c];

@@ -473,14 +473,14 @@ rr_status cholqr2(rr_factors* fa, int k, double2* Y, double2* Rout, Work& w, rr_
 
 }  // namespace
 
-// TMA tensor maps over all FP32 factors G [F][nx][b][b] (complex, viewed as
+// TMA tensor maps over all FP32 factors G [F][nx][b][ldg] (complex, viewed as
 // floats [F*nx][b][2b]): tiles of 128 rows x 16 complex (G) and of 16 rows x
 // 128 complex (for G^H).  The rows of the former are 128 bytes and each thread
-// reads one, so they arrive swizzled.  Used only when b >= 128 and the row pitch is a
-// multiple of 16 bytes (b even); otherwise the sweeps use cp.async kernels.
+// reads one, so they arrive swizzled.  The row pitch is a multiple of 16 bytes (ldg
+// is even).
 static int encode_factor_maps(rr_factors* fa) {
   const OpDev& d = fa->op->d;
-  if (d.b < 128 || (d.b & 1)) return 0;
+  if (d.b < 128) return 0;
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
     cudaDriverEntryPointQueryResult q;
@@ -494,7 +494,7 @@ static int encode_factor_maps(rr_factors* fa) {
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
   const cuuint64_t dims[3] = {(cuuint64_t)2 * d.b, (cuuint64_t)d.b, (cuuint64_t)fa->F * d.nx};
-  const cuuint64_t strides[2] = {(cuuint64_t)2 * d.b * 4, (cuuint64_t)2 * d.b * d.b * 4};
+  const cuuint64_t strides[2] = {(cuuint64_t)2 * fa->ldg * 4, (cuuint64_t)2 * d.b * fa->ldg * 4};
   const cuuint32_t boxN[3] = {32, 128, 1}, boxT[3] = {256, 16, 1}, es[3] = {1, 1, 1};
   CUresult r1 = encode(reinterpret_cast<CUtensorMap*>(fa->tmap[0]), CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                        3, fa->G, dims, strides, boxN, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -723,13 +723,14 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
   fa->prec = prec;
   fa->stream = reinterpret_cast<cudaStream_t>(stream);
   fa->csz = prec == RR_FP64 ? sizeof(double2) : sizeof(float2);
+  fa->ldg = tc_prec(prec) ? (d.b + 1) & ~1 : d.b;
   const size_t bb = (size_t)d.b * d.b;
   rr_status s;
   auto fail = [&](rr_status st) {
     rr_destroy_factors(fa);
     return st;
   };
-  if ((s = dalloc(&fa->G, (size_t)nshift * d.nx * bb * fa->csz)) != RR_OK) return fail(s);
+  if ((s = dalloc(&fa->G, (size_t)nshift * d.nx * d.b * fa->ldg * fa->csz)) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->X, (size_t)2 * nshift * bb * fa->csz)) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->M, (size_t)2 * nshift * bb * fa->csz)) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->Bbuf, (size_t)2 * nshift * 16 * d.b * fa->csz)) != RR_OK) return fail(s);
@@ -847,7 +848,8 @@ rr_status factors_view(rr_factors* parent, int f0, int nf, cudaStream_t st, rr_f
   v->stream = st;
   v->csz = parent->csz;
   v->is_view = 1;
-  v->G = static_cast<char*>(parent->G) + (size_t)f0 * d.nx * d.b * d.b * parent->csz;
+  v->ldg = parent->ldg;
+  v->G = static_cast<char*>(parent->G) + (size_t)f0 * d.nx * d.b * parent->ldg * parent->csz;
   v->shifts = parent->shifts + f0;
   v->tune_update = parent->tune_update;
   rr_status s;

@@ -137,7 +137,8 @@ struct rr_factors {
   cudaEvent_t ev_next, ev_panel;
   cudaEvent_t ev_ring[8];  // panel / update rings of the 16-column factorisation
   size_t csz;        // bytes of one complex element of the factors
-  void* G;           // [F][nx][b][b]   inverse of each Schur block
+  void* G;           // [F][nx][b][ldg]  inverse of each Schur block
+  int ldg;           // row pitch of G: b, for the tensor cores the next even number
   // The factorisation runs from both ends to the middle column (factor.cu):
   // its work buffers hold 2 F problems, problem f of half h at h F + f.
   void* X;           // [2F][b][b] X_i = G_i C_i (G_i A_i) of the current columns (transient)

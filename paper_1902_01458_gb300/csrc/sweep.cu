@@ -419,14 +419,17 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
     const int m0 = (p_ks * cpp + p_lc) * TC2_KC;
     const int s = p_s;
     if (++p_s == stages) p_s = 0;
-    const uint32_t rhs_bytes = (uint32_t)(min(TC2_KC, b - m0) * k * 8);
+    // an odd block and an odd k put every other right-hand side off 16 bytes: the
+    // copy starts an element early and ends on 16 bytes (inside the workspace)
+    const size_t e0 = p_h * hstride + p_f * rstride + (size_t)m0 * k;
+    const int off = (int)(e0 & 1);
+    const uint32_t rhs_bytes = (uint32_t)((min(TC2_KC, b - m0) * k + off) * 8 + 15) & ~15u;
     unsigned char* st = raw + s * stage_bytes;
     const int zblk = p_f * nx + step_col(step, p_h, nx);
     tc::mbar_expect_tx(&full_bar[s], TC2_TILE_BYTES + rhs_bytes);
     if (!TRANS) tc::tma_load_3d(st, &tmap, 2 * m0, p_rt * TC_RT, zblk, &full_bar[s]);
     else tc::tma_load_3d(st, &tmap, 2 * p_rt * TC_RT, m0, zblk, &full_bar[s]);
-    w = Rhs{st + TC2_TILE_BYTES, rhs + p_h * hstride + p_f * rstride + (size_t)m0 * k, rhs_bytes,
-            &full_bar[s]};
+    w = Rhs{st + TC2_TILE_BYTES, rhs + e0 - off, rhs_bytes, &full_bar[s]};
     ++issued;
     if (++p_lc == p_len) {
       p_lc = 0;
@@ -533,6 +536,7 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
       int half, f, rt, ks;
       item(t, half, f, rt, ks);
       const int nl = item_len(ks);
+      const int off = (int)((half * hstride + f * rstride) & 1);  // (issue_tile)
       for (int lc = 0; lc < nl; ++lc, ++g) {
         if ((g & 1) != gi) continue;
         const int q = g & (NB - 1);
@@ -545,7 +549,8 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
         }
         tc::fence_after_sync();
         const float* R = reinterpret_cast<const float*>(raw + s * stage_bytes);
-        const float2* Rt = reinterpret_cast<const float2*>(raw + s * stage_bytes + TC2_TILE_BYTES);
+        const float2* Rt =
+            reinterpret_cast<const float2*>(raw + s * stage_bytes + TC2_TILE_BYTES) + off;
         // A: the lane's row, reals 16 kh ..; the 16-byte units of a swizzled row are
         // exchanged by its number mod 8
         float v[2][8];
@@ -713,9 +718,9 @@ rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
 
 }  // namespace
 
-// The split tensor-core sweep (sweep_tc2_kernel) serves FP32 factors with an
-// even block of at least 128 and at most 64 columns (32 for the BF16 x6 split,
-// whose three orders need 6N accumulator columns).
+// The split tensor-core sweep (sweep_tc2_kernel) serves FP32 factors with a block
+// of at least 128 and at most 64 columns (32 for the BF16 x6 split, whose three
+// orders need 6N accumulator columns).
 bool sweep_tc2_ok(const rr_factors* fa, int k) {
   return tc_prec(fa->prec) && k <= (fa->prec == RR_FP32_BF16X6 ? 32 : 64) && fa->tma_ok;
 }

@@ -44,8 +44,9 @@ constexpr size_t SMEM_CAP = 220 * 1024;
 template <typename T>
 struct Args {
   OpView op;
-  const C_t<T>* G;     // [F][nx][b][b]
+  const C_t<T>* G;     // [F][nx][b][ldg]
   size_t gstride;      // one problem of G
+  int ldg;
   const C_t<T>* in;    // [F][N][k]
   C_t<T>* x;           // [F][N][k]
   C_t<T>* h;           // [F][N][k] scratch (adjoint)
@@ -118,7 +119,8 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
   unsigned char* ring = reinterpret_cast<unsigned char*>(ob + (size_t)(rmax + 2 * q) * NC) +
                         (size_t)warp * 2 * SB;
   const C* Gf = a.G + (size_t)f * a.gstride;
-  const size_t bb = (size_t)b * b, NK = (size_t)op.n * a.k;
+  const int ldg = a.ldg;
+  const size_t bb = (size_t)b * ldg, NK = (size_t)op.n * a.k;
   const C* in = a.in + (size_t)f * NK;
   C* x = a.x + (size_t)f * NK;
   C* h = TRANS ? a.h + (size_t)f * NK : nullptr;
@@ -158,12 +160,12 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
           const int c = row0 + u * (gb / CS);
           const bool ok = m0 + sg < b && c < row0 + rows;
           cp_async(dst + (uint32_t)(sg * rmax * CS + u * gb),
-                   ok ? Gi + (size_t)(m0 + sg) * b + c : Gi, gb, ok);
+                   ok ? Gi + (size_t)(m0 + sg) * ldg + c : Gi, gb, ok);
         } else {      // the CTA's row sg at columns m0 ..
           const int c = m0 + u * (gb / CS);
           const bool ok = c < b;
           cp_async(dst + (uint32_t)(sg * PITCH + u * gb),
-                   ok ? Gi + (size_t)(row0 + sg) * b + c : Gi, gb, ok);
+                   ok ? Gi + (size_t)(row0 + sg) * ldg + c : Gi, gb, ok);
         }
         sg += walk_s;
         u += walk_u;
@@ -555,7 +557,8 @@ rr_status launch_plan(rr_factors* fa, const Plan& p, int k, const void* in, void
   Args<T> a;
   a.op = view(d);
   a.G = reinterpret_cast<const C_t<T>*>(fa->G);
-  a.gstride = (size_t)d.nx * d.b * d.b;
+  a.ldg = fa->ldg;
+  a.gstride = (size_t)d.nx * d.b * fa->ldg;
   a.in = reinterpret_cast<const C_t<T>*>(in);
   a.x = reinterpret_cast<C_t<T>*>(x);
   a.h = reinterpret_cast<C_t<T>*>(h);

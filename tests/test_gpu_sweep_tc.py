@@ -1,5 +1,5 @@
-"""GPU parity of the tensor-core form of the sweeps over what it serves: odd numbers of
-right-hand sides, every operand split, tiles cut by the edge, both directions.  Each
+"""GPU parity of the tensor-core form of the sweeps over what it serves: odd blocks and
+numbers of right-hand sides, every operand split, tiles cut by the edge, both directions.  Each
 case is a batch that takes this form (its launches are counted: one per column
 pair and direction, where the cluster form has two in all).
 
@@ -60,6 +60,17 @@ def check(kind, nx, ny, k, F, precision, periodic=False, adjoint=False):
                           ("ns", 86, 7, 64, "fp32_bf16x6", True)])
 @pytest.mark.parametrize("adjoint", [False, True])
 def test_odd_columns(kind, ny, k, F, precision, periodic, adjoint):
+    check(kind, 5, ny, k, F, precision, periodic, adjoint)
+
+
+@pytest.mark.parametrize("kind,ny,k,F,precision,periodic",
+                         [("ns", 129, 32, 32, "fp32", False), ("ns", 129, 31, 32, "fp32", True),
+                          ("ns", 129, 64, 24, "fp32", False), ("ad", 341, 9, 40, "fp32", True),
+                          ("ns", 85, 3, 96, "fp32_bf16x6", False),
+                          ("ns", 129, 16, 40, "fp32_bf16x3", True)])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_odd_blocks(kind, ny, k, F, precision, periodic, adjoint):
+    """Rows of G, and with odd k the right-hand sides, do not start on 16 bytes."""
     check(kind, 5, ny, k, F, precision, periodic, adjoint)
 
 
