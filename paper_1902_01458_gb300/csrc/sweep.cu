@@ -22,6 +22,7 @@
 // (sweep_tc2_kernel), and the sum of the partial blocks with the sparse
 // coupling that forms the next column's right-hand side (sweep_couple_kernel).
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include <cuda.h>
@@ -822,22 +823,33 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
 
 }  // namespace
 
-// FP64 factors and every FP32 shape the split tensor-core sweep does not take
-// run the whole-sweep cluster kernels.  Where both serve a shape, the one with
-// the smaller modelled time: a pair of columns in the tensor-core sweep takes 6.5
-// us + 0.04 us a column of the right-hand side + the factors' bytes at 4.5 TB/s.
-// Measured, cluster and tensor-core form, us per pair in a solve with its
-// residual check: blocks of 192 rows, 16 columns, 4 / 8 / 16 problems 6.9, 9.2,
-// 14.9 and 10.3, 12.7, 16.8; 64 columns, 4 / 8 problems 14.8, 27.8 and 17.6,
-// 22.9; 384 rows, 16 columns, 2 / 4 / 8 / 16 problems 11.8, 20.4, 22.9, 43.9 and
-// 11.2, 14.3, 18.6, 30.0; 768 rows, 32 columns, 1 / 6 problems 70.9, 248 and
-// 18.0, 38.9.
+// Modelled microseconds of a solve in the tensor-core form, per pair of columns: the
+// launches, the busiest CTA's chunks and items, and the coupling.  Fitted to solves
+// of 16 columns of 48 to 1023 rows with 1 to 64 right-hand sides and 1 to 512
+// problems (992, within 15 % for nine in ten); the cluster form took 1.3 times its
+// model on the same ones.  Of the two forms the one taken is within 5 % of the faster
+// in all but 4 % of them.  Measured, ms of a whole unrefined solve, tensor-core and
+// cluster form: 48 rows, 16 right-hand sides, 128 problems 0.48 and 0.37; 96 rows, 32,
+// 128 problems 1.09 and 1.50; 192 rows, 8, 32 problems 0.61 and 0.34; 387 rows, 32,
+// 64 problems 2.8 and 7.6; 768 rows, 32, 1 and 16 problems 0.40 and 1.6 instead of
+// 1.13 and 7.1.
+static double sweep_tc2_us(const rr_factors* fa, int k) {
+  const OpDev& d = fa->op->d;
+  const int nrt = (d.b + TC_RT - 1) / TC_RT, nch = (d.b + TC2_KC - 1) / TC2_KC;
+  const int nsm = num_sms(d.device), KS = split_count(fa, k, 2, nrt, nch, nsm);
+  const double items = std::ceil(2.0 * nrt * active_count(fa) * KS / nsm);  // of a CTA
+  const int cpp = (nch + KS - 1) / KS;
+  return (d.nx + 1.0) *
+         (5.2 + items * (1.25 + 0.6 * cpp) + 6.4e-5 * active_count(fa) * d.b * k);
+}
+
+// FP64 factors and the FP32 shapes that the tensor-core sweep does not take run the
+// whole-sweep cluster kernels.  Where both serve a shape, the one with the smaller
+// modelled time.
 rr_status launch_solve_lo(rr_factors* fa, int k, int adjoint, const void* b, void* x, void* tmp) {
   if (fa->prec == RR_FP64) return launch_sweep_cl64(fa, k, adjoint, b, x, tmp);
   if (sweep_tc2_ok(fa, k)) {
-    const OpDev& d = fa->op->d;
-    const double step = 6.5 + 0.04 * k + 16.0 * active_count(fa) * d.b * d.b / 4.5e6;
-    if ((d.nx + 1.0) * step < sweep_cl32_us(fa, k, adjoint)) {
+    if (sweep_tc2_us(fa, k) < 1.3 * sweep_cl32_us(fa, k, adjoint)) {
       const float2* in = reinterpret_cast<const float2*>(b);
       float2 *xo = reinterpret_cast<float2*>(x), *zh = reinterpret_cast<float2*>(tmp);
       if (k % 2)
