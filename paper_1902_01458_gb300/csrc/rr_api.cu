@@ -477,10 +477,10 @@ rr_status cholqr2(rr_factors* fa, int k, double2* Y, double2* Rout, Work& w, rr_
 // floats [F*nx][b][2b]): tiles of 128 rows x 16 complex (G) and of 16 rows x
 // 128 complex (for G^H).  The rows of the former are 128 bytes and each thread
 // reads one, so they arrive swizzled.  The row pitch is a multiple of 16 bytes (ldg
-// is even).
+// is even); a tile larger than the block is filled with zeros.
 static int encode_factor_maps(rr_factors* fa) {
   const OpDev& d = fa->op->d;
-  if (d.b < 128) return 0;
+  if (d.b < 48) return 0;  // (smaller blocks are faster in the cluster sweeps)
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
     cudaDriverEntryPointQueryResult q;

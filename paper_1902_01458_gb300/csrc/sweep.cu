@@ -720,8 +720,10 @@ rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
 }  // namespace
 
 // The split tensor-core sweep (sweep_tc2_kernel) serves FP32 factors with a block
-// of at least 128 and at most 64 columns (32 for the BF16 x6 split, whose three
-// orders need 6N accumulator columns).
+// of at least 48 (one tile of 128 rows still beats the cluster form in large batches:
+// 126 rows, 32 right-hand sides, 128 problems 1.6 ms a solve instead of 2.2) and at most
+// 64 columns (32 for the BF16 x6 split, whose three orders need 6N accumulator
+// columns).
 bool sweep_tc2_ok(const rr_factors* fa, int k) {
   return tc_prec(fa->prec) && k <= (fa->prec == RR_FP32_BF16X6 ? 32 : 64) && fa->tma_ok;
 }

@@ -74,6 +74,15 @@ def test_odd_blocks(kind, ny, k, F, precision, periodic, adjoint):
     check(kind, 5, ny, k, F, precision, periodic, adjoint)
 
 
+@pytest.mark.parametrize("kind,ny,k,F,precision,periodic",
+                         [("ns", 42, 32, 64, "fp32", False), ("ns", 21, 63, 96, "fp32", True),
+                          ("kz", 12, 64, 128, "fp32", False), ("kz", 31, 32, 64, "fp32_bf16x3", True),
+                          ("ns", 32, 32, 96, "fp32_bf16x6", False)])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_blocks_smaller_than_a_tile(kind, ny, k, F, precision, periodic, adjoint):
+    check(kind, 5, ny, k, F, precision, periodic, adjoint)
+
+
 @pytest.mark.parametrize("kind,ny,k,F", [("ns", 128, 16, 40), ("ns", 130, 32, 24),
                                          ("ad", 130, 32, 96)])
 @pytest.mark.parametrize("precision", ["fp32", "fp32_bf16x3", "fp32_bf16x6"])
