@@ -722,10 +722,11 @@ rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
 // The split tensor-core sweep (sweep_tc2_kernel) serves FP32 factors with a block
 // of at least 48 (one tile of 128 rows still beats the cluster form in large batches:
 // 126 rows, 32 right-hand sides, 128 problems 1.6 ms a solve instead of 2.2) and at most
-// 64 columns (32 for the BF16 x6 split, whose three orders need 6N accumulator
-// columns).
+// 64 columns.  The three orders of the BF16 x6 split need 6N accumulator columns, so
+// beyond 32 its sweeps take the TF32 split (768 rows, 64 right-hand sides, 16
+// problems: 2.7 ms a solve instead of 20 in the cluster form, no larger an error).
 bool sweep_tc2_ok(const rr_factors* fa, int k) {
-  return tc_prec(fa->prec) && k <= (fa->prec == RR_FP32_BF16X6 ? 32 : 64) && fa->tma_ok;
+  return tc_prec(fa->prec) && k <= 64 && fa->tma_ok;
 }
 
 namespace {
@@ -793,7 +794,7 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
     }
     prof_begin(PROF_SWEEP, st);
     rr_status ls;
-    switch (fa->prec) {
+    switch (fa->prec == RR_FP32_BF16X6 && k > 32 ? RR_FP32 : fa->prec) {
       case RR_FP32_BF16X3:
         ls = launch_tc2<TRANS, tc::SPLIT_BF16X3>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
                                                 rstride, hstride, s == 0, fa, st);

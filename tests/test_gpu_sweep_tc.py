@@ -91,6 +91,12 @@ def test_operand_splits(kind, ny, k, F, precision, adjoint):
     check(kind, 5, ny, k, F, precision, False, adjoint)
 
 
+@pytest.mark.parametrize("ny,k,F", [(128, 64, 24), (129, 33, 32)])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_bf16x6_beyond_32_columns(ny, k, F, adjoint):
+    check("ns", 5, ny, k, F, "fp32_bf16x6", False, adjoint)
+
+
 @pytest.mark.parametrize("ny,k,F", [(64, 8, 32), (64, 7, 64), (16, 4, 128)])
 def test_small_batches_stay_in_the_cluster_form(ny, k, F):
     """Two launches a solve: the form that measured faster there."""
