@@ -737,9 +737,11 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
   if ((s = dalloc(&fa->rowpiv, (size_t)2 * nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->pivslot, (size_t)2 * nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->Tbuf, (size_t)nshift * 128 * d.b * fa->csz)) != RR_OK) return fail(s);
-  if (tc_prec(prec)) {
-    if ((s = dalloc(&fa->Pbuf, (size_t)4 * nshift * 64 * d.b * sizeof(float2))) != RR_OK)
+  if (prec != RR_FP64)
+    if ((s = dalloc(&fa->Pbuf, (size_t)(tc_prec(prec) ? 4 : 2) * nshift * 64 * d.b * sizeof(float2))) !=
+        RR_OK)
       return fail(s);
+  if (tc_prec(prec)) {
     fa->tma_ok = encode_factor_maps(fa);
     if (d.b >= 64 && d.b <= 768 && d.b % 8 == 0) {
       if ((s = dalloc(&fa->Wbuf, (size_t)2 * nshift * 128 * d.b * sizeof(float2))) != RR_OK)
@@ -858,8 +860,11 @@ rr_status factors_view(rr_factors* parent, int f0, int nf, cudaStream_t st, rr_f
     return r;
   };
   if ((s = dalloc(&v->Tbuf, (size_t)nf * 128 * d.b * v->csz)) != RR_OK) return fail(s);
+  if (v->prec != RR_FP64)
+    if ((s = dalloc(&v->Pbuf, (size_t)(tc_prec(v->prec) ? 4 : 2) * nf * 64 * d.b * sizeof(float2))) !=
+        RR_OK)
+      return fail(s);
   if (tc_prec(v->prec)) {
-    if ((s = dalloc(&v->Pbuf, (size_t)4 * nf * 64 * d.b * sizeof(float2))) != RR_OK) return fail(s);
     v->tma_ok = encode_factor_maps(v);
   }
   if ((s = dalloc(&v->flag, (size_t)(2 * nf + 1) * sizeof(int))) != RR_OK) return fail(s);

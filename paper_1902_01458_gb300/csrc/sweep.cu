@@ -19,7 +19,8 @@
 // per problem and half (sweep_cl.cuh), or, for large blocks and batches, two
 // launches per pair of streamwise columns for all problems of the batch: the dense (b x b) x
 // (b x k) product on the tensor cores, its contraction split over CTAs
-// (sweep_tc2_kernel), and the sum of the partial blocks with the sparse
+// (sweep_tc2_kernel), or for RR_FP32_SIMT on the CUDA cores (sweep_cc_kernel), and
+// the sum of the partial blocks with the sparse
 // coupling that forms the next column's right-hand side (sweep_couple_kernel).
 #include <algorithm>
 #include <cmath>
@@ -678,6 +679,120 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
   if (warp == 0) tc::tmem_dealloc(tmem, ncols);
 }
 
+// ---------------------------------------------------------------------------
+// The same product on the CUDA cores in FP32 (RR_FP32_SIMT), one contraction part:
+// a CTA forms RT = 2048 / kp rows by kp columns of one problem and half, 4 x 2
+// outputs a thread, over chunks of 32 columns of op(G) in three stages filled by
+// cp.async (16 bytes where every row starts on 16 bytes).
+// Bound: FP32 and shared memory; batches that fill the chip many times over, where
+// a cluster per problem, half and column group reads G again for each group.  Rows of a
+// chunk are swizzled, not padded: two CTAs an SM from kp = 16 on.
+constexpr int CC_THREADS = 256, CC_KC = 32, CC_STAGES = 3, CC_RT = 2048;
+template <bool TRANS>
+__host__ __device__ constexpr int cc_pitch(int kp) { return TRANS ? CC_RT / kp : CC_KC; }
+template <bool TRANS>
+__host__ __device__ constexpr int cc_stage(int kp) {  // complex values
+  return (TRANS ? CC_KC : CC_RT / kp) * cc_pitch<TRANS>(kp) + CC_KC * kp;
+}
+
+__device__ __forceinline__ void cc_copy(float2* smem, const float2* gmem, int bytes, bool ok) {
+  const uint32_t s = tc::smem_u32(smem);
+  if (bytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem),
+                 "r"(ok ? 16 : 0)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(s), "l"(gmem),
+                 "r"(ok ? 8 : 0)
+                 : "memory");
+}
+
+template <bool TRANS>
+__global__ void __launch_bounds__(CC_THREADS)
+sweep_cc_kernel(const float2* __restrict__ G, int b, int ldg, int k, int kp, SweepStep step, int nx,
+                int nrt, const float2* __restrict__ rhs, size_t rstride, size_t hstride,
+                float2* __restrict__ part, int F, int Fa, const int* __restrict__ amap) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* base = reinterpret_cast<float2*>(smem_raw);
+  const int RT = CC_RT / kp, pitch = cc_pitch<TRANS>(kp), stage_len = cc_stage<TRANS>(kp);
+  const int p = blockIdx.x / nrt, r0 = (blockIdx.x - p * nrt) * RT;
+  const int half = p >= Fa, f = active_problem(amap, half ? p - Fa : p);
+  const float2* Gi = G + ((size_t)f * nx + step_col(step, half, nx)) * b * ldg;
+  const float2* t = rhs + half * hstride + f * rstride;
+  const int tid = threadIdx.x, TX = kp >> 1, TY = CC_THREADS / TX;
+  const int tx = tid % TX, ty = tid / TX;
+  const int gv = (b & 1) ? 1 : 2;  // columns of G a copy
+  const int sw = (ty & 7) * 2;     // (rows of a chunk are swizzled; TY is a multiple of 8)
+  auto load = [&](int st, int m0) {
+    float2* Ms = base + st * stage_len;
+    float2* Ts = Ms + stage_len - CC_KC * kp;
+    const int nr = TRANS ? CC_KC : RT, per = (TRANS ? RT : CC_KC) / gv;
+    for (int e = tid; e < nr * per; e += CC_THREADS) {
+      const int a = e / per, u = (e - a * per) * gv;
+      const int row = (TRANS ? m0 : r0) + a, col = (TRANS ? r0 : m0) + u;
+      const bool ok = row < b && col < b;
+      cc_copy(&Ms[a * pitch + (TRANS ? u : u ^ (a & 7) * 2)], ok ? Gi + (size_t)row * ldg + col : Gi, 8 * gv, ok);
+    }
+    for (int e = tid; e < CC_KC * kp; e += CC_THREADS) {
+      const int mm = e / kp, j = e - mm * kp, m = m0 + mm;
+      const bool ok = m < b && j < k;
+      cc_copy(&Ts[e], ok ? t + (size_t)m * k + j : t, 8, ok);
+    }
+  };
+  float2 acc[4][2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+  const int nch = (b + CC_KC - 1) / CC_KC;
+#pragma unroll
+  for (int s = 0; s < CC_STAGES - 1; ++s) {
+    if (s < nch) load(s, s * CC_KC);
+    asm volatile("cp.async.commit_group;\n" ::);
+  }
+  for (int c = 0; c < nch; ++c) {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(CC_STAGES - 2) : "memory");
+    __syncthreads();
+    if (c + CC_STAGES - 1 < nch) load((c + CC_STAGES - 1) % CC_STAGES, (c + CC_STAGES - 1) * CC_KC);
+    asm volatile("cp.async.commit_group;\n" ::);
+    const float2* Ms = base + (c % CC_STAGES) * stage_len;
+    const float2* Ts = Ms + stage_len - CC_KC * kp;
+#pragma unroll 2
+    for (int mm = 0; mm < CC_KC; mm += 2) {
+      float2 a[2][4], v[2][2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (TRANS) {
+          a[0][i] = cconj(Ms[mm * pitch + ty + TY * i]);
+          a[1][i] = cconj(Ms[(mm + 1) * pitch + ty + TY * i]);
+        } else {
+          const float4 w = *reinterpret_cast<const float4*>(&Ms[(ty + TY * i) * pitch + (mm ^ sw)]);
+          a[0][i] = make_float2(w.x, w.y);
+          a[1][i] = make_float2(w.z, w.w);
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        v[h][0] = Ts[(mm + h) * kp + tx];
+        v[h][1] = Ts[(mm + h) * kp + tx + TX];
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          acc[i][0] = cfma(a[h][i], v[h][0], acc[i][0]);
+          acc[i][1] = cfma(a[h][i], v[h][1], acc[i][1]);
+        }
+    }
+  }
+  float2* pf = part + ((size_t)half * F + f) * b * k;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = r0 + ty + TY * i;
+    if (r >= b) continue;
+    if (tx < k) pf[(size_t)r * k + tx] = acc[i][0];
+    if (tx + TX < k) pf[(size_t)r * k + tx + TX] = acc[i][1];
+  }
+}
+
 // Launch that may start before its predecessor in the stream has finished; the
 // kernel orders itself by grid_wait
 cudaLaunchConfig_t dependent_launch(dim3 grid, int threads, size_t smem, cudaStream_t st,
@@ -714,6 +829,25 @@ rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
       &cfg, sweep_tc2_kernel<TRANS, SPLIT>, *tm, b, k, kp, step, nx, nrt, KS, cpp, reinterpret_cast<const float2*>(rhs), rstride, hstride,
       reinterpret_cast<float2*>(fa->Pbuf), fa->F, active_count(fa), (const int*)fa->amap, fa->flag + fa->F,
       wait_tries(), take_stall()));
+  return RR_OK;
+}
+
+}  // namespace
+
+namespace {
+
+template <bool TRANS>
+rr_status launch_cc(int k, int kp, const SweepStep& step, const float2* rhs, size_t rstride,
+                    size_t hstride, rr_factors* fa, cudaStream_t st) {
+  const OpDev& d = fa->op->d;
+  const int nrt = (d.b * kp + CC_RT - 1) / CC_RT, Fa = active_count(fa);
+  const size_t smem = (size_t)CC_STAGES * cc_stage<TRANS>(kp) * sizeof(float2);
+  RR_CUDA(cudaFuncSetAttribute(sweep_cc_kernel<TRANS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               227 * 1024));
+  sweep_cc_kernel<TRANS><<<nrt * Fa * step.nh, CC_THREADS, smem, st>>>(
+      reinterpret_cast<const float2*>(fa->G), d.b, fa->ldg, k, kp, step, d.nx, nrt, rhs, rstride,
+      hstride, reinterpret_cast<float2*>(fa->Pbuf), fa->F, Fa, fa->amap);
+  RR_CUDA(cudaGetLastError());
   return RR_OK;
 }
 
@@ -784,7 +918,8 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
     const float2* rhs = s == 0 ? in : tb;
     const size_t rstride = s == 0 ? (size_t)d.n * k : (size_t)b * k;
     const size_t hstride = s == 0 ? (size_t)(nx - 1) * b * k : (size_t)F * b * k;
-    const int KS = split_count(fa, k, step.nh, nrt, nch, nsm), cpp = (nch + KS - 1) / KS;
+    const bool cc = fa->prec == RR_FP32_SIMT;
+    const int KS = cc ? 1 : split_count(fa, k, step.nh, nrt, nch, nsm), cpp = (nch + KS - 1) / KS;
     const int grid_x = std::min(nrt * Fa * step.nh * KS, nsm);
     if (step.phase == SW_MID) {
       prof_begin(PROF_SWEEP, st);
@@ -795,6 +930,9 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
     prof_begin(PROF_SWEEP, st);
     rr_status ls;
     switch (fa->prec == RR_FP32_BF16X6 && k > 32 ? RR_FP32 : fa->prec) {
+      case RR_FP32_SIMT:
+        ls = launch_cc<TRANS>(k, kp, step, rhs, rstride, hstride, fa, st);
+        break;
       case RR_FP32_BF16X3:
         ls = launch_tc2<TRANS, tc::SPLIT_BF16X3>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
                                                 rstride, hstride, s == 0, fa, st);
@@ -846,13 +984,30 @@ static double sweep_tc2_us(const rr_factors* fa, int k) {
          (5.2 + items * (1.25 + 0.6 * cpp) + 6.4e-5 * active_count(fa) * d.b * k);
 }
 
+// The same for the product on the CUDA cores (RR_FP32_SIMT): the chunks' latency per
+// wave of resident CTAs and their arithmetic.  Measured, ms of a whole unrefined
+// forward solve of 16 columns, this and the cluster form: 192 rows, 8 right-hand sides,
+// 64 problems 0.76 and 0.58; 384 rows, 64, 16 problems 2.3 and 2.8; 768 rows, 64, 64
+// problems 23.6 and 55.
+static double sweep_cc_us(const rr_factors* fa, int k) {
+  const OpDev& d = fa->op->d;
+  int kp = 8;
+  while (kp < k) kp <<= 1;
+  const int nch = (d.b + CC_KC - 1) / CC_KC, Fa = active_count(fa), nsm = num_sms(d.device);
+  const double ctas = 2.0 * Fa * ((d.b * kp + CC_RT - 1) / CC_RT);
+  const double waves = std::ceil(ctas / (nsm * (kp <= 8 ? 1.0 : kp == 16 ? 2.0 : 3.0)));
+  return (d.nx + 1.0) *
+         (5.5 + nch * (2.55 * waves + 0.93 * ctas / nsm) + 6.4e-5 * Fa * d.b * k);
+}
+
 // FP64 factors and the FP32 shapes that the tensor-core sweep does not take run the
 // whole-sweep cluster kernels.  Where both serve a shape, the one with the smaller
 // modelled time.
 rr_status launch_solve_lo(rr_factors* fa, int k, int adjoint, const void* b, void* x, void* tmp) {
   if (fa->prec == RR_FP64) return launch_sweep_cl64(fa, k, adjoint, b, x, tmp);
-  if (sweep_tc2_ok(fa, k)) {
-    if (sweep_tc2_us(fa, k) < 1.3 * sweep_cl32_us(fa, k, adjoint)) {
+  const bool simt = fa->prec == RR_FP32_SIMT;
+  if (simt || sweep_tc2_ok(fa, k)) {
+    if ((simt ? sweep_cc_us(fa, k) : sweep_tc2_us(fa, k)) < 1.3 * sweep_cl32_us(fa, k, adjoint)) {
       const float2* in = reinterpret_cast<const float2*>(b);
       float2 *xo = reinterpret_cast<float2*>(x), *zh = reinterpret_cast<float2*>(tmp);
       if (k % 2)
