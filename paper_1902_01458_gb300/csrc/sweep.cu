@@ -59,7 +59,7 @@ __host__ __device__ __forceinline__ int step_col(const SweepStep& s, int half, i
 //   t = h + L_{i,i'}^T o (adjoint outward)
 // for the next column i'.  z goes to zh in the inward sweep, so the outward one's
 // results (x) never overwrite a value a neighbouring tile still needs.
-// One grid dimension: two halves of 65,535 problems exceed the second one's limit.
+// (A grid dimension holds 65,535 problems, not two halves of them.)
 // (part is not __restrict__: the product writes it while this kernel already runs,
 // until grid_wait, so no load of it may go through the read-only path or move up.)
 // Bound: L2 latency (the partials were just written), so the coefficients and
@@ -93,16 +93,15 @@ __device__ __forceinline__ float2 vfma(float a, float2 u, float2 t) {
 
 template <bool TRANS, typename V>
 __global__ void __launch_bounds__(CPL_MAXTHR)
-sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
+sweep_couple_kernel(OpView op, SweepStep s, int F, int k, int KS,
                     const float2* part, const float2* __restrict__ in, float2* x, float2* zh,
                     float2* __restrict__ tbuf, const int* __restrict__ amap) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int VW = sizeof(V) / sizeof(float2);  // columns of a unit
   V* o = reinterpret_cast<V*>(smem_raw);           // [(CPL_Y + 2) q][P]
   const int b = op.b, q = op.q, ny = op.ny, nx = op.nx, P = k / VW;
-  const int nty = (ny + CPL_Y - 1) / CPL_Y, p = blockIdx.x / nty;
-  const int half = p / Fa, f = active_problem(amap, p - half * Fa);
-  const int y0 = (blockIdx.x - p * nty) * CPL_Y, npt = min(CPL_Y, ny - y0);
+  const int half = blockIdx.z, f = active_problem(amap, blockIdx.y);
+  const int y0 = blockIdx.x * CPL_Y, npt = min(CPL_Y, ny - y0);
   const size_t NK = (size_t)op.n * k, total = (size_t)s.nh * F * b * k;
   const int i = step_col(s, half, nx);
   const bool inw = s.phase == SW_IN, outw = s.phase == SW_OUT;
@@ -538,7 +537,7 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
       int half, f, rt, ks;
       item(t, half, f, rt, ks);
       const int nl = item_len(ks);
-      const int off = (int)((half * hstride + f * rstride) & 1);  // (issue_tile)
+      const int off = (b & k & 1) ? (int)((half * hstride + f * rstride) & 1) : 0;  // (issue_tile)
       for (int lc = 0; lc < nl; ++lc, ++g) {
         if ((g & 1) != gi) continue;
         const int q = g & (NB - 1);
@@ -950,9 +949,9 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
     const int ch = step.phase == SW_MID ? 2 : step.nh;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg =
-        dependent_launch(dim3((d.ny + CPL_Y - 1) / CPL_Y * ch * Fa), couple_threads(d.q, units), csmem,
+        dependent_launch(dim3((d.ny + CPL_Y - 1) / CPL_Y, Fa, ch), couple_threads(d.q, units), csmem,
                          st, at, true);
-    RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_couple_kernel<TRANS, V>, view(d), step, F, Fa, k, KS,
+    RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_couple_kernel<TRANS, V>, view(d), step, F, k, KS,
                                reinterpret_cast<const float2*>(fa->Pbuf), in, x, zh, tb,
                                (const int*)fa->amap));
     prof_end(PROF_SWEEP, st);
