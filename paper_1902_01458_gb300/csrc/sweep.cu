@@ -297,9 +297,19 @@ __host__ __device__ constexpr int tc2_sets(int kp) {
   const int fit = 256 / (tc2_orders<SPLIT>() * 2 * kp);
   return fit < 1 ? 1 : fit < tc::ksteps32<SPLIT>() ? fit : tc::ksteps32<SPLIT>();
 }
+// Where one set fits (64 columns), a second accumulator of hi.hi alone takes every other
+// K step of the TF32 split (384 rows, 24 problems: unrefined residual 1.0e-5 instead
+// of 8.7e-6 without it, 4.7e-5 and 3.8e-5 adjoint; 0 to 2 % of a solve).  BF16x3's
+// errors are its products'.
+template <int SPLIT>
+__host__ __device__ constexpr int tc2_extra(int kp) {
+  return SPLIT == tc::SPLIT_TF32X3 && tc2_sets<SPLIT>(kp) == 1 ? 1 : 0;
+}
 template <int SPLIT>
 __host__ __device__ constexpr uint32_t tc2_acc_cols(int kp) {
-  return (uint32_t)(tc2_sets<SPLIT>(kp) * tc2_orders<SPLIT>() * 2 * kp + 31) & ~31u;
+  return (uint32_t)((tc2_sets<SPLIT>(kp) * tc2_orders<SPLIT>() + tc2_extra<SPLIT>(kp)) * 2 * kp +
+                    31) &
+         ~31u;
 }
 // operand buffers: two for each group of warps where shared memory has the room
 __host__ __device__ constexpr int tc2_bufs(int kp) { return kp > 32 ? 2 : TC2_MAXBUFS; }
@@ -328,7 +338,8 @@ constexpr int TC2_CONV = 512;                 // converter threads (warps 0-15)
 constexpr int TC2_GROUP = TC2_CONV / 2;       // threads of a group
 constexpr int TC2_THREADS = TC2_CONV + 64;    // + warp 16, issues the MMAs, and 17, the copies
 
-template <bool TRANS, int SPLIT>
+// (WIDE: more than 32 columns)
+template <bool TRANS, int SPLIT, bool WIDE>
 __global__ void __launch_bounds__(TC2_THREADS, 1)
 sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp, SweepStep step,
                  int nx, int nrt, int KS, int cpp, const float2* rhs, size_t rstride,
@@ -363,7 +374,8 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
   // A_lo x B_hi into cross.  BF16 x6 (up to 32 columns), three: p0 x [q0 | q1 | q2],
   // p1 x [q0 | q1], p2 x q0.
   constexpr int ORDERS = tc2_orders<SPLIT>();
-  const int SETS = tc2_sets<SPLIT>(kp);
+  const int SETS = WIDE ? 1 : tc2_sets<SPLIT>(kp);
+  constexpr int EXTRA = WIDE ? tc2_extra<SPLIT>(64) : 0;
   const uint32_t set_cols = (uint32_t)(ORDERS * N);
   const uint32_t ncols = tc2_tmem_cols<SPLIT>(kp) <= 256 ? 256u : 512u;
   // work item t of this CTA -> (half, problem, row tile, contraction part)
@@ -505,18 +517,35 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
         tc::fence_after_sync();
         const uint64_t dB = tc::smem_desc(tc::smem_u32(ops + q * buf_bytes), TC_LBO, SBO);
         const uint32_t aq = abuf + (uint32_t)(q * PIECES) * AC;
+        if constexpr (EXTRA) {
+          const uint64_t lo = bt_bytes >> 4;  // to B_lo
 #pragma unroll
-        for (int kk = 0; kk < tc::ksteps32<SPLIT>(); ++kk) {
-          const uint64_t bk = dB + (uint64_t)(kk * 2 * TC_LBO >> 4);
-          const uint32_t ak = aq + (uint32_t)kk * 8;
-          const uint32_t set = tmem + (uint32_t)(kk & (SETS - 1)) * set_cols;
-          const uint32_t acc = (lc > 0 || kk >= SETS) ? 1u : 0u;
-          mma(set, ak, bk, X6 ? id3 : id2, acc);
-          if (X6) {
-            mma(set + N, ak + AC, bk, id2, 1u);
-            mma(set + 2 * N, ak + 2 * AC, bk, id1, 1u);
-          } else {
-            mma(set + N, ak + AC, bk, id1, 1u);
+          for (int kk = 0; kk < tc::ksteps32<SPLIT>(); ++kk) {
+            const uint64_t bk = dB + (uint64_t)(kk * 2 * TC_LBO >> 4);
+            const uint32_t ak = aq + (uint32_t)kk * 8;
+            const uint32_t acc = (lc > 0 || kk > 1) ? 1u : 0u;
+            if (kk & 1) {
+              mma(tmem + 2 * N, ak, bk, id1, acc);
+              mma(tmem + N, ak, bk + lo, id1, 1u);
+            } else {
+              mma(tmem, ak, bk, id2, acc);
+            }
+            mma(tmem + N, ak + AC, bk, id1, 1u);
+          }
+        } else {
+#pragma unroll
+          for (int kk = 0; kk < tc::ksteps32<SPLIT>(); ++kk) {
+            const uint64_t bk = dB + (uint64_t)(kk * 2 * TC_LBO >> 4);
+            const uint32_t ak = aq + (uint32_t)kk * 8;
+            const uint32_t set = tmem + (uint32_t)(kk & (SETS - 1)) * set_cols;
+            const uint32_t acc = (lc > 0 || kk >= SETS) ? 1u : 0u;
+            mma(set, ak, bk, X6 ? id3 : id2, acc);
+            if (X6) {
+              mma(set + N, ak + AC, bk, id2, 1u);
+              mma(set + 2 * N, ak + 2 * AC, bk, id1, 1u);
+            } else {
+              mma(set + N, ak + AC, bk, id1, 1u);
+            }
           }
         }
         tc::mma_commit(&mma_bar[q]);
@@ -634,7 +663,7 @@ sweep_tc2_kernel(const __grid_constant__ CUtensorMap tmap, int b, int k, int kp,
             tmem + ((uint32_t)(lq * 32 + 16 * sb) << 16) + (uint32_t)(hh * 32);
         tc::tmem_ld_16x256b_x4(ta, v);
 #pragma unroll
-        for (int a = 1; a < SETS * ORDERS; ++a) {  // the partial sums
+        for (int a = 1; a < SETS * ORDERS + EXTRA; ++a) {  // the partial sums
           tc::tmem_ld_16x256b_x4(ta + (uint32_t)(a * N), w);
 #pragma unroll
           for (int tt = 0; tt < 16; ++tt) v[tt] += w[tt];
@@ -810,24 +839,24 @@ cudaLaunchConfig_t dependent_launch(dim3 grid, int threads, size_t smem, cudaStr
 
 // One launch of the TMA-fed tensor-core sweep step in the factors' operand
 // split (partial products into Pbuf).
-template <bool TRANS, int SPLIT, typename C>
+template <bool TRANS, int SPLIT, bool WIDE>
 rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
-                     const SweepStep& step, int nx, int nrt, int KS, int cpp, const C* rhs,
+                     const SweepStep& step, int nx, int nrt, int KS, int cpp, const float2* rhs,
                      size_t rstride, size_t hstride, bool first, rr_factors* fa, cudaStream_t st) {
   const size_t smem = tc2_smem_bytes<SPLIT>(kp) + 1024;
   static size_t attr = 0;  // dynamic shared memory opted in so far
   if (smem > attr) {
-    RR_CUDA(cudaFuncSetAttribute(sweep_tc2_kernel<TRANS, SPLIT>,
+    RR_CUDA(cudaFuncSetAttribute(sweep_tc2_kernel<TRANS, SPLIT, WIDE>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr = smem;
   }
   // dependent launch, but for the first: its predecessor is not of this solve
   cudaLaunchAttribute at[1];
   const cudaLaunchConfig_t cfg = dependent_launch(dim3(grid_x), TC2_THREADS, smem, st, at, !first);
-  RR_CUDA(cudaLaunchKernelEx(
-      &cfg, sweep_tc2_kernel<TRANS, SPLIT>, *tm, b, k, kp, step, nx, nrt, KS, cpp, reinterpret_cast<const float2*>(rhs), rstride, hstride,
-      reinterpret_cast<float2*>(fa->Pbuf), fa->F, active_count(fa), (const int*)fa->amap, fa->flag + fa->F,
-      wait_tries(), take_stall()));
+  RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_tc2_kernel<TRANS, SPLIT, WIDE>, *tm, b, k, kp, step, nx, nrt,
+                             KS, cpp, rhs, rstride, hstride, reinterpret_cast<float2*>(fa->Pbuf),
+                             fa->F, active_count(fa), (const int*)fa->amap, fa->flag + fa->F,
+                             wait_tries(), take_stall()));
   return RR_OK;
 }
 
@@ -927,23 +956,21 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
       prof_end(PROF_SWEEP, st);
     }
     prof_begin(PROF_SWEEP, st);
+    auto product = [&](auto launch) {
+      return launch(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs, rstride, hstride, s == 0, fa,
+                    st);
+    };
     rr_status ls;
-    switch (fa->prec == RR_FP32_BF16X6 && k > 32 ? RR_FP32 : fa->prec) {
-      case RR_FP32_SIMT:
-        ls = launch_cc<TRANS>(k, kp, step, rhs, rstride, hstride, fa, st);
-        break;
-      case RR_FP32_BF16X3:
-        ls = launch_tc2<TRANS, tc::SPLIT_BF16X3>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
-                                                rstride, hstride, s == 0, fa, st);
-        break;
-      case RR_FP32_BF16X6:
-        ls = launch_tc2<TRANS, tc::SPLIT_BF16X6>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
-                                                rstride, hstride, s == 0, fa, st);
-        break;
-      default:
-        ls = launch_tc2<TRANS, tc::SPLIT_TF32X3>(tm, grid_x, b, k, kp, step, nx, nrt, KS, cpp, rhs,
-                                                rstride, hstride, s == 0, fa, st);
-    }
+    if (cc)
+      ls = launch_cc<TRANS>(k, kp, step, rhs, rstride, hstride, fa, st);
+    else if (fa->prec == RR_FP32_BF16X3)
+      ls = kp > 32 ? product(launch_tc2<TRANS, tc::SPLIT_BF16X3, true>)
+                   : product(launch_tc2<TRANS, tc::SPLIT_BF16X3, false>);
+    else if (fa->prec == RR_FP32_BF16X6 && kp <= 32)
+      ls = product(launch_tc2<TRANS, tc::SPLIT_BF16X6, false>);
+    else
+      ls = kp > 32 ? product(launch_tc2<TRANS, tc::SPLIT_TF32X3, true>)
+                   : product(launch_tc2<TRANS, tc::SPLIT_TF32X3, false>);
     if (ls != RR_OK) return ls;
     // (the middle's result starts both halves' outward sweeps)
     const int ch = step.phase == SW_MID ? 2 : step.nh;

@@ -123,3 +123,24 @@ def test_small_batches_stay_in_the_cluster_form(ny, k, F):
 def test_cuda_core_product(kind, ny, k, F, periodic, adjoint):
     """Large batches of FP32 factors without tensor cores take the same form."""
     check(kind, 5, ny, k, F, "fp32_simt", periodic, adjoint)
+
+
+@pytest.mark.parametrize("seed", [0, 1, 2])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_sixty_four_columns_are_as_accurate_as_thirty_two(seed, adjoint):
+    """The same 32 right-hand sides twice: both widths sum hi.hi in two accumulators over
+    equally long parts of the contraction, so the unrefined residuals agree up to the
+    small orders; a tenth is allowed (one accumulator rounds towards zero twice as often)."""
+    torch = torch_cuda()
+    rr = lib()
+    g = W.ns_grid(24, 128)
+    o = rr.Operator(g, W.smooth_random_flow(g, seed))
+    F = 24
+    fa = o.factor(0.05 + 1j * np.linspace(0.4, 2.5, F), "fp32")
+    gen = torch.Generator(device="cuda:0").manual_seed(seed)
+    b = torch.randn(F, o.n, 32, dtype=torch.complex128, device="cuda:0", generator=gen)
+    res = [fa.solve(v, adjoint, refine_tol=0.0, max_refine=0, check=False)[1]["first_residual"]
+           for v in (b, torch.cat([b, b], dim=2))]
+    assert res[1] <= 1.1 * res[0]
+    fa.close()
+    o.close()
