@@ -159,6 +159,14 @@ __device__ __forceinline__ unsigned gp_mag(double2 x) {
   return max((unsigned)__double2hiint(x.x) & 0x7fffffffu, (unsigned)__double2hiint(x.y) & 0x7fffffffu) &
          ~31u;
 }
+// magnitudes below which a pivot counts as zero, because its square vanishes (2^-538;
+// FP32: a square of 2^-144), and below which 1 / square may overflow (2^-511; 2^-126)
+template <typename T> __device__ __forceinline__ constexpr unsigned gp_zero() {
+  return sizeof(T) == 8 ? 0x1e500000u : 32u;
+}
+template <typename T> __device__ __forceinline__ constexpr unsigned gp_small() {
+  return sizeof(T) == 8 ? 0x20000000u : 0x00800000u;
+}
 // a magnitude above this is not a number
 template <typename T> __device__ __forceinline__ constexpr unsigned gp_inf() {
   return sizeof(T) == 8 ? 0x7ff00000u : 0x7f800000u;
@@ -290,10 +298,15 @@ __global__ void __launch_bounds__(GP_MAXW * 32) gjp_panel_kernel(PanelArgs g, C_
       const unsigned char* src = wst + ((size_t)buf * GP_MAXW + cw) * SLOT;
       if (cw + warp == 15u) {  // 1 / pivot, by the warp that holds the candidate
         C pv = *reinterpret_cast<const C*>(src + j * CS);
-        if (gp_mag(pv) == 0u) pv = mk(sizeof(T) == 8 ? (T)1e-150 : (T)1e-18, (T)0);
-        const T rd = (T)1 / (pv.x * pv.x + pv.y * pv.y);
+        if (gp_mag(pv) < gp_zero<T>()) pv = mk(sizeof(T) == 8 ? (T)1e-150 : (T)1e-18, (T)0);
+        const T pd = pv.x * pv.x + pv.y * pv.y;
         alignas(16) C pi[16 / CS] = {};
-        pi[0] = mk(pv.x * rd, -pv.y * rd);
+        if (gp_mag(pv) < gp_small<T>()) {
+          pi[0] = mk(pv.x / pd, -pv.y / pd);
+        } else {
+          const T rd = (T)1 / pd;
+          pi[0] = mk(pv.x * rd, -pv.y * rd);
+        }
         const float4 val = *reinterpret_cast<const float4*>(pi);
         if (lane < CL)
           tc::st_async16(tc::cluster_map(cand_a + (uint32_t)(buf * CL * SLOT + NP * 16), lane), val,
@@ -315,7 +328,7 @@ __global__ void __launch_bounds__(GP_MAXW * 32) gjp_panel_kernel(PanelArgs g, C_
       const int sl = min(lane, CL - 1);
       const unsigned cmax = __reduce_max_sync(
           0xffffffffu, gp_mag(*reinterpret_cast<const C*>(cb + (size_t)sl * SLOT + j * CS)) | sl);
-      singular |= cmax < 32u || (cmax & ~31u) > gp_inf<T>();
+      singular |= cmax < gp_zero<T>() || (cmax & ~31u) > gp_inf<T>();
       const int pc = (int)(cmax & 31u);
       src = cb + (size_t)pc * SLOT;
       const C pinv = *reinterpret_cast<const C*>(src + NP * 16);

@@ -299,7 +299,7 @@ __host__ __device__ constexpr int tc2_sets(int kp) {
 }
 // Where one set fits (64 columns), a second accumulator of hi.hi alone takes every other
 // K step of the TF32 split (384 rows, 24 problems: unrefined residual 1.0e-5 instead
-// of 8.7e-6 without it, 4.7e-5 and 3.8e-5 adjoint; 0 to 2 % of a solve).  BF16x3's
+// of 8.7e-6 without it, 4.7e-5 and 3.8e-5 adjoint; 0 to 3 % of a solve).  BF16x3's
 // errors are its products'.
 template <int SPLIT>
 __host__ __device__ constexpr int tc2_extra(int kp) {
