@@ -788,12 +788,7 @@ rr_status launch_gram(int F, int N, int k, const double2* Y, double2* part, int 
 rr_status launch_cholesky(int F, int k, const double2* G, double2* R, double2* Rinv, int* bad,
                           double shift_rel, double* cond, cudaStream_t st) {
   size_t smem = (size_t)2 * k * k * sizeof(double2);
-  static bool attr = false;
-  if (!attr) {
-    RR_CUDA(cudaFuncSetAttribute(cholesky_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 2 * 64 * 64 * (int)sizeof(double2)));
-    attr = true;
-  }
+  RR_TRY(smem_opt_in<cholesky_kernel>(2 * 64 * 64 * sizeof(double2)));
   prof_begin(PROF_SMALL, st);
   cholesky_kernel<<<F, 256, smem, st>>>(k, G, R, Rinv, bad, shift_rel, cond);
   prof_end(PROF_SMALL, st);
@@ -805,14 +800,8 @@ rr_status launch_right_mul(int F, int N, int k, const double2* Y, const double2*
                            cudaStream_t st, int upper) {
   int RB = 64;
   size_t smem = ((size_t)k * k + (size_t)RB * k) * sizeof(double2);
-  static bool attr = false;
-  if (!attr) {
-    RR_CUDA(cudaFuncSetAttribute(right_mul_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 160 * 1024));
-    RR_CUDA(cudaFuncSetAttribute(right_mul_upper_kernel,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
-    attr = true;
-  }
+  RR_TRY(smem_opt_in<right_mul_kernel>(160 * 1024));
+  RR_TRY(smem_opt_in<right_mul_upper_kernel>(160 * 1024));
   int nb = (N + RB - 1) / RB;
   if (nb > 152 * 4 / (F > 0 ? F : 1) + 1) nb = 152 * 4 / (F > 0 ? F : 1) + 1;
   prof_begin(PROF_RIGHTMUL, st);

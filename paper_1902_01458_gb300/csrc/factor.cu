@@ -508,18 +508,14 @@ __global__ void gjp_finalize_kernel(OpView op, int ldg, int nh, int col0, int co
 }
 
 template <typename T>
-void launch_schur(const OpView& ov, const double2* shifts, int F, int nh, int col0, int col1,
+rr_status launch_schur(const OpView& ov, const double2* shifts, int F, int nh, int col0, int col1,
                   int dx0, int add, const C_t<T>* Xprev, C_t<T>* M, cudaStream_t st) {
   constexpr int CB = SchurCfg<T>::CB;
   const size_t smem = Xprev ? schur_smem<T>(ov.q) : 0;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(schur_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)schur_smem<T>(4));
-    attr = true;
-  }
+  RR_TRY(smem_opt_in<schur_kernel<T>>(schur_smem<T>(4)));
   dim3 gs((ov.ny + SCHUR_Y - 1) / SCHUR_Y * nh, (ov.b + CB - 1) / CB, F);
   schur_kernel<T><<<gs, CB, smem, st>>>(ov, shifts, nh, col0, col1, dx0, add, Xprev, M);
+  return RR_OK;
 }
 
 // M = S_i for step t of the factorisation (twist_steps)
@@ -531,12 +527,13 @@ rr_status schur_step(rr_factors* fa, const TwistStep& t, cudaStream_t st) {
   C* M = reinterpret_cast<C*>(fa->M);
   const C* X = reinterpret_cast<const C*>(fa->X);
   prof_begin(PROF_SCHUR, st);
-  launch_schur<T>(ov, fa->shifts, fa->F, t.nh, t.col0, t.col1, -1, 0, t.first ? nullptr : X, M, st);
+  RR_TRY(launch_schur<T>(ov, fa->shifts, fa->F, t.nh, t.col0, t.col1, -1, 0,
+                         t.first ? nullptr : X, M, st));
   prof_end(PROF_SCHUR, st);
   if (t.middle) {
     prof_begin(PROF_SCHUR, st);
-    launch_schur<T>(ov, fa->shifts, fa->F, 1, t.col0, t.col1, 1, 1, X + (size_t)fa->F * d.b * d.b,
-                    M, st);
+    RR_TRY(launch_schur<T>(ov, fa->shifts, fa->F, 1, t.col0, t.col1, 1, 1,
+                           X + (size_t)fa->F * d.b * d.b, M, st));
     prof_end(PROF_SCHUR, st);
   }
   RR_CUDA(cudaGetLastError());
@@ -559,12 +556,7 @@ rr_status launch_panel(rr_factors* fa, int nh, int k0, int nbk, int kp0, cudaStr
   a.flag = fa->flag;
   a.tries = wait_tries();
   const size_t smem = panel_smem<T>(a.rpc, a.CL);
-  static bool attr = false;
-  if (!attr) {
-    RR_CUDA(cudaFuncSetAttribute(gjp_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)panel_smem<T>(GP_MAXW * 8, GP_CLMAX)));
-    attr = true;
-  }
+  RR_TRY(smem_opt_in<gjp_panel_kernel<T>>(panel_smem<T>(GP_MAXW * 8, GP_CLMAX)));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.CL * fa->F * nh), 1, 1);
   cfg.blockDim = dim3((unsigned)((a.rpc * GP_LPR + 31) / 32 * 32), 1, 1);
@@ -595,11 +587,9 @@ rr_status factor_impl(rr_factors* fa) {
   C* G = reinterpret_cast<C*>(fa->G);
   C* X = reinterpret_cast<C*>(fa->X);
   C* Bbuf = reinterpret_cast<C*>(fa->Bbuf);
-  int RB = 4;
-  while (RB > 1 && (size_t)RB * b * sizeof(C) + b * sizeof(int) > 160 * 1024) RB >>= 1;
-  const size_t fsmem = (size_t)RB * b * sizeof(C) + b * sizeof(int);
-  RR_CUDA(cudaFuncSetAttribute(gjp_finalize_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)fsmem));
+  constexpr int RB = 4;
+  const size_t fsmem = (size_t)RB * b * sizeof(C) + b * sizeof(int);  // (b <= 1024)
+  RR_TRY(smem_opt_in<gjp_finalize_kernel<T>>(RB * 1024 * sizeof(C) + 1024 * sizeof(int)));
   constexpr int TR = UpdCfg<T>::TR;
   const int nt = (b + TR - 1) / TR, P = (b + NB - 1) / NB;
   rr_status s;

@@ -527,17 +527,9 @@ rr_status launch_slab(rr_factors* fa, int nh, int c0, int c1, cudaStream_t st) {
   a.tries = wait_tries();
   const size_t smem = slab_smem_bytes(a.rpc, a.CL);
   const int lpr = slab_lpr(a.rpc);
-  static bool attr = false;
-  if (!attr) {
-    constexpr int cap = (int)SL_SMEM_CAP;
-    RR_CUDA(cudaFuncSetAttribute(gjw_slab_kernel<true, 2>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-    RR_CUDA(cudaFuncSetAttribute(gjw_slab_kernel<true, 4>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-    RR_CUDA(cudaFuncSetAttribute(gjw_slab_kernel<false, 4>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-    attr = true;
-  }
+  RR_TRY((smem_opt_in<gjw_slab_kernel<true, 2>>(SL_SMEM_CAP)));
+  RR_TRY((smem_opt_in<gjw_slab_kernel<true, 4>>(SL_SMEM_CAP)));
+  RR_TRY((smem_opt_in<gjw_slab_kernel<false, 4>>(SL_SMEM_CAP)));
   prof_begin(PROF_PANEL, st);
   if (a.CL == 1) {
     if (lpr == 4) gjw_slab_kernel<true, 4><<<P, SL_THREADS, smem, st>>>(a);
@@ -980,12 +972,7 @@ rr_status launch_gemm(rr_factors* fa, int nh, const CUtensorMap* ta, const CUten
   // and the second stream's panels find SMs as they free up
   const long nsm = num_sms(d.device);
   const int grid = (int)(items <= 8 * nsm ? std::min<long>(items, nsm) : (items + 3) / 4);
-  static bool attr = false;
-  if (!attr) {
-    RR_CUDA(cudaFuncSetAttribute(gjw_gemm_kernel<SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)gg_smem_bytes<SPLIT>()));
-    attr = true;
-  }
+  RR_TRY(smem_opt_in<gjw_gemm_kernel<SPLIT>>(gg_smem_bytes<SPLIT>()));
   prof_begin(PROF_UPDATE, st);
   gjw_gemm_kernel<SPLIT><<<grid, GG_THREADS, gg_smem_bytes<SPLIT>(), st>>>(*ta, *tb, a);
   prof_end(PROF_UPDATE, st);
@@ -1006,8 +993,8 @@ rr_status factor_wide_impl(rr_factors* fa) {
   const CUtensorMap* tBout = reinterpret_cast<const CUtensorMap*>(fa->wmap[1]);
   const int RB = 8;
   const size_t fsmem = (size_t)RB * b * sizeof(float2) + b * sizeof(int);
-  RR_CUDA(cudaFuncSetAttribute(gjw_finalize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)fsmem));
+  RR_TRY(smem_opt_in<gjw_finalize_kernel>((size_t)RB * GW_MAX * sizeof(float2) +
+                                          GW_MAX * sizeof(int)));
   const int nct_all = (b + GG_CT - 1) / GG_CT;
   for (int step = 0; step < twist_steps(fa); ++step) {
     const TwistStep t = twist_step(fa, step);
@@ -1086,8 +1073,7 @@ int cluster_slots(int device, int cl) {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (cudaFuncSetAttribute(gjw_slab_kernel<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SL_SMEM_CAP) != cudaSuccess ||
+    if (smem_opt_in<gjw_slab_kernel<false, 4>>(SL_SMEM_CAP) != RR_OK ||
         cudaOccupancyMaxActiveClusters(&n, gjw_slab_kernel<false, 4>, &cfg) != cudaSuccess ||
         n <= 0) {
       cudaGetLastError();

@@ -2,6 +2,8 @@
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <atomic>
 #include <stdint.h>
 
 #include <string>
@@ -211,6 +213,26 @@ rr_status cuda_status(cudaError_t e, const char* what);
   do {                                                            \
     cudaError_t _e = (call);                                      \
     if (_e != cudaSuccess) return cuda_status(_e, #call);         \
+  } while (0)
+
+// Opts Kernel in to `bytes` of dynamic shared memory on the current device, once per
+// device: the attribute belongs to the device, and always the most that any call
+// takes, so that no thread lowers it under another's launch.
+template <auto Kernel>
+rr_status smem_opt_in(size_t bytes) {
+  static std::atomic<bool> done[64];
+  int dev = 0;
+  RR_CUDA(cudaGetDevice(&dev));
+  const bool known = dev >= 0 && dev < 64;
+  if (known && done[dev].load(std::memory_order_acquire)) return RR_OK;
+  RR_CUDA(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  if (known) done[dev].store(true, std::memory_order_release);
+  return RR_OK;
+}
+#define RR_TRY(call)                    \
+  do {                                  \
+    const rr_status _s = (call);        \
+    if (_s != RR_OK) return _s;         \
   } while (0)
 
 // ------------------------------------------------------- kernel launchers

@@ -844,12 +844,8 @@ rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
                      const SweepStep& step, int nx, int nrt, int KS, int cpp, const float2* rhs,
                      size_t rstride, size_t hstride, bool first, rr_factors* fa, cudaStream_t st) {
   const size_t smem = tc2_smem_bytes<SPLIT>(kp) + 1024;
-  static size_t attr = 0;  // dynamic shared memory opted in so far
-  if (smem > attr) {
-    RR_CUDA(cudaFuncSetAttribute(sweep_tc2_kernel<TRANS, SPLIT, WIDE>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = smem;
-  }
+  RR_TRY((smem_opt_in<sweep_tc2_kernel<TRANS, SPLIT, WIDE>>(
+      tc2_smem_bytes<SPLIT>(WIDE ? 64 : 32) + 1024)));
   // dependent launch, but for the first: its predecessor is not of this solve
   cudaLaunchAttribute at[1];
   const cudaLaunchConfig_t cfg = dependent_launch(dim3(grid_x), TC2_THREADS, smem, st, at, !first);
@@ -870,8 +866,7 @@ rr_status launch_cc(int k, int kp, const SweepStep& step, const float2* rhs, siz
   const OpDev& d = fa->op->d;
   const int nrt = (d.b * kp + CC_RT - 1) / CC_RT, Fa = active_count(fa);
   const size_t smem = (size_t)CC_STAGES * cc_stage<TRANS>(kp) * sizeof(float2);
-  RR_CUDA(cudaFuncSetAttribute(sweep_cc_kernel<TRANS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               227 * 1024));
+  RR_TRY(smem_opt_in<sweep_cc_kernel<TRANS>>(CC_STAGES * cc_stage<TRANS>(8) * sizeof(float2)));
   sweep_cc_kernel<TRANS><<<nrt * Fa * step.nh, CC_THREADS, smem, st>>>(
       reinterpret_cast<const float2*>(fa->G), d.b, fa->ldg, k, kp, step, d.nx, nrt, rhs, rstride,
       hstride, reinterpret_cast<float2*>(fa->Pbuf), fa->F, Fa, fa->amap);

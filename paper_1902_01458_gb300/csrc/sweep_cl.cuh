@@ -511,12 +511,7 @@ Plan make_plan(const OpDev& d, int Fa, int k, int trans) {
 
 template <typename T, bool TRANS, int LC, int CPL, int RPL>
 rr_status launch(const Args<T>& a, int clusters, size_t smem, int W, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    RR_CUDA(cudaFuncSetAttribute(sweep_cl_kernel<T, TRANS, LC, CPL, RPL>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_CAP));
-    attr = true;
-  }
+  RR_TRY((smem_opt_in<sweep_cl_kernel<T, TRANS, LC, CPL, RPL>>(SMEM_CAP)));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.CL * clusters), 1, 1);
   cfg.blockDim = dim3((unsigned)(32 * W), 1, 1);

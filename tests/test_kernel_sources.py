@@ -30,3 +30,15 @@ def test_data_of_a_running_predecessor_is_not_declared_constant():
     rhs = [p for p in _parameters(_source("sweep.cu"), "sweep_tc2_kernel")
            if re.search(r"\brhs$", p)]
     assert rhs == ["const float2* rhs"]
+
+
+def test_shared_memory_is_opted_in_per_device():
+    """The opt-in to more than 48 KB of dynamic shared memory belongs to a device and is
+    the same for every call: one helper sets it, and no process-wide flag skips it."""
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith((".cu", ".cuh")):
+            continue
+        src = _source(name)
+        assert not re.search(r"static\s+(bool|size_t|int)\s+\w*attr", src), name
+        calls = src.count("cudaFuncSetAttribute(")
+        assert calls == (1 if name == "rr_internal.cuh" else 0), name
