@@ -10,7 +10,7 @@
 //     S_0 = D_0,  G_i = S_i^{-1},  X_i = G_i C_i,  S_{i+1} = D_{i+1} - A_{i+1} X_i
 //     S_{nx-1} = D_{nx-1},  X_i = G_i A_i,  S_{i-1} = D_{i-1} - C_{i-1} X_i
 //     S_m = D_m - A_m X_{m-1} - C_m X_{m+1}.
-// Work buffers hold 2 F problems: problem f of half h at index h F + f.  Measured
+// Work buffers hold both halves: problem f of half h at index h F + f.  Measured
 // against the same kernels run from one end, factorisation and solves: two
 // frequencies of 128 x 64 points 13.5 ms instead of 25.5, six of 512 x 256 points
 // 401 instead of 619; in FP64 four of 128 x 64 points and their gradient 75
@@ -182,7 +182,8 @@ struct PanelArgs {
   int b, k0, nbk, kp0, rpc, CL, F;
   int* rowpiv;    // [F][b]
   int* pivslot;   // [F][b]
-  int* flag;      // [F] singular flags, [F] = wait timeout
+  int* flag;      // [F] singular flags
+  int* err;       // wait timeout
   uint32_t tries;
 };
 
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(GP_MAXW * 32) gjp_panel_kernel(PanelArgs g, C_
     }
   }
   if (rank == 0 && tid == 0 && singular) g.flag[f % g.F] = 1;
-  if (!ok && lane == 0) atomicExch(g.flag + g.F, 1);
+  if (!ok && lane == 0) atomicExch(g.err, 1);
   if (!ok) tc::cluster_settle();
   tc::cluster_sync();  // no CTA leaves while another may still send to it
 }
@@ -554,6 +555,7 @@ rr_status launch_panel(rr_factors* fa, int nh, int k0, int nbk, int kp0, cudaStr
   a.rowpiv = fa->rowpiv;
   a.pivslot = fa->pivslot;
   a.flag = fa->flag;
+  a.err = fa->err;
   a.tries = wait_tries();
   const size_t smem = panel_smem<T>(a.rpc, a.CL);
   RR_TRY(smem_opt_in<gjp_panel_kernel<T>>(panel_smem<T>(GP_MAXW * 8, GP_CLMAX)));
@@ -658,7 +660,21 @@ rr_status launch_schur_f32(rr_factors* fa, const TwistStep& t, cudaStream_t st) 
 }
 
 rr_status launch_factor(rr_factors* fa) {
-  if (fa->prec == RR_FP64) return factor_impl<double>(fa);
-  if (factor_wide_ok(fa) && fa->tune_update != 1) return launch_factor_wide(fa);
-  return factor_impl<float>(fa);
+  const OpDev& d = fa->op->d;
+  const bool wide = fa->prec != RR_FP64 && factor_wide_ok(fa) && fa->tune_update != 1;
+  if (fa->Fw < 1) {
+    set_error("no memory for the factorisation's work buffers");
+    return RR_ERR_NOMEM;
+  }
+  for (int f0 = 0; f0 < fa->F; f0 += fa->Fw) {
+    rr_factors part = *fa;  // the problems of this pass (the work buffers are shared)
+    part.F = std::min(fa->Fw, fa->F - f0);
+    part.G = static_cast<char*>(fa->G) + (size_t)f0 * d.nx * d.b * fa->ldg * fa->csz;
+    part.shifts = fa->shifts + f0;
+    part.flag = fa->flag + f0;
+    RR_TRY(fa->prec == RR_FP64 ? factor_impl<double>(&part)
+           : wide              ? launch_factor_wide(&part)
+                               : factor_impl<float>(&part));
+  }
+  return RR_OK;
 }

@@ -98,7 +98,8 @@ struct SlabArgs {
   float2* M;                     // [2F][b][b]
   int* rowpiv;                   // [2F][b]
   int* pivslot;                  // [2F][b]
-  int* flag;                     // [F] singular flags, [F] = wait timeout
+  int* flag;                     // [F] singular flags
+  int* err;                      // wait timeout
   int F;
   uint32_t tries;
 };
@@ -480,7 +481,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) gjw_slab_kernel(SlabArgs g) {
     }
   }
   if (rank == 0 && tid == 0 && singular) g.flag[f % g.F] = 1;
-  if (!ok && lane == 0) atomicExch(g.flag + g.F, 1);
+  if (!ok && lane == 0) atomicExch(g.err, 1);
   if (!ok) tc::cluster_settle();
   if (!SOLO) tc::cluster_sync();  // no CTA leaves while another may still send to it
 }
@@ -524,6 +525,7 @@ rr_status launch_slab(rr_factors* fa, int nh, int c0, int c1, cudaStream_t st) {
   a.rowpiv = fa->rowpiv;
   a.pivslot = fa->pivslot;
   a.flag = fa->flag;
+  a.err = fa->err;
   a.tries = wait_tries();
   const size_t smem = slab_smem_bytes(a.rpc, a.CL);
   const int lpr = slab_lpr(a.rpc);
@@ -962,7 +964,7 @@ rr_status launch_gemm(rr_factors* fa, int nh, const CUtensorMap* ta, const CUten
   a.x0 = x0; a.x1 = x1; a.y0 = y0; a.y1 = y1;
   a.M = reinterpret_cast<float2*>(fa->M);
   a.rowpiv = fa->rowpiv;
-  a.err = fa->flag + fa->F;
+  a.err = fa->err;
   a.tries = wait_tries();
   const int nrt = (d.b + GG_RT - 1) / GG_RT;
   const long items = (long)a.F * nrt * ((x1 - x0) + (y1 - y0));

@@ -18,6 +18,8 @@
 // ---------------------------------------------------------------- errors
 static thread_local std::string g_err;
 
+static rr_status shrink_factor_work(rr_factors* fa, int Fw);
+
 void set_error(const std::string& msg) { g_err = msg; }
 
 rr_status cuda_status(cudaError_t e, const char* what) {
@@ -163,6 +165,12 @@ rr_status get_work(rr_factors* fa, int k, Work* w) {
     }
     size_t bytes = carve(fa, k, nullptr, nullptr);
     rr_status s = dalloc(reinterpret_cast<char**>(&fa->ws), bytes);
+    // the factorisation gives way: it can run over fewer problems at a time
+    while (s == RR_ERR_NOMEM && !fa->is_view && fa->Fw > 1) {
+      cudaStreamSynchronize(fa->stream);
+      if ((s = shrink_factor_work(fa, fa->Fw)) == RR_OK)
+        s = dalloc(reinterpret_cast<char**>(&fa->ws), bytes);
+    }
     if (s != RR_OK) return s;
     fa->ws_bytes = bytes;
     fa->kmax = k;
@@ -187,10 +195,10 @@ void info_reset(rr_info* info) {
 rr_status sweep_status(rr_factors* fa) {
   int tc_err = 0;
   cudaStream_t st = fa->stream;
-  RR_CUDA(cudaMemcpyAsync(&tc_err, fa->flag + fa->F, sizeof(int), cudaMemcpyDeviceToHost, st));
+  RR_CUDA(cudaMemcpyAsync(&tc_err, fa->err, sizeof(int), cudaMemcpyDeviceToHost, st));
   RR_CUDA(cudaStreamSynchronize(st));
   if (!tc_err) return RR_OK;
-  RR_CUDA(cudaMemsetAsync(fa->flag + fa->F, 0, sizeof(int), st));
+  RR_CUDA(cudaMemsetAsync(fa->err, 0, sizeof(int), st));
   RR_CUDA(cudaStreamSynchronize(st));
   g_err = "a sweep kernel timed out in a bounded wait";
   return RR_ERR_TIMEOUT;
@@ -511,7 +519,7 @@ static int encode_factor_maps(rr_factors* fa) {
 // columns x 128 rows of M (the left operand of the rank-128 update, read in
 // place), and tiles of 16 rows x 64 complex of the gathered pivot rows Wbuf
 // [F][128][b] (its right operand).
-static int encode_wide_maps(rr_factors* fa) {
+static int encode_wide_maps(rr_factors* fa, int Fw) {
   const OpDev& d = fa->op->d;
   cudaDriverEntryPointQueryResult q;
   void* fn = nullptr;
@@ -523,10 +531,10 @@ static int encode_wide_maps(rr_factors* fa) {
   }
   auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   const cuuint32_t es[3] = {1, 1, 1};
-  const cuuint64_t dm[3] = {(cuuint64_t)2 * d.b, (cuuint64_t)d.b, (cuuint64_t)2 * fa->F};
+  const cuuint64_t dm[3] = {(cuuint64_t)2 * d.b, (cuuint64_t)d.b, (cuuint64_t)2 * Fw};
   const cuuint64_t sm[2] = {(cuuint64_t)2 * d.b * 4, (cuuint64_t)2 * d.b * d.b * 4};
   const cuuint32_t boxA[3] = {32, 128, 1}, boxB[3] = {128, 16, 1};
-  const cuuint64_t dw[3] = {(cuuint64_t)2 * d.b, 128, (cuuint64_t)2 * fa->F};
+  const cuuint64_t dw[3] = {(cuuint64_t)2 * d.b, 128, (cuuint64_t)2 * Fw};
   const cuuint64_t sw[2] = {(cuuint64_t)2 * d.b * 4, (cuuint64_t)2 * d.b * 128 * 4};
   CUresult r0 = encode(reinterpret_cast<CUtensorMap*>(fa->wmap[0]), CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                        3, fa->M, dm, sm, boxA, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -537,6 +545,46 @@ static int encode_wide_maps(rr_factors* fa) {
                        CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return (r0 == CUDA_SUCCESS && r1 == CUDA_SUCCESS) ? 1 : 0;
+}
+
+// Work buffers of the factorisation for passes over Fw problems; they hold nothing
+// between factorisations.
+static void free_factor_work(rr_factors* fa) {
+  for (void** p : {&fa->X, &fa->M, &fa->Bbuf, &fa->Wbuf}) {
+    cudaFree(*p);
+    *p = nullptr;
+  }
+  for (int** p : {&fa->rowpiv, &fa->pivslot}) {
+    cudaFree(*p);
+    *p = nullptr;
+  }
+}
+
+static rr_status alloc_factor_work(rr_factors* fa, int Fw) {
+  const OpDev& d = fa->op->d;
+  const size_t n = (size_t)2 * Fw;
+  free_factor_work(fa);
+  fa->Fw = 0;
+  RR_TRY(dalloc(&fa->X, n * d.b * d.b * fa->csz));
+  RR_TRY(dalloc(&fa->M, n * d.b * d.b * fa->csz));
+  RR_TRY(dalloc(&fa->Bbuf, n * 16 * d.b * fa->csz));
+  RR_TRY(dalloc(&fa->rowpiv, n * d.b * sizeof(int)));
+  RR_TRY(dalloc(&fa->pivslot, n * d.b * sizeof(int)));
+  if (tc_prec(fa->prec) && d.b >= 64 && d.b <= 768 && d.b % 8 == 0) {
+    RR_TRY(dalloc(&fa->Wbuf, n * 128 * d.b * sizeof(float2)));
+    fa->wide_ok = encode_wide_maps(fa, Fw);
+  }
+  // a row index in every entry, also of a factorisation that found no pivot
+  RR_CUDA(cudaMemsetAsync(fa->pivslot, 0, n * d.b * sizeof(int), fa->stream));
+  fa->Fw = Fw;
+  return RR_OK;
+}
+
+// The same for fewer problems at a time, half of them at most, as memory allows
+static rr_status shrink_factor_work(rr_factors* fa, int Fw) {
+  rr_status s = RR_ERR_NOMEM;
+  while (s == RR_ERR_NOMEM && Fw > 1) s = alloc_factor_work(fa, Fw = (Fw + 1) / 2);
+  return s;
 }
 
 // ----------------------------------------------------------------- operator
@@ -724,18 +772,12 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
   fa->stream = reinterpret_cast<cudaStream_t>(stream);
   fa->csz = prec == RR_FP64 ? sizeof(double2) : sizeof(float2);
   fa->ldg = tc_prec(prec) ? (d.b + 1) & ~1 : d.b;
-  const size_t bb = (size_t)d.b * d.b;
   rr_status s;
   auto fail = [&](rr_status st) {
     rr_destroy_factors(fa);
     return st;
   };
   if ((s = dalloc(&fa->G, (size_t)nshift * d.nx * d.b * fa->ldg * fa->csz)) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->X, (size_t)2 * nshift * bb * fa->csz)) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->M, (size_t)2 * nshift * bb * fa->csz)) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->Bbuf, (size_t)2 * nshift * 16 * d.b * fa->csz)) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->rowpiv, (size_t)2 * nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
-  if ((s = dalloc(&fa->pivslot, (size_t)2 * nshift * d.b * sizeof(int))) != RR_OK) return fail(s);
   if ((s = dalloc(&fa->Tbuf, (size_t)nshift * 128 * d.b * fa->csz)) != RR_OK) return fail(s);
   if (prec != RR_FP64)
     if ((s = dalloc(&fa->Pbuf, (size_t)(tc_prec(prec) ? 4 : 2) * nshift * 64 * d.b * sizeof(float2))) !=
@@ -743,17 +785,17 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
       return fail(s);
   if (tc_prec(prec)) {
     fa->tma_ok = encode_factor_maps(fa);
-    if (d.b >= 64 && d.b <= 768 && d.b % 8 == 0) {
-      if ((s = dalloc(&fa->Wbuf, (size_t)2 * nshift * 128 * d.b * sizeof(float2))) != RR_OK)
-        return fail(s);
-      fa->wide_ok = encode_wide_maps(fa);
-    }
   }
   // flags: one singular-pivot flag per shift, then the tensor-core wait flag,
   // then room for the active-problem list of the refinement
   if ((s = dalloc(&fa->flag, (size_t)(2 * nshift + 1) * sizeof(int))) != RR_OK) return fail(s);
+  fa->err = fa->flag + nshift;
   fa->amap_buf = fa->flag + nshift + 1;
   if ((s = dalloc(&fa->shifts, (size_t)nshift * sizeof(double2))) != RR_OK) return fail(s);
+  // both halves of all problems at once, or of as many as fit
+  s = alloc_factor_work(fa, nshift);
+  if (s == RR_ERR_NOMEM) s = shrink_factor_work(fa, nshift);
+  if (s != RR_OK) return fail(s);
   {
     // the look-ahead panel stream gets the highest priority so its CTAs are
     // scheduled ahead of the trailing update's as SMs free up
@@ -774,9 +816,6 @@ extern "C" rr_status rr_factor(rr_operator* op, int nshift, const double* shifts
   if (e != cudaSuccess) return fail(cuda_status(e, "rr_factor shifts"));
   e = cudaMemsetAsync(fa->flag, 0, (nshift + 1) * sizeof(int), st);
   if (e != cudaSuccess) return fail(cuda_status(e, "rr_factor flags"));
-  // a row index in every entry, also of a factorisation that found no pivot
-  e = cudaMemsetAsync(fa->pivslot, 0, (size_t)2 * nshift * d.b * sizeof(int), st);
-  if (e != cudaSuccess) return fail(cuda_status(e, "rr_factor pivots"));
   if ((s = launch_factor(fa)) != RR_OK) return fail(s);
   std::vector<int> flags(nshift + 1);
   e = cudaMemcpyAsync(flags.data(), fa->flag, (nshift + 1) * sizeof(int), cudaMemcpyDeviceToHost,
@@ -810,14 +849,9 @@ extern "C" rr_status rr_destroy_factors(rr_factors* fa) {
   cudaFree(fa->chk);
   delete fa->sched;
   delete fa->chk_desc;
-  cudaFree(fa->X);
-  cudaFree(fa->M);
-  cudaFree(fa->Bbuf);
+  free_factor_work(fa);
   cudaFree(fa->Tbuf);
   cudaFree(fa->Pbuf);
-  cudaFree(fa->rowpiv);
-  cudaFree(fa->pivslot);
-  cudaFree(fa->Wbuf);
   cudaFree(fa->flag);
   cudaFree(fa->ws);
   if (fa->stream2) {
@@ -868,6 +902,7 @@ rr_status factors_view(rr_factors* parent, int f0, int nf, cudaStream_t st, rr_f
     v->tma_ok = encode_factor_maps(v);
   }
   if ((s = dalloc(&v->flag, (size_t)(2 * nf + 1) * sizeof(int))) != RR_OK) return fail(s);
+  v->err = v->flag + nf;
   v->amap_buf = v->flag + nf + 1;
   RR_CUDA(cudaMemsetAsync(v->flag, 0, (nf + 1) * sizeof(int), st));
   v->shifts_h = new double2[nf];

@@ -141,22 +141,25 @@ struct rr_factors {
   size_t csz;        // bytes of one complex element of the factors
   void* G;           // [F][nx][b][ldg]  inverse of each Schur block
   int ldg;           // row pitch of G: b, for the tensor cores the next even number
-  // The factorisation runs from both ends to the middle column (factor.cu):
-  // its work buffers hold 2 F problems, problem f of half h at h F + f.
-  void* X;           // [2F][b][b] X_i = G_i C_i (G_i A_i) of the current columns (transient)
-  void* M;           // [2F][b][b] work matrices
-  void* Bbuf;        // [2F][16][b] saved pivot rows of the current panel
+  // The factorisation runs from both ends to the middle column (factor.cu), Fw
+  // problems at a time (F, or as many as the memory left holds): its work buffers
+  // hold 2 Fw problems, problem f of half h of a pass over n problems at h n + f.
+  int Fw;
+  void* X;           // [2Fw][b][b] X_i = G_i C_i (G_i A_i) of the current columns (transient)
+  void* M;           // [2Fw][b][b] work matrices
+  void* Bbuf;        // [2Fw][16][b] saved pivot rows of the current panel
   void* Tbuf;        // [2][F][b][64] right-hand sides (or edge blocks) of both halves
   void* Pbuf;        // [4][F][b][64] partial products of the split tensor-core sweep
   alignas(64) unsigned char tmap[2][128];  // TMA maps: G tiles, G^H tiles (FP32)
   int tma_ok;        // 1 if the maps of G were encoded
-  int* rowpiv;       // [2F][b] pivot column of each row (-1: not yet pivoted)
-  int* pivslot;      // [2F][b] pivot row of each column
+  int* rowpiv;       // [2Fw][b] pivot column of each row (-1: not yet pivoted)
+  int* pivslot;      // [2Fw][b] pivot row of each column
   // slab (two-level) factorisation of FP32 factors
   int wide_ok;       // 1 if the buffers and TMA maps below exist
-  void* Wbuf;        // [2F][128][b] gathered pivot rows of a slab (outer update)
+  void* Wbuf;        // [2Fw][128][b] gathered pivot rows of a slab (outer update)
   alignas(64) unsigned char wmap[2][128];  // TMA maps: A chunks of M, Wbuf rows
   int* flag;         // [F] singular-pivot flags
+  int* err;          // flag + F: a bounded wait gave up
   double2* shifts;   // [F] device
   double2* shifts_h; // [F] host copy
   // workspace for the sketch (allocated lazily, sized for kmax)

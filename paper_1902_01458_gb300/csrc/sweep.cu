@@ -851,7 +851,7 @@ rr_status launch_tc2(const CUtensorMap* tm, int grid_x, int b, int k, int kp,
   const cudaLaunchConfig_t cfg = dependent_launch(dim3(grid_x), TC2_THREADS, smem, st, at, !first);
   RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_tc2_kernel<TRANS, SPLIT, WIDE>, *tm, b, k, kp, step, nx, nrt,
                              KS, cpp, rhs, rstride, hstride, reinterpret_cast<float2*>(fa->Pbuf),
-                             fa->F, active_count(fa), (const int*)fa->amap, fa->flag + fa->F,
+                             fa->F, active_count(fa), (const int*)fa->amap, fa->err,
                              wait_tries(), take_stall()));
   return RR_OK;
 }

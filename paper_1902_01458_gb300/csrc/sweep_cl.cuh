@@ -564,7 +564,7 @@ rr_status launch_plan(rr_factors* fa, const Plan& p, int k, const void* in, void
   a.npt = p.npt;
   a.CL = p.CL;
   a.amap = fa->amap;
-  a.err = fa->flag + fa->F;
+  a.err = fa->err;
   a.tries = wait_tries();
   const int clusters = 2 * active_count(fa) * a.ng;
   const size_t smem = smem_bytes<T, TRANS>(d.b, p.npt * d.q, d.q, p.kc, p.W);
