@@ -365,7 +365,7 @@ rr_status tune(rr_batch* B) {
   // K-split of each view's tensor-core sweep
   for (auto& G : B->groups)
     for (auto& v : G.views) {
-      if (!sweep_tc2_ok(v.fa, v.k)) continue;
+      if (!sweep_tc2_taken(v.fa, v.k, 0) && !sweep_tc2_taken(v.fa, v.k, 1)) continue;
       float best = INFINITY;
       int best_ks = 0;
       for (int ks = 0; ks <= 4; ++ks) {

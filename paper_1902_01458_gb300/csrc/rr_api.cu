@@ -362,7 +362,6 @@ rr_status solve_refined(rr_factors* fa, int k, int adjoint, const double2* b, do
                               cudaMemcpyHostToDevice, st));
       fa->amap = fa->amap_buf;
       fa->Fa = (int)act.size();
-      fa->amap_h = act;
       if ((s = launch_convert_d2f_map(fa->Fa, fa->amap, nk, w.R64, (float2*)w.L1, st)) != RR_OK)
         return s;
       if ((s = launch_solve_lo(fa, k, adjoint, w.L1, w.L2, w.L3)) != RR_OK) return s;

@@ -54,10 +54,6 @@ template <typename C, typename R> __device__ __forceinline__ C crfma(R r, C b, C
   return c;
 }
 template <typename C> __device__ __forceinline__ auto cabs2(C a) -> decltype(a.x) { return a.x * a.x + a.y * a.y; }
-template <typename C> __device__ __forceinline__ C cinv(C a) {
-  auto d = a.x * a.x + a.y * a.y;
-  return mk(a.x / d, -a.y / d);
-}
 template <typename To, typename From> __device__ __forceinline__ To ccast(From a);
 template <> __device__ __forceinline__ double2 ccast<double2, double2>(double2 a) { return a; }
 template <> __device__ __forceinline__ float2 ccast<float2, float2>(float2 a) { return a; }
@@ -193,7 +189,6 @@ struct rr_factors {
   int* amap_buf;
   const int* amap;
   int Fa;
-  std::vector<int> amap_h;  // host copy of the list
 };
 
 // number of problems the solve path runs on, and the problem of slot s
@@ -284,10 +279,8 @@ rr_status launch_solve_lo(rr_factors* f, int k, int adjoint, const void* b, void
 rr_status launch_sweep_cl32(rr_factors* f, int k, int adjoint, const void* b, void* x, void* tmp);
 rr_status launch_sweep_cl64(rr_factors* f, int k, int adjoint, const void* b, void* x, void* tmp);
 double sweep_cl32_us(const rr_factors* f, int k, int adjoint);
-double sweep_cl64_us(const rr_factors* f, int k, int adjoint);
-// true when solves of k columns may take the split tensor-core sweep (both forms
-// run on a subset of the problems, rr_factors::amap)
-bool sweep_tc2_ok(const rr_factors* f, int k);
+// true when a solve of k columns takes the split tensor-core sweep
+bool sweep_tc2_taken(const rr_factors* f, int k, int adjoint);
 
 // dense.cu
 // kind: 0 Gaussian, 1 Rademacher, 2 sparse Rademacher of the given density
@@ -340,7 +333,7 @@ rr_status launch_gain_grad(const OpDev& d, const rr_grid& g, int F, int J, const
 enum {
   PROF_SCHUR = 0, PROF_PANEL = 1, PROF_ROWBLOCK = 2, PROF_UPDATE = 3, PROF_FINALIZE = 4,
   PROF_SWEEP = 5, PROF_RESIDUAL = 6, PROF_GRAM = 7, PROF_RIGHTMUL = 8, PROF_SMALL = 9,
-  PROF_INNER = 10, PROF_OTHER = 11, PROF_N = 12
+  PROF_OTHER = 11, PROF_N = 12  // (10 is unused)
 };
 // While a ProfSuspend lives (graph capture), launches are neither counted
 // nor timed.

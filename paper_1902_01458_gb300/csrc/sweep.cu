@@ -882,7 +882,7 @@ rr_status launch_cc(int k, int kp, const SweepStep& step, const float2* rhs, siz
 // 64 columns.  The three orders of the BF16 x6 split need 6N accumulator columns, so
 // beyond 32 its sweeps take the TF32 split (768 rows, 64 right-hand sides, 16
 // problems: 2.7 ms a solve instead of 20 in the cluster form, no larger an error).
-bool sweep_tc2_ok(const rr_factors* fa, int k) {
+static bool sweep_tc2_ok(const rr_factors* fa, int k) {
   return tc_prec(fa->prec) && k <= 64 && fa->tma_ok;
 }
 
@@ -1021,22 +1021,30 @@ static double sweep_cc_us(const rr_factors* fa, int k) {
          (5.5 + nch * (2.55 * waves + 0.93 * ctas / nsm) + 6.4e-5 * Fa * d.b * k);
 }
 
-// FP64 factors and the FP32 shapes that the tensor-core sweep does not take run the
-// whole-sweep cluster kernels.  Where both serve a shape, the one with the smaller
-// modelled time.
+// FP32 solves that take the column-pair form: where both forms serve a shape, the
+// one with the smaller modelled time.
+static bool sweep_steps_taken(const rr_factors* fa, int k, int adjoint) {
+  const bool simt = fa->prec == RR_FP32_SIMT;
+  if (!simt && !sweep_tc2_ok(fa, k)) return false;
+  return (simt ? sweep_cc_us(fa, k) : sweep_tc2_us(fa, k)) < 1.3 * sweep_cl32_us(fa, k, adjoint);
+}
+
+bool sweep_tc2_taken(const rr_factors* fa, int k, int adjoint) {
+  return tc_prec(fa->prec) && sweep_steps_taken(fa, k, adjoint);
+}
+
+// FP64 factors and FP32 shapes that the column-pair form does not take run the
+// whole-sweep cluster kernels.
 rr_status launch_solve_lo(rr_factors* fa, int k, int adjoint, const void* b, void* x, void* tmp) {
   if (fa->prec == RR_FP64) return launch_sweep_cl64(fa, k, adjoint, b, x, tmp);
-  const bool simt = fa->prec == RR_FP32_SIMT;
-  if (simt || sweep_tc2_ok(fa, k)) {
-    if ((simt ? sweep_cc_us(fa, k) : sweep_tc2_us(fa, k)) < 1.3 * sweep_cl32_us(fa, k, adjoint)) {
-      const float2* in = reinterpret_cast<const float2*>(b);
-      float2 *xo = reinterpret_cast<float2*>(x), *zh = reinterpret_cast<float2*>(tmp);
-      if (k % 2)
-        return adjoint ? solve_tc2<true, float2>(fa, k, in, xo, zh)
-                       : solve_tc2<false, float2>(fa, k, in, xo, zh);
-      return adjoint ? solve_tc2<true, float4>(fa, k, in, xo, zh)
-                     : solve_tc2<false, float4>(fa, k, in, xo, zh);
-    }
+  if (sweep_steps_taken(fa, k, adjoint)) {
+    const float2* in = reinterpret_cast<const float2*>(b);
+    float2 *xo = reinterpret_cast<float2*>(x), *zh = reinterpret_cast<float2*>(tmp);
+    if (k % 2)
+      return adjoint ? solve_tc2<true, float2>(fa, k, in, xo, zh)
+                     : solve_tc2<false, float2>(fa, k, in, xo, zh);
+    return adjoint ? solve_tc2<true, float4>(fa, k, in, xo, zh)
+                   : solve_tc2<false, float4>(fa, k, in, xo, zh);
   }
   return launch_sweep_cl32(fa, k, adjoint, b, x, tmp);
 }
