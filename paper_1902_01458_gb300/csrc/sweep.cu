@@ -59,7 +59,8 @@ __host__ __device__ __forceinline__ int step_col(const SweepStep& s, int half, i
 //   t = h + L_{i,i'}^T o (adjoint outward)
 // for the next column i'.  z goes to zh in the inward sweep, so the outward one's
 // results (x) never overwrite a value a neighbouring tile still needs.
-// (A grid dimension holds 65,535 problems, not two halves of them.)
+// One grid dimension: the others hold 65,535 problems, not two halves of them, and with
+// the halves in a third one an adjoint step of 384 rows took 4 % longer.
 // (part is not __restrict__: the product writes it while this kernel already runs,
 // until grid_wait, so no load of it may go through the read-only path or move up.)
 // Bound: L2 latency (the partials were just written), so the coefficients and
@@ -93,15 +94,16 @@ __device__ __forceinline__ float2 vfma(float a, float2 u, float2 t) {
 
 template <bool TRANS, typename V>
 __global__ void __launch_bounds__(CPL_MAXTHR)
-sweep_couple_kernel(OpView op, SweepStep s, int F, int k, int KS,
+sweep_couple_kernel(OpView op, SweepStep s, int F, int Fa, int k, int KS,
                     const float2* part, const float2* __restrict__ in, float2* x, float2* zh,
                     float2* __restrict__ tbuf, const int* __restrict__ amap) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int VW = sizeof(V) / sizeof(float2);  // columns of a unit
   V* o = reinterpret_cast<V*>(smem_raw);           // [(CPL_Y + 2) q][P]
   const int b = op.b, q = op.q, ny = op.ny, nx = op.nx, P = k / VW;
-  const int half = blockIdx.z, f = active_problem(amap, blockIdx.y);
-  const int y0 = blockIdx.x * CPL_Y, npt = min(CPL_Y, ny - y0);
+  const int nty = (ny + CPL_Y - 1) / CPL_Y, p = blockIdx.x / nty;
+  const int half = p >= Fa, f = active_problem(amap, half ? p - Fa : p);
+  const int y0 = (blockIdx.x - p * nty) * CPL_Y, npt = min(CPL_Y, ny - y0);
   const size_t NK = (size_t)op.n * k, total = (size_t)s.nh * F * b * k;
   const int i = step_col(s, half, nx);
   const bool inw = s.phase == SW_IN, outw = s.phase == SW_OUT;
@@ -971,9 +973,9 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
     const int ch = step.phase == SW_MID ? 2 : step.nh;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg =
-        dependent_launch(dim3((d.ny + CPL_Y - 1) / CPL_Y, Fa, ch), couple_threads(d.q, units), csmem,
-                         st, at, true);
-    RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_couple_kernel<TRANS, V>, view(d), step, F, k, KS,
+        dependent_launch(dim3((d.ny + CPL_Y - 1) / CPL_Y * Fa * ch), couple_threads(d.q, units),
+                         csmem, st, at, true);
+    RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_couple_kernel<TRANS, V>, view(d), step, F, Fa, k, KS,
                                reinterpret_cast<const float2*>(fa->Pbuf), in, x, zh, tb,
                                (const int*)fa->amap));
     prof_end(PROF_SWEEP, st);
@@ -985,24 +987,21 @@ rr_status solve_tc2(rr_factors* fa, int k, const float2* in, float2* x, float2* 
 
 }  // namespace
 
-// Modelled microseconds of a solve in the tensor-core form, per pair of columns: the
-// launches, the busiest CTA's chunks and items, and the coupling.  Fitted to solves
-// of 16 columns of 48 to 1023 rows with 1 to 64 right-hand sides and 1 to 512
-// problems (992, within 15 % for nine in ten); the cluster form took 1.3 times its
-// model on the same ones.  Of the two forms the one taken is within 5 % of the faster
-// in all but 4 % of them.  Measured, ms of a whole unrefined solve, tensor-core and
-// cluster form: 48 rows, 16 right-hand sides, 128 problems 0.48 and 0.37; 96 rows, 32,
-// 128 problems 1.09 and 1.50; 192 rows, 8, 32 problems 0.61 and 0.34; 387 rows, 32,
-// 64 problems 2.8 and 7.6; 768 rows, 32, 1 and 16 problems 0.40 and 1.6 instead of
-// 1.13 and 7.1.
+// Modelled microseconds of a solve in the tensor-core form, less what the cluster form
+// also takes: per pair of columns the launches, and the busiest CTA's chunks and
+// items.  Fitted together with form_step_us (sweep_cl.cuh) to 1467 shapes, forward and
+// adjoint: the form taken is the slower one by more than 5 % in 2 % of them.  Measured,
+// ms of a whole unrefined solve of 16 columns, tensor-core and cluster form: 48 rows, 16
+// right-hand sides, 128 problems 0.48 and 0.37; 96 rows, 32, 128 problems 1.09 and
+// 1.50; 192 rows, 8, 32 problems 0.61 and 0.34; 387 rows, 32, 64 problems 2.8 and
+// 7.6; 768 rows, 32, 1 and 16 problems 0.40 and 1.6 instead of 1.13 and 7.1.
 static double sweep_tc2_us(const rr_factors* fa, int k) {
   const OpDev& d = fa->op->d;
   const int nrt = (d.b + TC_RT - 1) / TC_RT, nch = (d.b + TC2_KC - 1) / TC2_KC;
   const int nsm = num_sms(d.device), KS = split_count(fa, k, 2, nrt, nch, nsm);
   const double items = std::ceil(2.0 * nrt * active_count(fa) * KS / nsm);  // of a CTA
   const int cpp = (nch + KS - 1) / KS;
-  return (d.nx + 1.0) *
-         (5.2 + items * (1.25 + 0.6 * cpp) + 6.4e-5 * active_count(fa) * d.b * k);
+  return (d.nx + 1.0) * (4.3 + items * (1.34 + 0.67 * cpp));
 }
 
 // The same for the product on the CUDA cores (RR_FP32_SIMT): the chunks' latency per
@@ -1017,8 +1016,7 @@ static double sweep_cc_us(const rr_factors* fa, int k) {
   const int nch = (d.b + CC_KC - 1) / CC_KC, Fa = active_count(fa), nsm = num_sms(d.device);
   const double ctas = 2.0 * Fa * ((d.b * kp + CC_RT - 1) / CC_RT);
   const double waves = std::ceil(ctas / (nsm * (kp <= 8 ? 1.0 : kp == 16 ? 2.0 : 3.0)));
-  return (d.nx + 1.0) *
-         (5.5 + nch * (2.55 * waves + 0.93 * ctas / nsm) + 6.4e-5 * Fa * d.b * k);
+  return (d.nx + 1.0) * (4.5 + nch * (2.8 * waves + 0.96 * ctas / nsm));
 }
 
 // FP32 solves that take the column-pair form: where both forms serve a shape, the
@@ -1026,7 +1024,7 @@ static double sweep_cc_us(const rr_factors* fa, int k) {
 static bool sweep_steps_taken(const rr_factors* fa, int k, int adjoint) {
   const bool simt = fa->prec == RR_FP32_SIMT;
   if (!simt && !sweep_tc2_ok(fa, k)) return false;
-  return (simt ? sweep_cc_us(fa, k) : sweep_tc2_us(fa, k)) < 1.3 * sweep_cl32_us(fa, k, adjoint);
+  return (simt ? sweep_cc_us(fa, k) : sweep_tc2_us(fa, k)) < sweep_cl32_us(fa, k, adjoint);
 }
 
 bool sweep_tc2_taken(const rr_factors* fa, int k, int adjoint) {

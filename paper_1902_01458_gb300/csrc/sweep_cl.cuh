@@ -90,8 +90,10 @@ template <typename T, int CPL, int RPL>
 constexpr int max_warps() { return sizeof(T) == 4 && CPL * RPL >= 20 ? 8 : MAXW; }
 
 // LR = 32 / LC lanes over rows x LC over columns; a lane holds RPL rows (LR
-// apart) x CPL adjacent columns
-template <typename T, bool TRANS, int LC, int CPL, int RPL>
+// apart) x CPL adjacent columns.  PITCHED: G's rows are a.ldg apart, else b.  (The forward
+// kernels are pitched always: up to a third faster at 384 and 768 rows than with b; the
+// adjoint ones were 2 to 5 % slower at 192 rows.)
+template <typename T, bool TRANS, int LC, int CPL, int RPL, bool PITCHED>
 __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_kernel(Args<T> a) {
   using C = C_t<T>;
   constexpr int CS = sizeof(C);
@@ -119,7 +121,7 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
   unsigned char* ring = reinterpret_cast<unsigned char*>(ob + (size_t)(rmax + 2 * q) * NC) +
                         (size_t)warp * 2 * SB;
   const C* Gf = a.G + (size_t)f * a.gstride;
-  const int ldg = a.ldg;
+  const int ldg = PITCHED ? a.ldg : b;
   const size_t bb = (size_t)b * ldg, NK = (size_t)op.n * a.k;
   const C* in = a.in + (size_t)f * NK;
   C* x = a.x + (size_t)f * NK;
@@ -454,7 +456,8 @@ __global__ void __launch_bounds__(max_warps<T, CPL, RPL>() * 32, 1) sweep_cl_ker
 // ------------------------------------------------------------------- plan
 struct Plan {
   int kc, CL, npt, W, rpl;
-  double us;  // modelled time of the solve
+  double us;       // modelled time of the solve
+  double form_us;  // the same by form_step_us
 };
 
 // Microseconds of a column step: the chain of a step plus a part that grows
@@ -470,6 +473,15 @@ inline double step_us(bool dp, int b, int rpl, int cpl) {
   return 1.6 + 1e-3 * b * (cpl == 2 ? two[rpl] : four[rpl]);
 }
 
+// The FP32 step beside the tensor-core form's (sweep.cu), for the choice between the
+// two: fitted to unrefined solves of 96 columns of 48 to 768 rows, 1 to 64 right-hand
+// sides and 1 to 128 problems in both forms.  Odd blocks take 8-byte copies.
+inline double form_step_us(int b, int rpl, int cpl) {
+  const double two[10] = {0, 9.7, 10.2, 13.4, 17.4, 25.6, 27.6, 42.7, 52.6, 70.2};
+  const double four[10] = {0, 8.8, 15.6, 18.6, 29.4, 35.9, 37.0, 43.6, 44, 70};
+  return 0.94 + 1e-3 * b * (cpl == 2 ? two[rpl] : four[rpl]) * (b % 2 ? 1.33 : 1.0);
+}
+
 // Column groups and cluster size with the least modelled time: waves of
 // clusters x steps.  us < 0 when the block does not fit.
 template <typename T>
@@ -477,7 +489,7 @@ Plan make_plan(const OpDev& d, int Fa, int k, int trans) {
   constexpr bool DP = sizeof(T) == 8;
   constexpr int KC = 64 / sizeof(C_t<T>);
   const int kcs[3] = {DP ? 1 : 4, DP ? 2 : 8, 4};
-  Plan best{0, 0, 0, 0, 0, -1.0};
+  Plan best{0, 0, 0, 0, 0, -1.0, -1.0};
   const int lr = DP ? 32 : 16, rplmax = DP ? 5 : 9;
   for (int ki = 0; ki < (DP ? 3 : 2); ++ki) {
     const int kc = kcs[ki], ng = (k + kc - 1) / kc, cpl = DP ? kc : kc / 2;
@@ -503,15 +515,19 @@ Plan make_plan(const OpDev& d, int Fa, int k, int trans) {
       const int slots = cluster_slots(d.device, CL);
       const int waves = (int)((2L * Fa * ng + slots - 1) / slots);
       const double us = waves * (d.nx + 1.0) * step_us(DP, d.b, rpl, cpl);
-      if (best.us < 0 || us < best.us) best = Plan{kc, CL, npt, W, rpl, us};
+      if (best.us < 0 || us < best.us)
+        best = Plan{kc, CL, npt, W, rpl, us,
+                    DP ? us : waves * (d.nx + 1.0) * form_step_us(d.b, rpl, cpl)};
     }
   }
   return best;
 }
 
-template <typename T, bool TRANS, int LC, int CPL, int RPL>
+template <typename T, bool TRANS, int LC, int CPL, int RPL, bool PITCHED = !TRANS>
 rr_status launch(const Args<T>& a, int clusters, size_t smem, int W, cudaStream_t st) {
-  RR_TRY((smem_opt_in<sweep_cl_kernel<T, TRANS, LC, CPL, RPL>>(SMEM_CAP)));
+  if constexpr (sizeof(T) == 4 && !PITCHED)
+    if (a.ldg != a.op.b) return launch<T, TRANS, LC, CPL, RPL, true>(a, clusters, smem, W, st);
+  RR_TRY((smem_opt_in<sweep_cl_kernel<T, TRANS, LC, CPL, RPL, PITCHED>>(SMEM_CAP)));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.CL * clusters), 1, 1);
   cfg.blockDim = dim3((unsigned)(32 * W), 1, 1);
@@ -524,7 +540,7 @@ rr_status launch(const Args<T>& a, int clusters, size_t smem, int W, cudaStream_
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_cl_kernel<T, TRANS, LC, CPL, RPL>, a));
+  RR_CUDA(cudaLaunchKernelEx(&cfg, sweep_cl_kernel<T, TRANS, LC, CPL, RPL, PITCHED>, a));
   return RR_OK;
 }
 

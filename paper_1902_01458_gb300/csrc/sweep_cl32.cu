@@ -2,7 +2,7 @@
 #include "sweep_cl.cuh"
 
 double sweep_cl32_us(const rr_factors* fa, int k, int adjoint) {
-  return sweepcl::make_plan<float>(fa->op->d, active_count(fa), k, adjoint).us;
+  return sweepcl::make_plan<float>(fa->op->d, active_count(fa), k, adjoint).form_us;
 }
 
 rr_status launch_sweep_cl32(rr_factors* fa, int k, int adjoint, const void* in, void* x, void* h) {

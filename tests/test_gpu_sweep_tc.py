@@ -118,7 +118,7 @@ def test_small_batches_stay_in_the_cluster_form(ny, k, F):
 
 @pytest.mark.parametrize("kind,ny,k,F,periodic", [("ns", 128, 32, 48, False), ("ns", 129, 16, 64, True),
                                                   ("ad", 257, 63, 32, False), ("kz", 33, 64, 64, True),
-                                                  ("ns", 256, 5, 64, False)])
+                                                  ("ns", 256, 16, 48, False)])
 @pytest.mark.parametrize("adjoint", [False, True])
 def test_cuda_core_product(kind, ny, k, F, periodic, adjoint):
     """Large batches of FP32 factors without tensor cores take the same form."""
