@@ -55,15 +55,16 @@ typedef enum {
 /* Arithmetic of the block factorisation and the block sweeps.  FP64 runs
  * everything in complex double.  FP32 stores the factors in complex float,
  * runs the factorisation's rank-128 updates and the sweep products of large
- * blocks and batches on the tensor cores (tcgen05 kind::tf32 with each operand split into a TF32 part
- * and its remainder, hi.hi + hi.lo + lo.hi: FP32-level products, FP32
- * accumulation; the pivoted 128-column slabs and the sweeps of small blocks
- * run in FP32 on the CUDA cores) and wins accuracy back by
- * iterative refinement against an FP64 residual.
+ * blocks and batches on the tensor cores (tcgen05 kind::tf32 with each operand
+ * split into a TF32 part and its remainder, hi.hi + hi.lo + lo.hi: FP32-level
+ * products, FP32 accumulation; the pivoted 128-column slabs and the sweeps of
+ * small blocks and batches run in FP32 on the CUDA cores) and wins accuracy back
+ * by iterative refinement against an FP64 residual.
  * FP32_BF16X3 and FP32_BF16X6 are the same with the operands split into
  * BF16 pieces on tcgen05 kind::f16: two pieces and three products (about 16
  * bits of each product) or three pieces and six products (hi.hi, hi.mid,
- * mid.hi, hi.lo, mid.mid, lo.hi: FP32-level).  FP32_SIMT is FP32 with every
+ * mid.hi, hi.lo, mid.mid, lo.hi: FP32-level; sweeps of more than 32 columns
+ * take the TF32 split).  FP32_SIMT is FP32 with every
  * product on the FP32 CUDA cores.  QR, SVD, norms and the refinement
  * residual stay FP64 in every mode. */
 typedef enum {
@@ -437,12 +438,12 @@ rr_status rr_profile_read(int cls, double* ms, long long* launches);
 
 /* Diagnostics of the bounded device-side waits (no counterpart in the paper;
  * for tests of the RR_ERR_TIMEOUT path).  Every mbarrier wait of the
- * tensor-core kernels polls at most `tries` times (0 restores the default,
- * 2^22) before the kernel records a timeout, drains what it has in flight,
- * frees its tensor memory and returns; the call that launched it then
+ * tensor-core and cluster kernels polls at most `tries` times (0 restores the
+ * default, 2^22) before the kernel records a timeout, drains what it has in
+ * flight, frees its tensor memory and returns; the call that launched it then
  * returns RR_ERR_TIMEOUT.  stall_launches > 0 makes that many of the next
- * tensor-core sweep launches stall on purpose: the first CTA of
- * each issues no copy and no MMA, so that CTA's first wait runs out with
+ * sweep launches of either form stall on purpose: the first CTA of each issues
+ * no copy and no MMA, or sends nothing, so that the waits for it run out with
  * nothing in flight.  Process-wide, not thread-safe; for tests only. */
 rr_status rr_debug_waits(unsigned tries, int stall_launches);
 

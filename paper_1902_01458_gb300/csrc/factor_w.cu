@@ -5,8 +5,8 @@
 // bulk of the work is a rank-128 complex update on the tensor cores.
 //
 // Pivoting is implicit: rows are never moved.  Column j is eliminated with
-// the pivot row p_j (the largest |.| among rows not yet pivoted, lowest row on
-// ties) by the elementary transformation E_j (row p_j scaled by 1/m_pj,
+// the pivot row p_j (the largest |.|^2, to 18 bits, among rows not yet pivoted;
+// ties: see gjw_slab_kernel) by the elementary transformation E_j (row p_j scaled by 1/m_pj,
 // m_pj times it subtracted from every other row; column j then holds E_j's
 // column p_j, the in-place inverse).  After all b columns the work matrix is
 // M = Q^T S^{-1} Q^T with (Q x)_j = x_{p_j}, so S^{-1}[j, p_m] = M[p_j, m].

@@ -272,10 +272,11 @@ bool factor_wide_ok(const rr_factors* f);
 rr_status launch_factor_wide(rr_factors* f);
 
 // sweep.cu: x = A^{-1} b or A^{-H} b with the factors in precision T.
-// b and x are [F][N][k] in the factor precision; tmp same size (adjoint only).
+// b and x are [F][N][k] in the factor precision; tmp, scratch of the same size (b may
+// be read 8 bytes past its end: both lie inside the workspace).
 rr_status launch_solve_lo(rr_factors* f, int k, int adjoint, const void* b, void* x, void* tmp);
-// sweep_cl32.cu, sweep_cl64.cu: the same in one launch per solve, and its
-// modelled time in microseconds
+// sweep_cl32.cu, sweep_cl64.cu: the same in two launches per solve; the FP32 one's
+// modelled time in microseconds, to compare with the other form's
 rr_status launch_sweep_cl32(rr_factors* f, int k, int adjoint, const void* b, void* x, void* tmp);
 rr_status launch_sweep_cl64(rr_factors* f, int k, int adjoint, const void* b, void* x, void* tmp);
 double sweep_cl32_us(const rr_factors* f, int k, int adjoint);

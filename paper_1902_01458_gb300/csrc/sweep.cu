@@ -2,10 +2,10 @@
 // Algorithm 1 (Sec. II.B, second, fourth and sixth steps), all reusing the
 // one factorisation of s I - L (Sec. III.A).
 //
-// With G_i = S_i^{-1} and C_i = -L_{i,i+1} (at most 3q entries per row):
-// and the factorisation run from both ends to the middle column m (factor.cu), a
-// solve goes inwards in both halves, through the middle, and outwards (written
-// for the left half, i < m; the right one is the mirror image):
+// With G_i = S_i^{-1}, C_i = -L_{i,i+1} (at most 3q entries per row) and the
+// factorisation run from both ends to the middle column m (factor.cu), a solve goes
+// inwards in both halves, through the middle, and outwards (written for the left
+// half, i < m; the right one is the mirror image):
 // Normal solve (s I - L) y = f:
 //   inward   z_0 = G_0 f_0,      z_i = G_i (f_i + L_{i,i-1} z_{i-1})
 //   middle   y_m = G_m (f_m + L_{m,m-1} z_{m-1} + L_{m,m+1} z_{m+1})
@@ -17,11 +17,11 @@
 // The chain is nx + 1 products instead of the 2 nx - 1 of a sweep from one end.
 // Only G_i is stored.  Two forms: two launches per solve with a cluster of CTAs
 // per problem and half (sweep_cl.cuh), or, for large blocks and batches, two
-// launches per pair of streamwise columns for all problems of the batch: the dense (b x b) x
-// (b x k) product on the tensor cores, its contraction split over CTAs
+// launches per pair of streamwise columns for all problems of the batch: the dense
+// (b x b) x (b x k) product on the tensor cores, its contraction split over CTAs
 // (sweep_tc2_kernel), or for RR_FP32_SIMT on the CUDA cores (sweep_cc_kernel), and
-// the sum of the partial blocks with the sparse
-// coupling that forms the next column's right-hand side (sweep_couple_kernel).
+// the sum of the partial blocks with the sparse coupling that forms the next
+// column's right-hand side (sweep_couple_kernel).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
