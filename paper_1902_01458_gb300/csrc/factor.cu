@@ -388,7 +388,10 @@ __global__ void gjp_gather_kernel(int b, int k0, int nbk, int nh, const C_t<T>* 
 
 // (Summing onto the matrix entries instead rounds them sixteen times a panel: the
 // unrefined residual of a 384-row FP64 adjoint solve was 6.3e-14 instead of 3.0e-14,
-// of a 768-row FP32 one 8.6e-5 instead of 2.3e-5, at the same speed.)
+// of a 768-row FP32 one 8.6e-5 instead of 2.3e-5.  In FP32 the sums go to the entries by
+// reductions in L2, no registers or latency for the old values: 960 rows, eight problems,
+// 16 columns 43.0 ms a factorisation; 55.9 with them requested ahead, 73 with them
+// read at the end.)
 // The rank-16 update on TR x TR tiles (16 x 16 threads) of the columns outside
 // [k0, k0 + nbk) and [n0, n1).  FP64 is bound by its pipe, so small tiles fill
 // the SMs; FP32 by shared memory, so a thread holds 4 x 4 outputs.
@@ -411,21 +414,11 @@ gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, int nh, C_t<T>* __rest
   auto col_live = [&](int c) {
     return c < b && !(c >= k0 && c < k0 + nbk) && !(c >= n0 && c < n1);
   };
-  // the old values are requested first and added last: the sixteen products are
-  // summed on their own, one rounding a panel against the matrix entry
-  C acc[PT][PT], old[PT][PT];
+  C acc[PT][PT];
 #pragma unroll
-  for (int a = 0; a < PT; ++a) {
-    const int r = r0 + ty + 16 * a;
-    const int rp = r < b ? rowpiv[r] : -1;
-    const bool keep = r < b && !(rp >= k0 && rp < k0 + nbk);
+  for (int a = 0; a < PT; ++a)
 #pragma unroll
-    for (int d = 0; d < PT; ++d) {
-      const int c = c0 + tx + 16 * d;
-      acc[a][d] = czero<C>();
-      old[a][d] = keep && col_live(c) ? M[(size_t)r * b + c] : czero<C>();
-    }
-  }
+    for (int d = 0; d < PT; ++d) acc[a][d] = czero<C>();
   for (int e = tid; e < TR * NB; e += 256) {
     const int rr = e / NB, m = e - rr * NB, r = r0 + rr;
     As[rr][m] = (r < b && m < nbk) ? M[(size_t)r * b + k0 + m] : czero<C>();
@@ -447,14 +440,23 @@ gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, int nh, C_t<T>* __rest
 #pragma unroll
       for (int d = 0; d < PT; ++d) acc[a][d] = cfma(av[a], bv[d], acc[a][d]);
   }
+  // one rounding a panel against the matrix entry: added where it lies in FP32, read
+  // back in FP64
 #pragma unroll
   for (int a = 0; a < PT; ++a) {
-    const int r = r0 + ty + 16 * a;
+    const int r = r0 + ty + 16 * a, rp = r < b ? rowpiv[r] : -1;
     if (r >= b) continue;
+    const bool keep = !(rp >= k0 && rp < k0 + nbk);
 #pragma unroll
     for (int d = 0; d < PT; ++d) {
       const int c = c0 + tx + 16 * d;
-      if (col_live(c)) M[(size_t)r * b + c] = cadd(old[a][d], acc[a][d]);
+      if (!col_live(c)) continue;
+      C* p = &M[(size_t)r * b + c];
+      if (!keep) *p = acc[a][d];
+      else if constexpr (sizeof(T) == 8) *p = cadd(*p, acc[a][d]);
+      else asm volatile("red.global.add.v2.f32 [%0], {%1, %2};\n" ::"l"(p), "f"(acc[a][d].x),
+                        "f"(acc[a][d].y)
+                        : "memory");
     }
   }
 }
