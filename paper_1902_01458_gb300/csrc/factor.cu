@@ -388,13 +388,21 @@ __global__ void gjp_gather_kernel(int b, int k0, int nbk, int nh, const C_t<T>* 
 
 // (Summing onto the matrix entries instead rounds them sixteen times a panel: the
 // unrefined residual of a 384-row FP64 adjoint solve was 6.3e-14 instead of 3.0e-14,
-// of a 768-row FP32 one 8.6e-5 instead of 2.3e-5.  In FP32 the sums go to the entries by
-// reductions in L2, no registers or latency for the old values: 960 rows, eight problems,
-// 16 columns 43.0 ms a factorisation; 55.9 with them requested ahead, 73 with them
-// read at the end.)
+// of a 768-row FP32 one 8.6e-5 instead of 2.3e-5.  The sums go to the entries by
+// reductions in L2, without registers, latency or FP64 operations for the old values.
+// FP32, 960 rows, eight problems, 16 columns: 43.0 ms a factorisation; 55.9 with them
+// requested ahead, 73 with them read at the end.  FP64, 192 rows, 64 problems: 64.2, and
+// 65.8 with either.)
 // The rank-16 update on TR x TR tiles (16 x 16 threads) of the columns outside
 // [k0, k0 + nbk) and [n0, n1).  FP64 is bound by its pipe, so small tiles fill
 // the SMs; FP32 by shared memory, so a thread holds 4 x 4 outputs.
+__device__ __forceinline__ void red_add(float2* p, float2 v) {
+  asm volatile("red.global.add.v2.f32 [%0], {%1, %2};\n" ::"l"(p), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void red_add(double2* p, double2 v) {
+  asm volatile("red.global.add.f64 [%0], %1;\n" ::"l"(&p->x), "d"(v.x) : "memory");
+  asm volatile("red.global.add.f64 [%0], %1;\n" ::"l"(&p->y), "d"(v.y) : "memory");
+}
 template <typename T> struct UpdCfg { static constexpr int TR = sizeof(T) == 8 ? 32 : 64; };
 template <typename T>
 __global__ void __launch_bounds__(256)
@@ -440,8 +448,7 @@ gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, int nh, C_t<T>* __rest
 #pragma unroll
       for (int d = 0; d < PT; ++d) acc[a][d] = cfma(av[a], bv[d], acc[a][d]);
   }
-  // one rounding a panel against the matrix entry: added where it lies in FP32, read
-  // back in FP64
+  // (an entry has one writer a launch: the order of the sums is fixed)
 #pragma unroll
   for (int a = 0; a < PT; ++a) {
     const int r = r0 + ty + 16 * a, rp = r < b ? rowpiv[r] : -1;
@@ -452,11 +459,8 @@ gjp_update_kernel(int b, int k0, int nbk, int n0, int n1, int nh, C_t<T>* __rest
       const int c = c0 + tx + 16 * d;
       if (!col_live(c)) continue;
       C* p = &M[(size_t)r * b + c];
-      if (!keep) *p = acc[a][d];
-      else if constexpr (sizeof(T) == 8) *p = cadd(*p, acc[a][d]);
-      else asm volatile("red.global.add.v2.f32 [%0], {%1, %2};\n" ::"l"(p), "f"(acc[a][d].x),
-                        "f"(acc[a][d].y)
-                        : "memory");
+      if (keep) red_add(p, acc[a][d]);
+      else *p = acc[a][d];
     }
   }
 }
